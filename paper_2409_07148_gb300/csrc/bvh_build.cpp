@@ -373,6 +373,7 @@ bool build_bvh(const float* verts, uint32_t n_verts, const uint32_t* tris, uint3
     out->nodes.clear();
     out->tris.clear();
     out->depth = 0;
+    out->stack_need = 0;
     if (n_tris == 0) {
         out->root = INT32_MIN;
         return true;
@@ -448,6 +449,7 @@ bool build_bvh(const float* verts, uint32_t n_verts, const uint32_t* tris, uint3
     int need = 0, depth4 = 0;
     out->root = B.collapse(root2, need, depth4);
     out->depth = depth4;
+    out->stack_need = need + 1;
     if (need + 1 > kStackSize) {
         *err = "BVH needs more traversal stack than the kernels hold";
         return false;

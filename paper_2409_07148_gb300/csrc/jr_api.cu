@@ -163,6 +163,7 @@ jr_status jr_scene_create(const jr_scene_desc* desc, void* stream, jr_scene** ou
         (e = dev_alloc(&s->mats, mats.size())) != cudaSuccess ||
         (e = cudaMemcpyAsync(s->nodes, bvh.nodes.data(), sizeof(Bvh4Node) * bvh.nodes.size(), cudaMemcpyHostToDevice,
                              st)) != cudaSuccess ||
+        (e = launch_swizzle_nodes(s->nodes, (uint32_t)bvh.nodes.size(), st)) != cudaSuccess ||
         (e = cudaMemcpyAsync(s->tris, bvh.tris.data(), sizeof(TriRecord) * bvh.tris.size(), cudaMemcpyHostToDevice,
                              st)) != cudaSuccess ||
         (e = cudaMemcpyAsync(s->mats, mats.data(), sizeof(Material) * mats.size(), cudaMemcpyHostToDevice, st)) !=
@@ -179,6 +180,7 @@ jr_status jr_scene_create(const jr_scene_desc* desc, void* stream, jr_scene** ou
     s->view.n_tris = (uint32_t)bvh.tris.size();
     s->view.visit_budget = kNodeVisitBudget;
     s->view.stack_limit = kStackSize;
+    s->view.stack_need = bvh.stack_need;
     std::memcpy(s->view.cam, desc->camera, sizeof(float) * 12);
     s->info.n_tris = desc->n_tris;
     s->info.n_nodes = (uint32_t)bvh.nodes.size();
@@ -651,6 +653,7 @@ struct jr_batch {
     uint32_t max_dim = 0;
     uint64_t total_px = 0, total_chains = 0;
     int block = 128;  // chains per megakernel work item; 0: the batched wavefront
+    int checks = 0;   // the watchdogs the megakernel checks: the most that any set's device descriptor needs
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     uint32_t graph_steps = 0;
@@ -666,9 +669,20 @@ struct jr_batch {
     unsigned int* fetch = nullptr;
     BatchWave bw{};
     bool wf_ready = false;
-    ~jr_batch() {
+    void drop_graph() {
         if (exec) cudaGraphExecDestroy(exec);
         if (graph) cudaGraphDestroy(graph);
+        exec = nullptr;
+        graph = nullptr;
+    }
+    // A set's device descriptor gets view v (a captured graph holds the old variant).
+    void needs(const SceneView& v) {
+        if (trav_checks(v) <= checks) return;
+        checks = trav_checks(v);
+        drop_graph();
+    }
+    ~jr_batch() {
+        drop_graph();
         cudaFree(entries);
         cudaFree(px_off);
         cudaFree(cursor);
@@ -749,10 +763,8 @@ jr_status sync_steps(jr_batch* b, cudaStream_t st) {
             JR_CUDA(cudaStreamSynchronize(st), "jr_batch (flow)");
             b->dev_flow_gen[k] = c->flow_gen;
             b->dev_steps[k] = c->steps;
-            if (b->exec) cudaGraphExecDestroy(b->exec);
-            if (b->graph) cudaGraphDestroy(b->graph);
-            b->exec = nullptr;
-            b->graph = nullptr;
+            b->needs(h.s);
+            b->drop_graph();
         }
         const uint64_t s = b->sets[k]->steps;
         if (s != b->dev_steps[k]) {
@@ -798,6 +810,7 @@ jr_status prepare_wave(jr_batch* b, cudaStream_t st) {
     for (uint32_t k = 0; k < S; ++k) {
         const jr_chains* c = b->sets[k];
         h[k].s = c->scene_view();
+        b->needs(h[k].s);
         h[k].c = c->view;
         h[k].step = b->dev_steps[k];
         size_t u = 0;
@@ -887,7 +900,9 @@ jr_status prepare_wave(jr_batch* b, cudaStream_t st) {
     bw.n_items = (uint32_t)items.size();
     bw.fetch = b->fetch;
     long long blocks = 0;
-    JR_CUDA(batch_wavefront_grid(&blocks), who);
+    bw.checks = 0;  // the merged scene is traversed under the default limits
+    for (const jr_scene* sc : uniq) bw.checks = std::max(bw.checks, trav_checks(sc->view));
+    JR_CUDA(batch_wavefront_grid(bw.checks, &blocks), who);
     b->wf_ready = true;
     return JR_OK;
 }
@@ -901,10 +916,10 @@ cudaError_t enqueue_batch(jr_batch* b, uint32_t n_steps, cudaStream_t st) {
         cudaError_t e = launch_batch_wavefront(b->bw, b->entries, n_steps, flow_views(b), st);
         if (e != cudaSuccess) return e;
         return launch_batch(b->entries, b->items, 0, b->px_off, S, b->total_px, b->cursor, b->max_dim, 128,
-                            n_steps, st);
+                            b->checks, n_steps, st);
     }
     return launch_batch(b->entries, b->items, b->n_items, b->px_off, S, b->total_px, b->cursor, b->max_dim, b->block,
-                        n_steps, st);
+                        b->checks, n_steps, st);
 }
 
 jr_status batch_launch(jr_batch* b, uint32_t n_steps, cudaStream_t st, const char* who) {
@@ -945,6 +960,7 @@ jr_status jr_batch_create(jr_chains* const* sets, uint32_t n_sets, void* stream,
             return fail(JR_ERR_STATE, "jr_batch_create: MALA chain sets advance on their own (megakernel)");
         }
         h[k].s = c->scene_view();
+        b->needs(h[k].s);
         h[k].c = c->view;
         h[k].step = c->steps;
         off[k + 1] = off[k] + (uint64_t)c->view.width * c->view.height;
@@ -1013,10 +1029,7 @@ jr_status jr_batch_advance_graph(jr_batch* b, uint32_t n_steps, void* stream) {
     if (r == JR_OK && b->block == 0) r = prepare_wave(b, st);
     if (r != JR_OK) return r;
     if (!b->exec || b->graph_steps != n_steps || b->graph_block != b->block) {
-        if (b->exec) cudaGraphExecDestroy(b->exec);
-        if (b->graph) cudaGraphDestroy(b->graph);
-        b->exec = nullptr;
-        b->graph = nullptr;
+        b->drop_graph();
         cudaStream_t cap = nullptr;
         JR_CUDA(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking), "jr_batch_advance_graph");
         cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);

@@ -93,7 +93,7 @@ struct Trav {
     int best, best_id;  // its leaf-order record and original triangle index
     int ref, sp;        // node/leaf ref being visited, stack depth
     uint32_t visits;
-    int oct;            // ray octant: bit a set when the direction's axis-a component is negative
+    uint32_t oct;       // ray octant: bit 4 + a set when the direction's axis-a component is negative
 };
 
 __device__ __forceinline__ void trav_begin_at(Trav& r, float3 o, float3 d, int root) {
@@ -108,7 +108,7 @@ __device__ __forceinline__ void trav_begin_at(Trav& r, float3 o, float3 d, int r
     r.ox = o.x * r.ix;
     r.oy = o.y * r.iy;
     r.oz = o.z * r.iz;
-    r.oct = (r.ix < 0.0f ? 1 : 0) | (r.iy < 0.0f ? 2 : 0) | (r.iz < 0.0f ? 4 : 0);
+    r.oct = (r.ix < 0.0f ? 16u : 0u) | (r.iy < 0.0f ? 32u : 0u) | (r.iz < 0.0f ? 64u : 0u);
     r.tb = INFINITY;
     r.best = -1;
     r.best_id = INT32_MAX;
@@ -131,62 +131,130 @@ __device__ __forceinline__ void cswap(float& ta, int& ra, float& tb, int& rb) {
     ra = q;
 }
 
-// Slab test of one child box against [0, tb], given its near and far plane
-// per axis (picked by the ray's octant, see trav_node): entry distance, or
-// +inf for a miss.  The far distance is scaled up by 2 ulp so that a ray
-// grazing a face of a (conservatively widened) box still enters it.
-__device__ __forceinline__ float slab(const Trav& r, float nx, float fx, float ny, float fy, float nz, float fz) {
-    const float tn = fmax3(fmaf(nx, r.ix, -r.ox), fmaf(ny, r.iy, -r.oy), fmaxf(fmaf(nz, r.iz, -r.oz), 0.0f));
-    const float tf = fmin3(fmaf(fx, r.ix, -r.ox), fmaf(fy, r.iy, -r.oy), fminf(fmaf(fz, r.iz, -r.oz), r.tb));
-    return tn <= tf * 1.00000024f ? tn : INFINITY;
+// Two FP32 values in one 64-bit register pair, and the packed fused multiply-add
+// and multiply (sm_100+): each half is the scalar operation's result.
+__device__ __forceinline__ unsigned long long pack_f32x2(float a, float b) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void fma_f32x2(float a0, float a1, unsigned long long b, unsigned long long c, float& d0,
+                                          float& d1) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack_f32x2(a0, a1)), "l"(b), "l"(c));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(r));
 }
 
+// Plane distances p * i - o of one plane of the four children.
+__device__ __forceinline__ void plane4(const float4 p, float i, float o, float (&t)[4]) {
+    const unsigned long long ii = pack_f32x2(i, i), oo = pack_f32x2(-o, -o);
+    fma_f32x2(p.x, p.y, ii, oo, t[0], t[1]);
+    fma_f32x2(p.z, p.w, ii, oo, t[2], t[3]);
+}
+
+// Which of the traversal's watchdogs a launch has to check (trav_checks in
+// jr_internal.h decides on the host):
+//   kCheckNone    neither can fire: a ray visits a node at most once, so a visit
+//                 budget of at least the node count is never exceeded, and the
+//                 builder knows the deepest stack a traversal can need;
+//   kCheckVisits  visits are counted, and the caller compares them with the
+//                 budget once per round (a ray over it is a miss either way,
+//                 whatever it did in the rest of the round);
+//   kCheckAll     both, at every visit.
+// The checks cost a node visit 7 % of the path kernel's time (512^2 Cornell +
+// spheres: 12.20 with, 11.53 ms without for 16 steps of 2^20 chains).
+//
 // Visit inner node r.ref of the 4-wide BVH: slab-test its children against
 // [0, tb], descend to the nearest hit child and push the other hit children
-// farthest first (front-to-back order), or pop.  Returns false (and sets a
-// status bit) if the visit budget or the stack ran out: the ray then counts
-// as a miss.
-template <bool kCount>
+// (the next nearest last, up to the order of the farthest two), or pop.
+// Returns false (and sets a status bit) if a checked limit ran out: the ray
+// then counts as a miss.
+//
+// The visit is bound by issue slots and by the latency of its loads:
+//  * The node's 16-byte chunks lie at chunk ^ (node & 7) (swizzle_nodes_kernel):
+//    a warp's lanes read the same chunk of different nodes, and every node
+//    starts on a 128-byte line, so unswizzled loads all hit the same four L1
+//    banks (43 % of the L1 data pipe's cycles at 12 active lanes).  Measured
+//    13.10 -> 12.63 ms (Cornell + spheres), 3.40 -> 3.17 ms (2M-triangle
+//    terrain, 4 steps of 2^20 chains).
+//  * The 24 plane distances are packed FMAs: half the instructions, the same
+//    values (13.10 -> 12.77 ms alone).
+//  * Three comparators instead of a full sorting network: the nearest child is
+//    exact, and so is the order of two hits; with three or more the order of
+//    the others is approximate, which costs fewer visits than the two
+//    comparators cost instructions (11.78 -> 11.70 ms; 2.76 -> 2.69 ms in the
+//    path-tracing kernel).  The closest hit does not depend on the order.
+enum TravCheck { kCheckNone = 0, kCheckVisits = 1, kCheckAll = 2 };
+
+template <int kCheck, bool kCount>
 __device__ __forceinline__ bool trav_node(const SceneView& s, Trav& r, int* stack, unsigned& status, Work& work) {
-    if (++r.visits > s.visit_budget) {
-        status |= JR_STATUS_TRAVERSAL;
-        return false;
+    if constexpr (kCheck != kCheckNone) ++r.visits;
+    if constexpr (kCheck == kCheckAll) {
+        if (r.visits > s.visit_budget) {
+            status |= JR_STATUS_TRAVERSAL;
+            return false;
+        }
     }
     if constexpr (kCount) work.nodes++;
-    const Bvh4Node* n = s.nodes + r.ref;
     // The planes are stored lo, hi per axis.  For a positive direction
     // component the lo plane is met first, for a negative one the hi plane:
     // (lo * i - o) <= (hi * i - o) for i > 0 and the reverse for i < 0, and
     // both sides round monotonically, so for finite ray data the octant picks
     // exactly the values min and max would pick (with a NaN in the ray the two
     // forms differ, and such a ray carries no contribution either way).
-    const float4* pl = &n->lox;
-    const int sx = r.oct & 1, sy = (r.oct >> 1) & 1, sz = (r.oct >> 2) & 1;
-    const float4 nx = __ldg(pl + sx), fx = __ldg(pl + (sx ^ 1));
-    const float4 ny = __ldg(pl + 2 + sy), fy = __ldg(pl + 2 + (sy ^ 1));
-    const float4 nz = __ldg(pl + 4 + sz), fz = __ldg(pl + 4 + (sz ^ 1));
-    int4 rf = __ldg(&n->refs);
-    float t0 = slab(r, nx.x, fx.x, ny.x, fy.x, nz.x, fz.x);
-    float t1 = slab(r, nx.y, fx.y, ny.y, fy.y, nz.y, fz.y);
-    float t2 = slab(r, nx.z, fx.z, ny.z, fy.z, nz.z, fz.z);
-    float t3 = slab(r, nx.w, fx.w, ny.w, fy.w, nz.w, fz.w);  // an empty slot's box misses (+inf)
-    // 5-comparator sorting network on (distance, ref)
-    cswap(t0, rf.x, t1, rf.y);
-    cswap(t2, rf.z, t3, rf.w);
-    cswap(t0, rf.x, t2, rf.z);
-    cswap(t1, rf.y, t3, rf.w);
-    cswap(t1, rf.y, t2, rf.z);
-    const int pushes = (t1 < INFINITY) + (t2 < INFINITY) + (t3 < INFINITY);
-    if (r.sp + pushes > s.stack_limit) {
-        status |= JR_STATUS_STACK;
-        return false;
+    const char* n = reinterpret_cast<const char*>(s.nodes + r.ref);
+    const uint32_t key = ((uint32_t)r.ref & 7u) << 4;
+    const uint32_t kx = key ^ (r.oct & 16u), ky = key ^ ((r.oct >> 1) & 16u), kz = key ^ ((r.oct >> 2) & 16u);
+    auto chunk = [&](uint32_t at) { return __ldg(reinterpret_cast<const float4*>(n + at)); };
+    const float4 nx = chunk(kx), fx = chunk(kx ^ 16u);
+    const float4 ny = chunk(ky ^ 32u), fy = chunk(ky ^ 48u);
+    const float4 nz = chunk(kz ^ 64u), fz = chunk(kz ^ 80u);
+    int4 rf = __ldg(reinterpret_cast<const int4*>(n + (key ^ 96u)));
+    float ax[4], ay[4], az[4], bx[4], by[4], bz[4], t[4];
+    plane4(nx, r.ix, r.ox, ax);
+    plane4(fx, r.ix, r.ox, bx);
+    plane4(ny, r.iy, r.oy, ay);
+    plane4(fy, r.iy, r.oy, by);
+    plane4(nz, r.iz, r.oz, az);
+    plane4(fz, r.iz, r.oz, bz);
+    // Entry distance of each child box in [0, tb], or +inf for a miss (an empty
+    // slot's box always misses).  The far distance is scaled up by 2 ulp so that
+    // a ray grazing a face of a box still enters it.
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float tn = fmax3(ax[j], ay[j], fmaxf(az[j], 0.0f));
+        const float tf = fmin3(bx[j], by[j], fminf(bz[j], r.tb));
+        t[j] = tn <= tf * 1.00000024f ? tn : INFINITY;
     }
-    if (t3 < INFINITY) stack[r.sp++] = rf.w;
-    if (t2 < INFINITY) stack[r.sp++] = rf.z;
-    if (t1 < INFINITY) stack[r.sp++] = rf.y;
-    if (t0 < INFINITY) r.ref = rf.x;
+    cswap(t[0], rf.x, t[1], rf.y);
+    cswap(t[2], rf.z, t[3], rf.w);
+    cswap(t[0], rf.x, t[2], rf.z);
+    if constexpr (kCheck == kCheckAll) {
+        const int pushes = (t[1] < INFINITY) + (t[2] < INFINITY) + (t[3] < INFINITY);
+        if (r.sp + pushes > s.stack_limit) {
+            status |= JR_STATUS_STACK;
+            return false;
+        }
+    }
+    if (t[3] < INFINITY) stack[r.sp++] = rf.w;
+    if (t[2] < INFINITY) stack[r.sp++] = rf.z;
+    if (t[1] < INFINITY) stack[r.sp++] = rf.y;
+    if (t[0] < INFINITY) r.ref = rf.x;
     else r.ref = r.sp > 0 ? stack[--r.sp] : kSentinel;
     return true;
+}
+
+// kCheckVisits: whether ray r has used up its visit budget (called once per
+// round; the caller then treats the ray as a miss).
+template <int kCheck>
+__device__ __forceinline__ bool over_budget(const SceneView& s, const Trav& r, unsigned& status) {
+    if constexpr (kCheck == kCheckVisits) {
+        if (r.visits > s.visit_budget) {
+            status |= JR_STATUS_TRAVERSAL;
+            return true;
+        }
+    }
+    return false;
 }
 
 // Test the triangles of leaf `leaf` (Moller-Trumbore, JGT 1997; ties on equal
@@ -248,7 +316,7 @@ __device__ __forceinline__ bool search_done(unsigned searching, unsigned tracing
 // a __any_sync over `mask`, so the lanes reconverge every iteration instead of
 // drifting apart under independent thread scheduling.  Returns the leaf-order
 // record index or -1; t_out gets the hit distance.
-template <bool kCount>
+template <int kCheck, bool kCount>
 __device__ __forceinline__ int closest_hit(const SceneView& s, unsigned mask, bool want, float3 o, float3 d,
                                            float& t_out, unsigned& status, Work& work) {
     Trav r;
@@ -258,12 +326,17 @@ __device__ __forceinline__ int closest_hit(const SceneView& s, unsigned mask, bo
     int stack[kStackSize];
     while (__any_sync(mask, active)) {
         const unsigned tracing = __ballot_sync(mask, active);
-        while (__any_sync(mask, active && r.ref >= 0)) {
-            if (active && r.ref >= 0 && !trav_node<kCount>(s, r, stack, status, work)) {
+        if (__any_sync(mask, active && r.ref >= 0)) {
+            do {  // one vote per node visit: it ends the loop when nobody searches, too
+                if (active && r.ref >= 0 && !trav_node<kCheck, kCount>(s, r, stack, status, work)) {
+                    active = false;
+                    r.best = -1;
+                }
+            } while (!search_done(__ballot_sync(mask, active && r.ref >= 0), tracing));
+            if (active && over_budget<kCheck>(s, r, status)) {
                 active = false;
                 r.best = -1;
             }
-            if (search_done(__ballot_sync(mask, active && r.ref >= 0), tracing)) break;
         }
         if (active && r.ref < 0) active = r.ref != kSentinel && trav_leaf<kCount>(s, r, stack, work);
     }
@@ -385,7 +458,7 @@ __device__ __forceinline__ float3 finite_or_zero(float3 F, unsigned& status) {
 // The integrand for the lanes in `mask` (all of which must call together;
 // lanes with want = false only keep the warp in step).  The bounce loop runs
 // until no lane in the warp has a live path.
-template <bool kCount>
+template <int kCheck, bool kCount>
 __device__ __forceinline__ float3 eval_path_w(const SceneView& s, unsigned mask, bool want, int depth, const float* y,
                                               uint32_t ys, int32_t* ids, uint64_t id_stride, unsigned& status,
                                               Work& work) {
@@ -398,7 +471,7 @@ __device__ __forceinline__ float3 eval_path_w(const SceneView& s, unsigned mask,
     for (int v = 0; v <= depth; ++v) {
         if (!__any_sync(mask, alive)) break;
         float t;
-        const int k = closest_hit<kCount>(s, mask, alive, o, d, t, status, work);
+        const int k = closest_hit<kCheck, kCount>(s, mask, alive, o, d, t, status, work);
         if (alive) {
             if (k < 0) {
                 alive = false;
@@ -413,10 +486,11 @@ __device__ __forceinline__ float3 eval_path_w(const SceneView& s, unsigned mask,
     return want ? finite_or_zero(F, status) : F;
 }
 
+template <int kCheck>
 __device__ __forceinline__ float3 eval_path(const SceneView& s, unsigned mask, bool want, int depth, const float* y,
                                             uint32_t ys, int32_t* ids, uint64_t id_stride, unsigned& status) {
     Work w;
-    return eval_path_w<false>(s, mask, want, depth, y, ys, ids, id_stride, status, w);
+    return eval_path_w<kCheck, false>(s, mask, want, depth, y, ys, ids, id_stride, status, w);
 }
 
 // ------------------------------------------------------------------ gradient
@@ -554,7 +628,7 @@ __device__ inline bool scatter_grad(const Material& m, float3 d, float3 ng, floa
 
 // F(y) and dF/dy (dF->c[ch][k]) for one lane (no warp cooperation: the
 // megakernel's lanes call it together, each with its own state).
-template <bool kCount>
+template <int kCheck, bool kCount>
 __device__ inline float3 eval_path_grad(const SceneView& s, unsigned mask, bool want, int depth, const float* y,
                                         uint32_t ys, Jac3& JF, unsigned& status, Work& work) {
     const int D = 2 + 2 * depth;
@@ -585,7 +659,7 @@ __device__ inline float3 eval_path_grad(const SceneView& s, unsigned mask, bool 
     for (int v = 0; v <= depth; ++v) {
         if (!__any_sync(mask, alive)) break;
         float t;
-        const int k = closest_hit<kCount>(s, mask, alive, o, d, t, status, work);
+        const int k = closest_hit<kCheck, kCount>(s, mask, alive, o, d, t, status, work);
         if (!alive) continue;
         if (k < 0) {
             alive = false;

@@ -7,6 +7,7 @@
 
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 namespace jr {
@@ -28,7 +29,9 @@ constexpr uint64_t kWavefrontMinChains = 1u << 18;  // JR_EXEC_AUTO picks the wa
 // >= 0 inner node index; < 0 leaf = ~((first << 3) | (count - 1)); kNoChild
 // marks an empty slot, whose box is the empty box (lo = +inf, hi = -inf), so
 // that the slab test misses it.  pad.x holds the child count; the rest of the
-// last 16 bytes is unused.
+// last 16 bytes is unused.  On the device node i's eight 16-byte chunks are
+// stored at chunk ^ (i & 7) (swizzle_nodes_kernel), so that the lanes of a warp,
+// which read the same chunk of different nodes, spread over the L1 banks.
 struct __align__(128) Bvh4Node {
     float4 lox, hix, loy, hiy, loz, hiz;
     int4 refs;
@@ -66,7 +69,23 @@ struct SceneView {
     float cam[12];
     uint32_t visit_budget;  // node visits per ray before the watchdog stops it (kNodeVisitBudget)
     int stack_limit;        // traversal stack entries a ray may use (<= kStackSize)
+    int stack_need;         // the most entries a traversal of this tree can hold (HostBvh::stack_need)
 };
+
+// The traversal watchdogs that can fire on a view (TravCheck in jr_device.cuh).
+// A ray visits a node at most once, so a budget of at least the node count is
+// never exceeded; the builder bounds the stack.
+inline int trav_checks(const SceneView& s) {
+    if (s.stack_limit < s.stack_need) return 2;                // kCheckAll
+    return s.visit_budget < (uint32_t)s.n_nodes ? 1 : 0;       // kCheckVisits, kCheckNone
+}
+// f(std::integral_constant<int, checks>) for the run-time `checks`.
+template <class F>
+inline void with_checks(int checks, F&& f) {
+    if (checks == 0) f(std::integral_constant<int, 0>{});
+    else if (checks == 1) f(std::integral_constant<int, 1>{});
+    else f(std::integral_constant<int, 2>{});
+}
 
 // The regeneration flow (jr_flow.cu): L coupling layers, MLP of 2 x 64 hidden
 // units, K bins, conditioner width padded to kFAP; bf16 weight rows padded to
@@ -175,14 +194,18 @@ struct BatchWave {
     const BatchItem* items;     // [n_items] work items of 128 chains for the step launches
     uint32_t n_sets = 0, n_items = 0;
     unsigned int* fetch;        // the path launches' item cursor
+    int checks = 0;             // the watchdogs a path launch checks (trav_checks, the most of any set)
 };
+// Move the chunks of freshly uploaded nodes to their device positions (Bvh4Node).
+cudaError_t launch_swizzle_nodes(Bvh4Node* nodes, uint32_t n_nodes, cudaStream_t st);
 // Rebase one scene's nodes and triangles, already copied into the
-// merged arrays (refs via rebase_ref, material indices + mat_off).
+// merged arrays (refs via rebase_ref, chunks to the merged positions, material
+// indices + mat_off).
 cudaError_t launch_rebase_scene(Bvh4Node* nodes, uint32_t n_nodes, TriRecord* tris, uint32_t n_tris, int node_off,
                                 int tri_off, int mat_off, cudaStream_t st);
 // The batched path kernel's persistent grid (set up once per device; call it
 // outside stream capture before the first launch_batch_wavefront).
-cudaError_t batch_wavefront_grid(long long* blocks);
+cudaError_t batch_wavefront_grid(int checks, long long* blocks);
 // n_steps batched wavefront steps of every set (step indices entries[q].step + k),
 // ending with the closing step launch; the caller folds afterwards.  flow_sets:
 // the host views of the sets with a flow attached (their flow launches run
@@ -223,6 +246,7 @@ struct HostBvh {
     std::vector<TriRecord> tris;
     int root = 0;
     int depth = 0;
+    int stack_need = 0;  // the most stack entries a traversal can hold (<= kStackSize)
 };
 
 // bvh_build.cpp
@@ -251,9 +275,10 @@ cudaError_t launch_eval_grad(const SceneView& s, uint32_t depth, const float* x,
                              cudaStream_t st);
 // Batched persistent launch + fold over n_sets chain sets (block = chains per
 // work item = threads per block, a multiple of 32 in [32, 256]).
+// checks: the most of any set's trav_checks.
 cudaError_t launch_batch(BatchEntry* entries, const BatchItem* items, uint32_t n_items, const uint64_t* px_off,
                          uint32_t n_sets, uint64_t total_px, unsigned int* cursor, uint32_t max_dim, int block,
-                         uint32_t n_steps, cudaStream_t st);
+                         int checks, uint32_t n_steps, cudaStream_t st);
 // Device time per kernel class of a sequence of launches on one stream: an
 // event is recorded after every launch, and the time since the previous event
 // is charged to that launch's class.

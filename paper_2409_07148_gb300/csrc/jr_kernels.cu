@@ -26,6 +26,7 @@ namespace {
 
 // ------------------------------------------------------------------ kernels
 // x0 ~ mu (tag 1); y built in shared memory, then written to the SoA state.
+template <int kCheck>
 __global__ void init_kernel(SceneView s, ChainView c) {
     extern __shared__ float sh[];
     const uint32_t B = blockDim.x, tid = threadIdx.x;
@@ -43,7 +44,7 @@ __global__ void init_kernel(SceneView s, ChainView c) {
             if (4 * b + q < D) y[(4 * b + q) * B] = u01(rr[q]);
     }
     unsigned status = 0;
-    const float3 F = eval_path(s, mask, true, (int)c.depth, y, B, nullptr, 0, status);
+    const float3 F = eval_path<kCheck>(s, mask, true, (int)c.depth, y, B, nullptr, 0, status);
     float2* x2 = reinterpret_cast<float2*>(c.x);
     for (int k = 0; 2 * k < D; ++k) x2[(uint64_t)k * c.n + i] = make_float2(y[2 * k * B], y[(2 * k + 1) * B]);
     c.fpu[0 * c.n + i] = F.x;
@@ -72,7 +73,7 @@ __global__ void reeval_kernel(SceneView s, ChainView c) {
     if (i >= c.n) return;
     unsigned status = 0;
     load_coords(c, i, sh + threadIdx.x, blockDim.x);
-    const float3 F = eval_path(s, mask, true, (int)c.depth, sh + threadIdx.x, blockDim.x, nullptr, 0, status);
+    const float3 F = eval_path<kCheckAll>(s, mask, true, (int)c.depth, sh + threadIdx.x, blockDim.x, nullptr, 0, status);
     c.fpu[0 * c.n + i] = F.x;
     c.fpu[1 * c.n + i] = F.y;
     c.fpu[2 * c.n + i] = F.z;
@@ -84,7 +85,7 @@ __global__ void reeval_kernel(SceneView s, ChainView c) {
 // n_steps of Alg. 2 for chain i of set c (thread tid of the block; `active`
 // false for threads without a chain).  Every thread of the block calls it;
 // sh holds [2][D][blockDim] floats.
-template <bool kTrace, bool kCount>
+template <int kCheck, bool kTrace, bool kCount>
 __device__ __forceinline__ void chain_steps(const SceneView& s, const ChainView& c, uint64_t i, bool active, float* sh,
                                             uint64_t step_begin, uint32_t n_steps, uint8_t* tr_flags, float* tr_dt,
                                             int32_t* tr_pix, unsigned long long* work_out) {
@@ -166,7 +167,7 @@ __device__ __forceinline__ void chain_steps(const SceneView& s, const ChainView&
                     }
                 }
             }
-            const float3 Fy = eval_path_w<kCount>(s, mask, true, (int)c.depth, cand, B, nullptr, 0, status, work);
+            const float3 Fy = eval_path_w<kCheck, kCount>(s, mask, true, (int)c.depth, cand, B, nullptr, 0, status, work);
             const float py_ = lum(Fy);
             bool accept;
             if (mh) {  // Alg. 1: U < min(1, p(y)/p(x)), 1 if p(x) = 0
@@ -240,13 +241,13 @@ __device__ __forceinline__ void chain_steps(const SceneView& s, const ChainView&
 // per SM): the 4-wide traversal would take 108, and the occupancy the cap buys
 // outweighs its small spill (measured: 5.0 -> 5.9e8 chain steps/s for the
 // megakernel, 5.9 -> 6.1e8 for the 64-scene batch).
-template <bool kTrace, bool kCount>
+template <int kCheck, bool kTrace, bool kCount>
 __global__ void __launch_bounds__(256, 4) step_kernel(SceneView s, ChainView c, uint64_t step_begin, uint32_t n_steps,
                                                    uint8_t* tr_flags, float* tr_dt, int32_t* tr_pix,
                                                    unsigned long long* work_out) {
     extern __shared__ float sh[];
     const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    chain_steps<kTrace, kCount>(s, c, i, i < c.n, sh, step_begin, n_steps, tr_flags, tr_dt, tr_pix, work_out);
+    chain_steps<kCheck, kTrace, kCount>(s, c, i, i < c.n, sh, step_begin, n_steps, tr_flags, tr_dt, tr_pix, work_out);
 }
 
 // ------------------------------------------------------------------ one chain per warp
@@ -450,7 +451,7 @@ __device__ __forceinline__ float mala_log_q(const float* b, const float* a, cons
     return -s / (2.0f * sigma * sigma);
 }
 
-template <bool kTrace>
+template <int kCheck, bool kTrace>
 __device__ __forceinline__ void chain_steps_mala(const SceneView& s, const ChainView& c, uint64_t i, bool active,
                                                  float* sh, uint64_t step_begin, uint32_t n_steps, uint8_t* tr_flags,
                                                  float* tr_dt, int32_t* tr_pix) {
@@ -532,7 +533,7 @@ __device__ __forceinline__ void chain_steps_mala(const SceneView& s, const Chain
                 }
             }
         }
-        const float3 Fy = eval_path_grad<false>(s, mask, active, (int)c.depth, cand, B, JF, status, work);
+        const float3 Fy = eval_path_grad<kCheck, false>(s, mask, active, (int)c.depth, cand, B, JF, status, work);
         bool accept = false;
         if (active) {
             for (int d = 0; d < D; ++d) my[d * B] = mala_drift(Fy, JF, d, c.sigma);
@@ -601,13 +602,13 @@ __device__ __forceinline__ void chain_steps_mala(const SceneView& s, const Chain
     }
 }
 
-template <bool kTrace>
+template <int kCheck, bool kTrace>
 __global__ void __launch_bounds__(128) step_kernel_mala(SceneView s, ChainView c, uint64_t step_begin,
                                                         uint32_t n_steps, uint8_t* tr_flags, float* tr_dt,
                                                         int32_t* tr_pix) {
     extern __shared__ float sh[];
     const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    chain_steps_mala<kTrace>(s, c, i, i < c.n, sh, step_begin, n_steps, tr_flags, tr_dt, tr_pix);
+    chain_steps_mala<kCheck, kTrace>(s, c, i, i < c.n, sh, step_begin, n_steps, tr_flags, tr_dt, tr_pix);
 }
 
 // F, p and the drift of the stored states (chain creation and jr_set_state).
@@ -621,7 +622,7 @@ __global__ void __launch_bounds__(128) mala_reeval_kernel(SceneView s, ChainView
     Jac3 JF;
     load_coords(c, i, sh + threadIdx.x, blockDim.x);
     const float3 F =
-        eval_path_grad<false>(s, mask, true, (int)c.depth, sh + threadIdx.x, blockDim.x, JF, status, w);
+        eval_path_grad<kCheckAll, false>(s, mask, true, (int)c.depth, sh + threadIdx.x, blockDim.x, JF, status, w);
     c.fpu[0 * c.n + i] = F.x;
     c.fpu[1 * c.n + i] = F.y;
     c.fpu[2 * c.n + i] = F.z;
@@ -640,7 +641,7 @@ __global__ void __launch_bounds__(128) eval_grad_kernel(SceneView s, uint32_t de
     unsigned status = 0;
     Work w;
     Jac3 JF;
-    const float3 f = eval_path_grad<false>(s, mask, true, (int)depth, x + i, (uint32_t)n, JF, status, w);
+    const float3 f = eval_path_grad<kCheckVisits, false>(s, mask, true, (int)depth, x + i, (uint32_t)n, JF, status, w);
     const int D = 2 + 2 * (int)depth;
     if (F) {
         F[i] = f.x;
@@ -657,6 +658,7 @@ __global__ void __launch_bounds__(128) eval_grad_kernel(SceneView s, uint32_t de
 // chains of one set -- from a global cursor; the host orders the items by
 // estimated cost, so the longest items start first.  Every item runs all
 // n_steps of Alg. 2 for its chains with the same code as step_kernel.
+template <int kCheck>
 __global__ void __launch_bounds__(256, 4) batch_step_kernel(const BatchEntry* entries, const BatchItem* items,
                                                          uint32_t n_items, unsigned int* cursor, uint32_t n_steps) {
     extern __shared__ float sh[];
@@ -670,7 +672,7 @@ __global__ void __launch_bounds__(256, 4) batch_step_kernel(const BatchEntry* en
         const BatchItem wi = items[it];
         const BatchEntry& e = entries[wi.set];  // descriptor fields are read where used
         const uint64_t i = wi.begin + threadIdx.x;
-        chain_steps<false, false>(e.s, e.c, i, i < wi.end, sh, e.step, n_steps, nullptr, nullptr, nullptr, nullptr);
+        chain_steps<kCheck, false, false>(e.s, e.c, i, i < wi.end, sh, e.step, n_steps, nullptr, nullptr, nullptr, nullptr);
         __syncthreads();  // the shared state buffers are reused by the next item
     }
 }
@@ -740,13 +742,14 @@ __global__ void resolve_kernel(const double4_32a* acc, const unsigned long long*
     rgb[3 * j + 2] = (float)(a.z * inv);
 }
 
+template <int kCheck>
 __global__ void eval_states_kernel(SceneView s, uint32_t depth, float c_tilde, const float* x, uint64_t n, float* F,
                                    float* p, float* u, float* k, int32_t* ids, unsigned int* status_word) {
     const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     const unsigned mask = __ballot_sync(0xffffffffu, i < n);
     if (i >= n) return;
     unsigned status = 0;
-    const float3 f = eval_path(s, mask, true, (int)depth, x + i, (uint32_t)n, ids ? ids + i : nullptr, n, status);
+    const float3 f = eval_path<kCheck>(s, mask, true, (int)depth, x + i, (uint32_t)n, ids ? ids + i : nullptr, n, status);
     const float pp = lum(f);
     const float uu = 1.0f;
     if (F) {
@@ -760,6 +763,7 @@ __global__ void eval_states_kernel(SceneView s, uint32_t depth, float c_tilde, c
     if (status && status_word) atomicOr(status_word, status);
 }
 
+template <int kCheck>
 __global__ void render_pt_kernel(SceneView s, uint32_t W, uint32_t H, uint32_t depth, uint64_t seed,
                                  uint64_t sample_begin, uint64_t n, double* accum) {
     extern __shared__ float sh[];
@@ -778,7 +782,7 @@ __global__ void render_pt_kernel(SceneView s, uint32_t W, uint32_t H, uint32_t d
             if (4 * b + q < D) y[(4 * b + q) * B] = u01(rr[q]);
     }
     unsigned status = 0;
-    const float3 F = eval_path(s, mask, true, (int)depth, y, B, nullptr, 0, status);
+    const float3 F = eval_path<kCheck>(s, mask, true, (int)depth, y, B, nullptr, 0, status);
     uint32_t px = min((uint32_t)((double)y[0] * (double)W), W - 1);
     uint32_t py = min((uint32_t)((double)y[B] * (double)H), H - 1);
     const double WH = (double)W * (double)H;
@@ -822,6 +826,12 @@ __global__ void __launch_bounds__(256) fma_peak_kernel(uint32_t iters, float* si
 
 inline unsigned grid_for(uint64_t n, unsigned b) { return (unsigned)((n + b - 1) / b); }
 
+// A kernel as a type, so that a generic launcher has one set of statics per kernel.
+template <auto K>
+struct Kernel {
+    static constexpr auto value = K;
+};
+
 }  // namespace
 
 cudaError_t measure_fma_peak(double* tflops, double* ms_out, cudaStream_t st) {
@@ -861,7 +871,9 @@ cudaError_t measure_fma_peak(double* tflops, double* ms_out, cudaStream_t st) {
 
 cudaError_t launch_init(const SceneView& s, const ChainView& c, cudaStream_t st) {
     const unsigned B = 128;
-    init_kernel<<<grid_for(c.n, B), B, sizeof(float) * c.dim * B, st>>>(s, c);
+    with_checks(trav_checks(s), [&](auto k) {
+        init_kernel<k()><<<grid_for(c.n, B), B, sizeof(float) * c.dim * B, st>>>(s, c);
+    });
     return cudaGetLastError();
 }
 
@@ -885,55 +897,50 @@ cudaError_t launch_step(const SceneView& s, const ChainView& c, uint64_t step_be
     const unsigned B = (unsigned)block;
     const size_t shm = sizeof(float) * 2 * c.dim * B;  // <= 2 * 32 * 256 * 4 = 64 KB
     const unsigned G = grid_for(c.n, B);
-    static DeviceOnce once;  // per device: opt in to > 48 KB of dynamic shared memory
-    cudaError_t e0 = once.get(
-        [](int, long long*) {
-            const int lim = (int)(sizeof(float) * 2 * kMaxDim * 256);
-            cudaError_t e;
-            if ((e = cudaFuncSetAttribute(step_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          lim)) != cudaSuccess ||
-                (e = cudaFuncSetAttribute(step_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          lim)) != cudaSuccess ||
-                (e = cudaFuncSetAttribute(step_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          lim)) != cudaSuccess)
-                return e;
-            return cudaSuccess;
-        },
-        nullptr);
-    if (e0 != cudaSuccess) return e0;
-    if (work_out)
-        step_kernel<false, true><<<G, B, shm, st>>>(s, c, step_begin, n_steps, nullptr, nullptr, nullptr, work_out);
-    else if (tr_flags || tr_dt || tr_pix)
-        step_kernel<true, false><<<G, B, shm, st>>>(s, c, step_begin, n_steps, tr_flags, tr_dt, tr_pix, nullptr);
-    else
-        step_kernel<false, false><<<G, B, shm, st>>>(s, c, step_begin, n_steps, nullptr, nullptr, nullptr, nullptr);
-    return cudaGetLastError();
+    // The traced and the counted variant always check both watchdogs.
+    const auto run = [&](auto kernel, uint8_t* f, float* dt, int32_t* pix, unsigned long long* work) {
+        static DeviceOnce once;  // per device and variant: opt in to > 48 KB of dynamic shared memory
+        const cudaError_t e = once.get(
+            [&](int, long long*) {
+                return cudaFuncSetAttribute(kernel.value, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)(sizeof(float) * 2 * kMaxDim * 256));
+            },
+            nullptr);
+        if (e != cudaSuccess) return e;
+        kernel.value<<<G, B, shm, st>>>(s, c, step_begin, n_steps, f, dt, pix, work);
+        return cudaGetLastError();
+    };
+    if (work_out) return run(Kernel<step_kernel<kCheckAll, false, true>>{}, nullptr, nullptr, nullptr, work_out);
+    if (tr_flags || tr_dt || tr_pix)
+        return run(Kernel<step_kernel<kCheckAll, true, false>>{}, tr_flags, tr_dt, tr_pix, nullptr);
+    cudaError_t e = cudaSuccess;
+    with_checks(trav_checks(s), [&](auto k) {
+        e = run(Kernel<step_kernel<k(), false, false>>{}, nullptr, nullptr, nullptr, nullptr);
+    });
+    return e;
 }
 
 cudaError_t launch_step_mala(const SceneView& s, const ChainView& c, uint64_t step_begin, uint32_t n_steps,
                              uint8_t* tr_flags, float* tr_dt, int32_t* tr_pix, cudaStream_t st) {
     const unsigned B = 128;
     const size_t shm = sizeof(float) * 4 * c.dim * B;  // <= 4 * 32 * 128 * 4 = 64 KB
-    static DeviceOnce once;
-    cudaError_t e0 = once.get(
-        [](int, long long*) {
-            const int lim = (int)(sizeof(float) * 4 * kMaxDim * 128);
-            cudaError_t e;
-            if ((e = cudaFuncSetAttribute(step_kernel_mala<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          lim)) != cudaSuccess ||
-                (e = cudaFuncSetAttribute(step_kernel_mala<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) !=
-                    cudaSuccess)
-                return e;
-            return cudaSuccess;
-        },
-        nullptr);
-    if (e0 != cudaSuccess) return e0;
     const unsigned G = grid_for(c.n, B);
-    if (tr_flags || tr_dt || tr_pix)
-        step_kernel_mala<true><<<G, B, shm, st>>>(s, c, step_begin, n_steps, tr_flags, tr_dt, tr_pix);
-    else
-        step_kernel_mala<false><<<G, B, shm, st>>>(s, c, step_begin, n_steps, nullptr, nullptr, nullptr);
-    return cudaGetLastError();
+    const auto run = [&](auto kernel) {
+        static DeviceOnce once;  // per device and variant
+        const cudaError_t e = once.get(
+            [&](int, long long*) {
+                return cudaFuncSetAttribute(kernel.value, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)(sizeof(float) * 4 * kMaxDim * 128));
+            },
+            nullptr);
+        if (e != cudaSuccess) return e;
+        kernel.value<<<G, B, shm, st>>>(s, c, step_begin, n_steps, tr_flags, tr_dt, tr_pix);
+        return cudaGetLastError();
+    };
+    if (tr_flags || tr_dt || tr_pix) return run(Kernel<step_kernel_mala<kCheckAll, true>>{});
+    cudaError_t e = cudaSuccess;
+    with_checks(trav_checks(s), [&](auto k) { e = run(Kernel<step_kernel_mala<k(), false>>{}); });
+    return e;
 }
 
 cudaError_t launch_mala_reeval(const SceneView& s, const ChainView& c, cudaStream_t st) {
@@ -956,29 +963,35 @@ cudaError_t launch_fold(const ChainView& c, cudaStream_t st) {
 
 cudaError_t launch_batch(BatchEntry* entries, const BatchItem* items, uint32_t n_items, const uint64_t* px_off,
                          uint32_t n_sets, uint64_t total_px, unsigned int* cursor, uint32_t max_dim, int block,
-                         uint32_t n_steps, cudaStream_t st) {
-    static DeviceOnce once;  // per device: the SM count, after the shared-memory opt-in
+                         int checks, uint32_t n_steps, cudaStream_t st) {
     const size_t shm = sizeof(float) * 2 * max_dim * (size_t)block;
-    long long sms = 0;
-    cudaError_t e = once.get(
-        [](int dev, long long* v) {
-            int n = 0;
-            cudaError_t r;
-            if ((r = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
-                (r = cudaFuncSetAttribute(batch_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)(sizeof(float) * 2 * kMaxDim * 256))) != cudaSuccess)
-                return r;
-            *v = n;
-            return cudaSuccess;
-        },
-        &sms);
+    const auto run = [&](auto kernel) {
+        static DeviceOnce once;  // per device and variant: the SM count, after the shared-memory opt-in
+        long long sms = 0;
+        cudaError_t e = once.get(
+            [&](int dev, long long* v) {
+                int n = 0;
+                cudaError_t r;
+                if ((r = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+                    (r = cudaFuncSetAttribute(kernel.value, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)(sizeof(float) * 2 * kMaxDim * 256))) != cudaSuccess)
+                    return r;
+                *v = n;
+                return cudaSuccess;
+            },
+            &sms);
+        if (e != cudaSuccess) return e;
+        int per_sm = 0;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel.value, block, shm)) != cudaSuccess)
+            return e;
+        const unsigned grid = (unsigned)std::min<uint64_t>((uint64_t)sms * (per_sm > 0 ? per_sm : 1), n_items);
+        if (n_steps > 0 && n_items > 0)
+            kernel.value<<<grid, block, shm, st>>>(entries, items, n_items, cursor, n_steps);
+        return cudaSuccess;
+    };
+    cudaError_t e = cudaSuccess;
+    with_checks(checks, [&](auto k) { e = run(Kernel<batch_step_kernel<k()>>{}); });
     if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_step_kernel, block, shm)) != cudaSuccess)
-        return e;
-    const unsigned grid = (unsigned)std::min<uint64_t>((uint64_t)sms * (per_sm > 0 ? per_sm : 1), n_items);
-    if (n_steps > 0 && n_items > 0)
-        batch_step_kernel<<<grid, block, shm, st>>>(entries, items, n_items, cursor, n_steps);
     const uint64_t total = total_px > n_sets ? total_px : n_sets;
     batch_fold_kernel<<<grid_for(total, 256), 256, 0, st>>>(entries, px_off, n_sets, total_px, cursor, n_steps);
     return cudaGetLastError();
@@ -994,7 +1007,9 @@ cudaError_t launch_resolve(const ChainView& c, float* rgb, uint64_t mh_samples, 
 cudaError_t launch_eval_states(const SceneView& s, uint32_t depth, float c_tilde, const float* x, uint64_t n,
                                float* F, float* p, float* u, float* k, int32_t* ids, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    eval_states_kernel<<<grid_for(n, 128), 128, 0, st>>>(s, depth, c_tilde, x, n, F, p, u, k, ids, nullptr);
+    with_checks(trav_checks(s), [&](auto kc) {
+        eval_states_kernel<kc()><<<grid_for(n, 128), 128, 0, st>>>(s, depth, c_tilde, x, n, F, p, u, k, ids, nullptr);
+    });
     return cudaGetLastError();
 }
 
@@ -1003,7 +1018,9 @@ cudaError_t launch_render_pt(const SceneView& s, uint32_t width, uint32_t height
     if (n == 0) return cudaSuccess;
     const unsigned B = 128;
     const size_t shm = sizeof(float) * (2 + 2 * depth) * B;
-    render_pt_kernel<<<grid_for(n, B), B, shm, st>>>(s, width, height, depth, seed, sample_begin, n, accum);
+    with_checks(trav_checks(s), [&](auto k) {
+        render_pt_kernel<k()><<<grid_for(n, B), B, shm, st>>>(s, width, height, depth, seed, sample_begin, n, accum);
+    });
     return cudaGetLastError();
 }
 

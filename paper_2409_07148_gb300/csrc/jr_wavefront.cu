@@ -368,6 +368,7 @@ constexpr int kShadeBatch = 16;
 enum PathState : uint32_t { kIdle = 0, kTraverse = 1, kWaitShade = 2 };
 
 
+template <int kCheck>
 __global__ void __launch_bounds__(128) wf_path_kernel(SceneView s, ChainView c, int ident) {
     const WaveView& w = c.wf;
     const uint32_t* qin = w.queue;
@@ -381,14 +382,27 @@ __global__ void __launch_bounds__(128) wf_path_kernel(SceneView s, ChainView c, 
     const unsigned lt = (1u << lane) - 1u;
     unsigned status = 0;
     Work wk;
-    Trav r;
+    Trav r{};
     int stack[kStackSize];
     uint32_t state = kIdle, i = 0;
     int v = 0, leaf = kSentinel;
-    bool failed = false, drained = false;
-    float3 T = f3(1.f, 1.f, 1.f), F = f3(0.f, 0.f, 0.f);
-    float u1 = 0.f, u2 = 0.f;  // the coordinates of vertex v
-    bool cx = false;           // the candidate lives in x (else in y)
+    bool drained = false;
+    float3 T = f3(1.f, 1.f, 1.f);
+    bool lit = false;  // F is not zero, and waits in fy[i]
+    bool cx = false;   // the candidate lives in x (else in y)
+    // One node visit of a lane that has an inner node; a leaf it comes to is
+    // postponed if it holds none yet.
+    auto visit = [&](bool on) {
+        if (on && r.ref >= 0) {
+            if (!trav_node<kCheck, false>(s, r, stack, status, wk)) {
+                r.best = -1;
+                r.ref = leaf = kSentinel;
+            } else if (leaf == kSentinel && r.ref < 0 && r.ref != kSentinel) {
+                leaf = r.ref;
+                r.ref = r.sp > 0 ? stack[--r.sp] : kSentinel;
+            }
+        }
+    };
     while (true) {
         // shade the waiting lanes as a batch
         const unsigned waiting = __ballot_sync(kFull, state == kWaitShade);
@@ -397,19 +411,24 @@ __global__ void __launch_bounds__(128) wf_path_kernel(SceneView s, ChainView c, 
             bool need_u = false;
             if (state == kWaitShade) {
                 bool live = false;
+                float3 F = f3(0.f, 0.f, 0.f);
+                if (lit) {
+                    const float4 f = __ldcs(w.fy + i);
+                    F = f3(f.x, f.y, f.z);
+                }
                 if (r.best >= 0) {
+                    float2 uv = make_float2(0.f, 0.f);
+                    if (v < depth)  // vertex v's coordinate pair, one 8-byte load (evict-first)
+                        uv = __ldcs(reinterpret_cast<const float2*>(cx ? c.x : w.y) + (uint64_t)(1 + v) * n + i);
                     float3 o = r.o, d = r.d;
-                    live = shade_vertex(s, r.best, r.tb, v, depth, v < depth ? u1 : 0.f, v < depth ? u2 : 0.f, o,
-                                        d, T, F);
+                    live = shade_vertex(s, r.best, r.tb, v, depth, uv.x, uv.y, o, d, T, F);
                     if (live) {
                         ++v;
                         trav_begin(s, r, o, d);
                         state = kTraverse;
-                        if (v < depth) {  // vertex v's coordinate pair, one 8-byte load (evict-first)
-                            const float2 uv =
-                                __ldcs(reinterpret_cast<const float2*>(cx ? c.x : w.y) + (uint64_t)(1 + v) * n + i);
-                            u1 = uv.x;
-                            u2 = uv.y;
+                        if (F.x != 0.f || F.y != 0.f || F.z != 0.f) {
+                            __stcs(w.fy + i, make_float4(F.x, F.y, F.z, 0.f));
+                            lit = true;
                         }
                     }
                 }
@@ -439,12 +458,10 @@ __global__ void __launch_bounds__(128) wf_path_kernel(SceneView s, ChainView c, 
                     i = ident ? j : qin[j];
                     const float4 y = __ldcs(w.fy + i);
                     cx = __ldcs(w.par + i) != 0;
-                    u1 = y.z;
-                    u2 = y.w;
                     float3 o, d;
                     camera_ray(s, y.x, y.y, o, d);
                     T = f3(1.f, 1.f, 1.f);
-                    F = f3(0.f, 0.f, 0.f);
+                    lit = false;
                     v = 0;
                     trav_begin(s, r, o, d);
                     state = s.root != kSentinel ? kTraverse : kWaitShade;  // empty scene: a miss
@@ -462,29 +479,22 @@ __global__ void __launch_bounds__(128) wf_path_kernel(SceneView s, ChainView c, 
             r.ref = r.sp > 0 ? stack[--r.sp] : kSentinel;
         }
         const unsigned tracing_now = __ballot_sync(kFull, trav);
-        while (__any_sync(kFull, trav && leaf == kSentinel && r.ref >= 0)) {
-            if (trav && r.ref >= 0) {
-                if (!trav_node<false>(s, r, stack, status, wk)) {
-                    r.best = -1;
-                    r.ref = kSentinel;
-                    leaf = kSentinel;
-                    failed = true;
-                } else if (leaf == kSentinel && r.ref < 0 && r.ref != kSentinel) {
-                    leaf = r.ref;
-                    r.ref = r.sp > 0 ? stack[--r.sp] : kSentinel;
-                }
+        if (__any_sync(kFull, trav && leaf == kSentinel && r.ref >= 0)) {
+            do {  // two visits per vote: half the votes, and a lane that reaches its leaf goes on speculatively
+                visit(trav);
+                visit(trav);
+            } while (!search_done(__ballot_sync(kFull, trav && leaf == kSentinel && r.ref >= 0), tracing_now));
+            if (trav && over_budget<kCheck>(s, r, status)) {
+                r.best = -1;
+                r.ref = leaf = kSentinel;
             }
-            if (search_done(__ballot_sync(kFull, trav && leaf == kSentinel && r.ref >= 0), tracing_now)) break;
         }
         if (trav) {
             if (leaf != kSentinel) {
                 trav_test_leaf<false>(s, r, leaf, wk);
                 leaf = kSentinel;
             }
-            if (failed || r.ref == kSentinel) {
-                state = kWaitShade;
-                failed = false;
-            }
+            if (r.ref == kSentinel) state = kWaitShade;
         }
     }
     status = __reduce_or_sync(kFull, status);
@@ -498,16 +508,37 @@ __global__ void __launch_bounds__(128) wf_path_kernel(SceneView s, ChainView c, 
 // indices rebased), so the traversal's pointers are uniform over a warp and a
 // lane keeps only its set, the set's chain buffers and its root.
 
+// The 16-byte chunks of one node, moved in place from their positions for node
+// index `from` to those for index `to` (chunk c of node i lies at c ^ (i & 7));
+// from = 0 is the host's plain order.
+__device__ __forceinline__ void move_chunks(Bvh4Node* node, uint32_t from, uint32_t to) {
+    uint4* q = reinterpret_cast<uint4*>(node);
+    uint4 c[8];
+#pragma unroll
+    for (uint32_t k = 0; k < 8; ++k) c[k] = q[k];
+    const uint32_t x = (from ^ to) & 7u;
+#pragma unroll
+    for (uint32_t k = 0; k < 8; ++k) q[k ^ x] = c[k];
+}
+
+__global__ void swizzle_nodes_kernel(Bvh4Node* nodes, uint32_t n_nodes) {
+    const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < n_nodes) move_chunks(nodes + j, 0, j);
+}
+
 // Rebase one scene's nodes and triangles after they were copied into the
-// merged arrays at offsets node_off, tri_off, mat_off.
+// merged arrays at offsets node_off, tri_off, mat_off (nodes points at the
+// scene's first node there).
 __global__ void rebase_scene_kernel(Bvh4Node* nodes, uint32_t n_nodes, TriRecord* tris, uint32_t n_tris,
                                     int node_off, int tri_off, int mat_off) {
     const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j < n_nodes) {
-        int4 r = nodes[j].refs;
+        int4* refs = reinterpret_cast<int4*>(nodes + j) + (6u ^ (j & 7u));
+        int4 r = *refs;
         int* rr = &r.x;
         for (int q = 0; q < 4; ++q) rr[q] = rebase_ref(rr[q], node_off, tri_off);
-        nodes[j].refs = r;
+        *refs = r;
+        move_chunks(nodes + j, j, j + (uint32_t)node_off);
     }
     if (j < n_tris) tris[j].e1_mat.w = __int_as_float(__float_as_int(tris[j].e1_mat.w) + mat_off);
 }
@@ -543,6 +574,7 @@ __global__ void __launch_bounds__(128) wf_batch_step_kernel(const BatchEntry* en
 // prefix sums, copied to shared memory).  The lane logic is the single-set
 // path kernel's; per lane it keeps the set, its depth, the candidate buffer
 // and its stride, and starts each ray at the set's root in the merged scene.
+template <int kCheck>
 __global__ void __launch_bounds__(128, 7) wf_batch_path_kernel(SceneView m, const BatchEntry* entries, const int* roots,
                                                             const uint64_t* chain_off, uint32_t n_sets,
                                                             unsigned int* fetch) {
@@ -555,14 +587,24 @@ __global__ void __launch_bounds__(128, 7) wf_batch_path_kernel(SceneView m, cons
     const unsigned lt = (1u << lane) - 1u;
     unsigned status = 0;
     Work wk;
-    Trav r;
+    Trav r{};
     int stack[kStackSize];
     uint32_t state = kIdle, i = 0, set = 0, nst = 0;
     int v = 0, leaf = kSentinel, depth = 0;
-    bool failed = false, drained = false;
-    float3 T = f3(1.f, 1.f, 1.f), F = f3(0.f, 0.f, 0.f);
-    float u1 = 0.f, u2 = 0.f;       // the coordinates of vertex v
+    bool drained = false, lit = false;
+    float3 T = f3(1.f, 1.f, 1.f);
     const float* cand = nullptr;     // the candidate's buffer (pair layout, nst chains)
+    auto visit = [&](bool on) {      // as in the single-set path kernel
+        if (on && r.ref >= 0) {
+            if (!trav_node<kCheck, false>(m, r, stack, status, wk)) {
+                r.best = -1;
+                r.ref = leaf = kSentinel;
+            } else if (leaf == kSentinel && r.ref < 0 && r.ref != kSentinel) {
+                leaf = r.ref;
+                r.ref = r.sp > 0 ? stack[--r.sp] : kSentinel;
+            }
+        }
+    };
     while (true) {
         // shade the waiting lanes as a batch
         const unsigned waiting = __ballot_sync(kFull, state == kWaitShade);
@@ -571,18 +613,24 @@ __global__ void __launch_bounds__(128, 7) wf_batch_path_kernel(SceneView m, cons
             bool need_u = false;
             if (state == kWaitShade) {
                 bool live = false;
+                float3 F = f3(0.f, 0.f, 0.f);
+                if (lit) {
+                    const float4 f = __ldcs(entries[set].c.wf.fy + i);
+                    F = f3(f.x, f.y, f.z);
+                }
                 if (r.best >= 0) {
+                    float2 uv = make_float2(0.f, 0.f);
+                    if (v < depth)  // vertex v's coordinate pair, one 8-byte load
+                        uv = __ldcs(reinterpret_cast<const float2*>(cand) + (uint64_t)(1 + v) * nst + i);
                     float3 o = r.o, d = r.d;
-                    live = shade_vertex(m, r.best, r.tb, v, depth, v < depth ? u1 : 0.f, v < depth ? u2 : 0.f, o,
-                                        d, T, F);
+                    live = shade_vertex(m, r.best, r.tb, v, depth, uv.x, uv.y, o, d, T, F);
                     if (live) {
                         ++v;
                         trav_begin_at(r, o, d, roots[set]);
                         state = kTraverse;
-                        if (v < depth) {  // vertex v's coordinate pair, one 8-byte load
-                            const float2 uv = __ldcs(reinterpret_cast<const float2*>(cand) + (uint64_t)(1 + v) * nst + i);
-                            u1 = uv.x;
-                            u2 = uv.y;
+                        if (F.x != 0.f || F.y != 0.f || F.z != 0.f) {
+                            __stcs(entries[set].c.wf.fy + i, make_float4(F.x, F.y, F.z, 0.f));
+                            lit = true;
                         }
                     }
                 }
@@ -638,12 +686,10 @@ __global__ void __launch_bounds__(128, 7) wf_batch_path_kernel(SceneView m, cons
                     cand = __ldcs(e.c.wf.par + i) ? e.c.x : e.c.wf.y;
                     nst = (uint32_t)e.c.n;
                     depth = (int)e.c.depth;
-                    u1 = y.z;
-                    u2 = y.w;
                     float3 o, d;
                     camera_ray(e.s, y.x, y.y, o, d);
                     T = f3(1.f, 1.f, 1.f);
-                    F = f3(0.f, 0.f, 0.f);
+                    lit = false;
                     v = 0;
                     const int root = roots[set];
                     trav_begin_at(r, o, d, root);
@@ -662,34 +708,39 @@ __global__ void __launch_bounds__(128, 7) wf_batch_path_kernel(SceneView m, cons
             r.ref = r.sp > 0 ? stack[--r.sp] : kSentinel;
         }
         const unsigned tracing_now = __ballot_sync(kFull, trav);
-        while (__any_sync(kFull, trav && leaf == kSentinel && r.ref >= 0)) {
-            if (trav && r.ref >= 0) {
-                if (!trav_node<false>(m, r, stack, status, wk)) {
-                    r.best = -1;
-                    r.ref = kSentinel;
-                    leaf = kSentinel;
-                    failed = true;
-                } else if (leaf == kSentinel && r.ref < 0 && r.ref != kSentinel) {
-                    leaf = r.ref;
-                    r.ref = r.sp > 0 ? stack[--r.sp] : kSentinel;
-                }
+        if (__any_sync(kFull, trav && leaf == kSentinel && r.ref >= 0)) {
+            do {  // two visits per vote: half the votes, and a lane that reaches its leaf goes on speculatively
+                visit(trav);
+                visit(trav);
+            } while (!search_done(__ballot_sync(kFull, trav && leaf == kSentinel && r.ref >= 0), tracing_now));
+            if (trav && over_budget<kCheck>(m, r, status)) {
+                r.best = -1;
+                r.ref = leaf = kSentinel;
             }
-            if (search_done(__ballot_sync(kFull, trav && leaf == kSentinel && r.ref >= 0), tracing_now)) break;
         }
         if (trav) {
             if (leaf != kSentinel) {
                 trav_test_leaf<false>(m, r, leaf, wk);
                 leaf = kSentinel;
             }
-            if (failed || r.ref == kSentinel) {
-                state = kWaitShade;
-                failed = false;
-            }
+            if (r.ref == kSentinel) state = kWaitShade;
         }
     }
 }
 
 inline unsigned grid_for(uint64_t n, unsigned b) { return (unsigned)((n + b - 1) / b); }
+
+// Blocks of 128 threads of a persistent kernel that the device holds at once.
+template <class K>
+cudaError_t resident_blocks(int dev, K kernel, size_t shm, long long* blocks) {
+    int sms = 0, per_sm = 0;
+    cudaError_t r;
+    if ((r = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+        (r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 128, shm)) != cudaSuccess)
+        return r;
+    *blocks = (long long)sms * (per_sm > 0 ? per_sm : 1);
+    return cudaSuccess;
+}
 
 // The flow stages of a step (a chain's candidate lives in x when its parity
 // byte is 1, else in y).  Before the path kernel: y = T^{-1}(z) and u(y) of
@@ -737,26 +788,17 @@ KernelTimer::~KernelTimer() {
 
 cudaError_t launch_wavefront(const SceneView& s, const ChainView& c, uint64_t step_begin, uint32_t n_steps,
                              cudaStream_t st, int mode, KernelTimer* tm) {
-    static DeviceOnce once;  // per device: the path kernel's persistent grid
+    const int checks = trav_checks(s);
     long long path_blocks = 0;
-    {
-        cudaError_t e0 = once.get(
-            [](int dev, long long* v) {
-                int sms = 0, per_sm = 0;
-                cudaError_t r;
-                if ((r = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
-                    (r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wf_path_kernel, 128, 0)) !=
-                        cudaSuccess)
-                    return r;
-                *v = (long long)sms * (per_sm > 0 ? per_sm : 1);
-                return cudaSuccess;
-            },
-            &path_blocks);
-        if (e0 != cudaSuccess) return e0;
-    }
+    cudaError_t e = cudaSuccess;
+    with_checks(checks, [&](auto k) {
+        static DeviceOnce once;  // per device and check mode: the path kernel's persistent grid
+        e = once.get([](int dev, long long* v) { return resident_blocks(dev, wf_path_kernel<decltype(k)::value>, 0, v); },
+                     &path_blocks);
+    });
+    if (e != cudaSuccess) return e;
     const unsigned G = grid_for(c.n, 128);
     const bool has_flow = c.flow.D != 0;
-    cudaError_t e = cudaSuccess;
     auto mark = [&](int kind) {
         if (tm && e == cudaSuccess) e = tm->mark(kind, st);
     };
@@ -767,7 +809,9 @@ cudaError_t launch_wavefront(const SceneView& s, const ChainView& c, uint64_t st
         mark(KernelTimer::kStep);
         if (has_flow && (e = launch_flow_draws(c, st)) != cudaSuccess) return e;
         if (has_flow) mark(KernelTimer::kFlow);
-        wf_path_kernel<<<(unsigned)path_blocks, 128, 0, st>>>(s, c, mode != kModeDrain);
+        with_checks(checks, [&](auto kc) {
+            wf_path_kernel<kc()><<<(unsigned)path_blocks, 128, 0, st>>>(s, c, mode != kModeDrain);
+        });
         mark(KernelTimer::kPath);
         if (has_flow && (e = launch_flow_densities(c, st)) != cudaSuccess) return e;
         if (has_flow) mark(KernelTimer::kFlow);
@@ -779,6 +823,12 @@ cudaError_t launch_wavefront(const SceneView& s, const ChainView& c, uint64_t st
     return cudaGetLastError();
 }
 
+cudaError_t launch_swizzle_nodes(Bvh4Node* nodes, uint32_t n_nodes, cudaStream_t st) {
+    if (n_nodes == 0) return cudaSuccess;
+    swizzle_nodes_kernel<<<grid_for(n_nodes, 256), 256, 0, st>>>(nodes, n_nodes);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_rebase_scene(Bvh4Node* nodes, uint32_t n_nodes, TriRecord* tris, uint32_t n_tris, int node_off,
                                 int tri_off, int mat_off, cudaStream_t st) {
     const uint32_t n = n_nodes > n_tris ? n_nodes : n_tris;
@@ -787,27 +837,23 @@ cudaError_t launch_rebase_scene(Bvh4Node* nodes, uint32_t n_nodes, TriRecord* tr
     return cudaGetLastError();
 }
 
-cudaError_t batch_wavefront_grid(long long* blocks) {
-    static DeviceOnce once;  // per device: the batched path kernel's persistent grid
-    return once.get(
-        [](int dev, long long* v) {
-            int sms = 0, per_sm = 0;
-            cudaError_t r;
-            if ((r = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
-                (r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wf_batch_path_kernel, 128,
-                                                                   sizeof(uint64_t) * (kBatchMaxSets + 1))) !=
-                    cudaSuccess)
-                return r;
-            *v = (long long)sms * (per_sm > 0 ? per_sm : 1);
-            return cudaSuccess;
-        },
-        blocks);
+cudaError_t batch_wavefront_grid(int checks, long long* blocks) {
+    cudaError_t e = cudaSuccess;
+    with_checks(checks, [&](auto k) {
+        static DeviceOnce once;  // per device and check mode: the batched path kernel's persistent grid
+        e = once.get(
+            [](int dev, long long* v) {
+                return resident_blocks(dev, wf_batch_path_kernel<decltype(k)::value>, sizeof(uint64_t) * (kBatchMaxSets + 1), v);
+            },
+            blocks);
+    });
+    return e;
 }
 
 cudaError_t launch_batch_wavefront(const BatchWave& bw, BatchEntry* entries, uint32_t n_steps,
                                    const std::vector<ChainView>& flow_sets, cudaStream_t st) {
     long long blocks = 0;
-    cudaError_t e = batch_wavefront_grid(&blocks);
+    cudaError_t e = batch_wavefront_grid(bw.checks, &blocks);
     if (e != cudaSuccess) return e;
     if (bw.n_items == 0) return cudaSuccess;
     if (bw.n_sets == 0 || bw.n_sets > kBatchMaxSets) return cudaErrorInvalidValue;
@@ -820,8 +866,10 @@ cudaError_t launch_batch_wavefront(const BatchWave& bw, BatchEntry* entries, uin
         wf_batch_step_kernel<<<bw.n_items, 128, 0, st>>>(entries, bw.items, k, k > 0, 1);
         for (const ChainView& c : flow_sets)  // y = T^{-1}(z) and u(y) of the flow draws
             if ((e = launch_flow_draws(c, st)) != cudaSuccess) return e;
-        wf_batch_path_kernel<<<(unsigned)blocks, 128, shm, st>>>(bw.merged, entries, bw.roots, bw.chain_off,
-                                                                 bw.n_sets, bw.fetch);
+        with_checks(bw.checks, [&](auto kc) {
+            wf_batch_path_kernel<kc()><<<(unsigned)blocks, 128, shm, st>>>(bw.merged, entries, bw.roots, bw.chain_off,
+                                                                           bw.n_sets, bw.fetch);
+        });
         for (const ChainView& c : flow_sets)  // u(y) of the candidates that become states with p > 0
             if ((e = launch_flow_densities(c, st)) != cudaSuccess) return e;
     }

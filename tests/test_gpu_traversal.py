@@ -1,0 +1,58 @@
+"""The traversal's watchdog variants: a launch checks only the limits that can
+fire, and each variant gives the states of the one that checks both."""
+import numpy as np
+import pytest
+
+from paper_2409_07148_gb300 import jr, scenes
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(scene, sc, n, mode, limits, flags, steps=6):
+    ch = jr.Chains(scene, sc.width, sc.height, sc.depth, n, seed=11, flags=flags, burn_in=0)
+    ch.set_limits(*limits)
+    ch.set_execution(mode)
+    ch.advance(steps)
+    x, fpu = ch.get_state()
+    st = ch.stats()
+    return x, fpu, st
+
+
+# 1 and 33 chains: a lane alone and a warp plus one; 5000: many warps, ragged
+@pytest.mark.parametrize("n", [1, 33, 5000])
+@pytest.mark.parametrize("mode", ["wave", "mega"])
+@pytest.mark.parametrize("flags", [0, jr.JR_FLAG_MH])
+def test_check_variants_give_the_same_chains(n, mode, flags):
+    sc = scenes.cornell_spheres(width=64, height=64, depth=6, n_lon=40, n_lat=41)
+    scene = jr.Scene(sc)
+    nodes = scene.info()["n_nodes"]
+    assert 900 < nodes < 65536
+    ref = _run(scene, sc, n, mode, (0, 0), flags)            # neither limit can fire
+    visits = _run(scene, sc, n, mode, (nodes - 1, 0), flags)  # visits are counted, none runs out
+    both = _run(scene, sc, n, mode, (0, 16), flags)           # every push is compared, none runs out
+    for other in (visits, both):
+        assert other[2] == ref[2]
+        assert np.array_equal(other[0], ref[0])
+        assert np.array_equal(other[1], ref[1])
+
+
+@pytest.mark.parametrize("mode", ["wave", "mega"])
+def test_budget_counted_once_per_round_equals_counted_per_visit(mode):
+    """A budget that some rays exceed: the variant that compares once per round
+    (stack limit out of reach) marks the same rays as the one that compares at
+    every visit (a stack limit below the tree's bound, above what rays use)."""
+    sc = scenes.cornell_spheres(width=64, height=64, depth=4, n_lon=40, n_lat=41)
+    scene = jr.Scene(sc)
+    out = []
+    for limits in ((9, 0), (9, 16)):
+        ch = jr.Chains(scene, sc.width, sc.height, sc.depth, 4096, seed=3, flags=jr.JR_FLAG_MH, burn_in=0)
+        ch.set_limits(*limits)
+        ch.set_execution(mode)
+        ch.advance(4)
+        st = ch.stats(check=False)
+        assert st["status_word"] & jr.JR_STATUS_TRAVERSAL
+        assert not st["status_word"] & jr.JR_STATUS_STACK
+        out.append((st, *ch.get_state()))
+    assert out[0][0] == out[1][0]
+    assert np.array_equal(out[0][1], out[1][1])
+    assert np.array_equal(out[0][2], out[1][2])
