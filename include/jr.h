@@ -205,7 +205,9 @@ jr_status jr_advance_timed(jr_chains* chains, uint32_t n_steps, double ms_out[4]
 jr_status jr_advance_counted(jr_chains* chains, uint32_t n_steps, uint64_t work_out[3], void* stream);
 
 /* Threads per block of the megakernel for this chain set: a multiple of 32
- * in [32, 256] (default 128).  Results do not depend on it. */
+ * in [32, 256] (default 128).  Results do not depend on it.  (A launch whose
+ * chains all fit on the device at once spreads them over one-warp blocks
+ * instead.) */
 jr_status jr_set_block_size(jr_chains* chains, uint32_t block);
 
 /* Execution mode of jr_advance for this chain set (jr_advance_traced and

@@ -266,7 +266,7 @@ cudaError_t launch_step(const SceneView& s, const ChainView& c, uint64_t step_be
                         cudaStream_t st);
 cudaError_t launch_fold(const ChainView& c, cudaStream_t st);
 // JR_FLAG_MALA chain sets: n steps with Langevin local moves (megakernel, one
-// chain per thread, 128 threads per block); F, p and drift of stored states;
+// chain per thread, one-warp blocks); F, p and drift of stored states;
 // F [3][n] and dF/dx [3][D][n] of given states x [D][n].
 cudaError_t launch_step_mala(const SceneView& s, const ChainView& c, uint64_t step_begin, uint32_t n_steps,
                              uint8_t* tr_flags, float* tr_dt, int32_t* tr_pix, cudaStream_t st);

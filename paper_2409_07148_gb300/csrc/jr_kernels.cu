@@ -238,7 +238,7 @@ __device__ __forceinline__ void chain_steps(const SceneView& s, const ChainView&
 }
 
 // Both persistent kernels are capped at 64 registers (4 blocks of 256 threads
-// per SM): the 4-wide traversal would take 108, and the occupancy the cap buys
+// per SM): the 4-wide traversal would take 110, and the occupancy the cap buys
 // outweighs its small spill (measured: 5.0 -> 5.9e8 chain steps/s for the
 // megakernel, 5.9 -> 6.1e8 for the 64-scene batch).
 template <int kCheck, bool kTrace, bool kCount>
@@ -248,6 +248,25 @@ __global__ void __launch_bounds__(256, 4) step_kernel(SceneView s, ChainView c, 
     extern __shared__ float sh[];
     const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     chain_steps<kCheck, kTrace, kCount>(s, c, i, i < c.n, sh, step_begin, n_steps, tr_flags, tr_dt, tr_pix, work_out);
+}
+
+// The megakernel where all chains fit on the device at once: a warp holds only
+// `per_warp` chains, in its first lanes, so that the chains spread over all the
+// warps that can be resident.  Such a launch is bound by latency: a warp's step
+// lasts as long as the divergent paths of all its lanes together, so fewer lanes
+// per warp shorten it (1 000 chains, 16 steps of Cornell + spheres: 1 377 us
+// with 32 chains per warp, 1 024 with 16, 770 with 8, 570 with 4, 426 with 2, 340 with
+// one) while issue slots are left over.  Blocks of one warp, so that warps spread
+// evenly over the SMs, and no register cap below what 16 warps per SM leave: a
+// spill would lengthen the step (1 587 -> 1 377 us) and more warps would not be
+// resident anyway.
+template <int kCheck>
+__global__ void __launch_bounds__(32, 16) step_kernel_spread(SceneView s, ChainView c, uint64_t step_begin,
+                                                             uint32_t n_steps, uint32_t per_warp) {
+    extern __shared__ float sh[];
+    const uint64_t i = blockIdx.x * (uint64_t)per_warp + threadIdx.x;
+    const bool active = threadIdx.x < per_warp && i < c.n;
+    chain_steps<kCheck, false, false>(s, c, i, active, sh, step_begin, n_steps, nullptr, nullptr, nullptr, nullptr);
 }
 
 // ------------------------------------------------------------------ one chain per warp
@@ -602,13 +621,16 @@ __device__ __forceinline__ void chain_steps_mala(const SceneView& s, const Chain
     }
 }
 
+// One-warp blocks of per_warp chains, as in step_kernel_spread (4 steps of 1 000
+// chains on Cornell + spheres 728 -> 285 us, 8 steps of 32 768 1 930 -> 1 687 us).
 template <int kCheck, bool kTrace>
-__global__ void __launch_bounds__(128) step_kernel_mala(SceneView s, ChainView c, uint64_t step_begin,
-                                                        uint32_t n_steps, uint8_t* tr_flags, float* tr_dt,
-                                                        int32_t* tr_pix) {
+__global__ void __launch_bounds__(32, 16) step_kernel_mala(SceneView s, ChainView c, uint64_t step_begin,
+                                                           uint32_t n_steps, uint32_t per_warp, uint8_t* tr_flags,
+                                                           float* tr_dt, int32_t* tr_pix) {
     extern __shared__ float sh[];
-    const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    chain_steps_mala<kCheck, kTrace>(s, c, i, i < c.n, sh, step_begin, n_steps, tr_flags, tr_dt, tr_pix);
+    const uint64_t i = blockIdx.x * (uint64_t)per_warp + threadIdx.x;
+    const bool active = threadIdx.x < per_warp && i < c.n;
+    chain_steps_mala<kCheck, kTrace>(s, c, i, active, sh, step_begin, n_steps, tr_flags, tr_dt, tr_pix);
 }
 
 // F, p and the drift of the stored states (chain creation and jr_set_state).
@@ -826,6 +848,36 @@ __global__ void __launch_bounds__(256) fma_peak_kernel(uint32_t iters, float* si
 
 inline unsigned grid_for(uint64_t n, unsigned b) { return (unsigned)((n + b - 1) / b); }
 
+// Chains per warp for a kernel that gives each one-warp block that many chains:
+// the fewest with which kSpreadWarps warps per SM hold them all, or 0 where the
+// device cannot hold them all at once even in full warps: there the launch is
+// bound by throughput, which full warps have the most of.  kSpreadWarps: three
+// warps per scheduler; more of them, with fewer chains each, wait for one another
+// (10 007 chains, 32 steps of Cornell + spheres: 1 702 us at 8, 1 578 at 12,
+// 1 600 at 16; 30 000 chains, 16 steps: 1 431, 1 357, 1 375 us; 6 000 chains in the
+// 24-triangle box, 64 steps: 785, 842, 892 us).
+constexpr int kSpreadWarps = 12;
+template <class K>
+cudaError_t chains_per_warp(K kernel, size_t shm, uint64_t n, unsigned* per_warp) {
+    static DeviceOnce once;  // per device: its SM count
+    long long sms = 0;
+    cudaError_t e = once.get(
+        [](int dev, long long* v) {
+            int n = 0;
+            const cudaError_t r = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+            *v = n;
+            return r;
+        },
+        &sms);
+    int per_sm = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32, shm);
+    if (e != cudaSuccess) return e;
+    const uint64_t warps = (uint64_t)sms * (uint64_t)std::min(per_sm, kSpreadWarps);
+    const bool fits = per_sm > 0 && n <= 32 * (uint64_t)sms * (uint64_t)per_sm;
+    *per_warp = fits ? (unsigned)std::min<uint64_t>(32, (n + warps - 1) / warps) : 0u;
+    return cudaSuccess;
+}
+
 // A kernel as a type, so that a generic launcher has one set of statics per kernel.
 template <auto K>
 struct Kernel {
@@ -915,31 +967,34 @@ cudaError_t launch_step(const SceneView& s, const ChainView& c, uint64_t step_be
         return run(Kernel<step_kernel<kCheckAll, true, false>>{}, tr_flags, tr_dt, tr_pix, nullptr);
     cudaError_t e = cudaSuccess;
     with_checks(trav_checks(s), [&](auto k) {
-        e = run(Kernel<step_kernel<k(), false, false>>{}, nullptr, nullptr, nullptr, nullptr);
+        const auto spread = step_kernel_spread<decltype(k)::value>;
+        const size_t wshm = sizeof(float) * 2 * c.dim * 32;  // <= 8 KB
+        unsigned per_warp = 0;
+        if ((e = chains_per_warp(spread, wshm, c.n, &per_warp)) != cudaSuccess) return;
+        if (per_warp) {
+            spread<<<grid_for(c.n, per_warp), 32, wshm, st>>>(s, c, step_begin, n_steps, per_warp);
+            e = cudaGetLastError();
+        } else {
+            e = run(Kernel<step_kernel<k(), false, false>>{}, nullptr, nullptr, nullptr, nullptr);
+        }
     });
     return e;
 }
 
 cudaError_t launch_step_mala(const SceneView& s, const ChainView& c, uint64_t step_begin, uint32_t n_steps,
                              uint8_t* tr_flags, float* tr_dt, int32_t* tr_pix, cudaStream_t st) {
-    const unsigned B = 128;
-    const size_t shm = sizeof(float) * 4 * c.dim * B;  // <= 4 * 32 * 128 * 4 = 64 KB
-    const unsigned G = grid_for(c.n, B);
+    const size_t shm = sizeof(float) * 4 * c.dim * 32;  // <= 16 KB
     const auto run = [&](auto kernel) {
-        static DeviceOnce once;  // per device and variant
-        const cudaError_t e = once.get(
-            [&](int, long long*) {
-                return cudaFuncSetAttribute(kernel.value, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)(sizeof(float) * 4 * kMaxDim * 128));
-            },
-            nullptr);
+        unsigned per_warp = 0;
+        const cudaError_t e = chains_per_warp(kernel, shm, c.n, &per_warp);
         if (e != cudaSuccess) return e;
-        kernel.value<<<G, B, shm, st>>>(s, c, step_begin, n_steps, tr_flags, tr_dt, tr_pix);
+        if (per_warp == 0) per_warp = 32;
+        kernel<<<grid_for(c.n, per_warp), 32, shm, st>>>(s, c, step_begin, n_steps, per_warp, tr_flags, tr_dt, tr_pix);
         return cudaGetLastError();
     };
-    if (tr_flags || tr_dt || tr_pix) return run(Kernel<step_kernel_mala<kCheckAll, true>>{});
+    if (tr_flags || tr_dt || tr_pix) return run(step_kernel_mala<kCheckAll, true>);
     cudaError_t e = cudaSuccess;
-    with_checks(trav_checks(s), [&](auto k) { e = run(Kernel<step_kernel_mala<k(), false>>{}); });
+    with_checks(trav_checks(s), [&](auto k) { e = run(step_kernel_mala<decltype(k)::value, false>); });
     return e;
 }
 

@@ -56,3 +56,18 @@ def test_budget_counted_once_per_round_equals_counted_per_visit(mode):
     assert out[0][0] == out[1][0]
     assert np.array_equal(out[0][1], out[1][1])
     assert np.array_equal(out[0][2], out[1][2])
+
+
+# 1 and 7: a single warp; 1824 and 1825: one chain per warp on 152 SMs x 12 warps, and the first with
+# two; 58369: full warps; 90001: more than the device holds at once
+@pytest.mark.parametrize("n", [1, 7, 1824, 1825, 58369, 90001])
+def test_spread_megakernel_equals_wavefront(n):
+    """The same device functions on the same streams: the chains agree except
+    where a rounding that the compiler places differently decides a tie."""
+    sc = scenes.cornell_spheres(width=64, height=64, depth=5, n_lon=40, n_lat=41)
+    scene = jr.Scene(sc)
+    (xa, fa, sa), (xb, fb, sb) = (_run(scene, sc, n, mode, (0, 0), jr.JR_FLAG_MH, steps=3) for mode in ("mega", "wave"))
+    same = np.all(xa == xb, axis=0)
+    assert np.mean(~same) <= 1e-4
+    assert np.allclose(fa[:, same], fb[:, same], rtol=1e-5, atol=0)
+    assert abs(sa["accepted"] - sb["accepted"]) <= 1e-4 * n
