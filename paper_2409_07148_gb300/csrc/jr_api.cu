@@ -1379,6 +1379,12 @@ jr_status jr_flow_train_rows(jr_flow* f, const float* x_dev, const float* w_dev,
 
 namespace {
 
+// Without a flow, a drain's steps run in the wavefront while more chains than
+// this may be open, then in launches of drain_kernel of at most kDrainTailSteps
+// steps (which bounds one launch).  The line is where the wavefront's packed
+// warps stop paying for its waiting on the longest path of every step.
+constexpr uint32_t kDrainTailChains = 1u << 16, kDrainTailSteps = 4096;
+
 // Drain: advance only the chains that are inside a tour until every tour has
 // ended (a kill ends the tour and the chain); the steps are regular steps of
 // Alg. 2 for those chains.  Returns the chains still in a tour after
@@ -1396,8 +1402,9 @@ jr_status drain_impl(jr_chains* c, uint32_t max_steps, uint64_t* remaining, cuda
     JR_CUDA(cudaMemsetAsync(c->view.counters + 3, 0, sizeof(unsigned long long), st), who);
     const uint64_t s0 = c->steps;
     uint32_t group = 1;
-    while (active > 0 && k < max_steps) {
-        const uint32_t g = std::min(group, max_steps - k);
+    const bool flow = c->view.flow.D != 0;  // u(y) of each candidate comes from the wavefront's flow launches
+    while (active > 0 && k < max_steps && (flow || active > kDrainTailChains)) {
+        const uint32_t g = flow ? std::min(group, max_steps - k) : 1u;
         // one launch sequence per group: a single closing finish launch, not one per step
         JR_CUDA(launch_wavefront(c->scene_view(), c->view, s0 + k, g, st, kModeDrain), who);
         k += g;
@@ -1405,6 +1412,16 @@ jr_status drain_impl(jr_chains* c, uint32_t max_steps, uint64_t* remaining, cuda
                 who);
         JR_CUDA(cudaStreamSynchronize(st), who);
         group = std::min<uint32_t>(2 * group, 16);
+    }
+    while (active > 0 && k < max_steps) {  // few open tours: each runs to its end without waiting for the others
+        const uint32_t g = std::min(kDrainTailSteps, max_steps - k);
+        unsigned long long* ctl = c->view.counters + kCounterDrain;
+        JR_CUDA(launch_drain(c->scene_view(), c->view, c->view.wf.done, s0 + k, g, ctl, st), who);
+        k += g;
+        unsigned long long open = 0;
+        JR_CUDA(cudaMemcpyAsync(&open, ctl + 1, sizeof(open), cudaMemcpyDeviceToHost, st), who);
+        JR_CUDA(cudaStreamSynchronize(st), who);
+        active = (unsigned int)open;
     }
     if (k > 0) {
         unsigned long long mark = 0;

@@ -21,6 +21,7 @@ constexpr uint32_t kNodeVisitBudget = 1u << 16;  // per ray; exceeding it is a w
 
 constexpr uint32_t kTagStep = 0, kTagInit = 1, kTagPt = 2, kTagRestart = 3;
 constexpr int kCounters = 8;   // ChainView::counters entries
+constexpr int kCounterDrain = 6;  // [6], [7]: launch_drain's ctl
 constexpr int kCounterPSum = 5;  // MH: sum of p over the large-step proposals (double)
 constexpr uint64_t kWavefrontMinChains = 1u << 18;  // JR_EXEC_AUTO picks the wavefront from here up
 
@@ -147,7 +148,8 @@ struct ChainView {
     double4_32a* acc64;  // [H*W]
     // [0] J (MH: large-step proposals), [1] local steps (MH: small-step
     // proposals), [2] accepted, [3] drain mark, [4] unused, [5] MH: the sum of
-    // p over the large-step proposals (a double's bits), [6..7] unused
+    // p over the large-step proposals (a double's bits), [6..7] the drain
+    // kernel's fetch cursor and open tours
     unsigned long long* counters;
     unsigned int* status;
     uint64_t n;
@@ -264,6 +266,11 @@ cudaError_t launch_step_warp(const SceneView& s, const ChainView& c, uint64_t st
 cudaError_t launch_step(const SceneView& s, const ChainView& c, uint64_t step_begin, uint32_t n_steps,
                         uint8_t* tr_flags, float* tr_dt, int32_t* tr_pix, unsigned long long* work_out, int block,
                         cudaStream_t st);
+// The open tours of a drain to their ends (no flow): every chain with skip[i] = 0
+// (all of them when skip is null) takes up to n_steps drain steps from step_begin.
+// ctl [2]: fetch cursor, chains still open afterwards.  Sets c.wf.done.
+cudaError_t launch_drain(const SceneView& s, const ChainView& c, const uint8_t* skip, uint64_t step_begin,
+                         uint32_t n_steps, unsigned long long* ctl, cudaStream_t st);
 cudaError_t launch_fold(const ChainView& c, cudaStream_t st);
 // JR_FLAG_MALA chain sets: n steps with Langevin local moves (megakernel, one
 // chain per thread, one-warp blocks); F, p and drift of stored states;

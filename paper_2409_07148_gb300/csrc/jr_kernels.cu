@@ -82,6 +82,50 @@ __global__ void reeval_kernel(SceneView s, ChainView c) {
     flush_status(status, c.status);
 }
 
+// Alg. 2: holding time t1 ~ Exp(1); killing time t2 ~ Exp(k), k = c~ u / p.  True:
+// the local branch; dt gets the time the state is held for.
+__device__ __forceinline__ bool restore_clocks(const ChainView& c, const uint4& r0, float p, float u, float& dt) {
+    const float E1 = -logf(1.0f - u01(r0.x));
+    const float E2 = -logf(1.0f - u01(r0.y));
+    const float t2 = p > 0.0f ? E2 * p / (c.c_tilde * u) : 0.0f;
+    const bool local = E1 < t2;  // a tie goes to the killing branch
+    dt = local ? E1 : t2;
+    if (c.flags & JR_FLAG_RAO_BLACKWELL) dt = p > 0.0f ? p / (p + c.c_tilde * u) : 0.0f;
+    return local;
+}
+
+// Candidate y of step `step` (cand[d * B]): a Gaussian small step from cur
+// (local) or a fresh draw from mu.
+__device__ __forceinline__ void propose(const ChainView& c, uint32_t chain, uint64_t step, bool local,
+                                        const float* cur, float* cand, uint32_t B) {
+    const int D = (int)c.dim;
+    const float sigma = c.sigma;
+    for (int b = 0; 4 * b < D; ++b) {
+        const uint4 r = draw(c.seed, kTagStep, (uint32_t)(b + 1), chain, step);
+        const int d0 = 4 * b;
+        if (local) {
+            float sn, cs;
+            float R = sqrtf(-2.0f * logf(1.0f - u01(r.x)));
+            sincospif(2.0f * u01(r.y), &sn, &cs);
+            cand[d0 * B] = wrap01(cur[d0 * B] + sigma * R * cs);
+            cand[(d0 + 1) * B] = wrap01(cur[(d0 + 1) * B] + sigma * R * sn);
+            if (d0 + 2 < D) {
+                R = sqrtf(-2.0f * logf(1.0f - u01(r.z)));
+                sincospif(2.0f * u01(r.w), &sn, &cs);
+                cand[(d0 + 2) * B] = wrap01(cur[(d0 + 2) * B] + sigma * R * cs);
+                cand[(d0 + 3) * B] = wrap01(cur[(d0 + 3) * B] + sigma * R * sn);
+            }
+        } else {
+            cand[d0 * B] = u01(r.x);
+            cand[(d0 + 1) * B] = u01(r.y);
+            if (d0 + 2 < D) {
+                cand[(d0 + 2) * B] = u01(r.z);
+                cand[(d0 + 3) * B] = u01(r.w);
+            }
+        }
+    }
+}
+
 // n_steps of Alg. 2 for chain i of set c (thread tid of the block; `active`
 // false for threads without a chain).  Every thread of the block calls it;
 // sh holds [2][D][blockDim] floats.
@@ -106,9 +150,7 @@ __device__ __forceinline__ void chain_steps(const SceneView& s, const ChainView&
         float* cur = buf0;
         float* cand = buf1;
         const uint32_t chain = c.chain_offset + (uint32_t)i;
-        const float c_tilde = c.c_tilde, sigma = c.sigma;
         const float WH = (float)c.width * (float)c.height;
-        const bool rb = (c.flags & JR_FLAG_RAO_BLACKWELL) != 0;
         for (uint32_t st = 0; st < n_steps; ++st) {
             const uint64_t step = step_begin + st;
             const uint4 r0 = draw(c.seed, kTagStep, 0, chain, step);
@@ -122,13 +164,7 @@ __device__ __forceinline__ void chain_steps(const SceneView& s, const ChainView&
                 local = !(u01(r0.x) < c.large_step);
                 dt = step >= c.burn_in ? 1.0f : 0.0f;
             } else {
-                // Alg. 2: holding time t1 ~ Exp(1); killing time t2 ~ Exp(k), k = c~ u / p.
-                const float E1 = -logf(1.0f - u01(r0.x));
-                const float E2 = -logf(1.0f - u01(r0.y));
-                const float t2 = p > 0.0f ? E2 * p / (c_tilde * u) : 0.0f;
-                local = E1 < t2;  // a tie goes to the killing branch
-                dt = local ? E1 : t2;
-                if (rb) dt = p > 0.0f ? p / (p + c_tilde * u) : 0.0f;
+                local = restore_clocks(c, r0, p, u, dt);
             }
             int32_t pix = -1;
             if (dt > 0.0f && p > 0.0f) {
@@ -139,34 +175,10 @@ __device__ __forceinline__ void chain_steps(const SceneView& s, const ChainView&
                 px = min(px, c.width - 1);
                 py = min(py, c.height - 1);
                 pix = (int32_t)(py * c.width + px);
-                const float wgt = mh ? WH / p : c_tilde * dt * WH / p;
+                const float wgt = mh ? WH / p : c.c_tilde * dt * WH / p;
                 atomicAdd(c.fb + pix, make_float4(wgt * Fr, wgt * Fg, wgt * Fb, dt));
             }
-            // candidate y: Gaussian small step (local) or a fresh draw from mu
-            for (int b = 0; 4 * b < D; ++b) {
-                const uint4 r = draw(c.seed, kTagStep, (uint32_t)(b + 1), chain, step);
-                const int d0 = 4 * b;
-                if (local) {
-                    float sn, cs;
-                    float R = sqrtf(-2.0f * logf(1.0f - u01(r.x)));
-                    sincospif(2.0f * u01(r.y), &sn, &cs);
-                    cand[d0 * B] = wrap01(cur[d0 * B] + sigma * R * cs);
-                    cand[(d0 + 1) * B] = wrap01(cur[(d0 + 1) * B] + sigma * R * sn);
-                    if (d0 + 2 < D) {
-                        R = sqrtf(-2.0f * logf(1.0f - u01(r.z)));
-                        sincospif(2.0f * u01(r.w), &sn, &cs);
-                        cand[(d0 + 2) * B] = wrap01(cur[(d0 + 2) * B] + sigma * R * cs);
-                        cand[(d0 + 3) * B] = wrap01(cur[(d0 + 3) * B] + sigma * R * sn);
-                    }
-                } else {
-                    cand[d0 * B] = u01(r.x);
-                    cand[(d0 + 1) * B] = u01(r.y);
-                    if (d0 + 2 < D) {
-                        cand[(d0 + 2) * B] = u01(r.z);
-                        cand[(d0 + 3) * B] = u01(r.w);
-                    }
-                }
-            }
+            propose(c, chain, step, local, cur, cand, B);
             const float3 Fy = eval_path_w<kCheck, kCount>(s, mask, true, (int)c.depth, cand, B, nullptr, 0, status, work);
             const float py_ = lum(Fy);
             bool accept;
@@ -267,6 +279,128 @@ __global__ void __launch_bounds__(32, 16) step_kernel_spread(SceneView s, ChainV
     const uint64_t i = blockIdx.x * (uint64_t)per_warp + threadIdx.x;
     const bool active = threadIdx.x < per_warp && i < c.n;
     chain_steps<kCheck, false, false>(s, c, i, active, sh, step_begin, n_steps, nullptr, nullptr, nullptr, nullptr);
+}
+
+// ------------------------------------------------------------------ drain tail
+// The open tours of a drain, each run to its end in one launch: lane = chain,
+// one-warp blocks, chains fetched from [0, n) (those with done[i] skipped) as
+// lanes become free.  A chain takes steps step_begin, step_begin + 1, ... of Alg. 2
+// until a kill ends its tour (J += 1, done = 1) or n_steps are taken; a chain
+// still open then is stored and counted in ctl[1] (ctl[0]: the fetch cursor).
+//
+// The tail of a drain is a few hundred chains with tours of up to several
+// hundred steps.  In the wavefront every step waits for the longest of their
+// paths and for three launches over all chains; here a chain waits for no other
+// but the few in its warp, so the drain lasts as long as its longest tour.
+template <int kCheck>
+__global__ void __launch_bounds__(32, 16) drain_kernel(SceneView s, ChainView c, const uint8_t* skip,
+                                                       uint64_t step_begin, uint32_t n_steps,
+                                                       unsigned long long* ctl) {
+    extern __shared__ float sh[];
+    constexpr uint32_t B = 32;
+    const int lane = threadIdx.x;
+    const float WH = (float)c.width * (float)c.height;
+    const uint64_t end = step_begin + n_steps;
+    float* cur = sh + lane;
+    float* cand = sh + (size_t)c.dim * B + lane;
+    uint32_t nJ = 0, nL = 0, nA = 0, open = 0;
+    unsigned status = 0;
+    Work work;
+    bool live = false, drained = false;
+    uint64_t i = 0, step = step_begin, mark = 0;
+    float Fr = 0.f, Fg = 0.f, Fb = 0.f, p = 0.f, u = 1.f;
+    // The start of step `step`: clocks and splat.  False: the tour ends here.
+    auto begin_step = [&](float x0, float x1) {
+        float dt;
+        const bool local = restore_clocks(c, draw(c.seed, kTagStep, 0, c.chain_offset + (uint32_t)i, step), p, u, dt);
+        if (dt > 0.0f && p > 0.0f) {
+            const uint32_t px = min((uint32_t)((double)x0 * (double)c.width), c.width - 1);
+            const uint32_t py = min((uint32_t)((double)x1 * (double)c.height), c.height - 1);
+            const float wgt = c.c_tilde * dt * WH / p;
+            atomicAdd(c.fb + (py * c.width + px), make_float4(wgt * Fr, wgt * Fg, wgt * Fb, dt));
+        }
+        if (local) {
+            mark = max(mark, step + 1);
+        } else {
+            nJ++;
+            c.wf.done[i] = 1;
+        }
+        return local;
+    };
+    while (true) {
+        while (__any_sync(0xffffffffu, !live && !drained)) {  // free lanes take chains until one is in a tour
+            const unsigned want = __ballot_sync(0xffffffffu, !live && !drained);
+            unsigned long long base = 0;
+            if (lane == 0) base = atomicAdd(ctl, (unsigned long long)__popc(want));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (!live && !drained) {
+                i = base + __popc(want & ((1u << lane) - 1u));
+                drained = i >= c.n;
+                if (!drained && !(skip && skip[i])) {
+                    p = c.fpu[3 * c.n + i];
+                    step = step_begin;
+                    if (!(p > 0.0f)) {  // k = inf: killed at once, nothing to splat
+                        nJ++;
+                        c.wf.done[i] = 1;
+                    } else {
+                        Fr = c.fpu[0 * c.n + i];
+                        Fg = c.fpu[1 * c.n + i];
+                        Fb = c.fpu[2 * c.n + i];
+                        u = c.fpu[4 * c.n + i];
+                        load_coords(c, i, cur, B);
+                        live = begin_step(cur[0], cur[B]);
+                    }
+                }
+            }
+        }
+        if (!__any_sync(0xffffffffu, live)) break;
+        if (live) propose(c, c.chain_offset + (uint32_t)i, step, true, cur, cand, B);
+        const float3 Fy = eval_path_w<kCheck, false>(s, 0xffffffffu, live, (int)c.depth, cand, B, nullptr, 0, status, work);
+        if (live) {
+            const float py = lum(Fy);
+            const bool accept = u01(draw(c.seed, kTagStep, 0, c.chain_offset + (uint32_t)i, step).z) * p < py;
+            nL++;
+            nA += accept;
+            if (accept) {
+                float* t = cur;
+                cur = cand;
+                cand = t;
+                Fr = Fy.x;
+                Fg = Fy.y;
+                Fb = Fy.z;
+                p = py;
+                u = 1.0f;
+            }
+            ++step;
+            const bool last = step == end;
+            if (last) open++;
+            else live = begin_step(cur[0], cur[B]);
+            if (last || !live) {
+                live = false;
+                float2* x2 = reinterpret_cast<float2*>(c.x);
+                for (int k = 0; 2 * k < (int)c.dim; ++k)
+                    x2[(uint64_t)k * c.n + i] = make_float2(cur[2 * k * B], cur[(2 * k + 1) * B]);
+                c.fpu[0 * c.n + i] = Fr;
+                c.fpu[1 * c.n + i] = Fg;
+                c.fpu[2 * c.n + i] = Fb;
+                c.fpu[3 * c.n + i] = p;
+                c.fpu[4 * c.n + i] = u;
+            }
+        }
+    }
+    nJ = __reduce_add_sync(0xffffffffu, nJ);
+    nL = __reduce_add_sync(0xffffffffu, nL);
+    nA = __reduce_add_sync(0xffffffffu, nA);
+    open = __reduce_add_sync(0xffffffffu, open);
+    status = __reduce_or_sync(0xffffffffu, status);
+    if (mark) atomicMax(c.counters + 3, (unsigned long long)mark);
+    if (lane == 0) {
+        if (nJ) atomicAdd(c.counters + 0, (unsigned long long)nJ);
+        if (nL) atomicAdd(c.counters + 1, (unsigned long long)nL);
+        if (nA) atomicAdd(c.counters + 2, (unsigned long long)nA);
+        if (open) atomicAdd(ctl + 1, (unsigned long long)open);
+        flush_status(status, c.status);
+    }
 }
 
 // ------------------------------------------------------------------ one chain per warp
@@ -977,6 +1111,33 @@ cudaError_t launch_step(const SceneView& s, const ChainView& c, uint64_t step_be
         } else {
             e = run(Kernel<step_kernel<k(), false, false>>{}, nullptr, nullptr, nullptr, nullptr);
         }
+    });
+    return e;
+}
+
+cudaError_t launch_drain(const SceneView& s, const ChainView& c, const uint8_t* skip, uint64_t step_begin,
+                         uint32_t n_steps, unsigned long long* ctl, cudaStream_t st) {
+    const size_t shm = sizeof(float) * 2 * c.dim * 32;  // <= 8 KB
+    cudaError_t e = cudaMemsetAsync(ctl, 0, 2 * sizeof(unsigned long long), st);
+    if (e != cudaSuccess) return e;
+    with_checks(trav_checks(s), [&](auto k) {
+        static DeviceOnce once;  // per device and variant: its SM count
+        const auto kernel = drain_kernel<decltype(k)::value>;
+        long long sms = 0;
+        e = once.get(
+            [](int dev, long long* v) {
+                int n = 0;
+                const cudaError_t r = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+                *v = n;
+                return r;
+            },
+            &sms);
+        int per_sm = 0;
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32, shm);
+        if (e != cudaSuccess) return;
+        const uint64_t blocks = std::min<uint64_t>((uint64_t)sms * (per_sm > 0 ? per_sm : 1), (c.n + 31) / 32);
+        kernel<<<(unsigned)blocks, 32, shm, st>>>(s, c, skip, step_begin, n_steps, ctl);
+        e = cudaGetLastError();
     });
     return e;
 }

@@ -71,3 +71,29 @@ def test_spread_megakernel_equals_wavefront(n):
     assert np.mean(~same) <= 1e-4
     assert np.allclose(fa[:, same], fb[:, same], rtol=1e-5, atol=0)
     assert abs(sa["accepted"] - sb["accepted"]) <= 1e-4 * n
+
+
+# 70000 chains drain in the wavefront first and in the drain kernel afterwards, their shards in the
+# drain kernel alone; 1 step: every tour that survives it is reported open; 4097: more than one launch
+@pytest.mark.parametrize("max_steps", [1, 3, 4097])
+@pytest.mark.parametrize("rao", [0, jr.JR_FLAG_RAO_BLACKWELL])
+def test_drain_kernel_equals_wavefront_drain(max_steps, rao):
+    sc = scenes.furnace(width=32, height=32, depth=3, albedo=0.6, emission=20.0)
+    scene = jr.Scene(sc)
+
+    def drain(offset, n):
+        ch = jr.Chains(scene, sc.width, sc.height, sc.depth, n, seed=5, chain_offset=offset, flags=rao)
+        ch.advance(2)
+        left = jr.complete_tours(ch, max_steps)
+        return left, ch.stats(), ch.accumulator()
+
+    whole = drain(0, 70000)
+    parts = [drain(0, 35000), drain(35000, 35000)]
+    assert whole[0] == sum(p[0] for p in parts)
+    assert (whole[0] > 0) == (max_steps < 4097)
+    for key in ("regenerations", "local_steps", "accepted"):
+        assert whole[1][key] == sum(p[1][key] for p in parts)
+    assert whole[1]["steps_per_chain"] == max(p[1]["steps_per_chain"] for p in parts)
+    acc = sum(p[2] for p in parts)
+    # FP32 sums of up to a few thousand positive terms per pixel in another order
+    assert np.allclose(whole[2], acc, rtol=1e-4, atol=0)
