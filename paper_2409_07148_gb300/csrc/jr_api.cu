@@ -1306,6 +1306,7 @@ jr_status jr_flow_gradient(jr_flow* f, const float* x_dev, const float* w_dev, u
     float* buf = nullptr;  // gradient, then the weight sum and the loss
     JR_CUDA(dev_alloc(&buf, P + 2), "jr_flow_gradient");
     cudaError_t e = cudaMemsetAsync(buf, 0, sizeof(float) * (P + 2), st);
+    if (e == cudaSuccess) e = launch_flow_wsum(w_dev, nullptr, off, batch, buf + P, 1, 1, st);
     if (e == cudaSuccess) e = launch_flow_train_step(f->view(0.f), x_dev, w_dev, n, off, batch, buf, buf + P, buf + P + 1, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(grad_host, buf, sizeof(float) * P, cudaMemcpyDeviceToHost, st);
     float tail[2] = {0.f, 0.f};
@@ -1345,23 +1346,32 @@ jr_status jr_flow_train_rows(jr_flow* f, const float* x_dev, const float* w_dev,
             return cuda_fail(e, "jr_flow_train (optimiser state)");
         }
     }
-    float* scal = nullptr;  // [iters][2]: minibatch weight sum, loss
-    JR_CUDA(dev_alloc(&scal, 2 * (size_t)std::max<uint32_t>(iters, 1)), "jr_flow_train");
-    cudaError_t e = cudaMemsetAsync(scal, 0, sizeof(float) * 2 * std::max<uint32_t>(iters, 1), st);
+    std::vector<uint64_t> offs(iters);
     uint64_t rng = seed * 0x9E3779B97F4A7C15ull + 0xD1B54A32D192ED03ull;
-    for (uint32_t it = 0; it < iters && e == cudaSuccess; ++it) {
+    for (uint32_t it = 0; it < iters; ++it) {
         rng ^= rng >> 30;  // splitmix64 (Steele, Lea, Flood 2014): the minibatch window
         rng *= 0xBF58476D1CE4E5B9ull;
         rng ^= rng >> 27;
         rng *= 0x94D049BB133111EBull;
         rng ^= rng >> 31;
-        const uint64_t off = rng % (n_rows - batch + 1);
-        if ((e = cudaMemsetAsync(f->grad, 0, sizeof(float) * P, st)) != cudaSuccess) break;
-        if ((e = launch_flow_train_step(f->view(0.f), x_dev, w_dev, n, off, batch, f->grad, scal + 2 * it,
+        offs[it] = rng % (n_rows - batch + 1);
+    }
+    // [iters][2] minibatch weight sum and loss, then the windows' offsets [iters]
+    float* scal = nullptr;
+    JR_CUDA(dev_alloc(&scal, 4 * (size_t)std::max<uint32_t>(iters, 1)), "jr_flow_train");
+    uint64_t* offs_dev = reinterpret_cast<uint64_t*>(scal + 2 * (size_t)std::max<uint32_t>(iters, 1));
+    cudaError_t e = cudaMemsetAsync(scal, 0, sizeof(float) * 2 * std::max<uint32_t>(iters, 1), st);
+    if (iters > 0) {
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(offs_dev, offs.data(), sizeof(uint64_t) * iters, cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = launch_flow_wsum(w_dev, offs_dev, 0, batch, scal, 2, iters, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(f->grad, 0, sizeof(float) * P, st);
+    }
+    for (uint32_t it = 0; it < iters && e == cudaSuccess; ++it) {
+        if ((e = launch_flow_train_step(f->view(0.f), x_dev, w_dev, n, offs[it], batch, f->grad, scal + 2 * it,
                                         scal + 2 * it + 1, st)) != cudaSuccess)
             break;
-        if ((e = launch_adam(f->master, f->grad, f->adam_m, f->adam_v, P, lr, ++f->adam_t, st)) != cudaSuccess) break;
-        if ((e = launch_flow_pack(f->master, f->wb, f->bias, f->AK, st)) != cudaSuccess) break;
+        e = launch_adam(f->master, f->grad, f->adam_m, f->adam_v, f->D, lr, ++f->adam_t, f->wb, f->bias, st);
     }
     if (e == cudaSuccess) e = launch_flow_pack_ws(f->master, f->ws, f->AK, st);
     std::vector<float> h(2 * (size_t)std::max<uint32_t>(iters, 1));

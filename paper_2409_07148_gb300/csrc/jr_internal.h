@@ -339,12 +339,18 @@ __host__ __device__ inline size_t flow_layer_floats(uint32_t D) {
 cudaError_t launch_snapshot(const ChainView& c, float* x_out, float* w_out, cudaStream_t st);
 cudaError_t launch_snapshot_append(const ChainView& c, float* x_ring, float* w_ring, uint64_t cap,
                                    unsigned long long* total, cudaStream_t st);
+// Weight sums of `count` minibatch windows w[off_k .. off_k + batch) into out[k * stride];
+// off_k = offs[k] (device), or off when offs is null.
+cudaError_t launch_flow_wsum(const float* w, const uint64_t* offs, uint64_t off, uint32_t batch, float* out,
+                             uint32_t stride, uint32_t count, cudaStream_t st);
 // One minibatch of the time-weighted maximum-likelihood loss: gradient into
-// grad (added), minibatch weight sum into *wsum (added), loss into *loss (added).
+// grad (added), loss into *loss (added); wsum: the minibatch's weight sum (device).
 cudaError_t launch_flow_train_step(const FlowView& f, const float* x, const float* w, uint64_t n, uint64_t off,
-                                   uint32_t batch, float* grad, float* wsum, float* loss, cudaStream_t st);
-cudaError_t launch_adam(float* p, const float* g, float* m, float* v, uint64_t count, float lr, uint64_t t,
-                        cudaStream_t st);
+                                   uint32_t batch, float* grad, const float* wsum, float* loss, cudaStream_t st);
+// One Adam step of a flow over D dimensions on its master parameters p; zeroes g
+// and brings the training copy (wb, bias) up to date.
+cudaError_t launch_adam(float* p, float* g, float* m, float* v, uint32_t D, float lr, uint64_t t, __nv_bfloat16* wb,
+                        float* bias, cudaStream_t st);
 // image = accumulator / J (Jump Restore), or b_hat accumulator / mh_samples
 // with b_hat = (sum of p over large steps) / (large steps) (MH, JR_FLAG_MH).
 cudaError_t launch_resolve(const ChainView& c, float* rgb, uint64_t mh_samples, cudaStream_t st);

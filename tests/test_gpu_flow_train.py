@@ -82,3 +82,42 @@ def test_training_fits_a_known_density(J):
     p = f.get_params().reshape(w.shape)
     q = np.exp(FL.log_density(perm, p, G.astype(np.float64))[0])
     assert abs(q.mean() - 1.0) < 0.05
+
+
+# one row, one row short of a tile, a tile and a row; the smallest D, an odd number of
+# coordinate pairs, and the largest D
+@pytest.mark.parametrize("D", [2, 6, 32])
+@pytest.mark.parametrize("rows", [1, 63, 65])
+def test_gradient_at_the_tile_edges(J, D, rows):
+    import torch
+    perm, w = _flow(D, 60 + D, 0.1)
+    f = J.Flow(D, perm, w)
+    rng = np.random.default_rng(100 * D + rows)
+    n = rows + 7
+    x = rng.random((n, D)).astype(np.float32)
+    wt = (rng.random(n) + 0.05).astype(np.float32)
+    loss, g = f.gradient(torch.from_numpy(np.ascontiguousarray(x.T)).cuda(), torch.from_numpy(wt).cuda(), off=3,
+                         batch=rows)
+    lo, go = FL.nll_and_grad_torch(perm, w, x[3:3 + rows].astype(np.float64), wt[3:3 + rows].astype(np.float64))
+    assert abs(loss - lo) <= 1e-3 * max(1.0, abs(lo)), (loss, lo)
+    g = g.reshape(w.shape).astype(np.float64)
+    # a single row's bf16 roundings do not average out: the module's 3e-2 in norm, over all layers together
+    assert np.linalg.norm(g - go) <= 3e-2 * np.linalg.norm(go), np.linalg.norm(g - go) / np.linalg.norm(go)
+
+
+def test_adam_keeps_the_training_copy_in_step(J):
+    """Two calls of one step each equal one call of two steps: the packed
+    weights and the zeroed gradient carry over."""
+    import torch
+    D = 8
+    perm, w = _flow(D, 71, 0.1)
+    rng = np.random.default_rng(5)
+    x = torch.from_numpy(rng.random((D, 256)).astype(np.float32)).cuda()
+    wt = torch.from_numpy((rng.random(256) + 0.05).astype(np.float32)).cuda()
+    a, b = J.Flow(D, perm, w), J.Flow(D, perm, w)
+    la = a.train(x, wt, 2, 256, lr=1e-3, seed=1)
+    lb = [float(b.train(x, wt, 1, 256, lr=1e-3, seed=s)[0]) for s in (1, 2)]
+    # the window is the whole set either way; atomic sums differ in their last bits
+    assert np.allclose(la, lb, rtol=1e-5), (la, lb)
+    c = J.Flow(D, perm, b.get_params())  # a fresh flow packs b's parameters itself
+    assert abs(c.gradient(x, wt)[0] - b.gradient(x, wt)[0]) <= 1e-6 * abs(lb[1]) + 1e-6
