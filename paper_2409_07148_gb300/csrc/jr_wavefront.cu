@@ -32,7 +32,6 @@ namespace jr {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kRefill = 4;  // refill a warp once this many lanes are idle
 
 // Append chain i to a queue if `live`; one atomic per warp.  All 32 lanes call.
 __device__ __forceinline__ void enqueue(bool live, uint32_t i, uint32_t* q, unsigned int* count) {
@@ -339,166 +338,82 @@ __global__ void __launch_bounds__(128, 10) wf_step_kernel(ChainView c, uint64_t 
     count_and_flush_last(bc, nJ, nL, nA, status, ps, c);
 }
 
-// Whole paths of every queued chain in one persistent launch.  A lane keeps
-// its path (ray, throughput T, emission F, vertex v) in registers and moves
-// between three states: traversing its current ray; waiting to shade (its
-// closest hit is known); idle (no path).  Traversal rounds are warp-
-// synchronous while-while rounds with speculative traversal (Aila & Laine
-// 2009): a lane that meets a leaf postpones it and keeps descending inner
-// nodes until all but kSearchExit lanes hold a leaf.  A warp shades its
-// waiting lanes together once kShadeBatch of them wait, or once they are at
-// least as many as the traversing lanes (measured: 1.22 -> 1.25e9 chain
-// steps/s against the batch rule alone); a shaded path either continues with
-// its next ray or ends (F
-// goes to fy, and, with a flow, the row joins the density queue: when its
-// candidate will become a state with p > 0 and still lacks u(y); the finish of
-// the next step kernel takes the same decision from the same values).  Idle lanes take new
-// paths from the queue (dynamic fetch, so a warp does not idle for its
-// longest path); a new path starts at the camera ray through the candidate's
-// film point (y0, y1) with T = 1, F = 0.  ident = 1: the queue is the identity
-// over all n chains (every step but a drain step).
-// A path's loads never wait on one another: the start record fy[i] =
-// (y0, y1, y2, y3) and the parity byte arrive together, and the two
-// coordinates of vertex v + 1 are loaded when vertex v is shaded, so they
-// arrive while the next ray traverses.  These per-chain loads and the store of
-// F are marked evict-first (ld/st .cs): each is touched once per launch, and
-// L1 is better kept for the BVH nodes, the triangles and the traversal stacks
-// (measured: +0.3 %).
-constexpr int kShadeBatch = 16;
-enum PathState : uint32_t { kIdle = 0, kTraverse = 1, kWaitShade = 2 };
+// Whole paths of every queued chain in one persistent launch (trace_paths).  The
+// paths are the queue's chains, fetched dynamically; ident = 1: the queue is the
+// identity over all n chains (every step but a drain step).  A path starts from
+// the record fy[i] = (y0, y1, y2, y3), and F goes back to fy; with a flow, the row
+// joins the density queue when its candidate will become a state with p > 0 and
+// still lacks u(y) (the finish of the next step kernel takes the same decision
+// from the same values).  The per-chain loads and the store of F are marked
+// evict-first (ld/st .cs): each is touched once per launch, and L1 is better kept
+// for the BVH nodes, the triangles and the traversal stacks (measured: +0.3 %).
+struct ChainPaths {
+    const ChainView& c;
+    unsigned count;
+    bool ident;
+    bool drained = false;
+    uint32_t i = 0;
+    bool lit = false;     // F is not zero, and waits in fy[i]
+    bool cx = false;      // the candidate lives in x (else in y)
+    bool need_u = false;
 
+    __device__ __forceinline__ bool take(unsigned idle, bool mine, float& y0, float& y1) {
+        const int lane = threadIdx.x & 31;
+        unsigned base = 0;
+        if (lane == 0) base = atomicAdd(c.wf.qcount + (kMaxDepth + 2), (unsigned)__popc(idle));
+        base = __shfl_sync(kFull, base, 0);
+        if (base + (unsigned)__popc(idle) >= count) drained = true;
+        const unsigned j = base + __popc(idle & ((1u << lane) - 1u));
+        if (!mine || j >= count) return false;
+        i = ident ? j : c.wf.queue[j];
+        const float4 y = __ldcs(c.wf.fy + i);
+        cx = __ldcs(c.wf.par + i) != 0;
+        lit = false;
+        y0 = y.x;
+        y1 = y.y;
+        return true;
+    }
+    __device__ __forceinline__ const SceneView& camera(const SceneView& s) const { return s; }
+    __device__ __forceinline__ int root(const SceneView& s) const { return s.root; }
+    __device__ __forceinline__ int depth() const { return (int)c.depth; }
+    __device__ __forceinline__ float2 coords(int v) const {  // one 8-byte load
+        return __ldcs(reinterpret_cast<const float2*>(cx ? c.x : c.wf.y) + (uint64_t)(1 + v) * c.n + i);
+    }
+    __device__ __forceinline__ float3 emission() const {
+        if (!lit) return f3(0.f, 0.f, 0.f);
+        const float4 f = __ldcs(c.wf.fy + i);
+        return f3(f.x, f.y, f.z);
+    }
+    __device__ __forceinline__ void keep(float3 F) {
+        if (F.x != 0.f || F.y != 0.f || F.z != 0.f) {
+            __stcs(c.wf.fy + i, make_float4(F.x, F.y, F.z, 0.f));
+            lit = true;
+        }
+    }
+    __device__ __forceinline__ void finish(float3 F, unsigned&) {
+        __stcs(c.wf.fy + i, make_float4(F.x, F.y, F.z, 0.f));
+        if (c.flow.D != 0) {
+            unsigned ignored = 0;
+            const float py = lum(finite_or_zero(F, ignored));
+            const float ua = c.wf.ua[i];
+            need_u = ua >= 0.0f ? ua * c.fpu[3 * c.n + i] < py : (ua == -1.0f && py > 0.0f);
+        }
+    }
+    __device__ __forceinline__ void batch_done() {
+        if (c.flow.D != 0) enqueue(need_u, i, c.wf.fq, c.wf.qcount + kQFlowDensity);
+        need_u = false;
+    }
+};
 
 template <int kCheck>
 __global__ void __launch_bounds__(128) wf_path_kernel(SceneView s, ChainView c, int ident) {
-    const WaveView& w = c.wf;
-    const uint32_t* qin = w.queue;
-    const unsigned count = ident ? (unsigned)c.n : w.qcount[0];
+    const unsigned count = ident ? (unsigned)c.n : c.wf.qcount[0];
     if ((uint64_t)blockIdx.x * blockDim.x >= count) return;
-    unsigned int* fetch = w.qcount + (kMaxDepth + 2);
-    const uint64_t n = c.n;
-    const int depth = (int)c.depth;
-    const bool has_flow = c.flow.D != 0;
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
     unsigned status = 0;
-    Work wk;
-    Trav r{};
-    int stack[kStackSize];
-    uint32_t state = kIdle, i = 0;
-    int v = 0, leaf = kSentinel;
-    bool drained = false;
-    float3 T = f3(1.f, 1.f, 1.f);
-    bool lit = false;  // F is not zero, and waits in fy[i]
-    bool cx = false;   // the candidate lives in x (else in y)
-    // One node visit of a lane that has an inner node; a leaf it comes to is
-    // postponed if it holds none yet.
-    auto visit = [&](bool on) {
-        if (on && r.ref >= 0) {
-            if (!trav_node<kCheck, false>(s, r, stack, status, wk)) {
-                r.best = -1;
-                r.ref = leaf = kSentinel;
-            } else if (leaf == kSentinel && r.ref < 0 && r.ref != kSentinel) {
-                leaf = r.ref;
-                r.ref = r.sp > 0 ? stack[--r.sp] : kSentinel;
-            }
-        }
-    };
-    while (true) {
-        // shade the waiting lanes as a batch
-        const unsigned waiting = __ballot_sync(kFull, state == kWaitShade);
-        const unsigned tracing = __ballot_sync(kFull, state == kTraverse);
-        if (waiting && (__popc(waiting) >= kShadeBatch || __popc(waiting) >= __popc(tracing))) {
-            bool need_u = false;
-            if (state == kWaitShade) {
-                bool live = false;
-                float3 F = f3(0.f, 0.f, 0.f);
-                if (lit) {
-                    const float4 f = __ldcs(w.fy + i);
-                    F = f3(f.x, f.y, f.z);
-                }
-                if (r.best >= 0) {
-                    float2 uv = make_float2(0.f, 0.f);
-                    if (v < depth)  // vertex v's coordinate pair, one 8-byte load (evict-first)
-                        uv = __ldcs(reinterpret_cast<const float2*>(cx ? c.x : w.y) + (uint64_t)(1 + v) * n + i);
-                    float3 o = r.o, d = r.d;
-                    live = shade_vertex(s, r.best, r.tb, v, depth, uv.x, uv.y, o, d, T, F);
-                    if (live) {
-                        ++v;
-                        trav_begin(s, r, o, d);
-                        state = kTraverse;
-                        if (F.x != 0.f || F.y != 0.f || F.z != 0.f) {
-                            __stcs(w.fy + i, make_float4(F.x, F.y, F.z, 0.f));
-                            lit = true;
-                        }
-                    }
-                }
-                if (!live) {
-                    __stcs(w.fy + i, make_float4(F.x, F.y, F.z, 0.f));
-                    if (has_flow) {
-                        unsigned ignored = 0;
-                        const float py = lum(finite_or_zero(F, ignored));
-                        const float ua = w.ua[i];
-                        need_u = ua >= 0.0f ? ua * c.fpu[3 * n + i] < py : (ua == -1.0f && py > 0.0f);
-                    }
-                    state = kIdle;
-                }
-            }
-            if (has_flow) enqueue(need_u, i, w.fq, w.qcount + kQFlowDensity);
-        }
-        // take new paths for idle lanes
-        const unsigned idle = __ballot_sync(kFull, state == kIdle);
-        if (!drained && idle && (__popc(idle) >= kRefill || idle == kFull)) {
-            unsigned base = 0;
-            if (lane == 0) base = atomicAdd(fetch, (unsigned)__popc(idle));
-            base = __shfl_sync(kFull, base, 0);
-            if (base + (unsigned)__popc(idle) >= count) drained = true;
-            if (state == kIdle) {
-                const unsigned j = base + __popc(idle & lt);
-                if (j < count) {
-                    i = ident ? j : qin[j];
-                    const float4 y = __ldcs(w.fy + i);
-                    cx = __ldcs(w.par + i) != 0;
-                    float3 o, d;
-                    camera_ray(s, y.x, y.y, o, d);
-                    T = f3(1.f, 1.f, 1.f);
-                    lit = false;
-                    v = 0;
-                    trav_begin(s, r, o, d);
-                    state = s.root != kSentinel ? kTraverse : kWaitShade;  // empty scene: a miss
-                }
-            }
-        }
-        if (!__any_sync(kFull, state != kIdle)) {
-            if (drained) break;
-            continue;
-        }
-        // one speculative while-while traversal round
-        const bool trav = state == kTraverse;
-        if (trav && leaf == kSentinel && r.ref < 0 && r.ref != kSentinel) {
-            leaf = r.ref;
-            r.ref = r.sp > 0 ? stack[--r.sp] : kSentinel;
-        }
-        const unsigned tracing_now = __ballot_sync(kFull, trav);
-        if (__any_sync(kFull, trav && leaf == kSentinel && r.ref >= 0)) {
-            do {  // two visits per vote: half the votes, and a lane that reaches its leaf goes on speculatively
-                visit(trav);
-                visit(trav);
-            } while (!search_done(__ballot_sync(kFull, trav && leaf == kSentinel && r.ref >= 0), tracing_now));
-            if (trav && over_budget<kCheck>(s, r, status)) {
-                r.best = -1;
-                r.ref = leaf = kSentinel;
-            }
-        }
-        if (trav) {
-            if (leaf != kSentinel) {
-                trav_test_leaf<false>(s, r, leaf, wk);
-                leaf = kSentinel;
-            }
-            if (r.ref == kSentinel) state = kWaitShade;
-        }
-    }
+    ChainPaths src{c, count, ident != 0};
+    trace_paths<kCheck>(s, src, status);
     status = __reduce_or_sync(kFull, status);
-    if (lane == 0 && status) atomicOr(c.status, status);
+    if ((threadIdx.x & 31) == 0 && status) atomicOr(c.status, status);
 }
 
 // ---------------------------------------------------------------------------
@@ -571,161 +486,108 @@ __global__ void __launch_bounds__(128) wf_batch_step_kernel(const BatchEntry* en
 
 // The path kernel over every set's candidates: item j of the launch is chain
 // j - off[q] of set q, off[q] <= j < off[q + 1] (off = the sets' chain
-// prefix sums, copied to shared memory).  The lane logic is the single-set
-// path kernel's; per lane it keeps the set, its depth, the candidate buffer
-// and its stride, and starts each ray at the set's root in the merged scene.
+// prefix sums, copied to shared memory).  As ChainPaths; per lane it keeps the
+// set, its depth, the candidate buffer and its stride, and starts each ray at the
+// set's root in the merged scene.
+struct BatchPaths {
+    const BatchEntry* entries;
+    const int* roots;
+    const uint64_t* off;   // shared memory
+    uint32_t n_sets;
+    unsigned int* fetch;
+    bool drained = false;
+    uint32_t i = 0, set = 0, nst = 0;
+    int dep = 0;
+    const float* cand = nullptr;  // the candidate's buffer (pair layout, nst chains)
+    bool lit = false;
+    bool need_u = false;
+
+    __device__ __forceinline__ bool take(unsigned idle, bool mine, float& y0, float& y1) {
+        const int lane = threadIdx.x & 31;
+        const unsigned count = (unsigned)off[n_sets];
+        unsigned base = 0;
+        if (lane == 0) base = atomicAdd(fetch, (unsigned)__popc(idle));
+        base = __shfl_sync(kFull, base, 0);
+        if (base + (unsigned)__popc(idle) >= count) drained = true;
+        const unsigned j = base + __popc(idle & ((1u << lane) - 1u));
+        if (!mine || j >= count) return false;
+        uint32_t lo = 0, hi = n_sets;  // the set whose chain range holds j
+        while (hi - lo > 1) {
+            const uint32_t mid = (lo + hi) / 2;
+            if (off[mid] <= j) lo = mid;
+            else hi = mid;
+        }
+        set = lo;
+        i = j - (uint32_t)off[lo];
+        const BatchEntry& e = entries[set];
+        const float4 y = __ldcs(e.c.wf.fy + i);
+        cand = __ldcs(e.c.wf.par + i) ? e.c.x : e.c.wf.y;
+        nst = (uint32_t)e.c.n;
+        dep = (int)e.c.depth;
+        lit = false;
+        y0 = y.x;
+        y1 = y.y;
+        return true;
+    }
+    __device__ __forceinline__ const SceneView& camera(const SceneView&) const { return entries[set].s; }
+    __device__ __forceinline__ int root(const SceneView&) const { return roots[set]; }
+    __device__ __forceinline__ int depth() const { return dep; }
+    __device__ __forceinline__ float2 coords(int v) const {
+        return __ldcs(reinterpret_cast<const float2*>(cand) + (uint64_t)(1 + v) * nst + i);
+    }
+    __device__ __forceinline__ float3 emission() const {
+        if (!lit) return f3(0.f, 0.f, 0.f);
+        const float4 f = __ldcs(entries[set].c.wf.fy + i);
+        return f3(f.x, f.y, f.z);
+    }
+    __device__ __forceinline__ void keep(float3 F) {
+        if (F.x != 0.f || F.y != 0.f || F.z != 0.f) {
+            __stcs(entries[set].c.wf.fy + i, make_float4(F.x, F.y, F.z, 0.f));
+            lit = true;
+        }
+    }
+    __device__ __forceinline__ void finish(float3 F, unsigned& status) {
+        const ChainView& c = entries[set].c;
+        __stcs(c.wf.fy + i, make_float4(F.x, F.y, F.z, 0.f));
+        if (status) {
+            atomicOr(c.status, status);
+            status = 0;
+        }
+        if (c.flow.D != 0) {  // as in the single-set path kernel
+            unsigned ignored = 0;
+            const float py = lum(finite_or_zero(F, ignored));
+            const float ua = c.wf.ua[i];
+            need_u = ua >= 0.0f ? ua * c.fpu[3 * c.n + i] < py : (ua == -1.0f && py > 0.0f);
+        }
+    }
+    // Rows whose u(y) the density pass must fill, appended to their set's queue:
+    // lanes of one warp may hold different sets, so the lanes of each set share
+    // one atomic.
+    __device__ __forceinline__ void batch_done() {
+        const unsigned peers = __match_any_sync(kFull, need_u ? set : 0xffffffffu);
+        if (need_u) {
+            const int lane = threadIdx.x & 31, leader = __ffs(peers) - 1;
+            unsigned base = 0;
+            if (lane == leader)
+                base = atomicAdd(entries[set].c.wf.qcount + kQFlowDensity, (unsigned)__popc(peers));
+            base = __shfl_sync(peers, base, leader);
+            entries[set].c.wf.fq[base + __popc(peers & ((1u << lane) - 1u))] = i;
+        }
+        need_u = false;
+    }
+};
+
 template <int kCheck>
-__global__ void __launch_bounds__(128, 7) wf_batch_path_kernel(SceneView m, const BatchEntry* entries, const int* roots,
-                                                            const uint64_t* chain_off, uint32_t n_sets,
-                                                            unsigned int* fetch) {
+__global__ void __launch_bounds__(128, 7) wf_batch_path_kernel(SceneView m, const BatchEntry* entries,
+                                                               const int* roots, const uint64_t* chain_off,
+                                                               uint32_t n_sets, unsigned int* fetch) {
     extern __shared__ uint64_t off_s[];
     for (uint32_t q = threadIdx.x; q <= n_sets; q += blockDim.x) off_s[q] = chain_off[q];
     __syncthreads();
-    const unsigned count = (unsigned)off_s[n_sets];
-    if ((uint64_t)blockIdx.x * blockDim.x >= count) return;
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
+    if ((uint64_t)blockIdx.x * blockDim.x >= off_s[n_sets]) return;
     unsigned status = 0;
-    Work wk;
-    Trav r{};
-    int stack[kStackSize];
-    uint32_t state = kIdle, i = 0, set = 0, nst = 0;
-    int v = 0, leaf = kSentinel, depth = 0;
-    bool drained = false, lit = false;
-    float3 T = f3(1.f, 1.f, 1.f);
-    const float* cand = nullptr;     // the candidate's buffer (pair layout, nst chains)
-    auto visit = [&](bool on) {      // as in the single-set path kernel
-        if (on && r.ref >= 0) {
-            if (!trav_node<kCheck, false>(m, r, stack, status, wk)) {
-                r.best = -1;
-                r.ref = leaf = kSentinel;
-            } else if (leaf == kSentinel && r.ref < 0 && r.ref != kSentinel) {
-                leaf = r.ref;
-                r.ref = r.sp > 0 ? stack[--r.sp] : kSentinel;
-            }
-        }
-    };
-    while (true) {
-        // shade the waiting lanes as a batch
-        const unsigned waiting = __ballot_sync(kFull, state == kWaitShade);
-        const unsigned tracing = __ballot_sync(kFull, state == kTraverse);
-        if (waiting && (__popc(waiting) >= kShadeBatch || __popc(waiting) >= __popc(tracing))) {
-            bool need_u = false;
-            if (state == kWaitShade) {
-                bool live = false;
-                float3 F = f3(0.f, 0.f, 0.f);
-                if (lit) {
-                    const float4 f = __ldcs(entries[set].c.wf.fy + i);
-                    F = f3(f.x, f.y, f.z);
-                }
-                if (r.best >= 0) {
-                    float2 uv = make_float2(0.f, 0.f);
-                    if (v < depth)  // vertex v's coordinate pair, one 8-byte load
-                        uv = __ldcs(reinterpret_cast<const float2*>(cand) + (uint64_t)(1 + v) * nst + i);
-                    float3 o = r.o, d = r.d;
-                    live = shade_vertex(m, r.best, r.tb, v, depth, uv.x, uv.y, o, d, T, F);
-                    if (live) {
-                        ++v;
-                        trav_begin_at(r, o, d, roots[set]);
-                        state = kTraverse;
-                        if (F.x != 0.f || F.y != 0.f || F.z != 0.f) {
-                            __stcs(entries[set].c.wf.fy + i, make_float4(F.x, F.y, F.z, 0.f));
-                            lit = true;
-                        }
-                    }
-                }
-                if (!live) {
-                    const ChainView& c = entries[set].c;
-                    __stcs(c.wf.fy + i, make_float4(F.x, F.y, F.z, 0.f));
-                    if (status) {
-                        atomicOr(c.status, status);
-                        status = 0;
-                    }
-                    if (c.flow.D != 0) {  // as in the single-set path kernel
-                        unsigned ignored = 0;
-                        const float py = lum(finite_or_zero(F, ignored));
-                        const float ua = c.wf.ua[i];
-                        need_u = ua >= 0.0f ? ua * c.fpu[3 * c.n + i] < py : (ua == -1.0f && py > 0.0f);
-                    }
-                    state = kIdle;
-                }
-            }
-            // rows whose u(y) the density pass must fill, appended to their set's
-            // queue: lanes of one warp may hold different sets, so the lanes of
-            // each set share one atomic (all 32 lanes take part)
-            const unsigned peers = __match_any_sync(kFull, need_u ? set : 0xffffffffu);
-            if (need_u) {
-                const int leader = __ffs(peers) - 1;
-                unsigned base = 0;
-                if (lane == leader)
-                    base = atomicAdd(entries[set].c.wf.qcount + kQFlowDensity, (unsigned)__popc(peers));
-                base = __shfl_sync(peers, base, leader);
-                entries[set].c.wf.fq[base + __popc(peers & lt)] = i;
-            }
-        }
-        // take new paths for idle lanes
-        const unsigned idle = __ballot_sync(kFull, state == kIdle);
-        if (!drained && idle && (__popc(idle) >= kRefill || idle == kFull)) {
-            unsigned base = 0;
-            if (lane == 0) base = atomicAdd(fetch, (unsigned)__popc(idle));
-            base = __shfl_sync(kFull, base, 0);
-            if (base + (unsigned)__popc(idle) >= count) drained = true;
-            if (state == kIdle) {
-                const unsigned j = base + __popc(idle & lt);
-                if (j < count) {
-                    uint32_t lo = 0, hi = n_sets;  // the set whose chain range holds j
-                    while (hi - lo > 1) {
-                        const uint32_t mid = (lo + hi) / 2;
-                        if (off_s[mid] <= j) lo = mid;
-                        else hi = mid;
-                    }
-                    set = lo;
-                    i = j - (uint32_t)off_s[lo];
-                    const BatchEntry& e = entries[set];
-                    const float4 y = __ldcs(e.c.wf.fy + i);
-                    cand = __ldcs(e.c.wf.par + i) ? e.c.x : e.c.wf.y;
-                    nst = (uint32_t)e.c.n;
-                    depth = (int)e.c.depth;
-                    float3 o, d;
-                    camera_ray(e.s, y.x, y.y, o, d);
-                    T = f3(1.f, 1.f, 1.f);
-                    lit = false;
-                    v = 0;
-                    const int root = roots[set];
-                    trav_begin_at(r, o, d, root);
-                    state = root != kSentinel ? kTraverse : kWaitShade;  // empty scene: a miss
-                }
-            }
-        }
-        if (!__any_sync(kFull, state != kIdle)) {
-            if (drained) break;
-            continue;
-        }
-        // one speculative while-while traversal round
-        const bool trav = state == kTraverse;
-        if (trav && leaf == kSentinel && r.ref < 0 && r.ref != kSentinel) {
-            leaf = r.ref;
-            r.ref = r.sp > 0 ? stack[--r.sp] : kSentinel;
-        }
-        const unsigned tracing_now = __ballot_sync(kFull, trav);
-        if (__any_sync(kFull, trav && leaf == kSentinel && r.ref >= 0)) {
-            do {  // two visits per vote: half the votes, and a lane that reaches its leaf goes on speculatively
-                visit(trav);
-                visit(trav);
-            } while (!search_done(__ballot_sync(kFull, trav && leaf == kSentinel && r.ref >= 0), tracing_now));
-            if (trav && over_budget<kCheck>(m, r, status)) {
-                r.best = -1;
-                r.ref = leaf = kSentinel;
-            }
-        }
-        if (trav) {
-            if (leaf != kSentinel) {
-                trav_test_leaf<false>(m, r, leaf, wk);
-                leaf = kSentinel;
-            }
-            if (r.ref == kSentinel) state = kWaitShade;
-        }
-    }
+    BatchPaths src{entries, roots, off_s, n_sets, fetch};
+    trace_paths<kCheck>(m, src, status);
 }
 
 inline unsigned grid_for(uint64_t n, unsigned b) { return (unsigned)((n + b - 1) / b); }
