@@ -1,0 +1,498 @@
+// Look-ahead execution of Jump Restore with uniform regeneration (sm_103a).
+//
+// A regeneration of Alg. 2 (Section 7.2) draws its state from mu, so the candidate
+// of step s of chain i depends on (i, s) only, not on the chain's state: its path
+// can be traced before it is known whether step s regenerates at all.  In the
+// stationary jump chain a share p_lambda / (p_lambda + c~) of the steps is local
+// (Section 6.1), often around one percent, and all the others regenerate.  So an
+// advance goes in windows of K steps:
+//
+//   1. ahead_path_kernel: F of the regeneration candidate of every (chain, step) of
+//      the window, n K independent paths in one persistent launch (trace_paths).
+//      The coordinates are drawn where they are used; 16 bytes per path go out.
+//   2. settle_kernel, one thread per chain: the window's steps in order.  A state
+//      with p = 0 is killed at once (k = inf), so a dark step is one 16-byte read;
+//      a lit state draws its clocks and is splatted.  A chain whose step turns out
+//      local stops and joins a queue.
+//   3. tail_kernel: the queued chains, each carried to the window's end by one lane,
+//      with the local moves' paths traced there (or settle_warp_kernel does 2 and 3
+//      with one warp per chain, for scenes of at most kWarpChainMaxTris triangles).
+//
+// The wavefront (jr_wavefront.cu) has to end every step's path launch before the
+// next step, so it pays a launch's tail per step (12 % of the warp slots at 2^20
+// chains), and few chains leave the device idle whatever the step does.  Here a
+// launch has K times the paths, and the state is read and written once per window.
+// What it costs: a local step's regeneration candidate is traced for nothing.
+// Measured (start of the change -> with it): 400 steps of 256 chains in the
+// 24-triangle box 1 024 -> 453 us, 32 steps of 10 007 chains on Cornell + spheres
+// 1 578 -> 988 us, 16 steps of 2^20 11.23 -> 9.65 ms, 400 steps of 10 007 20.6 -> 4.2 ms.
+//
+// The draws, the arithmetic and the order of a chain's steps are the other modes',
+// so the chains are the same.
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+#include "../../include/jr.h"
+#include "jr_device.cuh"
+#include "jr_internal.h"
+
+namespace jr {
+namespace {
+
+constexpr unsigned kFull = 0xffffffffu;
+
+// Path j of a window is the regeneration candidate of chain j % n at step
+// step0 + j / n; out[j] = (F, status bits).
+struct AheadPaths {
+    const ChainView& c;
+    uint64_t step0;
+    unsigned count;
+    unsigned int* fetch;
+    float4* out;
+    bool drained = false;
+    uint32_t j = 0;
+    float3 F = f3(0.f, 0.f, 0.f);
+
+    __device__ __forceinline__ uint4 block(uint32_t b) const {
+        const uint32_t n = (uint32_t)c.n, k = j / n;
+        return draw(c.seed, kTagStep, b + 1u, c.chain_offset + (j - k * n), step0 + k);
+    }
+    __device__ __forceinline__ bool take(unsigned idle, bool mine, float& y0, float& y1) {
+        const int lane = threadIdx.x & 31;
+        unsigned base = 0;
+        if (lane == 0) base = atomicAdd(fetch, (unsigned)__popc(idle));
+        base = __shfl_sync(kFull, base, 0);
+        if (base + (unsigned)__popc(idle) >= count) drained = true;
+        const unsigned q = base + __popc(idle & ((1u << lane) - 1u));
+        if (!mine || q >= count) return false;
+        j = q;
+        F = f3(0.f, 0.f, 0.f);
+        const uint4 r = block(0);
+        y0 = u01(r.x);
+        y1 = u01(r.y);
+        return true;
+    }
+    __device__ __forceinline__ const SceneView& camera(const SceneView& s) const { return s; }
+    __device__ __forceinline__ int root(const SceneView& s) const { return s.root; }
+    __device__ __forceinline__ int depth() const { return (int)c.depth; }
+    __device__ __forceinline__ float2 coords(int v) const {  // coordinates 2 + 2v, 3 + 2v
+        const uint4 r = block((uint32_t)(1 + v) >> 1);
+        return v & 1 ? make_float2(u01(r.x), u01(r.y)) : make_float2(u01(r.z), u01(r.w));
+    }
+    __device__ __forceinline__ float3 emission() const { return F; }
+    __device__ __forceinline__ void keep(float3 f) { F = f; }
+    __device__ __forceinline__ void finish(float3 f, unsigned& status) {
+        // the status belongs to the path: it counts only if the chain takes it
+        __stcs(out + j, make_float4(f.x, f.y, f.z, __uint_as_float(status)));
+        status = 0;
+    }
+    __device__ __forceinline__ void batch_done() {}
+};
+
+template <int kCheck>
+__global__ void __launch_bounds__(128, 7) ahead_path_kernel(SceneView s, ChainView c, uint64_t step0, uint32_t count,
+                                                            unsigned int* fetch, float4* out) {
+    if ((uint64_t)blockIdx.x * blockDim.x >= count) return;
+    AheadPaths src{c, step0, count, fetch, out};
+    unsigned status = 0;
+    trace_paths<kCheck>(s, src, status);
+}
+
+// A chain on its way through a window.  org: where the state's coordinates are:
+// 0 in c.x, q > 0: the regeneration of the window's step q - 1.
+struct Walk {
+    float Fr, Fg, Fb, p, u;
+    uint32_t k, org;
+    __device__ __forceinline__ void load(const ChainView& c, uint64_t i) {
+        Fr = c.fpu[0 * c.n + i];
+        Fg = c.fpu[1 * c.n + i];
+        Fb = c.fpu[2 * c.n + i];
+        p = c.fpu[3 * c.n + i];
+        u = c.fpu[4 * c.n + i];
+    }
+    __device__ __forceinline__ void store(const ChainView& c, uint64_t i) const {
+        c.fpu[0 * c.n + i] = Fr;
+        c.fpu[1 * c.n + i] = Fg;
+        c.fpu[2 * c.n + i] = Fb;
+        c.fpu[3 * c.n + i] = p;
+        c.fpu[4 * c.n + i] = u;
+    }
+    // Regenerate at step k: f = the candidate's (F, status).
+    __device__ __forceinline__ void regenerate(const float4 f, unsigned& status) {
+        status |= __float_as_uint(f.w);
+        const float3 F = finite_or_zero(f3(f.x, f.y, f.z), status);
+        Fr = F.x;
+        Fg = F.y;
+        Fb = F.z;
+        p = lum(F);
+        u = 1.0f;
+        org = ++k;
+    }
+};
+
+__device__ __forceinline__ void splat(const ChainView& c, const Walk& w, float x0, float x1, float dt) {
+    if (!(dt > 0.0f && w.p > 0.0f)) return;
+    const uint32_t px = min((uint32_t)((double)x0 * (double)c.width), c.width - 1);
+    const uint32_t py = min((uint32_t)((double)x1 * (double)c.height), c.height - 1);
+    const float WH = (float)c.width * (float)c.height;
+    const float wgt = c.c_tilde * dt * WH / w.p;
+    atomicAdd(c.fb + (py * c.width + px), make_float4(wgt * w.Fr, wgt * w.Fg, wgt * w.Fb, dt));
+}
+
+// The coordinates of the regeneration of step `step` into chain i's state.
+__device__ __forceinline__ void store_regeneration(const ChainView& c, uint64_t i, uint64_t step) {
+    float2* x2 = reinterpret_cast<float2*>(c.x);
+    for (int b = 0; 4 * b < (int)c.dim; ++b) {
+        const uint4 r = draw(c.seed, kTagStep, (uint32_t)(b + 1), c.chain_offset + (uint32_t)i, step);
+        x2[(uint64_t)(2 * b) * c.n + i] = make_float2(u01(r.x), u01(r.y));
+        if (4 * b + 2 < (int)c.dim) x2[(uint64_t)(2 * b + 1) * c.n + i] = make_float2(u01(r.z), u01(r.w));
+    }
+}
+
+// ctl: [0] the path kernel's cursor, [1] queue length, [2] the tail's cursor.
+enum { kCtlPaths = 0, kCtlQueue = 1, kCtlTail = 2, kCtlCount = 4 };
+
+// Bound by reading the window's F (16 bytes per step and chain, four steps in
+// flight); the lit states' clocks are rare.
+__global__ void __launch_bounds__(128) settle_kernel(ChainView c, uint64_t step0, uint32_t K, const float4* Fw,
+                                                     uint4* queue, unsigned int* ctl) {
+    const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    const bool valid = i < c.n;
+    uint32_t nJ = 0;
+    unsigned status = 0;
+    bool local = false;
+    Walk w;
+    w.k = w.org = 0;
+    w.p = 0.f;
+    if (valid) {
+        const uint32_t chain = c.chain_offset + (uint32_t)i;
+        w.load(c, i);
+        const float4* f = Fw + i;
+        float4 next[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) next[q] = q < (int)K ? __ldcs(f + (uint64_t)q * c.n) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (uint32_t k0 = 0; k0 < K && !local; k0 += 4) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t k = k0 + q;
+                if (k >= K || local) break;
+                if (w.p > 0.0f) {
+                    float dt;
+                    local = restore_clocks(c, draw(c.seed, kTagStep, 0, chain, step0 + k), w.p, w.u, dt);
+                    float2 x;
+                    if (w.org == 0) {
+                        x = reinterpret_cast<const float2*>(c.x)[i];
+                    } else {
+                        const uint4 r = draw(c.seed, kTagStep, 1, chain, step0 + w.org - 1);
+                        x = make_float2(u01(r.x), u01(r.y));
+                    }
+                    splat(c, w, x.x, x.y, dt);
+                }
+                if (!local) {
+                    nJ++;
+                    w.regenerate(next[q], status);
+                    next[q] = k + 4 < K ? __ldcs(f + (uint64_t)(k + 4) * c.n) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+            }
+        }
+        w.store(c, i);
+        if (!local && w.org) store_regeneration(c, i, step0 + w.org - 1);
+    }
+    // one queue atomic per warp
+    const unsigned m = __ballot_sync(kFull, local);
+    if (m) {
+        const int lane = threadIdx.x & 31;
+        unsigned base = 0;
+        if (lane == 0) base = atomicAdd(ctl + kCtlQueue, (unsigned)__popc(m));
+        base = __shfl_sync(kFull, base, 0);
+        if (local) queue[base + __popc(m & ((1u << lane) - 1u))] = make_uint4((uint32_t)i, w.k, w.org, 0u);
+    }
+    nJ = __reduce_add_sync(kFull, nJ);
+    status = __reduce_or_sync(kFull, status);
+    if ((threadIdx.x & 31) == 0) {
+        if (nJ) atomicAdd(c.counters + 0, (unsigned long long)nJ);
+        flush_status(status, c.status);
+    }
+}
+
+// The queued chains to the window's end: lane = chain, one-warp blocks, chains
+// fetched as lanes become free (drain_kernel's scheme: a local step waits for no
+// other chain but the few in its warp).
+template <int kCheck>
+__global__ void __launch_bounds__(32, 16) tail_kernel(SceneView s, ChainView c, uint64_t step0, uint32_t K,
+                                                      const float4* Fw, const uint4* queue, unsigned int* ctl) {
+    extern __shared__ float sh[];
+    constexpr uint32_t B = 32;
+    const int lane = threadIdx.x;
+    const unsigned count = ctl[kCtlQueue];
+    // Few chains spread over all warps: the first lanes of each take part.
+    const unsigned lanes = (count + gridDim.x - 1) / gridDim.x;
+    float* cur = sh + lane;
+    float* cand = sh + (size_t)c.dim * B + lane;
+    uint32_t nJ = 0, nL = 0, nA = 0;
+    unsigned status = 0;
+    Work work;
+    bool live = false, drained = (unsigned)lane >= lanes;
+    uint64_t i = 0;
+    uint32_t chain = 0;
+    Walk w;
+    w.k = w.org = 0;
+    while (true) {
+        if (__any_sync(kFull, !live && !drained)) {
+            const unsigned want = __ballot_sync(kFull, !live && !drained);
+            unsigned base = 0;
+            if (lane == 0) base = atomicAdd(ctl + kCtlTail, (unsigned)__popc(want));
+            base = __shfl_sync(kFull, base, 0);
+            if (!live && !drained) {
+                const unsigned q = base + __popc(want & ((1u << lane) - 1u));
+                drained = q >= count;
+                if (!drained) {
+                    const uint4 e = queue[q];
+                    i = e.x;
+                    w.k = e.y;
+                    w.org = e.z;
+                    chain = c.chain_offset + (uint32_t)i;
+                    w.load(c, i);
+                    if (w.org) propose(c, chain, step0 + w.org - 1, false, cur, cur, B);
+                    else load_coords(c, i, cur, B);
+                    live = true;
+                }
+            }
+        }
+        if (!__any_sync(kFull, live)) break;
+        if (live) propose(c, chain, step0 + w.k, true, cur, cand, B);
+        const float3 Fy = eval_path_w<kCheck, false>(s, kFull, live, (int)c.depth, cand, B, nullptr, 0, status, work);
+        if (live) {
+            const float py = lum(Fy);
+            const bool accept = u01(draw(c.seed, kTagStep, 0, chain, step0 + w.k).z) * w.p < py;
+            nL++;
+            nA += accept;
+            if (accept) {
+                float* t = cur;
+                cur = cand;
+                cand = t;
+                w.Fr = Fy.x;
+                w.Fg = Fy.y;
+                w.Fb = Fy.z;
+                w.p = py;
+                w.u = 1.0f;
+            }
+            w.org = 0;  // the coordinates are in cur
+            ++w.k;
+            bool local = false;
+            while (w.k < K && !local) {
+                if (w.p > 0.0f) {
+                    float dt;
+                    if (w.org) {  // lit after a regeneration: its coordinates are needed now
+                        propose(c, chain, step0 + w.org - 1, false, cur, cur, B);
+                        w.org = 0;
+                    }
+                    local = restore_clocks(c, draw(c.seed, kTagStep, 0, chain, step0 + w.k), w.p, w.u, dt);
+                    splat(c, w, cur[0], cur[B], dt);
+                }
+                if (!local) {
+                    nJ++;
+                    w.regenerate(__ldcs(Fw + (uint64_t)w.k * c.n + i), status);
+                }
+            }
+            if (!local) {  // the window's end
+                live = false;
+                w.store(c, i);
+                if (w.org) {
+                    store_regeneration(c, i, step0 + w.org - 1);
+                } else {
+                    float2* x2 = reinterpret_cast<float2*>(c.x);
+                    for (int k = 0; 2 * k < (int)c.dim; ++k)
+                        x2[(uint64_t)k * c.n + i] = make_float2(cur[2 * k * B], cur[(2 * k + 1) * B]);
+                }
+            }
+        }
+    }
+    nJ = __reduce_add_sync(kFull, nJ);
+    nL = __reduce_add_sync(kFull, nL);
+    nA = __reduce_add_sync(kFull, nA);
+    status = __reduce_or_sync(kFull, status);
+    if (lane == 0) {
+        if (nJ) atomicAdd(c.counters + 0, (unsigned long long)nJ);
+        if (nL) atomicAdd(c.counters + 1, (unsigned long long)nL);
+        if (nA) atomicAdd(c.counters + 2, (unsigned long long)nA);
+        flush_status(status, c.status);
+    }
+}
+
+// Settle and tail in one, a warp per chain (small scenes): lane d holds coordinate
+// d, a local move's path is traced by the whole warp (eval_path_warp), and a dark
+// state looks at the next 32 steps' candidates at once for the first lit one.
+__global__ void __launch_bounds__(128) settle_warp_kernel(SceneView s, ChainView c, uint64_t step0, uint32_t K,
+                                                          const float4* Fw) {
+    const uint64_t i = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
+    if (i >= c.n) return;  // a whole warp
+    const int lane = threadIdx.x & 31;
+    const bool mine = lane < (int)c.dim;
+    const uint32_t chain = c.chain_offset + (uint32_t)i;
+    uint32_t nJ = 0, nL = 0, nA = 0;
+    unsigned status = 0;
+    float xd = mine ? c.x[xidx((uint32_t)lane, i, c.n)] : 0.0f;
+    Walk w;
+    w.k = w.org = 0;
+    w.load(c, i);
+    // coordinate `lane` of the regeneration of the window's step q - 1
+    auto regenerated = [&](uint32_t q) {
+        if (!mine) return 0.0f;
+        const uint4 r = draw(c.seed, kTagStep, (uint32_t)(lane >> 2) + 1u, chain, step0 + q - 1);
+        return u01(lane & 2 ? ((lane & 1) ? r.w : r.z) : ((lane & 1) ? r.y : r.x));
+    };
+    while (w.k < K) {
+        if (!(w.p > 0.0f)) {  // regenerate up to the first lit candidate
+            const uint32_t left = min(32u, K - w.k);
+            float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (lane < (int)left) f = __ldcs(Fw + (uint64_t)(w.k + lane) * c.n + i);
+            // lit, or not to be skipped: not finite, or with a status to report
+            const bool stop = lum(f3(f.x, f.y, f.z)) > 0.0f || !isfinite(f.x) || !isfinite(f.y) || !isfinite(f.z) ||
+                              __float_as_uint(f.w) != 0u;
+            const unsigned m = __ballot_sync(kFull, stop);
+            const uint32_t skip = m ? (uint32_t)__ffs(m) - 1u : left;  // dark ones before it
+            nJ += skip;
+            w.k += skip;
+            if (skip) {  // the last skipped candidate is the state (p = 0)
+                const int src = (int)skip - 1;
+                w.Fr = __shfl_sync(kFull, f.x, src);
+                w.Fg = __shfl_sync(kFull, f.y, src);
+                w.Fb = __shfl_sync(kFull, f.z, src);
+                w.p = lum(f3(w.Fr, w.Fg, w.Fb));
+                w.u = 1.0f;
+                w.org = w.k;
+            }
+            if (m) {
+                const int src = (int)skip;
+                const float4 g = make_float4(__shfl_sync(kFull, f.x, src), __shfl_sync(kFull, f.y, src),
+                                             __shfl_sync(kFull, f.z, src), __shfl_sync(kFull, f.w, src));
+                nJ++;
+                w.regenerate(g, status);
+            }
+            continue;
+        }
+        if (w.org) {
+            xd = regenerated(w.org);
+            w.org = 0;
+        }
+        const uint4 r0 = draw(c.seed, kTagStep, 0, chain, step0 + w.k);
+        float dt;
+        const bool local = restore_clocks(c, r0, w.p, w.u, dt);
+        const float x0 = __shfl_sync(kFull, xd, 0), x1 = __shfl_sync(kFull, xd, 1);
+        if (lane == 0) splat(c, w, x0, x1, dt);
+        if (!local) {
+            nJ++;
+            w.regenerate(__ldcs(Fw + (uint64_t)w.k * c.n + i), status);
+            continue;
+        }
+        float yd = 0.0f;
+        if (mine) {
+            const uint4 r = draw(c.seed, kTagStep, (uint32_t)(lane >> 2) + 1u, chain, step0 + w.k);
+            const bool second = (lane & 2) != 0;
+            float sn, cs;
+            const float R = sqrtf(-2.0f * logf(1.0f - u01(second ? r.z : r.x)));
+            sincospif(2.0f * u01(second ? r.w : r.y), &sn, &cs);
+            yd = wrap01(xd + c.sigma * R * ((lane & 1) ? sn : cs));
+        }
+        const float3 Fy = eval_path_warp(s, (int)c.depth, yd, status);
+        const float py = lum(Fy);
+        const bool accept = u01(r0.z) * w.p < py;
+        nL++;
+        nA += accept;
+        if (accept) {
+            xd = yd;
+            w.Fr = Fy.x;
+            w.Fg = Fy.y;
+            w.Fb = Fy.z;
+            w.p = py;
+            w.u = 1.0f;
+        }
+        ++w.k;
+    }
+    if (w.org) xd = regenerated(w.org);
+    if (mine) c.x[xidx((uint32_t)lane, i, c.n)] = xd;
+    if (lane == 0) {
+        w.store(c, i);
+        if (nJ) atomicAdd(c.counters + 0, (unsigned long long)nJ);
+        if (nL) atomicAdd(c.counters + 1, (unsigned long long)nL);
+        if (nA) atomicAdd(c.counters + 2, (unsigned long long)nA);
+        flush_status(status, c.status);
+    }
+}
+
+// Sum of p over the chains (double), for the estimate of p_lambda.
+__global__ void __launch_bounds__(256) sum_p_kernel(ChainView c, double* out) {
+    double s = 0.0;
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < c.n; i += (uint64_t)gridDim.x * blockDim.x)
+        s += (double)c.fpu[3 * c.n + i];
+    s = warp_sum(s);
+    if ((threadIdx.x & 31) == 0 && s != 0.0) atomicAdd(out, s);
+}
+
+inline unsigned grid_for(uint64_t n, unsigned b) { return (unsigned)((n + b - 1) / b); }
+
+// Resident one-warp or 128-thread blocks of a kernel on the current device.
+template <class K>
+cudaError_t resident(K kernel, int threads, size_t shm, long long* blocks) {
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaError_t e;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+        (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, shm)) != cudaSuccess)
+        return e;
+    *blocks = (long long)sms * (per_sm > 0 ? per_sm : 1);
+    return cudaSuccess;
+}
+
+}  // namespace
+
+cudaError_t launch_sum_p(const ChainView& c, double* out, cudaStream_t st) {
+    const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(double), st);
+    if (e != cudaSuccess) return e;
+    sum_p_kernel<<<(unsigned)std::min<uint64_t>(608, (c.n + 255) / 256), 256, 0, st>>>(c, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_ahead(const SceneView& s, const ChainView& c, const AheadView& a, uint64_t step_begin,
+                         uint32_t n_steps, bool warp_tail, cudaStream_t st, KernelTimer* tm) {
+    if (c.n == 0 || n_steps == 0) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    with_checks(trav_checks(s), [&](auto kc) {
+        constexpr int kCheck = decltype(kc)::value;
+        const auto paths = ahead_path_kernel<kCheck>;
+        const auto tail = tail_kernel<kCheck>;
+        const size_t shm = sizeof(float) * 2 * c.dim * 32;  // <= 8 KB
+        long long path_blocks = 0, tail_blocks = 0;
+        if ((e = resident(paths, 128, 0, &path_blocks)) != cudaSuccess) return;
+        if (!warp_tail && (e = resident(tail, 32, shm, &tail_blocks)) != cudaSuccess) return;
+        auto mark = [&](int kind) {
+            if (tm && e == cudaSuccess) e = tm->mark(kind, st);
+        };
+        mark(-1);
+        for (uint32_t done = 0; done < n_steps && e == cudaSuccess;) {
+            const uint32_t K = std::min(a.window, n_steps - done);
+            const uint64_t step0 = step_begin + done;
+            const uint32_t count = (uint32_t)(c.n * K);
+            if ((e = cudaMemsetAsync(a.ctl, 0, sizeof(unsigned int) * kCtlCount, st)) != cudaSuccess) return;
+            paths<<<(unsigned)std::min<uint64_t>((uint64_t)path_blocks, grid_for(count, 128)), 128, 0, st>>>(
+                s, c, step0, count, a.ctl + kCtlPaths, a.F);
+            mark(KernelTimer::kPath);
+            if (warp_tail) {
+                settle_warp_kernel<<<grid_for(32 * c.n, 128), 128, 0, st>>>(s, c, step0, K, a.F);
+            } else {
+                settle_kernel<<<grid_for(c.n, 128), 128, 0, st>>>(c, step0, K, a.F, a.queue, a.ctl);
+                tail<<<(unsigned)std::min<uint64_t>((uint64_t)tail_blocks, c.n), 32, shm, st>>>(s, c, step0, K, a.F,
+                                                                                               a.queue, a.ctl);
+            }
+            mark(KernelTimer::kStep);
+            if (e == cudaSuccess) e = cudaGetLastError();
+            done += K;
+        }
+    });
+    return e;
+}
+
+}  // namespace jr

@@ -79,6 +79,8 @@ struct jr_chains {
     uint64_t flow_gen = 0;      // bumped whenever the attached flow (or its weight) changes
     uint32_t visit_budget = 0;  // traversal watchdog limits of this set's launches (0: the scene's)
     int stack_limit = 0;
+    AheadView ahead{};          // look-ahead buffers (JR_EXEC_AUTO), and whether they are worth having
+    enum Ahead { kUnknown, kYes, kNo } ahead_use = kUnknown;
     // The scene as this set's launches see it (with the set's traversal limits).
     SceneView scene_view() const {
         SceneView v = scene->view;
@@ -87,6 +89,9 @@ struct jr_chains {
         return v;
     }
     ~jr_chains() {
+        cudaFree(ahead.F);
+        cudaFree(ahead.queue);
+        cudaFree(ahead.ctl);
         cudaFree(view.wf.y);
         cudaFree(view.wf.par);
         cudaFree(view.wf.ua);
@@ -319,6 +324,75 @@ static bool warp_per_chain(const jr_chains* c) {
     return c->view.n < (uint64_t)(32 * sms);
 }
 
+// Whether JR_EXEC_AUTO runs this advance in look-ahead windows (jr_ahead.cu); sets
+// their buffers up on first use.  A window costs the latency of one path launch and
+// of its longest run of local steps, whatever the number of steps, so it takes the
+// more steps the fewer chains there are.  Measured against the best of the other
+// modes (us per advance; Cornell + spheres / slit caustic / terrain):
+//   2^20 chains, 2 steps     1 381, 1 416  /    842,   895  / 1 333, 1 338
+//   2^18 chains, 2 steps       533,   584  /    448,   511  /   608,   606
+//   2^16 chains, 8 steps       703, 1 148  /    611,   663  /   898,   911  (4: 467, 610 / 421, 381 / 567, 485)
+//   30 000 chains, 16 steps    844, 1 576  /    864,   923  / 1 207, 1 234  (8: 540, 841 / 548, 496 / 682, 658)
+//   3 000 chains, 64 steps   1 009, 1 901  /  1 740, 1 783  / 1 901, 2 054  (16: 485, 572 / 649, 551 / 767, 657)
+// and one warp per chain in the 24-triangle box: 256 chains, 64 steps 159, 198 (16: 88,
+// 69).  Such scenes with more chains than that stay in the megakernel: their paths
+// are short and alike, so it loses little (2^16 chains, 16 steps: 514, 369).
+//
+// It pays while few steps are local, because a local step's regeneration candidate
+// is traced for nothing.  The stationary share of local steps is p_lambda /
+// (p_lambda + c~) (Section 6.1); p_lambda = E_mu[p] is estimated once, from the chains'
+// own states (at first samples of mu).  Where the buffers cannot be had, or the
+// stream is being captured before they exist, the other modes run.
+constexpr double kAheadShare = 0.25;
+static bool use_ahead(jr_chains* c, uint32_t n_steps, cudaStream_t st) {
+    if (c->exec != JR_EXEC_AUTO || c->view.flow.D != 0 || (c->view.flags & (JR_FLAG_MH | JR_FLAG_MALA)) ||
+        c->ahead_use == jr_chains::kNo)
+        return false;
+    const uint64_t n = c->view.n;
+    const uint32_t least = n >= (1u << 18) ? 2 : n >= (1u << 16) ? 8 : n >= (1u << 14) ? 16 : 32;
+    if (n_steps < least || n > kAheadItems / least) return false;
+    if (c->scene->view.n_tris <= kWarpChainMaxTris && !warp_per_chain(c)) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool captured = cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+    if (c->ahead_use == jr_chains::kUnknown) {
+        if (captured) return false;
+        double sum = 0.0;
+        double* at = reinterpret_cast<double*>(c->view.counters + kCounterDrain);
+        c->ahead_use = jr_chains::kNo;
+        if (launch_sum_p(c->view, at, st) != cudaSuccess ||
+            cudaMemcpyAsync(&sum, at, sizeof(sum), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaStreamSynchronize(st) != cudaSuccess)
+            return false;
+        const double p = sum / (double)n;
+        if (!(p / (p + (double)c->view.c_tilde) < kAheadShare)) return false;
+        c->ahead_use = jr_chains::kYes;
+    }
+    AheadView& a = c->ahead;
+    uint64_t window = least;  // a power of two, so that advances of growing lengths rarely grow it
+    while (window < n_steps) window *= 2;
+    window = std::min<uint64_t>(window, kAheadItems / n);
+    if (a.window < window && !captured) {
+        AheadView b;
+        b.window = (uint32_t)window;
+        if (dev_alloc(&b.F, (size_t)window * n) == cudaSuccess && dev_alloc(&b.queue, n) == cudaSuccess &&
+            dev_alloc(&b.ctl, 4) == cudaSuccess)
+            std::swap(a, b);
+        else
+            (void)cudaGetLastError();
+        cudaFree(b.F);  // the old buffers (this waits for the launches that use them), or a part of the new ones
+        cudaFree(b.queue);
+        cudaFree(b.ctl);
+    }
+    return a.window != 0;
+}
+
+// One warp per chain has no traversal, so no traversal limits either: there the
+// look-ahead paths run under the scene's own.
+static cudaError_t run_ahead(jr_chains* c, uint32_t n_steps, cudaStream_t st, KernelTimer* tm) {
+    const bool warp = warp_per_chain(c);
+    return launch_ahead(warp ? c->scene->view : c->scene_view(), c->view, c->ahead, c->steps, n_steps, warp, st, tm);
+}
+
 static jr_status advance_impl(jr_chains* c, uint32_t n_steps, uint8_t* f, float* dt, int32_t* pix,
                               unsigned long long* work, void* stream, const char* who) {
     if (!c) return fail(JR_ERR_INVALID_ARG, std::string(who) + ": null chains");
@@ -337,7 +411,9 @@ static jr_status advance_impl(jr_chains* c, uint32_t n_steps, uint8_t* f, float*
         return fail(JR_ERR_STATE, std::string(who) + ": traced and counted advances do not run with a flow attached");
     const bool wave = plain && (has_flow || c->exec == JR_EXEC_WAVEFRONT ||
                                 (c->exec == JR_EXEC_AUTO && c->view.n >= kWavefrontMinChains));
-    if (wave) {
+    if (plain && use_ahead(c, n_steps, st)) {
+        JR_CUDA(run_ahead(c, n_steps, st, nullptr), who);
+    } else if (wave) {
         jr_status a = ensure_wavefront(c, st);
         if (a != JR_OK) return a;
         JR_CUDA(launch_wavefront(c->scene_view(), c->view, c->steps, n_steps, st), who);
@@ -374,7 +450,9 @@ jr_status jr_advance_timed(jr_chains* c, uint32_t n_steps, double ms_out[4], uin
         JR_CUDA(launch_fold(c->view, st), "jr_advance_timed");
         c->steps += n_steps;
     } else if (n_steps > 0) {
-        if (wave) {
+        if (use_ahead(c, n_steps, st)) {
+            JR_CUDA(run_ahead(c, n_steps, st, &tm), "jr_advance_timed");
+        } else if (wave) {
             jr_status a = ensure_wavefront(c, st);
             if (a != JR_OK) return a;
             JR_CUDA(launch_wavefront(c->scene_view(), c->view, c->steps, n_steps, st, kModeStep, &tm),

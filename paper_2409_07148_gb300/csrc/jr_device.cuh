@@ -619,6 +619,121 @@ __device__ __forceinline__ void trace_paths(const SceneView& s, Source& src, uns
     }
 }
 
+// ------------------------------------------------------------------ one step of Alg. 2
+// Load chain i's coordinates (pair layout) into shared memory y[d * B].
+__device__ __forceinline__ void load_coords(const ChainView& c, uint64_t i, float* y, uint32_t B) {
+    const float2* x2 = reinterpret_cast<const float2*>(c.x);
+    for (int k = 0; 2 * k < (int)c.dim; ++k) {
+        const float2 v = x2[(uint64_t)k * c.n + i];
+        y[2 * k * B] = v.x;
+        y[(2 * k + 1) * B] = v.y;
+    }
+}
+
+// Alg. 2: holding time t1 ~ Exp(1); killing time t2 ~ Exp(k), k = c~ u / p.  True:
+// the local branch; dt gets the time the state is held for.
+__device__ __forceinline__ bool restore_clocks(const ChainView& c, const uint4& r0, float p, float u, float& dt) {
+    const float E1 = -logf(1.0f - u01(r0.x));
+    const float E2 = -logf(1.0f - u01(r0.y));
+    const float t2 = p > 0.0f ? E2 * p / (c.c_tilde * u) : 0.0f;
+    const bool local = E1 < t2;  // a tie goes to the killing branch
+    dt = local ? E1 : t2;
+    if (c.flags & JR_FLAG_RAO_BLACKWELL) dt = p > 0.0f ? p / (p + c.c_tilde * u) : 0.0f;
+    return local;
+}
+
+// Candidate y of step `step` (cand[d * B]): a Gaussian small step from cur
+// (local) or a fresh draw from mu.
+__device__ __forceinline__ void propose(const ChainView& c, uint32_t chain, uint64_t step, bool local,
+                                        const float* cur, float* cand, uint32_t B) {
+    const int D = (int)c.dim;
+    const float sigma = c.sigma;
+    for (int b = 0; 4 * b < D; ++b) {
+        const uint4 r = draw(c.seed, kTagStep, (uint32_t)(b + 1), chain, step);
+        const int d0 = 4 * b;
+        if (local) {
+            float sn, cs;
+            float R = sqrtf(-2.0f * logf(1.0f - u01(r.x)));
+            sincospif(2.0f * u01(r.y), &sn, &cs);
+            cand[d0 * B] = wrap01(cur[d0 * B] + sigma * R * cs);
+            cand[(d0 + 1) * B] = wrap01(cur[(d0 + 1) * B] + sigma * R * sn);
+            if (d0 + 2 < D) {
+                R = sqrtf(-2.0f * logf(1.0f - u01(r.z)));
+                sincospif(2.0f * u01(r.w), &sn, &cs);
+                cand[(d0 + 2) * B] = wrap01(cur[(d0 + 2) * B] + sigma * R * cs);
+                cand[(d0 + 3) * B] = wrap01(cur[(d0 + 3) * B] + sigma * R * sn);
+            }
+        } else {
+            cand[d0 * B] = u01(r.x);
+            cand[(d0 + 1) * B] = u01(r.y);
+            if (d0 + 2 < D) {
+                cand[(d0 + 2) * B] = u01(r.z);
+                cand[(d0 + 3) * B] = u01(r.w);
+            }
+        }
+    }
+}
+
+// ------------------------------------------------------------------ a whole warp on one path
+// Closest hit of the ray (o, d) over all n triangle records, for the whole
+// warp (every lane calls with the same ray).  Returns the record index or -1.
+__device__ __forceinline__ int closest_hit_warp(const SceneView& s, float3 o, float3 d, float& t_out) {
+    const int lane = threadIdx.x & 31;
+    float tb = INFINITY;
+    int best = -1, bid = INT32_MAX;
+    for (uint32_t k = lane; k < s.n_tris; k += 32) {
+        const TriRecord* tr = s.tris + k;
+        const float4 q0 = __ldg(&tr->v0_id), q1 = __ldg(&tr->e1_mat), q2 = __ldg(&tr->e2);
+        const float3 e1 = f3(q1.x, q1.y, q1.z), e2 = f3(q2.x, q2.y, q2.z);
+        const float3 pv = cross(d, e2);
+        const float det = dot(e1, pv);
+        const float inv = 1.0f / det;
+        const float3 tv = o - f3(q0.x, q0.y, q0.z);
+        const float u = dot(tv, pv) * inv;
+        const float3 qv = cross(tv, e1);
+        const float v = dot(d, qv) * inv;
+        const float t = dot(e2, qv) * inv;
+        const int id = __float_as_int(q0.w);
+        const bool hit = det != 0.0f && !(u < 0.0f || u > 1.0f) && !(v < 0.0f || u + v > 1.0f) && t > 0.0f &&
+                         (t < tb || (t == tb && id < bid));
+        tb = hit ? t : tb;
+        best = hit ? (int)k : best;
+        bid = hit ? id : bid;
+    }
+    // The warp's closest hit, ties to the smaller original index.  Every tb is
+    // a hit distance t > 0 or +inf, and for such floats the bit patterns order
+    // as the values do, so two warp-wide integer minima find it: the nearest
+    // distance, then the smallest index among the lanes at that distance (the
+    // indices are distinct); the lane holding it hands over its record.
+    const unsigned tbits = __float_as_uint(tb);
+    const unsigned tmin = __reduce_min_sync(0xffffffffu, tbits);
+    if (tmin == __float_as_uint(INFINITY)) {  // no lane has a hit
+        t_out = INFINITY;
+        return -1;
+    }
+    const unsigned imin = __reduce_min_sync(0xffffffffu, tbits == tmin ? (unsigned)bid : 0xffffffffu);
+    const int src = __ffs(__ballot_sync(0xffffffffu, tbits == tmin && (unsigned)bid == imin)) - 1;
+    best = __shfl_sync(0xffffffffu, best, src);
+    t_out = __uint_as_float(tmin);
+    return best;
+}
+
+// The integrand F(y) for the warp's chain, y[d] in lane d (eval_path_w's steps).
+__device__ __forceinline__ float3 eval_path_warp(const SceneView& s, int depth, float yd, unsigned& status) {
+    float3 F = f3(0.f, 0.f, 0.f), T = f3(1.f, 1.f, 1.f);
+    float3 o, d;
+    camera_ray(s, __shfl_sync(0xffffffffu, yd, 0), __shfl_sync(0xffffffffu, yd, 1), o, d);
+    for (int v = 0; v <= depth; ++v) {
+        float t;
+        const int k = closest_hit_warp(s, o, d, t);
+        if (k < 0) break;
+        const float u1 = __shfl_sync(0xffffffffu, yd, (2 + 2 * v) & 31);
+        const float u2 = __shfl_sync(0xffffffffu, yd, (3 + 2 * v) & 31);
+        if (!shade_vertex(s, k, t, v, depth, v < depth ? u1 : 0.0f, v < depth ? u2 : 0.0f, o, d, T, F)) break;
+    }
+    return finite_or_zero(F, status);
+}
+
 // ------------------------------------------------------------------ gradient
 // dF/dx for the Langevin local dynamics (MALA), forward mode.  F depends on x
 // continuously only through the directions (camera, scattered) and the modified

@@ -141,6 +141,14 @@ __host__ __device__ inline uint64_t xidx(uint32_t d, uint64_t i, uint64_t n) {
     return ((((uint64_t)(d >> 1)) * n + i) << 1) | (uint64_t)(d & 1u);
 }
 
+// Buffers of the look-ahead execution (jr_ahead.cu; allocated on first use).
+struct AheadView {
+    float4* F = nullptr;          // [window][n] F of the regeneration candidates, and their status bits
+    uint4* queue = nullptr;       // [n] chains whose step is local: (chain, step of the window, origin, 0)
+    unsigned int* ctl = nullptr;  // [4] cursors and the queue length
+    uint32_t window = 0;          // steps per window
+};
+
 struct ChainView {
     float* x;        // PSS coordinates, D x n floats as n float2 per coordinate pair (xidx)
     float* fpu;      // [5][n] F.r F.g F.b p u
@@ -255,6 +263,19 @@ struct HostBvh {
 bool build_bvh(const float* verts, uint32_t n_verts, const uint32_t* tris, uint32_t n_tris,
                const uint32_t* tri_mat, HostBvh* out, std::string* err);
 
+// Device time per kernel class of a sequence of launches on one stream: an
+// event is recorded after every launch, and the time since the previous event
+// is charged to that launch's class.
+struct KernelTimer {
+    enum Kind { kStep = 0, kPath = 1, kReserved = 2, kFlow = 3, kKinds = 4 };
+    std::vector<cudaEvent_t> ev;
+    std::vector<int> kind;  // class of the launch that ends at ev[i] (-1: the start mark)
+    cudaError_t mark(int k, cudaStream_t st);
+    // After the stream is synchronised: ms[k] and launches[k] per class.
+    cudaError_t totals(double ms[kKinds], uint64_t launches[kKinds]) const;
+    ~KernelTimer();
+};
+
 // jr_kernels.cu -- launch wrappers; all return the cudaGetLastError() of the launch.
 cudaError_t launch_init(const SceneView& s, const ChainView& c, cudaStream_t st);
 // One chain per warp (JR_EXEC_WARP): brute-force intersection over every
@@ -286,19 +307,6 @@ cudaError_t launch_eval_grad(const SceneView& s, uint32_t depth, const float* x,
 cudaError_t launch_batch(BatchEntry* entries, const BatchItem* items, uint32_t n_items, const uint64_t* px_off,
                          uint32_t n_sets, uint64_t total_px, unsigned int* cursor, uint32_t max_dim, int block,
                          int checks, uint32_t n_steps, cudaStream_t st);
-// Device time per kernel class of a sequence of launches on one stream: an
-// event is recorded after every launch, and the time since the previous event
-// is charged to that launch's class.
-struct KernelTimer {
-    enum Kind { kStep = 0, kPath = 1, kReserved = 2, kFlow = 3, kKinds = 4 };
-    std::vector<cudaEvent_t> ev;
-    std::vector<int> kind;  // class of the launch that ends at ev[i] (-1: the start mark)
-    cudaError_t mark(int k, cudaStream_t st);
-    // After the stream is synchronised: ms[k] and launches[k] per class.
-    cudaError_t totals(double ms[kKinds], uint64_t launches[kKinds]) const;
-    ~KernelTimer();
-};
-
 // jr_wavefront.cu
 // n_steps wavefront steps in `mode` (WaveMode); for kModeRestart step_begin is
 // the restart epoch and n_steps is 1.  tm (optional) times every launch.
@@ -316,6 +324,14 @@ cudaError_t launch_wavefront_static(const SceneView& s, const ChainView& c, uint
 // Load the module that holds the static scratch on the current device and cache
 // the array's device address (the first call on a device allocates the array).
 cudaError_t prepare_static_scratch();
+
+// jr_ahead.cu: n steps of Alg. 2 in look-ahead windows (uniform mu, no flow, not
+// MH or MALA).  warp_tail: one warp per chain settles the window (small scenes).
+cudaError_t launch_ahead(const SceneView& s, const ChainView& c, const AheadView& a, uint64_t step_begin,
+                         uint32_t n_steps, bool warp_tail, cudaStream_t st, KernelTimer* tm = nullptr);
+// Sum of p over the chains' states into *out (device).
+cudaError_t launch_sum_p(const ChainView& c, double* out, cudaStream_t st);
+constexpr uint64_t kAheadItems = 1u << 24;  // paths per look-ahead window (256 MB of F)
 
 // jr_flow.cu: flow rows through the tensor cores.  Density: u_out[i] = beta q
 // + 1 - beta (and lq_out[i] = log q) for rows i of buf [D][n]; sample: buf

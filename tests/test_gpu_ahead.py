@@ -1,0 +1,85 @@
+"""Look-ahead execution (the auto mode's choice where few steps are local)
+against the megakernel and the wavefront on the same streams."""
+import numpy as np
+import pytest
+
+from paper_2409_07148_gb300 import jr, scenes
+
+pytestmark = pytest.mark.gpu
+
+SCENES = {
+    "box": lambda: scenes.cornell(width=32, height=32, depth=3),          # 24 triangles: one warp per chain settles
+    "spheres": lambda: scenes.cornell_spheres(width=64, height=64, depth=5, n_lon=40, n_lat=41),
+    "flat": lambda: scenes.cornell(width=8, height=8, depth=0),           # D = 2: no bounce, one Philox block, half used
+    "empty": lambda: scenes.empty(),
+}
+
+
+def _run(sc, scene, n, mode, advances, flags, c_tilde):
+    ch = jr.Chains(scene, sc.width, sc.height, sc.depth, n, seed=17, flags=flags, c_tilde=c_tilde, chain_offset=5)
+    ch.set_execution(mode)
+    for k in advances:
+        ch.advance(k)
+    return ch.get_state(), ch.stats(), ch.accumulator()
+
+
+# 1 chain; 256: the latency case, over several calls; 4000: full warps of chains; 5000 and 20000: lanes of
+# a warp at different steps; 1100000: windows of 15 steps, so a ragged last one and states carried over
+@pytest.mark.parametrize("name,n,advances,other", [
+    ("box", 1, [3, 70], "warp"), ("box", 256, [2, 33, 100], "warp"), ("box", 4000, [40], "mega"),
+    ("flat", 1000, [50], "mega"), ("empty", 100, [39], "mega"), ("spheres", 1, [32], "mega"),
+    ("spheres", 5000, [1, 2, 40], "mega"), ("spheres", 20000, [17], "mega"), ("spheres", 1100000, [20], "wave"),
+])
+@pytest.mark.parametrize("flags,c_tilde", [(0, 1.0), (jr.JR_FLAG_RAO_BLACKWELL, 0.3)])
+def test_ahead_equals_the_other_modes(name, n, advances, other, flags, c_tilde):
+    sc = SCENES[name]()
+    scene = jr.Scene(sc)
+    (xa, fa), sa, aa = _run(sc, scene, n, "auto", advances, flags, c_tilde)
+    (xb, fb), sb, ab = _run(sc, scene, n, other, advances, flags, c_tilde)
+    # the same device functions on the same draws: chains part only where a rounding that the
+    # compiler places differently decides a tie
+    same = np.all(xa == xb, axis=0)
+    assert np.mean(~same) <= 1e-4
+    assert np.allclose(fa[:, same], fb[:, same], rtol=1e-5, atol=0)
+    steps = n * sum(advances)
+    assert sa["regenerations"] + sa["local_steps"] == steps == sb["regenerations"] + sb["local_steps"]
+    for key in ("regenerations", "local_steps", "accepted"):
+        assert abs(sa[key] - sb[key]) <= 1e-5 * steps
+    assert sa["status_word"] == sb["status_word"] == 0
+    if np.all(same) and sa == sb:  # FP32 sums per pixel in another order
+        assert np.allclose(aa, ab, rtol=1e-4, atol=1e-6 * np.abs(ab).max())
+
+
+def test_ahead_reports_only_the_paths_a_chain_takes():
+    """A budget that some rays exceed: the same status and the same chains as the
+    wavefront, whatever was traced for nothing."""
+    sc = SCENES["spheres"]()
+    scene = jr.Scene(sc)
+    out = []
+    for mode in ("auto", "wave"):
+        ch = jr.Chains(scene, sc.width, sc.height, sc.depth, 3000, seed=2)
+        ch.set_execution(mode)
+        ch.set_limits(node_visit_budget=12)
+        ch.advance(40)
+        out.append((ch.stats(check=False), *ch.get_state()))
+    assert out[0][0]["status_word"] & jr.JR_STATUS_TRAVERSAL
+    assert out[0][0] == out[1][0]
+    assert np.array_equal(out[0][1], out[1][1])
+    assert np.allclose(out[0][2], out[1][2], rtol=1e-5, atol=0)
+
+
+def test_ahead_without_memory_falls_back():
+    sc = SCENES["spheres"]()
+    scene = jr.Scene(sc)
+    states = []
+    for fail in (False, True):
+        ch = jr.Chains(scene, sc.width, sc.height, sc.depth, 3000, seed=2)
+        if fail:
+            jr.lib().jr_debug_fail_alloc(0)
+        try:
+            ch.advance(33)
+        finally:
+            jr.lib().jr_debug_fail_alloc(-1)
+        ch.advance(32)
+        states.append(ch.get_state()[0])
+    assert np.mean(np.all(states[0] == states[1], axis=0)) >= 1 - 1e-3
