@@ -164,45 +164,79 @@ __device__ __forceinline__ void relu_to_frags(const float (&acc)[8][4], const fl
     }
 }
 
-// One coordinate's CDF step for one row, all 16 bins in this lane.  L: the
-// logits in base 2 (log2 e times the network's output: the layer's bias is
-// stored scaled and the accumulator is scaled in the same FMA), so the softmax
-// e_k = 2^(L_k - max L) = exp(l_k - max l) takes one ex2 per bin (base-2
+// Two FP32 sums in one instruction (sm_100+): each half is the scalar sum.
+__device__ __forceinline__ void add_f32x2(float a0, float a1, float b0, float b1, float& d0, float& d1) {
+    const unsigned long long a = pack_f32x2(a0, a1), b = pack_f32x2(b0, b1);
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(r));
+}
+
+// One coordinate's CDF step for one row, all 16 bins in this lane.  tile: the row's
+// 16 logits in shared memory, in base 2 (log2 e times the network's output: the
+// layer's bias is stored scaled and the accumulator is scaled in the same FMA), so
+// the softmax e_k = 2^(L_k - max L) = exp(l_k - max l) takes one ex2 per bin (base-2
 // softmax, as in FlashAttention-2, Dao 2023; measured -3.6 % per density row).
 // density: v = t in [0,1) becomes CDF(t); sampling: v = c becomes
 // CDF^{-1}(c).  Returns log(K Q[bin]).  With S = sum e, Q_k = sc e_k + E/K,
 // sc = (1 - E)/S.
+//
+// The kernel is bound by the instructions of this step, so it keeps them few: the
+// subtractions and the sum are packed; the mass below the bin is collected under
+// the predicate that finds the bin (the cumulative masses grow, so it holds for
+// exactly the bins below); and the bin's own mass is one more ex2 of a logit read
+// back from the tile, instead of a select per bin.  The sums' order is
+// unchanged.
 template <bool kSample>
-__device__ __forceinline__ float cdf_row(const float (&L)[kFK], float& v) {
+__device__ __forceinline__ float cdf_row(const float* tile, float& v) {
+    float L[kFK];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float4 q4 = reinterpret_cast<const float4*>(tile)[k];
+        L[4 * k] = q4.x;
+        L[4 * k + 1] = q4.y;
+        L[4 * k + 2] = q4.z;
+        L[4 * k + 3] = q4.w;
+    }
     float m = fmax3(fmax3(L[0], L[1], L[2]), fmax3(L[3], L[4], L[5]), fmax3(L[6], L[7], L[8]));
     m = fmax3(m, fmax3(L[9], L[10], L[11]), fmax3(L[12], L[13], fmaxf(L[14], L[15])));
     float e[kFK];
 #pragma unroll
-    for (int k = 0; k < kFK; ++k) e[k] = exp2_approx(L[k] - m);
-    float s4[4];
+    for (int k = 0; k < kFK; k += 2) {
+        add_f32x2(L[k], L[k + 1], -m, -m, e[k], e[k + 1]);
+        e[k] = exp2_approx(e[k]);
+        e[k + 1] = exp2_approx(e[k + 1]);
+    }
+    // (e0 + e1) + (e2 + e3) of each group of four, two groups at a time
+    float a[4], b4[4], s4[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) s4[k] = (e[4 * k] + e[4 * k + 1]) + (e[4 * k + 2] + e[4 * k + 3]);
+    for (int k = 0; k < 4; k += 2) {
+        add_f32x2(e[4 * k], e[4 * k + 4], e[4 * k + 1], e[4 * k + 5], a[k], a[k + 1]);
+        add_f32x2(e[4 * k + 2], e[4 * k + 6], e[4 * k + 3], e[4 * k + 7], b4[k], b4[k + 1]);
+        add_f32x2(a[k], a[k + 1], b4[k], b4[k + 1], s4[k], s4[k + 1]);
+    }
     const float S = (s4[0] + s4[1]) + (s4[2] + s4[3]);
     const float sc = __fdividef(1.0f - kFE, S);  // S in [1, 16]
     int b;
+    float lo_e = 0.f;
     if (!kSample) {
         b = min((int)(v * (float)kFK), kFK - 1);
+#pragma unroll
+        for (int k = 0; k < kFK - 1; ++k)
+            if (k < b) lo_e += e[k];
     } else {
         float cum = 0.f;
-        int cnt = 0;
+        b = 0;
 #pragma unroll
-        for (int k = 0; k < kFK; ++k) {
+        for (int k = 0; k < kFK - 1; ++k) {
             cum += fmaf(e[k], sc, kFE / kFK);
-            cnt += cum <= v;
+            if (cum <= v) {
+                lo_e += e[k];
+                b = k + 1;
+            }
         }
-        b = min(cnt, kFK - 1);
     }
-    float lo_e = 0.f, qb_e = 0.f;
-#pragma unroll
-    for (int k = 0; k < kFK; ++k) {
-        lo_e += k < b ? e[k] : 0.f;
-        qb_e = k == b ? e[k] : qb_e;
-    }
+    const float qb_e = exp2_approx(tile[b] - m);
     const float lo = fmaf(sc, lo_e, (float)b * (kFE / kFK));
     const float qb = fmaf(sc, qb_e, kFE / kFK);
     if (!kSample) {
@@ -290,19 +324,9 @@ __device__ __forceinline__ void coupling(const unsigned char* wl, const uint8_t*
             }
         __syncwarp();
         if (2 * jj < nq) {
-            float L[kFK];
-            const float4* src = reinterpret_cast<const float4*>(lg + r * kLgStride + 16 * jj);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float4 q4 = src[k];
-                L[4 * k] = q4.x;
-                L[4 * k + 1] = q4.y;
-                L[4 * k + 2] = q4.z;
-                L[4 * k + 3] = q4.w;
-            }
             const int cb = pm[A + j0 + jj];
             float vv = xw[r * xs + cb];
-            lqp += cdf_row<kSample>(L, vv);
+            lqp += cdf_row<kSample>(lg + r * kLgStride + 16 * jj, vv);
             xw[r * xs + cb] = vv;
         }
         __syncwarp();
