@@ -50,9 +50,17 @@ constexpr uint32_t kWaitIters = 1u << 26;
 
 // Shared-memory layout (bytes): two mbarriers, perm [kFL][D], row ids
 // [kTile], the rows' states [kTile][D + 1] FP32, per warp a logits tile
-// [16][kLgStride] FP32 (two coordinates' 32 logits per row), one layer buffer
+// [16][32] FP32 (two coordinates' 32 logits per row), one layer buffer
 // (bar[0] counts its copies).
-constexpr int kLgStride = 36;  // conflict-free 16-byte row reads by quarter warps
+//
+// The logits tile's 16-byte chunk c of row r lies at chunk c ^ lg_key(r): the key
+// runs through all eight values over eight rows, so a quarter warp's 16-byte reads
+// of one chunk hit eight bank groups, and through the even (odd) ones over rows
+// 0..3 (4..7), so a half warp's 8-byte writes of two neighbouring chunks do, too.
+// The kernel is bound by shared-memory bandwidth (85 % of it at D = 22); rows padded
+// to 36 floats read without conflicts but wrote with two-way ones.
+constexpr int kLgStride = 32;
+__device__ __forceinline__ int lg_key(int r) { return ((2 * r) & 7) | ((r >> 2) & 1); }
 constexpr size_t kOffBar = 0, kOffPerm = 64, kOffRows = 256, kOffX = kOffRows + 4 * kTile;
 constexpr size_t kLgBytes = sizeof(float) * kWarps * 16 * kLgStride;
 __host__ __device__ constexpr size_t round128(size_t b) { return (b + 127) & ~(size_t)127; }
@@ -173,7 +181,7 @@ __device__ __forceinline__ void add_f32x2(float a0, float a1, float b0, float b1
 }
 
 // One coordinate's CDF step for one row, all 16 bins in this lane.  tile: the row's
-// 16 logits in shared memory, in base 2 (log2 e times the network's output: the
+// logits in shared memory (chunk k of the coordinate's 16 at chunk key ^ k), in base 2 (log2 e times the network's output: the
 // layer's bias is stored scaled and the accumulator is scaled in the same FMA), so
 // the softmax e_k = 2^(L_k - max L) = exp(l_k - max l) takes one ex2 per bin (base-2
 // softmax, as in FlashAttention-2, Dao 2023; measured -3.6 % per density row).
@@ -188,11 +196,11 @@ __device__ __forceinline__ void add_f32x2(float a0, float a1, float b0, float b1
 // back from the tile, instead of a select per bin.  The sums' order is
 // unchanged.
 template <bool kSample>
-__device__ __forceinline__ float cdf_row(const float* tile, float& v) {
+__device__ __forceinline__ float cdf_row(const float* tile, int key, float& v) {
     float L[kFK];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const float4 q4 = reinterpret_cast<const float4*>(tile)[k];
+        const float4 q4 = reinterpret_cast<const float4*>(tile)[key ^ k];
         L[4 * k] = q4.x;
         L[4 * k + 1] = q4.y;
         L[4 * k + 2] = q4.z;
@@ -236,7 +244,7 @@ __device__ __forceinline__ float cdf_row(const float* tile, float& v) {
             }
         }
     }
-    const float qb_e = exp2_approx(tile[b] - m);
+    const float qb_e = exp2_approx(tile[4 * (key ^ (b >> 2)) + (b & 3)] - m);
     const float lo = fmaf(sc, lo_e, (float)b * (kFE / kFK));
     const float qb = fmaf(sc, qb_e, kFE / kFK);
     if (!kSample) {
@@ -317,16 +325,17 @@ __device__ __forceinline__ void coupling(const unsigned char* wl, const uint8_t*
             if (q < nq) {
                 const int c = 8 * q + 2 * t;
                 const float2 bb = *reinterpret_cast<const float2*>(b3 + 16 * j0 + c);
-                *reinterpret_cast<float2*>(lg + g * kLgStride + c) =
+                float* at = lg + g * kLgStride + 4 * ((2 * q + (t >> 1)) ^ lg_key(g)) + 2 * (t & 1);
+                *reinterpret_cast<float2*>(at) =
                     make_float2(fmaf(acc[q][0], kLog2e, bb.x), fmaf(acc[q][1], kLog2e, bb.y));
-                *reinterpret_cast<float2*>(lg + (g + 8) * kLgStride + c) =
+                *reinterpret_cast<float2*>(at + 8 * kLgStride) =  // row g + 8 has row g's key
                     make_float2(fmaf(acc[q][2], kLog2e, bb.x), fmaf(acc[q][3], kLog2e, bb.y));
             }
         __syncwarp();
         if (2 * jj < nq) {
             const int cb = pm[A + j0 + jj];
             float vv = xw[r * xs + cb];
-            lqp += cdf_row<kSample>(lg + r * kLgStride + 16 * jj, vv);
+            lqp += cdf_row<kSample>(lg + r * kLgStride, (4 * jj) ^ lg_key(r), vv);
             xw[r * xs + cb] = vv;
         }
         __syncwarp();
