@@ -27,6 +27,10 @@
 // 24-triangle box 1 024 -> 453 us, 32 steps of 10 007 chains on Cornell + spheres
 // 1 578 -> 988 us, 16 steps of 2^20 11.23 -> 9.65 ms, 400 steps of 10 007 20.6 -> 4.2 ms.
 //
+// MALA Restore chains (JR_FLAG_MALA without JR_FLAG_MH) go the same way: their
+// regenerations need F only, which the megakernel gets from the gradient's
+// evaluation.
+//
 // The draws, the arithmetic and the order of a chain's steps are the other modes',
 // so the chains are the same.
 #include <cuda_runtime.h>
@@ -155,7 +159,9 @@ __device__ __forceinline__ void store_regeneration(const ChainView& c, uint64_t 
 enum { kCtlPaths = 0, kCtlQueue = 1, kCtlTail = 2, kCtlCount = 4 };
 
 // Bound by reading the window's F (16 bytes per step and chain, four steps in
-// flight); the lit states' clocks are rare.
+// flight); the lit states' clocks are rare.  kMala: a chain whose window ends lit
+// also joins the queue, at step K, for its state's drift.
+template <bool kMala>
 __global__ void __launch_bounds__(128) settle_kernel(ChainView c, uint64_t step0, uint32_t K, const float4* Fw,
                                                      uint4* queue, unsigned int* ctl) {
     const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
@@ -198,7 +204,10 @@ __global__ void __launch_bounds__(128) settle_kernel(ChainView c, uint64_t step0
             }
         }
         w.store(c, i);
+        if (kMala && !local && w.p > 0.0f) local = true;
         if (!local && w.org) store_regeneration(c, i, step0 + w.org - 1);
+        if (kMala && !local)  // the drift is 0 where p = 0
+            for (uint32_t d = 0; d < c.dim; ++d) c.drift[d * c.n + i] = 0.0f;
     }
     // one queue atomic per warp
     const unsigned m = __ballot_sync(kFull, local);
@@ -306,6 +315,142 @@ __global__ void __launch_bounds__(32, 16) tail_kernel(SceneView s, ChainView c, 
                     float2* x2 = reinterpret_cast<float2*>(c.x);
                     for (int k = 0; 2 * k < (int)c.dim; ++k)
                         x2[(uint64_t)k * c.n + i] = make_float2(cur[2 * k * B], cur[(2 * k + 1) * B]);
+                }
+            }
+        }
+    }
+    nJ = __reduce_add_sync(kFull, nJ);
+    nL = __reduce_add_sync(kFull, nL);
+    nA = __reduce_add_sync(kFull, nA);
+    status = __reduce_or_sync(kFull, status);
+    if (lane == 0) {
+        if (nJ) atomicAdd(c.counters + 0, (unsigned long long)nJ);
+        if (nL) atomicAdd(c.counters + 1, (unsigned long long)nL);
+        if (nA) atomicAdd(c.counters + 2, (unsigned long long)nA);
+        flush_status(status, c.status);
+    }
+}
+
+// The tail with Langevin local moves (MALA Restore; the kernel of chain_steps_mala's
+// steps).  Only states that a local move starts from or is accepted to, and those a
+// window ends in, need the drift, and so the gradient of their path: a lane's round
+// evaluates either the candidate's (its F and drift) or, for a lit state that came
+// from a regeneration, the state's own drift.
+template <int kCheck>
+__global__ void __launch_bounds__(32, 16) mala_tail_kernel(SceneView s, ChainView c, uint64_t step0, uint32_t K,
+                                                           const float4* Fw, const uint4* queue, unsigned int* ctl) {
+    extern __shared__ float sh[];  // [4][D][32]: x, y, m(x), m(y)
+    constexpr uint32_t B = 32;
+    const int lane = threadIdx.x, D = (int)c.dim;
+    const unsigned count = ctl[kCtlQueue];
+    const unsigned lanes = (count + gridDim.x - 1) / gridDim.x;  // few chains spread over all warps
+    float* cur = sh + lane;
+    float* cand = sh + (size_t)D * B + lane;
+    float* mc = sh + (size_t)2 * D * B + lane;
+    float* my = sh + (size_t)3 * D * B + lane;
+    uint32_t nJ = 0, nL = 0, nA = 0;
+    unsigned status = 0;
+    Work work;
+    Jac3 JF;
+    bool live = false, known = false, drained = (unsigned)lane >= lanes;  // known: mc is the state's drift
+    uint64_t i = 0;
+    uint32_t chain = 0;
+    Walk w;
+    w.k = w.org = 0;
+    while (true) {
+        if (__any_sync(kFull, !live && !drained)) {
+            const unsigned want = __ballot_sync(kFull, !live && !drained);
+            unsigned base = 0;
+            if (lane == 0) base = atomicAdd(ctl + kCtlTail, (unsigned)__popc(want));
+            base = __shfl_sync(kFull, base, 0);
+            if (!live && !drained) {
+                const unsigned q = base + __popc(want & ((1u << lane) - 1u));
+                drained = q >= count;
+                if (!drained) {
+                    const uint4 e = queue[q];
+                    i = e.x;
+                    w.k = e.y;
+                    w.org = e.z;
+                    chain = c.chain_offset + (uint32_t)i;
+                    w.load(c, i);
+                    known = w.org == 0;
+                    if (known) {
+                        load_coords(c, i, cur, B);
+                        for (int d = 0; d < D; ++d) mc[d * B] = c.drift[d * c.n + i];
+                    } else {
+                        propose(c, chain, step0 + w.org - 1, false, cur, cur, B);
+                        w.org = 0;
+                    }
+                    live = true;
+                }
+            }
+        }
+        if (!__any_sync(kFull, live)) break;
+        if (live && known) mala_propose(c, chain, step0 + w.k, cur, mc, cand, B);
+        const float3 Fy = eval_path_grad<kCheck, false>(s, kFull, live, (int)c.depth, known ? cand : cur, B, JF, status,
+                                                        work);
+        if (live) {
+            bool local = true;  // a local step is pending
+            if (!known) {
+                for (int d = 0; d < D; ++d) mc[d * B] = mala_drift(Fy, JF, d, c.sigma);
+                known = true;
+                local = w.k < K;
+            } else {
+                for (int d = 0; d < D; ++d) my[d * B] = mala_drift(Fy, JF, d, c.sigma);
+                const float py = lum(Fy);
+                const float Ua = u01(draw(c.seed, kTagStep, 0, chain, step0 + w.k).z);
+                const bool accept = mala_accept(c, Ua, w.p, py, cur, mc, cand, my, B);
+                nL++;
+                nA += accept;
+                if (accept) {
+                    float* t = cur;
+                    cur = cand;
+                    cand = t;
+                    t = mc;
+                    mc = my;
+                    my = t;
+                    w.Fr = Fy.x;
+                    w.Fg = Fy.y;
+                    w.Fb = Fy.z;
+                    w.p = py;
+                    w.u = 1.0f;
+                }
+                ++w.k;
+                local = false;
+                while (w.k < K && !local) {
+                    if (w.p > 0.0f) {
+                        float dt;
+                        if (w.org) {  // lit after a regeneration: its coordinates are needed now
+                            propose(c, chain, step0 + w.org - 1, false, cur, cur, B);
+                            w.org = 0;
+                            known = false;
+                        }
+                        local = restore_clocks(c, draw(c.seed, kTagStep, 0, chain, step0 + w.k), w.p, w.u, dt);
+                        splat(c, w, cur[0], cur[B], dt);
+                    }
+                    if (!local) {
+                        nJ++;
+                        w.regenerate(__ldcs(Fw + (uint64_t)w.k * c.n + i), status);
+                    }
+                }
+                if (!local && w.org && w.p > 0.0f) {  // the window ends lit: one more round for the drift
+                    propose(c, chain, step0 + w.org - 1, false, cur, cur, B);
+                    w.org = 0;
+                    known = false;
+                    local = true;
+                }
+            }
+            if (!local) {  // the window's end
+                live = false;
+                w.store(c, i);
+                if (w.org) {  // dark
+                    store_regeneration(c, i, step0 + w.org - 1);
+                    for (int d = 0; d < D; ++d) c.drift[d * c.n + i] = 0.0f;
+                } else {
+                    float2* x2 = reinterpret_cast<float2*>(c.x);
+                    for (int k = 0; 2 * k < D; ++k)
+                        x2[(uint64_t)k * c.n + i] = make_float2(cur[2 * k * B], cur[(2 * k + 1) * B]);
+                    for (int d = 0; d < D; ++d) c.drift[d * c.n + i] = mc[d * B];
                 }
             }
         }
@@ -463,8 +608,10 @@ cudaError_t launch_ahead(const SceneView& s, const ChainView& c, const AheadView
     with_checks(trav_checks(s), [&](auto kc) {
         constexpr int kCheck = decltype(kc)::value;
         const auto paths = ahead_path_kernel<kCheck>;
-        const auto tail = tail_kernel<kCheck>;
-        const size_t shm = sizeof(float) * 2 * c.dim * 32;  // <= 8 KB
+        const bool mala = (c.flags & JR_FLAG_MALA) != 0;
+        const auto tail = mala ? mala_tail_kernel<kCheck> : tail_kernel<kCheck>;
+        const auto settle = mala ? settle_kernel<true> : settle_kernel<false>;
+        const size_t shm = sizeof(float) * (mala ? 4 : 2) * c.dim * 32;  // <= 16 KB
         long long path_blocks = 0, tail_blocks = 0;
         if ((e = resident(paths, 128, 0, &path_blocks)) != cudaSuccess) return;
         if (!warp_tail && (e = resident(tail, 32, shm, &tail_blocks)) != cudaSuccess) return;
@@ -483,7 +630,7 @@ cudaError_t launch_ahead(const SceneView& s, const ChainView& c, const AheadView
             if (warp_tail) {
                 settle_warp_kernel<<<grid_for(32 * c.n, 128), 128, 0, st>>>(s, c, step0, K, a.F);
             } else {
-                settle_kernel<<<grid_for(c.n, 128), 128, 0, st>>>(c, step0, K, a.F, a.queue, a.ctl);
+                settle<<<grid_for(c.n, 128), 128, 0, st>>>(c, step0, K, a.F, a.queue, a.ctl);
                 tail<<<(unsigned)std::min<uint64_t>((uint64_t)tail_blocks, c.n), 32, shm, st>>>(s, c, step0, K, a.F,
                                                                                                a.queue, a.ctl);
             }

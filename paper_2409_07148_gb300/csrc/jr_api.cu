@@ -337,6 +337,10 @@ static bool warp_per_chain(const jr_chains* c) {
 // and one warp per chain in the 24-triangle box: 256 chains, 64 steps 159, 198 (16: 88,
 // 69).  Such scenes with more chains than that stay in the megakernel: their paths
 // are short and alike, so it loses little (2^16 chains, 16 steps: 514, 369).
+// MALA Restore, whose megakernel takes the gradient of every candidate, gains from
+// fewer steps on (131 072 chains, 2 steps 497, 1 052 / 542, 863 / 717, 865; 32 768
+// chains, 4 steps 532, 887 / 569, 778 / 719, 729; 10 007 chains, 8 steps 594, 1 161 /
+// 783, 900 / 874, 958; 3 000 chains, 32 steps 1 143, 2 738 / 1 958, 2 039 / 2 388, 2 623).
 //
 // It pays while few steps are local, because a local step's regeneration candidate
 // is traced for nothing.  The stationary share of local steps is p_lambda /
@@ -345,13 +349,15 @@ static bool warp_per_chain(const jr_chains* c) {
 // stream is being captured before they exist, the other modes run.
 constexpr double kAheadShare = 0.25;
 static bool use_ahead(jr_chains* c, uint32_t n_steps, cudaStream_t st) {
-    if (c->exec != JR_EXEC_AUTO || c->view.flow.D != 0 || (c->view.flags & (JR_FLAG_MH | JR_FLAG_MALA)) ||
+    if (c->exec != JR_EXEC_AUTO || c->view.flow.D != 0 || (c->view.flags & JR_FLAG_MH) ||
         c->ahead_use == jr_chains::kNo)
         return false;
     const uint64_t n = c->view.n;
-    const uint32_t least = n >= (1u << 18) ? 2 : n >= (1u << 16) ? 8 : n >= (1u << 14) ? 16 : 32;
+    const bool mala = (c->view.flags & JR_FLAG_MALA) != 0;
+    const uint32_t least = mala ? (n >= (1u << 17) ? 2 : n >= (1u << 15) ? 4 : n >= (1u << 13) ? 8 : 32)
+                                : n >= (1u << 18) ? 2 : n >= (1u << 16) ? 8 : n >= (1u << 14) ? 16 : 32;
     if (n_steps < least || n > kAheadItems / least) return false;
-    if (c->scene->view.n_tris <= kWarpChainMaxTris && !warp_per_chain(c)) return false;
+    if (c->scene->view.n_tris <= kWarpChainMaxTris && (mala || !warp_per_chain(c))) return false;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const bool captured = cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
     if (c->ahead_use == jr_chains::kUnknown) {
@@ -389,7 +395,7 @@ static bool use_ahead(jr_chains* c, uint32_t n_steps, cudaStream_t st) {
 // One warp per chain has no traversal, so no traversal limits either: there the
 // look-ahead paths run under the scene's own.
 static cudaError_t run_ahead(jr_chains* c, uint32_t n_steps, cudaStream_t st, KernelTimer* tm) {
-    const bool warp = warp_per_chain(c);
+    const bool warp = warp_per_chain(c) && !(c->view.flags & JR_FLAG_MALA);
     return launch_ahead(warp ? c->scene->view : c->scene_view(), c->view, c->ahead, c->steps, n_steps, warp, st, tm);
 }
 
@@ -400,9 +406,10 @@ static jr_status advance_impl(jr_chains* c, uint32_t n_steps, uint8_t* f, float*
     cudaStream_t st = (cudaStream_t)stream;
     const bool plain = !f && !dt && !pix && !work;
     const bool has_flow = c->view.flow.D != 0;
-    if (c->view.flags & JR_FLAG_MALA) {  // Langevin moves: the megakernel only
+    if (c->view.flags & JR_FLAG_MALA) {  // Langevin moves: the megakernel, or look-ahead windows
         if (work) return fail(JR_ERR_STATE, std::string(who) + ": the counted advance does not run MALA chains");
-        JR_CUDA(launch_step_mala(c->scene_view(), c->view, c->steps, n_steps, f, dt, pix, st), who);
+        if (plain && use_ahead(c, n_steps, st)) JR_CUDA(run_ahead(c, n_steps, st, nullptr), who);
+        else JR_CUDA(launch_step_mala(c->scene_view(), c->view, c->steps, n_steps, f, dt, pix, st), who);
         JR_CUDA(launch_fold(c->view, st), who);
         c->steps += n_steps;
         return JR_OK;
@@ -443,10 +450,14 @@ jr_status jr_advance_timed(jr_chains* c, uint32_t n_steps, double ms_out[4], uin
                       (c->exec == JR_EXEC_AUTO && c->view.n >= kWavefrontMinChains);
     KernelTimer tm;
     if (n_steps > 0 && (c->view.flags & JR_FLAG_MALA)) {
-        JR_CUDA(tm.mark(-1, st), "jr_advance_timed");
-        JR_CUDA(launch_step_mala(c->scene_view(), c->view, c->steps, n_steps, nullptr, nullptr, nullptr, st),
-                "jr_advance_timed");
-        JR_CUDA(tm.mark(KernelTimer::kStep, st), "jr_advance_timed");
+        if (use_ahead(c, n_steps, st)) {
+            JR_CUDA(run_ahead(c, n_steps, st, &tm), "jr_advance_timed");
+        } else {
+            JR_CUDA(tm.mark(-1, st), "jr_advance_timed");
+            JR_CUDA(launch_step_mala(c->scene_view(), c->view, c->steps, n_steps, nullptr, nullptr, nullptr, st),
+                    "jr_advance_timed");
+            JR_CUDA(tm.mark(KernelTimer::kStep, st), "jr_advance_timed");
+        }
         JR_CUDA(launch_fold(c->view, st), "jr_advance_timed");
         c->steps += n_steps;
     } else if (n_steps > 0) {

@@ -966,6 +966,54 @@ __device__ inline float mala_drift(float3 F, const Jac3& JF, int k, float sigma)
     return fminf(fmaxf(0.5f * sigma * sigma * g, -2.0f * sigma), 2.0f * sigma);
 }
 
+__device__ __forceinline__ float torus_delta(float to, float from) {
+    const float d = to - from;
+    return d - floorf(d + 0.5f);
+}
+
+// log q(b | a) up to the constant, from a's drift ma (all [D] with stride B).
+__device__ __forceinline__ float mala_log_q(const float* b, const float* a, const float* ma, int D, uint32_t B,
+                                            float sigma) {
+    float s = 0.f;
+    for (int d = 0; d < D; ++d) {
+        const float e = torus_delta(b[d * B], a[d * B]) - ma[d * B];
+        s += e * e;
+    }
+    return -s / (2.0f * sigma * sigma);
+}
+
+// The MALA proposal y = x + m(x) + sigma N of step `step` (cand[d * B]).
+__device__ __forceinline__ void mala_propose(const ChainView& c, uint32_t chain, uint64_t step, const float* cur,
+                                             const float* mc, float* cand, uint32_t B) {
+    const int D = (int)c.dim;
+    for (int b = 0; 4 * b < D; ++b) {
+        const uint4 r = draw(c.seed, kTagStep, (uint32_t)(b + 1), chain, step);
+        const int d0 = 4 * b;
+        float sn, cs;
+        float R = sqrtf(-2.0f * logf(1.0f - u01(r.x)));
+        sincospif(2.0f * u01(r.y), &sn, &cs);
+        cand[d0 * B] = wrap01(cur[d0 * B] + mc[d0 * B] + c.sigma * R * cs);
+        cand[(d0 + 1) * B] = wrap01(cur[(d0 + 1) * B] + mc[(d0 + 1) * B] + c.sigma * R * sn);
+        if (d0 + 2 < D) {
+            R = sqrtf(-2.0f * logf(1.0f - u01(r.z)));
+            sincospif(2.0f * u01(r.w), &sn, &cs);
+            cand[(d0 + 2) * B] = wrap01(cur[(d0 + 2) * B] + mc[(d0 + 2) * B] + c.sigma * R * cs);
+            cand[(d0 + 3) * B] = wrap01(cur[(d0 + 3) * B] + mc[(d0 + 3) * B] + c.sigma * R * sn);
+        }
+    }
+}
+
+// Its acceptance, U_a < min(1, p(y) q(x|y) / (p(x) q(y|x))), 1 if p(x) = 0.
+__device__ __forceinline__ bool mala_accept(const ChainView& c, float Ua, float p, float py, const float* cur,
+                                            const float* mc, const float* cand, const float* my, uint32_t B) {
+    if (!(p > 0.0f)) return true;
+    if (!(py > 0.0f)) return false;
+    const int D = (int)c.dim;
+    const float la = logf(py) - logf(p) + mala_log_q(cur, cand, my, D, B, c.sigma) -
+                     mala_log_q(cand, cur, mc, D, B, c.sigma);
+    return Ua > 0.0f ? logf(Ua) < la : true;
+}
+
 __device__ __forceinline__ void flush_status(unsigned status, unsigned int* word) {
     if (status) atomicOr(word, status);
 }

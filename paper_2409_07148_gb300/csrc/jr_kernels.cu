@@ -475,22 +475,6 @@ __global__ void __launch_bounds__(kWarpChainThreads) step_kernel_warp(SceneView 
 // - m_d(a)) on the signed torus difference.  With JR_FLAG_MH the chain is the
 // MALA baseline (large steps from mu with probability l, MALA small steps);
 // otherwise MALA Restore (Alg. 2, local move = the MALA step, k = c~ u / p).
-__device__ __forceinline__ float torus_delta(float to, float from) {
-    const float d = to - from;
-    return d - floorf(d + 0.5f);
-}
-
-// log q(b | a) up to the constant, from a's drift ma (all [D] with stride B).
-__device__ __forceinline__ float mala_log_q(const float* b, const float* a, const float* ma, int D, uint32_t B,
-                                            float sigma) {
-    float s = 0.f;
-    for (int d = 0; d < D; ++d) {
-        const float e = torus_delta(b[d * B], a[d * B]) - ma[d * B];
-        s += e * e;
-    }
-    return -s / (2.0f * sigma * sigma);
-}
-
 template <int kCheck, bool kTrace>
 __device__ __forceinline__ void chain_steps_mala(const SceneView& s, const ChainView& c, uint64_t i, bool active,
                                                  float* sh, uint64_t step_begin, uint32_t n_steps, uint8_t* tr_flags,
@@ -548,30 +532,8 @@ __device__ __forceinline__ void chain_steps_mala(const SceneView& s, const Chain
             atomicAdd(c.fb + pix, make_float4(wgt * Fr, wgt * Fg, wgt * Fb, dt));
         }
         if (active) {
-            for (int b = 0; 4 * b < D; ++b) {
-                const uint4 r = draw(c.seed, kTagStep, (uint32_t)(b + 1), chain, step);
-                const int d0 = 4 * b;
-                if (local) {  // the MALA proposal: drift plus Gaussian pairs
-                    float sn, cs;
-                    float R = sqrtf(-2.0f * logf(1.0f - u01(r.x)));
-                    sincospif(2.0f * u01(r.y), &sn, &cs);
-                    cand[d0 * B] = wrap01(cur[d0 * B] + mc[d0 * B] + c.sigma * R * cs);
-                    cand[(d0 + 1) * B] = wrap01(cur[(d0 + 1) * B] + mc[(d0 + 1) * B] + c.sigma * R * sn);
-                    if (d0 + 2 < D) {
-                        R = sqrtf(-2.0f * logf(1.0f - u01(r.z)));
-                        sincospif(2.0f * u01(r.w), &sn, &cs);
-                        cand[(d0 + 2) * B] = wrap01(cur[(d0 + 2) * B] + mc[(d0 + 2) * B] + c.sigma * R * cs);
-                        cand[(d0 + 3) * B] = wrap01(cur[(d0 + 3) * B] + mc[(d0 + 3) * B] + c.sigma * R * sn);
-                    }
-                } else {
-                    cand[d0 * B] = u01(r.x);
-                    cand[(d0 + 1) * B] = u01(r.y);
-                    if (d0 + 2 < D) {
-                        cand[(d0 + 2) * B] = u01(r.z);
-                        cand[(d0 + 3) * B] = u01(r.w);
-                    }
-                }
-            }
+            if (local) mala_propose(c, chain, step, cur, mc, cand, B);
+            else propose(c, chain, step, false, cur, cand, B);
         }
         const float3 Fy = eval_path_grad<kCheck, false>(s, mask, active, (int)c.depth, cand, B, JF, status, work);
         bool accept = false;
@@ -579,13 +541,7 @@ __device__ __forceinline__ void chain_steps_mala(const SceneView& s, const Chain
             for (int d = 0; d < D; ++d) my[d * B] = mala_drift(Fy, JF, d, c.sigma);
             const float py_ = lum(Fy);
             if (local) {
-                if (!(p > 0.0f)) {
-                    accept = true;
-                } else if (py_ > 0.0f) {
-                    const float la = logf(py_) - logf(p) + mala_log_q(cur, cand, my, D, B, c.sigma) -
-                                     mala_log_q(cand, cur, mc, D, B, c.sigma);
-                    accept = Ua > 0.0f ? logf(Ua) < la : true;
-                }
+                accept = mala_accept(c, Ua, p, py_, cur, mc, cand, my, B);
                 nL++;
                 nA += accept;
             } else if (mh) {  // a large step: uniform and symmetric

@@ -83,3 +83,29 @@ def test_ahead_without_memory_falls_back():
         ch.advance(32)
         states.append(ch.get_state()[0])
     assert np.mean(np.all(states[0] == states[1], axis=0)) >= 1 - 1e-3
+
+
+# several calls, so that the drifts stored at a window's end are used by the next; 1 chain; 3000: lanes
+# at different steps, some with a drift to find first
+@pytest.mark.parametrize("n,advances", [(1, [2, 40]), (3000, [3, 32, 33]), (40000, [5, 4])])
+@pytest.mark.parametrize("c_tilde", [1.0, 0.05])
+def test_ahead_mala_equals_the_megakernel(n, advances, c_tilde):
+    sc = scenes.cornell_spheres(width=64, height=64, depth=4, n_lon=40, n_lat=41)
+    scene = jr.Scene(sc)
+    out = []
+    for mode in ("auto", "mega"):
+        ch = jr.Chains(scene, sc.width, sc.height, sc.depth, n, seed=23, flags=jr.JR_FLAG_MALA, sigma=0.02,
+                       c_tilde=c_tilde)
+        ch.set_execution(mode)
+        for k in advances:
+            ch.advance(k)
+        out.append((ch.get_state(), ch.stats()))
+    ((xa, fa), sa), ((xb, fb), sb) = out
+    # a drift may differ in its last bit (the same function, compiled apart): 2 sigma 2^-23 in x
+    same = np.all(np.abs(xa - xb) <= 1e-6, axis=0)
+    assert np.mean(~same) <= 1e-3
+    assert np.allclose(fa[:, same], fb[:, same], rtol=1e-4, atol=0)
+    steps = n * sum(advances)
+    assert sa["regenerations"] + sa["local_steps"] == steps
+    for key in ("regenerations", "local_steps", "accepted"):
+        assert abs(sa[key] - sb[key]) <= max(1, 1e-4 * steps)
