@@ -14,18 +14,22 @@
 //      with p = 0 is killed at once (k = inf), so a dark step is one 16-byte read;
 //      a lit state draws its clocks and is splatted.  A chain whose step turns out
 //      local stops and joins a queue.
-//   3. tail_kernel: the queued chains, each carried to the window's end by one lane,
-//      with the local moves' paths traced there (or settle_warp_kernel does 2 and 3
-//      with one warp per chain, for scenes of at most kWarpChainMaxTris triangles).
+//   3. The tail: the queued chains, each carried to the window's end by one lane, with
+//      the local moves' paths traced on the way.  It runs inside the next window's
+//      path launch; the last window's is a launch of its own.  With one warp per chain
+//      (scenes of at most kWarpChainMaxTris triangles) settle_warp_kernel does 2 and 3.
 //
 // The wavefront (jr_wavefront.cu) has to end every step's path launch before the
 // next step, so it pays a launch's tail per step (12 % of the warp slots at 2^20
 // chains), and few chains leave the device idle whatever the step does.  Here a
 // launch has K times the paths, and the state is read and written once per window.
 // What it costs: a local step's regeneration candidate is traced for nothing.
-// Measured (start of the change -> with it): 400 steps of 256 chains in the
+// Measured (against the other modes): 400 steps of 256 chains in the
 // 24-triangle box 1 024 -> 453 us, 32 steps of 10 007 chains on Cornell + spheres
-// 1 578 -> 988 us, 16 steps of 2^20 11.23 -> 9.65 ms, 400 steps of 10 007 20.6 -> 4.2 ms.
+// 1 578 -> 988 us, 16 steps of 2^20 11.23 -> 9.65 ms, 400 steps of 10 007 20.6 -> 4.2 ms;
+// with the tail inside the next launch against after its own window, 64 steps of 2^20
+// chains 38.4 -> 36.7 ms, on the slit caustic 20.7 -> 19.0 ms, 32 on the terrain 20.1
+// -> 18.0 ms.
 //
 // MALA Restore chains (JR_FLAG_MALA without JR_FLAG_MH) go the same way: their
 // regenerations need F only, which the megakernel gets from the gradient's
@@ -46,63 +50,6 @@ namespace jr {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-
-// Path j of a window is the regeneration candidate of chain j % n at step
-// step0 + j / n; out[j] = (F, status bits).
-struct AheadPaths {
-    const ChainView& c;
-    uint64_t step0;
-    unsigned count;
-    unsigned int* fetch;
-    float4* out;
-    bool drained = false;
-    uint32_t j = 0;
-    float3 F = f3(0.f, 0.f, 0.f);
-
-    __device__ __forceinline__ uint4 block(uint32_t b) const {
-        const uint32_t n = (uint32_t)c.n, k = j / n;
-        return draw(c.seed, kTagStep, b + 1u, c.chain_offset + (j - k * n), step0 + k);
-    }
-    __device__ __forceinline__ bool take(unsigned idle, bool mine, float& y0, float& y1) {
-        const int lane = threadIdx.x & 31;
-        unsigned base = 0;
-        if (lane == 0) base = atomicAdd(fetch, (unsigned)__popc(idle));
-        base = __shfl_sync(kFull, base, 0);
-        if (base + (unsigned)__popc(idle) >= count) drained = true;
-        const unsigned q = base + __popc(idle & ((1u << lane) - 1u));
-        if (!mine || q >= count) return false;
-        j = q;
-        F = f3(0.f, 0.f, 0.f);
-        const uint4 r = block(0);
-        y0 = u01(r.x);
-        y1 = u01(r.y);
-        return true;
-    }
-    __device__ __forceinline__ const SceneView& camera(const SceneView& s) const { return s; }
-    __device__ __forceinline__ int root(const SceneView& s) const { return s.root; }
-    __device__ __forceinline__ int depth() const { return (int)c.depth; }
-    __device__ __forceinline__ float2 coords(int v) const {  // coordinates 2 + 2v, 3 + 2v
-        const uint4 r = block((uint32_t)(1 + v) >> 1);
-        return v & 1 ? make_float2(u01(r.x), u01(r.y)) : make_float2(u01(r.z), u01(r.w));
-    }
-    __device__ __forceinline__ float3 emission() const { return F; }
-    __device__ __forceinline__ void keep(float3 f) { F = f; }
-    __device__ __forceinline__ void finish(float3 f, unsigned& status) {
-        // the status belongs to the path: it counts only if the chain takes it
-        __stcs(out + j, make_float4(f.x, f.y, f.z, __uint_as_float(status)));
-        status = 0;
-    }
-    __device__ __forceinline__ void batch_done() {}
-};
-
-template <int kCheck>
-__global__ void __launch_bounds__(128, 7) ahead_path_kernel(SceneView s, ChainView c, uint64_t step0, uint32_t count,
-                                                            unsigned int* fetch, float4* out) {
-    if ((uint64_t)blockIdx.x * blockDim.x >= count) return;
-    AheadPaths src{c, step0, count, fetch, out};
-    unsigned status = 0;
-    trace_paths<kCheck>(s, src, status);
-}
 
 // A chain on its way through a window.  org: where the state's coordinates are:
 // 0 in c.x, q > 0: the regeneration of the window's step q - 1.
@@ -157,6 +104,187 @@ __device__ __forceinline__ void store_regeneration(const ChainView& c, uint64_t 
 
 // ctl: [0] the path kernel's cursor, [1] queue length, [2] the tail's cursor.
 enum { kCtlPaths = 0, kCtlQueue = 1, kCtlTail = 2, kCtlCount = 4 };
+
+// The paths of one launch: the tail of a window (chains queued with a local step,
+// each carried to the window's end by one lane), and the regeneration candidates of
+// the next.  The two do not depend on one another, and a tail is a serial chain of
+// local steps for its longest run: beside the next window's paths it costs their
+// issue slots only.
+//
+// A lane's path belongs to chain i.  org = kRegen: the regeneration candidate of the
+// new window's step k; next.F[k n + i] gets (F, status bits).  Otherwise: the local
+// candidate of the tail window's step k, from the state at org (Walk); when it ends
+// the lane takes the acceptance, and goes on through the window until the next local
+// step (cont: its path is to be taken) or the window's end.
+constexpr uint32_t kRegen = 0xffffffffu;
+struct Window {
+    uint64_t step0;
+    uint32_t K;
+    float4* F;  // [K][n]
+};
+// kTail = false: a launch without a tail (1 to 2 % faster without its code).
+template <bool kTail>
+struct MixedPaths {
+    const ChainView& c;
+    Window next, tail;          // next.K = 0: no candidates; tail_count = 0: no tail
+    uint32_t tail_count;
+    int tail_lanes;             // lanes of a warp that take queued chains (few chains spread over all warps)
+    const uint4* queue;
+    unsigned int* ctl;
+    unsigned int* counts;       // shared memory: J, local steps, accepted
+    bool tails_done = false, regens_done = false, drained = false;
+    uint32_t i = 0, k = 0, org = kRegen;
+    bool cont = false;
+    float3 F = f3(0.f, 0.f, 0.f);
+
+    __device__ __forceinline__ bool regen() const { return !kTail || org == kRegen; }
+    __device__ __forceinline__ uint64_t step() const { return (regen() ? next.step0 : tail.step0) + k; }
+    __device__ __forceinline__ uint4 block(uint32_t b, uint64_t st) const {
+        return draw(c.seed, kTagStep, b + 1u, c.chain_offset + i, st);
+    }
+    __device__ __forceinline__ static float2 half_of(const uint4& r, uint32_t pair) {
+        return pair & 1 ? make_float2(u01(r.z), u01(r.w)) : make_float2(u01(r.x), u01(r.y));
+    }
+    // Coordinate pair `pair` of the state at origin o, and of the lane's candidate.
+    __device__ __forceinline__ float2 state_pair(uint32_t o, uint32_t pair) const {
+        if (o == 0) return reinterpret_cast<const float2*>(c.x)[(uint64_t)pair * c.n + i];
+        return half_of(block(pair >> 1, tail.step0 + o - 1), pair);
+    }
+    __device__ __forceinline__ float2 cand_pair(uint32_t pair) const {
+        const float2 z = half_of(block(pair >> 1, step()), pair);
+        if (regen()) return z;
+        const float2 x = state_pair(org, pair);
+        float sn, cs;
+        const float R = sqrtf(-2.0f * logf(1.0f - z.x));
+        sincospif(2.0f * z.y, &sn, &cs);
+        return make_float2(wrap01(x.x + c.sigma * R * cs), wrap01(x.y + c.sigma * R * sn));
+    }
+    __device__ __forceinline__ bool take(unsigned idle, bool mine, float& y0, float& y1) {
+        const int lane = threadIdx.x & 31;
+        const unsigned lt = (1u << lane) - 1u;
+        bool got = kTail && mine && cont;
+        cont = false;
+        if (kTail && !tails_done) {
+            const unsigned want = __ballot_sync(kFull, mine && !got && lane < tail_lanes);
+            if (want) {
+                unsigned base = 0;
+                if (lane == 0) base = atomicAdd(ctl + kCtlTail, (unsigned)__popc(want));
+                base = __shfl_sync(kFull, base, 0);
+                tails_done = base + (unsigned)__popc(want) >= tail_count;
+                const unsigned q = base + __popc(want & lt);
+                if (((want >> lane) & 1u) && q < tail_count) {
+                    const uint4 e = queue[q];
+                    i = e.x;
+                    k = e.y;
+                    org = e.z;
+                    got = true;
+                }
+            }
+        }
+        if (!regens_done) {
+            const unsigned want = __ballot_sync(kFull, mine && !got);
+            if (want) {
+                const uint32_t n = (uint32_t)c.n, count = n * next.K;
+                unsigned base = 0;
+                if (lane == 0) base = atomicAdd(ctl + kCtlPaths, (unsigned)__popc(want));
+                base = __shfl_sync(kFull, base, 0);
+                regens_done = base + (unsigned)__popc(want) >= count;
+                const unsigned q = base + __popc(want & lt);
+                if (((want >> lane) & 1u) && q < count) {
+                    k = q / n;
+                    i = q - k * n;
+                    org = kRegen;
+                    got = true;
+                }
+            }
+        }
+        drained = tails_done && regens_done;
+        if (!got) return false;
+        F = f3(0.f, 0.f, 0.f);
+        const float2 y = cand_pair(0);
+        y0 = y.x;
+        y1 = y.y;
+        return true;
+    }
+    __device__ __forceinline__ const SceneView& camera(const SceneView& s) const { return s; }
+    __device__ __forceinline__ int root(const SceneView& s) const { return s.root; }
+    __device__ __forceinline__ int depth() const { return (int)c.depth; }
+    __device__ __forceinline__ float2 coords(int v) const { return cand_pair(1u + (uint32_t)v); }
+    __device__ __forceinline__ float3 emission() const { return F; }
+    __device__ __forceinline__ void keep(float3 f) { F = f; }
+    __device__ __forceinline__ void finish(float3 f, unsigned& status) {
+        if (regen()) {  // the status belongs to the path: it counts only if the chain takes it
+            __stcs(next.F + (uint64_t)k * c.n + i, make_float4(f.x, f.y, f.z, __uint_as_float(status)));
+        } else {
+            local_step_done(f, status);
+            flush_status(status, c.status);
+        }
+        status = 0;
+    }
+    __device__ __forceinline__ void local_step_done(float3 f, unsigned& status) {
+        Walk w;
+        w.load(c, i);
+        w.k = k;
+        w.org = org;
+        f = finite_or_zero(f, status);
+        const float py = lum(f);
+        const bool accept = u01(draw(c.seed, kTagStep, 0, c.chain_offset + i, step()).z) * w.p < py;
+        atomicAdd(counts + 1, 1u);
+        if (accept) {
+            atomicAdd(counts + 2, 1u);
+            for (uint32_t q = 0; 2 * q < c.dim; ++q)
+                reinterpret_cast<float2*>(c.x)[(uint64_t)q * c.n + i] = cand_pair(q);
+            w.Fr = f.x;
+            w.Fg = f.y;
+            w.Fb = f.z;
+            w.p = py;
+            w.u = 1.0f;
+            w.org = 0;
+        }
+        ++w.k;
+        uint32_t nJ = 0;
+        while (w.k < tail.K && !cont) {
+            if (w.p > 0.0f) {
+                float dt;
+                cont = restore_clocks(c, draw(c.seed, kTagStep, 0, c.chain_offset + i, tail.step0 + w.k), w.p, w.u, dt);
+                const float2 x = state_pair(w.org, 0);
+                splat(c, w, x.x, x.y, dt);
+            }
+            if (!cont) {
+                nJ++;
+                w.regenerate(__ldcs(tail.F + (uint64_t)w.k * c.n + i), status);
+            }
+        }
+        if (nJ) atomicAdd(counts, nJ);
+        w.store(c, i);
+        if (!cont && w.org) store_regeneration(c, i, tail.step0 + w.org - 1);
+        k = w.k;
+        org = w.org;
+    }
+    __device__ __forceinline__ void batch_done() {
+        if (kTail && __any_sync(kFull, cont)) drained = false;
+    }
+};
+
+template <int kCheck, bool kTail>
+__global__ void __launch_bounds__(128, 7) ahead_path_kernel(SceneView s, ChainView c, Window next, Window tail,
+                                                            const uint4* queue, unsigned int* ctl) {
+    __shared__ unsigned int counts[3];
+    if (threadIdx.x < 3) counts[threadIdx.x] = 0;
+    __syncthreads();
+    const uint32_t tails = kTail ? ctl[kCtlQueue] : 0u;
+    const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+    MixedPaths<kTail> src{c, next, tail, tails, (int)((tails + warps - 1) / warps), queue, ctl, counts};
+    src.tails_done = tails == 0;
+    src.regens_done = next.K == 0;
+    src.drained = src.tails_done && src.regens_done;
+    unsigned status = 0;
+    trace_paths<kCheck>(s, src, status);
+    if (!kTail) return;
+    __syncthreads();
+    if (threadIdx.x < 3 && counts[threadIdx.x])
+        atomicAdd(c.counters + threadIdx.x, (unsigned long long)counts[threadIdx.x]);
+}
 
 // Bound by reading the window's F (16 bytes per step and chain, four steps in
 // flight); the lit states' clocks are rare.  kMala: a chain whose window ends lit
@@ -226,9 +354,13 @@ __global__ void __launch_bounds__(128) settle_kernel(ChainView c, uint64_t step0
     }
 }
 
-// The queued chains to the window's end: lane = chain, one-warp blocks, chains
-// fetched as lanes become free (drain_kernel's scheme: a local step waits for no
-// other chain but the few in its warp).
+// The tail by itself: the queued chains to the window's end, lane = chain, one-warp
+// blocks, chains fetched as lanes become free (drain_kernel's scheme: a local step
+// waits for no other chain but the few in its warp).  For an advance's last window,
+// which has no next one to hide in: there the longest run of local steps counts, and
+// this kernel takes a step in less time than trace_paths, whose lanes wait for
+// shading batches and refills (10 007 chains, 32 steps of Cornell + spheres: 596
+// against 680 us).
 template <int kCheck>
 __global__ void __launch_bounds__(32, 16) tail_kernel(SceneView s, ChainView c, uint64_t step0, uint32_t K,
                                                       const float4* Fw, const uint4* queue, unsigned int* ctl) {
@@ -607,36 +739,47 @@ cudaError_t launch_ahead(const SceneView& s, const ChainView& c, const AheadView
     cudaError_t e = cudaSuccess;
     with_checks(trav_checks(s), [&](auto kc) {
         constexpr int kCheck = decltype(kc)::value;
-        const auto paths = ahead_path_kernel<kCheck>;
         const bool mala = (c.flags & JR_FLAG_MALA) != 0;
-        const auto tail = mala ? mala_tail_kernel<kCheck> : tail_kernel<kCheck>;
+        const auto paths = ahead_path_kernel<kCheck, false>, mixed = ahead_path_kernel<kCheck, true>;
         const auto settle = mala ? settle_kernel<true> : settle_kernel<false>;
+        const auto alone = mala ? mala_tail_kernel<kCheck> : tail_kernel<kCheck>;
         const size_t shm = sizeof(float) * (mala ? 4 : 2) * c.dim * 32;  // <= 16 KB
-        long long path_blocks = 0, tail_blocks = 0;
-        if ((e = resident(paths, 128, 0, &path_blocks)) != cudaSuccess) return;
-        if (!warp_tail && (e = resident(tail, 32, shm, &tail_blocks)) != cudaSuccess) return;
+        long long path_blocks = 0, mixed_blocks = 0, tail_blocks = 0;
+        if ((e = resident(paths, 128, 0, &path_blocks)) != cudaSuccess ||
+            (e = resident(mixed, 128, 0, &mixed_blocks)) != cudaSuccess)
+            return;
+        if (!warp_tail && (e = resident(alone, 32, shm, &tail_blocks)) != cudaSuccess) return;
         auto mark = [&](int kind) {
             if (tm && e == cudaSuccess) e = tm->mark(kind, st);
         };
         mark(-1);
-        for (uint32_t done = 0; done < n_steps && e == cudaSuccess;) {
+        Window tail{0, 0, nullptr};  // the window whose tail is still to run
+        for (uint32_t done = 0, k = 0; done < n_steps && e == cudaSuccess; ++k) {
             const uint32_t K = std::min(a.window, n_steps - done);
-            const uint64_t step0 = step_begin + done;
-            const uint32_t count = (uint32_t)(c.n * K);
-            if ((e = cudaMemsetAsync(a.ctl, 0, sizeof(unsigned int) * kCtlCount, st)) != cudaSuccess) return;
-            paths<<<(unsigned)std::min<uint64_t>((uint64_t)path_blocks, grid_for(count, 128)), 128, 0, st>>>(
-                s, c, step0, count, a.ctl + kCtlPaths, a.F);
+            const Window w{step_begin + done, K, a.F + (a.buffers > 1 ? k & 1 : 0) * (uint64_t)a.window * c.n};
+            done += K;
+            if ((e = cudaMemsetAsync(a.ctl + kCtlPaths, 0, sizeof(unsigned int), st)) != cudaSuccess) return;
+            if (tail.K)
+                mixed<<<(unsigned)mixed_blocks, 128, 0, st>>>(s, c, w, tail, a.queue, a.ctl);
+            else
+                paths<<<(unsigned)std::min<uint64_t>((uint64_t)path_blocks, grid_for(c.n * K, 128)), 128, 0, st>>>(
+                    s, c, w, tail, a.queue, a.ctl);
             mark(KernelTimer::kPath);
+            tail.K = 0;
             if (warp_tail) {
-                settle_warp_kernel<<<grid_for(32 * c.n, 128), 128, 0, st>>>(s, c, step0, K, a.F);
+                settle_warp_kernel<<<grid_for(32 * c.n, 128), 128, 0, st>>>(s, c, w.step0, K, w.F);
             } else {
-                settle<<<grid_for(c.n, 128), 128, 0, st>>>(c, step0, K, a.F, a.queue, a.ctl);
-                tail<<<(unsigned)std::min<uint64_t>((uint64_t)tail_blocks, c.n), 32, shm, st>>>(s, c, step0, K, a.F,
-                                                                                               a.queue, a.ctl);
+                if (e == cudaSuccess)
+                    e = cudaMemsetAsync(a.ctl + kCtlQueue, 0, sizeof(unsigned int) * 2, st);  // and kCtlTail
+                settle<<<grid_for(c.n, 128), 128, 0, st>>>(c, w.step0, K, w.F, a.queue, a.ctl);
+                if (mala || a.buffers < 2 || done == n_steps)
+                    alone<<<(unsigned)std::min<uint64_t>((uint64_t)tail_blocks, c.n), 32, shm, st>>>(
+                        s, c, w.step0, K, w.F, a.queue, a.ctl);
+                else
+                    tail = w;
             }
             mark(KernelTimer::kStep);
             if (e == cudaSuccess) e = cudaGetLastError();
-            done += K;
         }
     });
     return e;

@@ -377,10 +377,12 @@ static bool use_ahead(jr_chains* c, uint32_t n_steps, cudaStream_t st) {
     uint64_t window = least;  // a power of two, so that advances of growing lengths rarely grow it
     while (window < n_steps) window *= 2;
     window = std::min<uint64_t>(window, kAheadItems / n);
-    if (a.window < window && !captured) {
+    const uint32_t buffers = n_steps > window ? 2 : 1;
+    if ((a.window < window || a.buffers < buffers) && !captured) {
         AheadView b;
-        b.window = (uint32_t)window;
-        if (dev_alloc(&b.F, (size_t)window * n) == cudaSuccess && dev_alloc(&b.queue, n) == cudaSuccess &&
+        b.window = (uint32_t)std::max<uint64_t>(window, a.window);
+        b.buffers = std::max(buffers, a.buffers);
+        if (dev_alloc(&b.F, (size_t)b.buffers * b.window * n) == cudaSuccess && dev_alloc(&b.queue, n) == cudaSuccess &&
             dev_alloc(&b.ctl, 4) == cudaSuccess)
             std::swap(a, b);
         else

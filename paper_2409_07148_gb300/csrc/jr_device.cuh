@@ -304,7 +304,7 @@ __device__ __forceinline__ bool trav_leaf(const SceneView& s, Trav& r, const int
 // x 10^9 chain steps/s.  The exit waits while the searching lanes outnumber
 // the others (a sparse warp, late in a drain, has nobody to release and would
 // only pay an extra round per node visit).
-constexpr int kSearchExit = 6;
+constexpr int kSearchExit = 8;
 __device__ __forceinline__ bool search_done(unsigned searching, unsigned tracing) {
     const int ns = __popc(searching);
     return ns <= kSearchExit && 2 * ns <= __popc(tracing);

@@ -143,10 +143,11 @@ __host__ __device__ inline uint64_t xidx(uint32_t d, uint64_t i, uint64_t n) {
 
 // Buffers of the look-ahead execution (jr_ahead.cu; allocated on first use).
 struct AheadView {
-    float4* F = nullptr;          // [window][n] F of the regeneration candidates, and their status bits
+    float4* F = nullptr;          // [buffers][window][n] F of the regeneration candidates, and their status bits
     uint4* queue = nullptr;       // [n] chains whose step is local: (chain, step of the window, origin, 0)
     unsigned int* ctl = nullptr;  // [4] cursors and the queue length
     uint32_t window = 0;          // steps per window
+    uint32_t buffers = 0;         // 2: a window's tail runs beside the next window's paths
 };
 
 struct ChainView {
@@ -331,7 +332,11 @@ cudaError_t launch_ahead(const SceneView& s, const ChainView& c, const AheadView
                          uint32_t n_steps, bool warp_tail, cudaStream_t st, KernelTimer* tm = nullptr);
 // Sum of p over the chains' states into *out (device).
 cudaError_t launch_sum_p(const ChainView& c, double* out, cudaStream_t st);
-constexpr uint64_t kAheadItems = 1u << 24;  // paths per look-ahead window (256 MB of F)
+// Paths per look-ahead window (128 MB of F; an advance of several windows keeps two).
+// Shorter windows pay the path launch's end more often, longer ones a longer last
+// tail: 16 steps of 2^20 chains on Cornell + spheres 10.19 (2^21), 9.68 (2^22), 9.64
+// (2^23), 9.88 ms (2^24); slit caustic 6.03, 5.31, 5.30, 5.70 ms.
+constexpr uint64_t kAheadItems = 1u << 23;
 
 // jr_flow.cu: flow rows through the tensor cores.  Density: u_out[i] = beta q
 // + 1 - beta (and lq_out[i] = log q) for rows i of buf [D][n]; sample: buf
