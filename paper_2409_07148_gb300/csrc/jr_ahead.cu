@@ -16,8 +16,9 @@
 //      local stops and joins a queue.
 //   3. The tail: the queued chains, each carried to the window's end by one lane, with
 //      the local moves' paths traced on the way.  It runs inside the next window's
-//      path launch; the last window's is a launch of its own.  With one warp per chain
-//      (scenes of at most kWarpChainMaxTris triangles) settle_warp_kernel does 2 and 3.
+//      path launch; the last window's is a launch of its own, or, with few chains queued,
+//      jr_runs.cu's.  For few chains in scenes of at most kWarpChainMaxTris triangles
+//      jr_runs.cu does 2 and 3.
 //
 // The wavefront (jr_wavefront.cu) has to end every step's path launch before the
 // next step, so it pays a launch's tail per step (12 % of the warp slots at 2^20
@@ -50,60 +51,6 @@ namespace jr {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-
-// A chain on its way through a window.  org: where the state's coordinates are:
-// 0 in c.x, q > 0: the regeneration of the window's step q - 1.
-struct Walk {
-    float Fr, Fg, Fb, p, u;
-    uint32_t k, org;
-    __device__ __forceinline__ void load(const ChainView& c, uint64_t i) {
-        Fr = c.fpu[0 * c.n + i];
-        Fg = c.fpu[1 * c.n + i];
-        Fb = c.fpu[2 * c.n + i];
-        p = c.fpu[3 * c.n + i];
-        u = c.fpu[4 * c.n + i];
-    }
-    __device__ __forceinline__ void store(const ChainView& c, uint64_t i) const {
-        c.fpu[0 * c.n + i] = Fr;
-        c.fpu[1 * c.n + i] = Fg;
-        c.fpu[2 * c.n + i] = Fb;
-        c.fpu[3 * c.n + i] = p;
-        c.fpu[4 * c.n + i] = u;
-    }
-    // Regenerate at step k: f = the candidate's (F, status).
-    __device__ __forceinline__ void regenerate(const float4 f, unsigned& status) {
-        status |= __float_as_uint(f.w);
-        const float3 F = finite_or_zero(f3(f.x, f.y, f.z), status);
-        Fr = F.x;
-        Fg = F.y;
-        Fb = F.z;
-        p = lum(F);
-        u = 1.0f;
-        org = ++k;
-    }
-};
-
-__device__ __forceinline__ void splat(const ChainView& c, const Walk& w, float x0, float x1, float dt) {
-    if (!(dt > 0.0f && w.p > 0.0f)) return;
-    const uint32_t px = min((uint32_t)((double)x0 * (double)c.width), c.width - 1);
-    const uint32_t py = min((uint32_t)((double)x1 * (double)c.height), c.height - 1);
-    const float WH = (float)c.width * (float)c.height;
-    const float wgt = c.c_tilde * dt * WH / w.p;
-    atomicAdd(c.fb + (py * c.width + px), make_float4(wgt * w.Fr, wgt * w.Fg, wgt * w.Fb, dt));
-}
-
-// The coordinates of the regeneration of step `step` into chain i's state.
-__device__ __forceinline__ void store_regeneration(const ChainView& c, uint64_t i, uint64_t step) {
-    float2* x2 = reinterpret_cast<float2*>(c.x);
-    for (int b = 0; 4 * b < (int)c.dim; ++b) {
-        const uint4 r = draw(c.seed, kTagStep, (uint32_t)(b + 1), c.chain_offset + (uint32_t)i, step);
-        x2[(uint64_t)(2 * b) * c.n + i] = make_float2(u01(r.x), u01(r.y));
-        if (4 * b + 2 < (int)c.dim) x2[(uint64_t)(2 * b + 1) * c.n + i] = make_float2(u01(r.z), u01(r.w));
-    }
-}
-
-// ctl: [0] the path kernel's cursor, [1] queue length, [2] the tail's cursor.
-enum { kCtlPaths = 0, kCtlQueue = 1, kCtlTail = 2, kCtlCount = 4 };
 
 // The paths of one launch: the tail of a window (chains queued with a local step,
 // each carried to the window's end by one lane), and the regeneration candidates of
@@ -248,7 +195,7 @@ struct MixedPaths {
                 float dt;
                 cont = restore_clocks(c, draw(c.seed, kTagStep, 0, c.chain_offset + i, tail.step0 + w.k), w.p, w.u, dt);
                 const float2 x = state_pair(w.org, 0);
-                splat(c, w, x.x, x.y, dt);
+                splat_state(c, w, x.x, x.y, dt);
             }
             if (!cont) {
                 nJ++;
@@ -322,7 +269,7 @@ __global__ void __launch_bounds__(128) settle_kernel(ChainView c, uint64_t step0
                         const uint4 r = draw(c.seed, kTagStep, 1, chain, step0 + w.org - 1);
                         x = make_float2(u01(r.x), u01(r.y));
                     }
-                    splat(c, w, x.x, x.y, dt);
+                    splat_state(c, w, x.x, x.y, dt);
                 }
                 if (!local) {
                     nJ++;
@@ -363,11 +310,13 @@ __global__ void __launch_bounds__(128) settle_kernel(ChainView c, uint64_t step0
 // against 680 us).
 template <int kCheck>
 __global__ void __launch_bounds__(32, 16) tail_kernel(SceneView s, ChainView c, uint64_t step0, uint32_t K,
-                                                      const float4* Fw, const uint4* queue, unsigned int* ctl) {
+                                                      const float4* Fw, const uint4* queue, unsigned int* ctl,
+                                                      uint32_t few) {
     extern __shared__ float sh[];
     constexpr uint32_t B = 32;
     const int lane = threadIdx.x;
     const unsigned count = ctl[kCtlQueue];
+    if (count <= few) return;
     // Few chains spread over all warps: the first lanes of each take part.
     const unsigned lanes = (count + gridDim.x - 1) / gridDim.x;
     float* cur = sh + lane;
@@ -431,7 +380,7 @@ __global__ void __launch_bounds__(32, 16) tail_kernel(SceneView s, ChainView c, 
                         w.org = 0;
                     }
                     local = restore_clocks(c, draw(c.seed, kTagStep, 0, chain, step0 + w.k), w.p, w.u, dt);
-                    splat(c, w, cur[0], cur[B], dt);
+                    splat_state(c, w, cur[0], cur[B], dt);
                 }
                 if (!local) {
                     nJ++;
@@ -470,11 +419,13 @@ __global__ void __launch_bounds__(32, 16) tail_kernel(SceneView s, ChainView c, 
 // from a regeneration, the state's own drift.
 template <int kCheck>
 __global__ void __launch_bounds__(32, 16) mala_tail_kernel(SceneView s, ChainView c, uint64_t step0, uint32_t K,
-                                                           const float4* Fw, const uint4* queue, unsigned int* ctl) {
+                                                           const float4* Fw, const uint4* queue, unsigned int* ctl,
+                                                           uint32_t few) {
     extern __shared__ float sh[];  // [4][D][32]: x, y, m(x), m(y)
     constexpr uint32_t B = 32;
     const int lane = threadIdx.x, D = (int)c.dim;
     const unsigned count = ctl[kCtlQueue];
+    if (count <= few) return;
     const unsigned lanes = (count + gridDim.x - 1) / gridDim.x;  // few chains spread over all warps
     float* cur = sh + lane;
     float* cand = sh + (size_t)D * B + lane;
@@ -558,7 +509,7 @@ __global__ void __launch_bounds__(32, 16) mala_tail_kernel(SceneView s, ChainVie
                             known = false;
                         }
                         local = restore_clocks(c, draw(c.seed, kTagStep, 0, chain, step0 + w.k), w.p, w.u, dt);
-                        splat(c, w, cur[0], cur[B], dt);
+                        splat_state(c, w, cur[0], cur[B], dt);
                     }
                     if (!local) {
                         nJ++;
@@ -592,107 +543,6 @@ __global__ void __launch_bounds__(32, 16) mala_tail_kernel(SceneView s, ChainVie
     nA = __reduce_add_sync(kFull, nA);
     status = __reduce_or_sync(kFull, status);
     if (lane == 0) {
-        if (nJ) atomicAdd(c.counters + 0, (unsigned long long)nJ);
-        if (nL) atomicAdd(c.counters + 1, (unsigned long long)nL);
-        if (nA) atomicAdd(c.counters + 2, (unsigned long long)nA);
-        flush_status(status, c.status);
-    }
-}
-
-// Settle and tail in one, a warp per chain (small scenes): lane d holds coordinate
-// d, a local move's path is traced by the whole warp (eval_path_warp), and a dark
-// state looks at the next 32 steps' candidates at once for the first lit one.
-__global__ void __launch_bounds__(128) settle_warp_kernel(SceneView s, ChainView c, uint64_t step0, uint32_t K,
-                                                          const float4* Fw) {
-    const uint64_t i = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
-    if (i >= c.n) return;  // a whole warp
-    const int lane = threadIdx.x & 31;
-    const bool mine = lane < (int)c.dim;
-    const uint32_t chain = c.chain_offset + (uint32_t)i;
-    uint32_t nJ = 0, nL = 0, nA = 0;
-    unsigned status = 0;
-    float xd = mine ? c.x[xidx((uint32_t)lane, i, c.n)] : 0.0f;
-    Walk w;
-    w.k = w.org = 0;
-    w.load(c, i);
-    // coordinate `lane` of the regeneration of the window's step q - 1
-    auto regenerated = [&](uint32_t q) {
-        if (!mine) return 0.0f;
-        const uint4 r = draw(c.seed, kTagStep, (uint32_t)(lane >> 2) + 1u, chain, step0 + q - 1);
-        return u01(lane & 2 ? ((lane & 1) ? r.w : r.z) : ((lane & 1) ? r.y : r.x));
-    };
-    while (w.k < K) {
-        if (!(w.p > 0.0f)) {  // regenerate up to the first lit candidate
-            const uint32_t left = min(32u, K - w.k);
-            float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (lane < (int)left) f = __ldcs(Fw + (uint64_t)(w.k + lane) * c.n + i);
-            // lit, or not to be skipped: not finite, or with a status to report
-            const bool stop = lum(f3(f.x, f.y, f.z)) > 0.0f || !isfinite(f.x) || !isfinite(f.y) || !isfinite(f.z) ||
-                              __float_as_uint(f.w) != 0u;
-            const unsigned m = __ballot_sync(kFull, stop);
-            const uint32_t skip = m ? (uint32_t)__ffs(m) - 1u : left;  // dark ones before it
-            nJ += skip;
-            w.k += skip;
-            if (skip) {  // the last skipped candidate is the state (p = 0)
-                const int src = (int)skip - 1;
-                w.Fr = __shfl_sync(kFull, f.x, src);
-                w.Fg = __shfl_sync(kFull, f.y, src);
-                w.Fb = __shfl_sync(kFull, f.z, src);
-                w.p = lum(f3(w.Fr, w.Fg, w.Fb));
-                w.u = 1.0f;
-                w.org = w.k;
-            }
-            if (m) {
-                const int src = (int)skip;
-                const float4 g = make_float4(__shfl_sync(kFull, f.x, src), __shfl_sync(kFull, f.y, src),
-                                             __shfl_sync(kFull, f.z, src), __shfl_sync(kFull, f.w, src));
-                nJ++;
-                w.regenerate(g, status);
-            }
-            continue;
-        }
-        if (w.org) {
-            xd = regenerated(w.org);
-            w.org = 0;
-        }
-        const uint4 r0 = draw(c.seed, kTagStep, 0, chain, step0 + w.k);
-        float dt;
-        const bool local = restore_clocks(c, r0, w.p, w.u, dt);
-        const float x0 = __shfl_sync(kFull, xd, 0), x1 = __shfl_sync(kFull, xd, 1);
-        if (lane == 0) splat(c, w, x0, x1, dt);
-        if (!local) {
-            nJ++;
-            w.regenerate(__ldcs(Fw + (uint64_t)w.k * c.n + i), status);
-            continue;
-        }
-        float yd = 0.0f;
-        if (mine) {
-            const uint4 r = draw(c.seed, kTagStep, (uint32_t)(lane >> 2) + 1u, chain, step0 + w.k);
-            const bool second = (lane & 2) != 0;
-            float sn, cs;
-            const float R = sqrtf(-2.0f * logf(1.0f - u01(second ? r.z : r.x)));
-            sincospif(2.0f * u01(second ? r.w : r.y), &sn, &cs);
-            yd = wrap01(xd + c.sigma * R * ((lane & 1) ? sn : cs));
-        }
-        const float3 Fy = eval_path_warp(s, (int)c.depth, yd, status);
-        const float py = lum(Fy);
-        const bool accept = u01(r0.z) * w.p < py;
-        nL++;
-        nA += accept;
-        if (accept) {
-            xd = yd;
-            w.Fr = Fy.x;
-            w.Fg = Fy.y;
-            w.Fb = Fy.z;
-            w.p = py;
-            w.u = 1.0f;
-        }
-        ++w.k;
-    }
-    if (w.org) xd = regenerated(w.org);
-    if (mine) c.x[xidx((uint32_t)lane, i, c.n)] = xd;
-    if (lane == 0) {
-        w.store(c, i);
         if (nJ) atomicAdd(c.counters + 0, (unsigned long long)nJ);
         if (nL) atomicAdd(c.counters + 1, (unsigned long long)nL);
         if (nA) atomicAdd(c.counters + 2, (unsigned long long)nA);
@@ -767,16 +617,20 @@ cudaError_t launch_ahead(const SceneView& s, const ChainView& c, const AheadView
             mark(KernelTimer::kPath);
             tail.K = 0;
             if (warp_tail) {
-                settle_warp_kernel<<<grid_for(32 * c.n, 128), 128, 0, st>>>(s, c, w.step0, K, w.F);
+                if (e == cudaSuccess) e = launch_runs_settle(s, c, w.step0, K, w.F, st);
             } else {
                 if (e == cudaSuccess)
                     e = cudaMemsetAsync(a.ctl + kCtlQueue, 0, sizeof(unsigned int) * 2, st);  // and kCtlTail
                 settle<<<grid_for(c.n, 128), 128, 0, st>>>(c, w.step0, K, w.F, a.queue, a.ctl);
-                if (mala || a.buffers < 2 || done == n_steps)
+                if (mala || a.buffers < 2 || done == n_steps) {
+                    uint32_t few = 0;  // queues this short are launch_runs_tail's
+                    if (!mala && e == cudaSuccess)
+                        e = launch_runs_tail(s, c, w.step0, K, w.F, a.queue, a.ctl, &few, st);
                     alone<<<(unsigned)std::min<uint64_t>((uint64_t)tail_blocks, c.n), 32, shm, st>>>(
-                        s, c, w.step0, K, w.F, a.queue, a.ctl);
-                else
+                        s, c, w.step0, K, w.F, a.queue, a.ctl, few);
+                } else {
                     tail = w;
+                }
             }
             mark(KernelTimer::kStep);
             if (e == cudaSuccess) e = cudaGetLastError();

@@ -1480,11 +1480,14 @@ jr_status jr_flow_train_rows(jr_flow* f, const float* x_dev, const float* w_dev,
 
 namespace {
 
-// Without a flow, a drain's steps run in the wavefront while more chains than
-// this may be open, then in launches of drain_kernel of at most kDrainTailSteps
-// steps (which bounds one launch).  The line is where the wavefront's packed
-// warps stop paying for its waiting on the longest path of every step.
-constexpr uint32_t kDrainTailChains = 1u << 16, kDrainTailSteps = 4096;
+// Without a flow, a drain's steps run in the wavefront while more than
+// kDrainTailChains chains may be open (there its packed warps pay), then in launches
+// of drain_kernel of 8, 16, 32 ... at most kDrainTailSteps steps, and once at most
+// kRunsDrainMost are open, a block takes each tour several steps at a time (jr_runs.cu).
+// A checkpoint of 2^18 chains on the slit caustic: 37.0 ms in the wavefront alone, 8.5
+// ms with drain_kernel, and with the blocks from 400, 1 400, 2 500, 10 000 open tours on
+// 7.9, 6.0, 5.8, 5.8 ms; 100 000 chains on the terrain 28.8, 5.9; 5.4, 4.9, 4.7, 4.8 ms.
+constexpr uint32_t kDrainTailChains = 1u << 16, kDrainFirstSteps = 8, kDrainTailSteps = 4096, kRunsDrainMost = 2500;
 
 // Drain: advance only the chains that are inside a tour until every tour has
 // ended (a kill ends the tour and the chain); the steps are regular steps of
@@ -1514,10 +1517,15 @@ jr_status drain_impl(jr_chains* c, uint32_t max_steps, uint64_t* remaining, cuda
         JR_CUDA(cudaStreamSynchronize(st), who);
         group = std::min<uint32_t>(2 * group, 16);
     }
-    while (active > 0 && k < max_steps) {  // few open tours: each runs to its end without waiting for the others
-        const uint32_t g = std::min(kDrainTailSteps, max_steps - k);
+    // Few open tours: each runs without waiting for the others, in launches of growing
+    // length until only the longest are left, which a block each then takes several
+    // steps at a time.
+    for (uint32_t len = kDrainFirstSteps; active > 0 && k < max_steps; len = std::min(2 * len, kDrainTailSteps)) {
+        const bool runs = k > 0 && active <= kRunsDrainMost;
+        const uint32_t g = std::min(runs ? kDrainTailSteps : len, max_steps - k);
         unsigned long long* ctl = c->view.counters + kCounterDrain;
-        JR_CUDA(launch_drain(c->scene_view(), c->view, c->view.wf.done, s0 + k, g, ctl, st), who);
+        if (runs) JR_CUDA(launch_runs_drain(c->scene_view(), c->view, s0 + k, g, ctl, st), who);
+        else JR_CUDA(launch_drain(c->scene_view(), c->view, c->view.wf.done, s0 + k, g, ctl, st), who);
         k += g;
         unsigned long long open = 0;
         JR_CUDA(cudaMemcpyAsync(&open, ctl + 1, sizeof(open), cudaMemcpyDeviceToHost, st), who);

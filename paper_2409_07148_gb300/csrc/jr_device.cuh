@@ -632,14 +632,16 @@ __device__ __forceinline__ void load_coords(const ChainView& c, uint64_t i, floa
 
 // Alg. 2: holding time t1 ~ Exp(1); killing time t2 ~ Exp(k), k = c~ u / p.  True:
 // the local branch; dt gets the time the state is held for.
-__device__ __forceinline__ bool restore_clocks(const ChainView& c, const uint4& r0, float p, float u, float& dt) {
-    const float E1 = -logf(1.0f - u01(r0.x));
-    const float E2 = -logf(1.0f - u01(r0.y));
+__device__ __forceinline__ bool restore_clocks_at(const ChainView& c, float E1, float E2, float p, float u,
+                                                  float& dt) {
     const float t2 = p > 0.0f ? E2 * p / (c.c_tilde * u) : 0.0f;
     const bool local = E1 < t2;  // a tie goes to the killing branch
     dt = local ? E1 : t2;
     if (c.flags & JR_FLAG_RAO_BLACKWELL) dt = p > 0.0f ? p / (p + c.c_tilde * u) : 0.0f;
     return local;
+}
+__device__ __forceinline__ bool restore_clocks(const ChainView& c, const uint4& r0, float p, float u, float& dt) {
+    return restore_clocks_at(c, -logf(1.0f - u01(r0.x)), -logf(1.0f - u01(r0.y)), p, u, dt);
 }
 
 // Candidate y of step `step` (cand[d * B]): a Gaussian small step from cur
@@ -671,6 +673,57 @@ __device__ __forceinline__ void propose(const ChainView& c, uint32_t chain, uint
                 cand[(d0 + 3) * B] = u01(r.w);
             }
         }
+    }
+}
+
+// A chain on its way through a window.  org: where the state's coordinates are:
+// 0 in c.x, q > 0: the regeneration of the window's step q - 1.
+struct Walk {
+    float Fr, Fg, Fb, p, u;
+    uint32_t k, org;
+    __device__ __forceinline__ void load(const ChainView& c, uint64_t i) {
+        Fr = c.fpu[0 * c.n + i];
+        Fg = c.fpu[1 * c.n + i];
+        Fb = c.fpu[2 * c.n + i];
+        p = c.fpu[3 * c.n + i];
+        u = c.fpu[4 * c.n + i];
+    }
+    __device__ __forceinline__ void store(const ChainView& c, uint64_t i) const {
+        c.fpu[0 * c.n + i] = Fr;
+        c.fpu[1 * c.n + i] = Fg;
+        c.fpu[2 * c.n + i] = Fb;
+        c.fpu[3 * c.n + i] = p;
+        c.fpu[4 * c.n + i] = u;
+    }
+    // Regenerate at step k: f = the candidate's (F, status).
+    __device__ __forceinline__ void regenerate(const float4 f, unsigned& status) {
+        status |= __float_as_uint(f.w);
+        const float3 F = finite_or_zero(f3(f.x, f.y, f.z), status);
+        Fr = F.x;
+        Fg = F.y;
+        Fb = F.z;
+        p = lum(F);
+        u = 1.0f;
+        org = ++k;
+    }
+};
+
+__device__ __forceinline__ void splat_state(const ChainView& c, const Walk& w, float x0, float x1, float dt) {
+    if (!(dt > 0.0f && w.p > 0.0f)) return;
+    const uint32_t px = min((uint32_t)((double)x0 * (double)c.width), c.width - 1);
+    const uint32_t py = min((uint32_t)((double)x1 * (double)c.height), c.height - 1);
+    const float WH = (float)c.width * (float)c.height;
+    const float wgt = c.c_tilde * dt * WH / w.p;
+    atomicAdd(c.fb + (py * c.width + px), make_float4(wgt * w.Fr, wgt * w.Fg, wgt * w.Fb, dt));
+}
+
+// The coordinates of the regeneration of step `step` into chain i's state.
+__device__ __forceinline__ void store_regeneration(const ChainView& c, uint64_t i, uint64_t step) {
+    float2* x2 = reinterpret_cast<float2*>(c.x);
+    for (int b = 0; 4 * b < (int)c.dim; ++b) {
+        const uint4 r = draw(c.seed, kTagStep, (uint32_t)(b + 1), c.chain_offset + (uint32_t)i, step);
+        x2[(uint64_t)(2 * b) * c.n + i] = make_float2(u01(r.x), u01(r.y));
+        if (4 * b + 2 < (int)c.dim) x2[(uint64_t)(2 * b + 1) * c.n + i] = make_float2(u01(r.z), u01(r.w));
     }
 }
 

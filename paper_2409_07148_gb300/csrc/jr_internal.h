@@ -326,6 +326,23 @@ cudaError_t launch_wavefront_static(const SceneView& s, const ChainView& c, uint
 // the array's device address (the first call on a device allocates the array).
 cudaError_t prepare_static_scratch();
 
+// Look-ahead control words: the path kernel's cursor, the queue's length, the
+// tail's cursor.
+enum AheadCtl { kCtlPaths = 0, kCtlQueue = 1, kCtlTail = 2, kCtlCount = 4 };
+
+// jr_runs.cu: local moves of few chains, one block per chain, several steps at a
+// time by speculation.
+// A window's steps for every chain (scenes of at most kWarpChainMaxTris triangles).
+cudaError_t launch_runs_settle(const SceneView& s, const ChainView& c, uint64_t step0, uint32_t K, const float4* F,
+                               cudaStream_t st);
+// A window's queued chains, if there are at most *most of them (set by the call);
+// tail_kernel takes them otherwise.
+cudaError_t launch_runs_tail(const SceneView& s, const ChainView& c, uint64_t step0, uint32_t K, const float4* F,
+                             const uint4* queue, unsigned int* ctl, uint32_t* most, cudaStream_t st);
+// As launch_drain with skip = c.wf.done, for few open tours.
+cudaError_t launch_runs_drain(const SceneView& s, const ChainView& c, uint64_t step_begin, uint32_t n_steps,
+                              unsigned long long* ctl, cudaStream_t st);
+
 // jr_ahead.cu: n steps of Alg. 2 in look-ahead windows (uniform mu, no flow, not
 // MH or MALA).  warp_tail: one warp per chain settles the window (small scenes).
 cudaError_t launch_ahead(const SceneView& s, const ChainView& c, const AheadView& a, uint64_t step_begin,
