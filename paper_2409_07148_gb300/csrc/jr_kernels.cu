@@ -765,7 +765,9 @@ __global__ void eval_states_kernel(SceneView s, uint32_t depth, float c_tilde, c
 // Plain path tracing by persistent warps (trace_paths).  Warp w of the grid traces
 // samples [w n / warps, (w + 1) n / warps): no cursor in memory, so calls on
 // several streams share nothing.  The coordinates are drawn where they are used (one Philox
-// block per vertex), so a path reads and writes nothing but its pixel.  Against
+// block per vertex), so a path reads and writes nothing but its pixel.  list (scenes
+// with a modified Phong material, see launch_render_pt): the lit samples are listed
+// instead of accumulated.  Against
 // one thread per path, whose warp waits for the longest ray of every vertex and
 // for its longest path: 2.76 -> 1.27 ms for 2^21 samples of Cornell + spheres.
 struct PtPaths {
@@ -773,7 +775,10 @@ struct PtPaths {
     int dep;
     uint64_t seed, next, end;  // next sample of the warp, end of its range
     double* accum;
-    bool drained = false;
+    uint32_t* list;              // offsets from sample `begin`
+    unsigned int* listed;
+    uint64_t begin;
+    bool drained = false, lit = false;
     uint64_t smp = 0;
     float3 F = f3(0.f, 0.f, 0.f);
 
@@ -802,8 +807,12 @@ struct PtPaths {
     __device__ __forceinline__ float3 emission() const { return F; }
     __device__ __forceinline__ void keep(float3 f) { F = f; }
     __device__ __forceinline__ void finish(float3 f, unsigned& status) {
-        f = finite_or_zero(f, status);
         if (f.x == 0.f && f.y == 0.f && f.z == 0.f) return;
+        if (list) {
+            lit = true;
+            return;
+        }
+        f = finite_or_zero(f, status);
         const uint4 r = block(0);
         const uint32_t px = min((uint32_t)((double)u01(r.x) * (double)W), W - 1);
         const uint32_t py = min((uint32_t)((double)u01(r.y) * (double)H), H - 1);
@@ -814,21 +823,65 @@ struct PtPaths {
         if (f.z != 0.f) atomicAdd(a + 2, WH * f.z);
         // channel 3 is left to the caller: the sample count is n, known on the host
     }
-    __device__ __forceinline__ void batch_done() {}
+    __device__ __forceinline__ void batch_done() {
+        if (!list) return;
+        const unsigned m = __ballot_sync(0xffffffffu, lit);
+        if (m) {
+            const int lane = threadIdx.x & 31;
+            unsigned base = 0;
+            if (lane == 0) base = atomicAdd(listed, (unsigned)__popc(m));
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (lit) list[base + __popc(m & ((1u << lane) - 1u))] = (uint32_t)(smp - begin);
+        }
+        lit = false;
+    }
 };
 
 template <int kCheck>
 __global__ void __launch_bounds__(128, 7) render_pt_kernel(SceneView s, uint32_t W, uint32_t H, uint32_t depth,
                                                            uint64_t seed, uint64_t sample_begin, uint64_t n,
-                                                           double* accum) {
+                                                           double* accum, uint32_t* list, unsigned int* listed) {
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
     const uint64_t w = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
     const uint64_t per = n / warps, more = n % warps;  // the first `more` warps take one sample more
     const uint64_t first = sample_begin + w * per + min(w, more);
-    PtPaths src{W, H, (int)depth, seed, first, first + per + (w < more ? 1 : 0), accum};
+    PtPaths src{W, H, (int)depth, seed, first, first + per + (w < more ? 1 : 0), accum, list, listed, sample_begin};
     unsigned status = 0;
     src.drained = src.next >= src.end;
     trace_paths<kCheck>(s, src, status);
+}
+
+// One thread per path: samples sample_begin + list[i] for i < *listed, or sample_begin
+// + i for i < n when list is null.
+template <int kCheck>
+__global__ void render_pt_each_kernel(SceneView s, uint32_t W, uint32_t H, uint32_t depth, uint64_t seed,
+                                      uint64_t sample_begin, uint64_t n, double* accum, const uint32_t* list,
+                                      const unsigned int* listed) {
+    extern __shared__ float sh[];
+    const uint32_t B = blockDim.x, tid = threadIdx.x;
+    const uint64_t i = blockIdx.x * (uint64_t)B + tid;
+    const uint64_t count = list ? *listed : n;
+    const unsigned mask = __ballot_sync(0xffffffffu, i < count);
+    if (i >= count) return;
+    const int D = 2 + 2 * (int)depth;
+    float* y = sh + tid;
+    const uint64_t smp = sample_begin + (list ? list[i] : i);
+    for (int b = 0; 4 * b < D; ++b) {
+        const uint4 r = draw(seed, kTagPt, (uint32_t)(b + 1), (uint32_t)smp, smp >> 32);
+        const uint32_t rr[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (4 * b + q < D) y[(4 * b + q) * B] = u01(rr[q]);
+    }
+    unsigned status = 0;
+    const float3 F = eval_path<kCheck>(s, mask, true, (int)depth, y, B, nullptr, 0, status);
+    uint32_t px = min((uint32_t)((double)y[0] * (double)W), W - 1);
+    uint32_t py = min((uint32_t)((double)y[B] * (double)H), H - 1);
+    const double WH = (double)W * (double)H;
+    double* a = accum + 4 * ((size_t)py * W + px);
+    if (F.x != 0.f) atomicAdd(a, WH * F.x);
+    if (F.y != 0.f) atomicAdd(a + 1, WH * F.y);
+    if (F.z != 0.f) atomicAdd(a + 2, WH * F.z);
 }
 
 __global__ void philox_kernel(uint64_t seed, uint32_t tag, uint32_t block, uint64_t chain_begin, uint64_t step,
@@ -1111,11 +1164,33 @@ cudaError_t launch_eval_states(const SceneView& s, uint32_t depth, float c_tilde
     return cudaGetLastError();
 }
 
+// Scenes with a modified Phong material: the lobe's arithmetic rounds in the last bit
+// as the compiler contracts it, and it does so differently in the two kernels; the
+// FP64 sums would differ by 3e-9.  So there the persistent kernel only finds the lit
+// samples (1 % of them on Cornell + spheres), and one thread per path evaluates those
+// (and every sample of a small call, where the list would cost more than it saves).
+constexpr uint64_t kRenderListMin = 1u << 19, kRenderListMax = 1u << 24;
+
 cudaError_t launch_render_pt(const SceneView& s, uint32_t width, uint32_t height, uint32_t depth, uint64_t seed,
                              uint64_t sample_begin, uint64_t n, double* accum, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     cudaError_t e = cudaSuccess;
+    const bool each = s.phong && n < kRenderListMin;
+    const size_t shm = sizeof(float) * (2 + 2 * depth) * 128;
+    unsigned int* listed = nullptr;  // the count, then the list (256 bytes on)
+    uint32_t* list = nullptr;
+    if (s.phong && !each) {
+        const uint64_t most = std::min(n, kRenderListMax);
+        if ((e = cudaMallocAsync((void**)&listed, 256 + sizeof(uint32_t) * most, st)) != cudaSuccess) return e;
+        list = listed + 64;
+    }
     with_checks(trav_checks(s), [&](auto k) {
+        if (each) {
+            render_pt_each_kernel<k()><<<grid_for(n, 128), 128, shm, st>>>(s, width, height, depth, seed, sample_begin,
+                                                                           n, accum, nullptr, nullptr);
+            e = cudaGetLastError();
+            return;
+        }
         static DeviceOnce once;  // per device and variant: the persistent grid
         const auto kernel = render_pt_kernel<decltype(k)::value>;
         long long packed = 0;    // SMs, and resident blocks per SM above them
@@ -1130,18 +1205,30 @@ cudaError_t launch_render_pt(const SceneView& s, uint32_t width, uint32_t height
                 return cudaSuccess;
             },
             &packed);
-        if (e != cudaSuccess) return;
         const long long sms = packed & 0xffffffffll;
-        long long blocks = sms * (packed >> 32);
-        // Two samples per lane while that fills three blocks per SM (a warp that
-        // refills hides its longest path), then one per lane: 100 000 samples of
-        // Cornell + spheres take 175 us over every resident warp, 152 us over 391
-        // blocks; 50 000 take 152 us, 133 us over 391 blocks and 146 us over 196.
-        const uint64_t want = std::max<uint64_t>((n + 255) / 256, std::min<uint64_t>((n + 127) / 128, 3 * (uint64_t)sms));
-        blocks = (long long)std::min<uint64_t>((uint64_t)blocks, want);
-        kernel<<<(unsigned)blocks, 128, 0, st>>>(s, width, height, depth, seed, sample_begin, n, accum);
-        e = cudaGetLastError();
+        const uint64_t blocks = (uint64_t)(sms * (packed >> 32));
+        for (uint64_t done = 0; done < n && e == cudaSuccess;) {
+            const uint64_t m = list ? std::min(n - done, kRenderListMax) : n;
+            // Two samples per lane while that fills three blocks per SM (a warp that
+            // refills hides its longest path), then one per lane: 100 000 samples of
+            // Cornell + spheres take 175 us over every resident warp, 152 us over 391
+            // blocks; 50 000 take 152 us, 133 us over 391 blocks and 146 us over 196.
+            const uint64_t want =
+                std::max<uint64_t>((m + 255) / 256, std::min<uint64_t>((m + 127) / 128, 3 * (uint64_t)sms));
+            if (list && (e = cudaMemsetAsync(listed, 0, sizeof(unsigned int), st)) != cudaSuccess) break;
+            kernel<<<(unsigned)std::min(blocks, want), 128, 0, st>>>(s, width, height, depth, seed, sample_begin + done,
+                                                                     m, accum, list, listed);
+            if (list)
+                render_pt_each_kernel<k()><<<grid_for(m, 128), 128, shm, st>>>(
+                    s, width, height, depth, seed, sample_begin + done, m, accum, list, listed);
+            e = cudaGetLastError();
+            done += m;
+        }
     });
+    if (listed) {
+        const cudaError_t f = cudaFreeAsync(listed, st);
+        if (e == cudaSuccess) e = f;
+    }
     return e;
 }
 
