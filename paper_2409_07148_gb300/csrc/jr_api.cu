@@ -81,6 +81,7 @@ struct jr_chains {
     int stack_limit = 0;
     AheadView ahead{};          // look-ahead buffers (JR_EXEC_AUTO), and whether they are worth having
     enum Ahead { kUnknown, kYes, kNo } ahead_use = kUnknown;
+    bool ahead_fixed = false;   // a captured graph holds the buffers' addresses: they stay as they are
     // The scene as this set's launches see it (with the set's traversal limits).
     SceneView scene_view() const {
         SceneView v = scene->view;
@@ -349,6 +350,16 @@ static bool warp_per_chain(const jr_chains* c) {
 // own states (at first samples of mu).  Where the buffers cannot be had, or the
 // stream is being captured before they exist, the other modes run.
 constexpr double kAheadShare = 0.25;
+
+// Lets this thread allocate while some other stream of it captures in the global mode.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { (void)cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { (void)cudaThreadExchangeStreamCaptureMode(&mode); }
+    RelaxedCapture(const RelaxedCapture&) = delete;
+    RelaxedCapture& operator=(const RelaxedCapture&) = delete;
+};
+
 static bool use_ahead(jr_chains* c, uint32_t n_steps, cudaStream_t st) {
     if (c->exec != JR_EXEC_AUTO || c->view.flow.D != 0 || (c->view.flags & JR_FLAG_MH) ||
         c->ahead_use == jr_chains::kNo)
@@ -361,8 +372,12 @@ static bool use_ahead(jr_chains* c, uint32_t n_steps, cudaStream_t st) {
     if (c->scene->view.n_tris <= kWarpChainMaxTris && (mala || !warp_per_chain(c))) return false;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const bool captured = cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+    if (captured) {  // with the buffers an advance outside a capture left, or not at all
+        c->ahead_fixed = c->ahead_fixed || c->ahead.window != 0;
+        return c->ahead.window != 0;
+    }
+    RelaxedCapture relaxed;  // another stream of this thread may be capturing
     if (c->ahead_use == jr_chains::kUnknown) {
-        if (captured) return false;
         double sum = 0.0;
         double* at = reinterpret_cast<double*>(c->view.counters + kCounterDrain);
         c->ahead_use = jr_chains::kNo;
@@ -373,13 +388,16 @@ static bool use_ahead(jr_chains* c, uint32_t n_steps, cudaStream_t st) {
         const double p = sum / (double)n;
         if (!(p / (p + (double)c->view.c_tilde) < kAheadShare)) return false;
         c->ahead_use = jr_chains::kYes;
+        // A later advance of fewer steps is the wavefront's, and may be captured: its
+        // buffers have to exist by then.
+        if (!mala && n >= kWavefrontMinChains && ensure_wavefront(c, st) != JR_OK) (void)cudaGetLastError();
     }
     AheadView& a = c->ahead;
     uint64_t window = least;  // a power of two, so that advances of growing lengths rarely grow it
     while (window < n_steps) window *= 2;
     window = std::min<uint64_t>(window, kAheadItems / n);
     const uint32_t buffers = n_steps > window ? 2 : 1;
-    if ((a.window < window || a.buffers < buffers) && !captured) {
+    if ((a.window < window || a.buffers < buffers) && !c->ahead_fixed) {
         AheadView b;
         b.window = (uint32_t)std::max<uint64_t>(window, a.window);
         b.buffers = std::max(buffers, a.buffers);

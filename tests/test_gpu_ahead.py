@@ -109,3 +109,41 @@ def test_ahead_mala_equals_the_megakernel(n, advances, c_tilde):
     assert sa["regenerations"] + sa["local_steps"] == steps
     for key in ("regenerations", "local_steps", "accepted"):
         assert abs(sa[key] - sb[key]) <= max(1, 1e-4 * steps)
+
+
+def test_a_captured_advance_keeps_its_buffers():
+    """A captured advance runs in the windows that an advance outside a capture left;
+    a later, longer one leaves them where the graph has them; a captured advance too
+    short for windows (2^18 chains: the wavefront's) still captures."""
+    import torch
+    sc = SCENES["spheres"]()
+    scene = jr.Scene(sc)
+    n = 1 << 18
+    ends = []
+    for capture in (False, True):
+        st = torch.cuda.Stream()
+        with torch.cuda.stream(st):
+            ch = jr.Chains(scene, sc.width, sc.height, sc.depth, n, seed=17, stream=st)
+            ch.advance(4, stream=st)
+            st.synchronize()
+            if not capture:
+                ch.advance(4, stream=st)
+                ch.advance(1, stream=st)
+            else:
+                g = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(g, stream=st):
+                    ch.advance(4, stream=st)
+                    ch.advance(1, stream=st)
+                g.replay()
+            ch.advance(24, stream=st)
+            st.synchronize()
+            if capture:
+                x, _ = ch.get_state(stream=st)
+                g.replay()  # steps 4 to 8 once more, from the present states: in its own buffers
+                st.synchronize()
+                assert ch.stats()["status_word"] == 0
+                ends.append(x)
+            else:
+                ends.append(ch.get_state(stream=st)[0])
+    # windows of other lengths: other kernels for the tails, so ties as above
+    assert np.mean(np.any(ends[0] != ends[1], axis=0)) <= 1e-4
