@@ -767,9 +767,10 @@ __global__ void eval_states_kernel(SceneView s, uint32_t depth, float c_tilde, c
 // several streams share nothing.  The coordinates are drawn where they are used (one Philox
 // block per vertex), so a path reads and writes nothing but its pixel.  list (scenes
 // with a modified Phong material, see launch_render_pt): the lit samples are listed
-// instead of accumulated.  Against
-// one thread per path, whose warp waits for the longest ray of every vertex and
-// for its longest path: 2.76 -> 1.27 ms for 2^21 samples of Cornell + spheres.
+// instead of accumulated.  Bound by the divergent traversal's L1/L2 latency and issue,
+// as the chains' path kernel.  Against one thread per path, whose warp waits for the
+// longest ray of every vertex and for its longest path: 3.16 -> 1.40 ms for 2^21
+// samples of Cornell + spheres (with the list), 97.7 -> 37.8 ms for 2^26.
 struct PtPaths {
     uint32_t W, H;
     int dep;
@@ -1164,25 +1165,39 @@ cudaError_t launch_eval_states(const SceneView& s, uint32_t depth, float c_tilde
     return cudaGetLastError();
 }
 
+// Small calls keep one thread per path: the persistent warps' tail is then most of the
+// launch (one thread per path against persistent: 60 000 samples of the terrain 125 / 135 us,
+// of the caustic 129 / 144; 100 000 of the 24-triangle box 35 / 41, 200 000 55 / 56, at depth 6
+// 53 / 53 and 85 / 76; 200 000 of the terrain 206 / 193, of the caustic 214 / 187).
+//
 // Scenes with a modified Phong material: the lobe's arithmetic rounds in the last bit
 // as the compiler contracts it, and it does so differently in the two kernels; the
 // FP64 sums would differ by 3e-9.  So there the persistent kernel only finds the lit
-// samples (1 % of them on Cornell + spheres), and one thread per path evaluates those
-// (and every sample of a small call, where the list would cost more than it saves).
-constexpr uint64_t kRenderListMin = 1u << 19, kRenderListMax = 1u << 24;
+// samples (1 % of them on Cornell + spheres), and one thread per path evaluates those.
+// The second pass moves the line (one thread per path / listed, Cornell + spheres:
+// 60 000 samples 157 / 253 us, 200 000 317 / 346, 400 000 535 / 435, 600 000 754 / 522).
+constexpr uint64_t kRenderPersistentMin = 1u << 17, kRenderListMin = 1u << 18, kRenderListMax = 1u << 24;
 
 cudaError_t launch_render_pt(const SceneView& s, uint32_t width, uint32_t height, uint32_t depth, uint64_t seed,
                              uint64_t sample_begin, uint64_t n, double* accum, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     cudaError_t e = cudaSuccess;
-    const bool each = s.phong && n < kRenderListMin;
+    // A captured call keeps to one launch (a graph that allocates can't be a child graph).
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    bool each = n < (s.phong ? kRenderListMin : kRenderPersistentMin) ||
+                (s.phong && (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone));
     const size_t shm = sizeof(float) * (2 + 2 * depth) * 128;
     unsigned int* listed = nullptr;  // the count, then the list (256 bytes on)
     uint32_t* list = nullptr;
     if (s.phong && !each) {
         const uint64_t most = std::min(n, kRenderListMax);
-        if ((e = cudaMallocAsync((void**)&listed, 256 + sizeof(uint32_t) * most, st)) != cudaSuccess) return e;
-        list = listed + 64;
+        if (cudaMallocAsync((void**)&listed, 256 + sizeof(uint32_t) * most, st) == cudaSuccess) {
+            list = listed + 64;
+        } else {  // no memory for the list: every sample by its own thread
+            (void)cudaGetLastError();
+            listed = nullptr;
+            each = true;
+        }
     }
     with_checks(trav_checks(s), [&](auto k) {
         if (each) {
@@ -1209,12 +1224,7 @@ cudaError_t launch_render_pt(const SceneView& s, uint32_t width, uint32_t height
         const uint64_t blocks = (uint64_t)(sms * (packed >> 32));
         for (uint64_t done = 0; done < n && e == cudaSuccess;) {
             const uint64_t m = list ? std::min(n - done, kRenderListMax) : n;
-            // Two samples per lane while that fills three blocks per SM (a warp that
-            // refills hides its longest path), then one per lane: 100 000 samples of
-            // Cornell + spheres take 175 us over every resident warp, 152 us over 391
-            // blocks; 50 000 take 152 us, 133 us over 391 blocks and 146 us over 196.
-            const uint64_t want =
-                std::max<uint64_t>((m + 255) / 256, std::min<uint64_t>((m + 127) / 128, 3 * (uint64_t)sms));
+            const uint64_t want = (m + 255) / 256;  // two samples per lane: a warp that refills hides its longest path
             if (list && (e = cudaMemsetAsync(listed, 0, sizeof(unsigned int), st)) != cudaSuccess) break;
             kernel<<<(unsigned)std::min(blocks, want), 128, 0, st>>>(s, width, height, depth, seed, sample_begin + done,
                                                                      m, accum, list, listed);

@@ -97,3 +97,24 @@ def test_drain_kernel_equals_wavefront_drain(max_steps, rao):
     acc = sum(p[2] for p in parts)
     # FP32 sums of up to a few thousand positive terms per pixel in another order
     assert np.allclose(whole[2], acc, rtol=1e-4, atol=0)
+
+
+# 2^19 + 77 samples go to persistent warps, and a Phong scene's lit samples are listed (a
+# ragged last block); calls below 2^17 samples take one thread per path.  FP64 sums
+# of one pixel in another order: 2^20 additions at most, each 2^-53 relative, all
+# terms of one sign: 1.2e-10.
+@pytest.mark.parametrize("phong", [True, False])
+def test_render_in_one_call_equals_split_calls(phong):
+    if phong:
+        sc = scenes.cornell_spheres(width=32, height=32, depth=6, n_lon=40, n_lat=41)
+    else:
+        sc = scenes.cornell(width=32, height=32, depth=6)
+    scene = jr.Scene(sc)
+    n, first = (1 << 19) + 77, (1 << 32) - 1000
+    whole = jr.render_pt(scene, sc.width, sc.height, sc.depth, n, seed=5, sample_begin=first)
+    parts = 0
+    for a in range(0, n, 130_001):
+        b = min(a + 130_001, n)
+        parts = parts + jr.render_pt(scene, sc.width, sc.height, sc.depth, b - a, seed=5, sample_begin=first + a)
+    assert whole[..., :3].sum() > 0
+    np.testing.assert_allclose(whole[..., :3].cpu(), parts[..., :3].cpu(), rtol=1.2e-10, atol=0)
