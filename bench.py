@@ -32,11 +32,11 @@ METRIC = "Restore chain steps/s on 1 GB300; time to relMSE 1e-2, learned vs plai
 UNIT = "chain steps/s"
 # FP32 operations issued per unit of traversal work (counted from the kernel
 # source: a visit of a 4-wide node = 4 slab tests of 6 FMA (2 FLOP each) on
-# the octant's near and far planes + 4 min/max + 1 scaled compare (2), then 5
-# compares of the sorting network;
+# the octant's near and far planes + 4 min/max + 1 scaled compare (2), then 3
+# compares to order the hits;
 # a triangle test = Moller-Trumbore: 2 cross, 4 dot, 1 reciprocal, 3 scaled
 # products, 3 subtractions, 5 compares).
-FLOP_PER_NODE = 77
+FLOP_PER_NODE = 75
 FLOP_PER_TRI = 45
 FP32_LANES = 128   # FP32 lanes per SM on sm_103a (the nominal-peak cross-check only)
 # DRAM traffic of one wf_path_kernel launch (dram__bytes_read.sum +
@@ -739,6 +739,12 @@ def main():
         n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
         warp = args.exec == "warp" or (args.exec == "auto" and C < 32 * n_sm and sc.n_tris <= 128)
         step_kernel_name = "step_kernel_warp" if warp else "step_kernel"
+        # auto runs look-ahead windows: their path launch is ahead_path_kernel, and the window's steps
+        # are a step launch (jr_runs.cu's for small scenes)
+        path_kernel_name = "wf_path_kernel"
+        if args.exec == "auto" and split["path"]["launches"] and split["path"]["launches"] < K:
+            path_kernel_name = "ahead_path_kernel"
+            step_kernel_name = "runs_window_kernel" if warp else "settle_kernel"
         if dom == "path":    # the traversal work runs in the path kernel
             achieved = flop / 1e12 / (split["path"]["ms"] / 1e3)
         else:                # one launch does everything (megakernel)
@@ -770,7 +776,7 @@ def main():
     if ws == 1:
         rg1, tg1 = gpu_config1(stream)
         small = {"workload": "cornell_64x64_depth3: the whole 256 chains x 10^4 steps", "value": rg1, "unit": UNIT,
-                 "seconds": round(tg1, 4), "kernel": "step_kernel_warp"}
+                 "seconds": round(tg1, 4), "kernel": "runs_window_kernel"}
     cpu = None
     if not args.no_cpu_baseline and ws == 1:
         r, cores, sample = cpu_oracle_rate(sc, wl)
@@ -790,7 +796,7 @@ def main():
                    "c_tilde": 1.0, "sigma": 0.01, "regen": "uniform", "global_batch": ws * C, "seq_len": K,
                    "parallelism": f"chains sharded over {ws} GPU(s)", "l2": "flushed by a 512 MB write between timed launches",
                    "block": args.block or 128, "exec": args.exec},
-        "roofline": {"bound": "alu", "kernel": "wf_path_kernel" if dom == "path" else step_kernel_name,
+        "roofline": {"bound": "alu", "kernel": path_kernel_name if dom == "path" else step_kernel_name,
                      "achieved": achieved, "peak": alu_peak, "unit": "TFLOP/s",
                      "frac": achieved / alu_peak,
                      "traffic": path_traffic(args.workload, C) if dom == "path" else None,

@@ -192,7 +192,9 @@ jr_status jr_advance_traced(jr_chains* chains, uint32_t n_steps, uint8_t* flags_
  * every launch and the time since the previous one is charged to that launch's
  * class; ms_out[k] / launches_out[k] (host, 4 each) for k = 0 step kernels,
  * 1 path kernels (tracing and shading whole paths), 2 reserved (always 0),
- * 3 flow kernels (the megakernel counts as one step launch).  Same
+ * 3 flow kernels (the megakernel counts as one step launch; of a look-ahead
+ * advance, the path launches are path kernels, also where they carry the
+ * local steps of the window before, and the rest are step kernels).  Same
  * chains and results as jr_advance; the events add a little time between
  * launches, so use it to split a step, not to time it.  Synchronises. */
 jr_status jr_advance_timed(jr_chains* chains, uint32_t n_steps, double ms_out[4], uint64_t launches_out[4],
@@ -227,10 +229,19 @@ jr_status jr_set_block_size(jr_chains* chains, uint32_t block);
  *                       triangles and few chains, where one thread per chain is
  *                       bound by the latency of its serial steps; chain sets
  *                       with a flow run in the wavefront instead;
- *   JR_EXEC_AUTO        wavefront from 2^18 chains up; below that, one warp per
- *                       chain for scenes of at most 128 triangles and fewer
- *                       than 32 chains per SM (4 864 on a 152-SM GB300), else
- *                       the megakernel.
+ *   JR_EXEC_AUTO        look-ahead where it applies: the regeneration candidates
+ *                       of a window of steps are traced in one launch before the
+ *                       steps are settled (jr_advance and jr_advance_timed of
+ *                       Jump Restore chains without a flow, uniform or MALA, few
+ *                       local steps expected, enough steps in the call; it holds
+ *                       16 bytes per chain and step of the window, 256 MB at
+ *                       most, until the chains are destroyed, and the first such
+ *                       advance reads one number back).  Otherwise, also where
+ *                       that memory is not to be had and while a capture has
+ *                       nothing to use, wavefront from 2^18 chains up; below
+ *                       that, one warp per chain for scenes of at most 128
+ *                       triangles and fewer than 32 chains per SM (4 864 on a
+ *                       152-SM GB300), else the megakernel.
  * All modes run the same per-chain arithmetic on the same Philox streams and
  * give the same closest hits (the least (t, original triangle index) with
  * t > 0). */

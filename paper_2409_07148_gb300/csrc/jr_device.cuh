@@ -300,8 +300,9 @@ __device__ __forceinline__ bool trav_leaf(const SceneView& s, Trav& r, const int
 // visit), instead of when none is: the few lanes with the longest way no
 // longer hold the warp's other lanes, which test their leaves and go on; the
 // rest carry on in the next round.  Measured on the 512^2 Cornell + spheres
-// workload (wavefront): 1.04 (exit at 0), 1.17 (4), 1.19 (6 and 8), 1.14 (16)
-// x 10^9 chain steps/s.  The exit waits while the searching lanes outnumber
+// workload (look-ahead windows, two visits per vote), relative to an exit at 6:
+// 0.96 (4), 1.014 (8), 1.015 (10), 1.008 (14); with one visit per vote and an exit
+// at 0, 0.87.  The exit waits while the searching lanes outnumber
 // the others (a sparse warp, late in a drain, has nobody to release and would
 // only pay an extra round per node visit).
 constexpr int kSearchExit = 8;
