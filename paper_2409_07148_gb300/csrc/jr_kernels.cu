@@ -919,16 +919,24 @@ __global__ void __launch_bounds__(256) fma_peak_kernel(uint32_t iters, float* si
 inline unsigned grid_for(uint64_t n, unsigned b) { return (unsigned)((n + b - 1) / b); }
 
 // Chains per warp for a kernel that gives each one-warp block that many chains:
-// the fewest with which kSpreadWarps warps per SM hold them all, or 0 where the
+// the fewest with which `most` warps per SM hold them all, or 0 where the
 // device cannot hold them all at once even in full warps: there the launch is
 // bound by throughput, which full warps have the most of.  kSpreadWarps: three
 // warps per scheduler; more of them, with fewer chains each, wait for one another
 // (10 007 chains, 32 steps of Cornell + spheres: 1 702 us at 8, 1 578 at 12,
 // 1 600 at 16; 30 000 chains, 16 steps: 1 431, 1 357, 1 375 us; 6 000 chains in the
 // 24-triangle box, 64 steps: 785, 842, 892 us).
-constexpr int kSpreadWarps = 12;
+//
+// kSpreadWarpsMalaSmall: MALA in scenes of at most kWarpChainMaxTris triangles.  There a
+// step is the gradient's Jacobians in local memory, whose lines a warp with few lanes
+// fills with as few of its chains; and the rays, which end after a visit or two, do not
+// hold one another up (24-triangle box, depth 6, 8 steps, warps per SM 4 / 8 / 12 / full
+// warps: 2 522 chains 272, 349, 391, 332 us; 8 000 chains 317, 498, 549, 333 us; 20 925
+// chains 458, 586, 668, 461 us; but 2 steps of 16 000 chains on Cornell + spheres 448,
+// 432, 419 and on the terrain 326, 309, 304 us).
+constexpr int kSpreadWarps = 12, kSpreadWarpsMalaSmall = 4;
 template <class K>
-cudaError_t chains_per_warp(K kernel, size_t shm, uint64_t n, unsigned* per_warp) {
+cudaError_t chains_per_warp(K kernel, size_t shm, uint64_t n, int most, unsigned* per_warp) {
     static DeviceOnce once;  // per device: its SM count
     long long sms = 0;
     cudaError_t e = once.get(
@@ -942,7 +950,7 @@ cudaError_t chains_per_warp(K kernel, size_t shm, uint64_t n, unsigned* per_warp
     int per_sm = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32, shm);
     if (e != cudaSuccess) return e;
-    const uint64_t warps = (uint64_t)sms * (uint64_t)std::min(per_sm, kSpreadWarps);
+    const uint64_t warps = (uint64_t)sms * (uint64_t)std::min(per_sm, most);
     const bool fits = per_sm > 0 && n <= 32 * (uint64_t)sms * (uint64_t)per_sm;
     *per_warp = fits ? (unsigned)std::min<uint64_t>(32, (n + warps - 1) / warps) : 0u;
     return cudaSuccess;
@@ -1040,7 +1048,7 @@ cudaError_t launch_step(const SceneView& s, const ChainView& c, uint64_t step_be
         const auto spread = step_kernel_spread<decltype(k)::value>;
         const size_t wshm = sizeof(float) * 2 * c.dim * 32;  // <= 8 KB
         unsigned per_warp = 0;
-        if ((e = chains_per_warp(spread, wshm, c.n, &per_warp)) != cudaSuccess) return;
+        if ((e = chains_per_warp(spread, wshm, c.n, kSpreadWarps, &per_warp)) != cudaSuccess) return;
         if (per_warp) {
             spread<<<grid_for(c.n, per_warp), 32, wshm, st>>>(s, c, step_begin, n_steps, per_warp);
             e = cudaGetLastError();
@@ -1083,7 +1091,8 @@ cudaError_t launch_step_mala(const SceneView& s, const ChainView& c, uint64_t st
     const size_t shm = sizeof(float) * 4 * c.dim * 32;  // <= 16 KB
     const auto run = [&](auto kernel) {
         unsigned per_warp = 0;
-        const cudaError_t e = chains_per_warp(kernel, shm, c.n, &per_warp);
+        const cudaError_t e = chains_per_warp(
+            kernel, shm, c.n, s.n_tris <= kWarpChainMaxTris ? kSpreadWarpsMalaSmall : kSpreadWarps, &per_warp);
         if (e != cudaSuccess) return e;
         if (per_warp == 0) per_warp = 32;
         kernel<<<grid_for(c.n, per_warp), 32, shm, st>>>(s, c, step_begin, n_steps, per_warp, tr_flags, tr_dt, tr_pix);

@@ -118,3 +118,22 @@ def test_render_in_one_call_equals_split_calls(phong):
         parts = parts + jr.render_pt(scene, sc.width, sc.height, sc.depth, b - a, seed=5, sample_begin=first + a)
     assert whole[..., :3].sum() > 0
     np.testing.assert_allclose(whole[..., :3].cpu(), parts[..., :3].cpu(), rtol=1.2e-10, atol=0)
+
+
+# 609 and 19 457 chains: one more than four warps per SM hold with one and with 32 chains each
+# (152 SMs); the last 100 alone go one to a warp.  The same kernel on the same draws: equal.
+@pytest.mark.parametrize("n", [609, 19457])
+@pytest.mark.parametrize("name", ["cornell", "cornell_spheres"])
+def test_mala_chains_do_not_depend_on_their_warps(n, name):
+    sc = scenes.cornell(width=32, height=32, depth=3) if name == "cornell" else \
+        scenes.cornell_spheres(width=32, height=32, depth=3, n_lon=40, n_lat=41)
+    scene = jr.Scene(sc)
+    x = []
+    for chains, first in ((n, 0), (100, n - 100)):
+        ch = jr.Chains(scene, sc.width, sc.height, sc.depth, chains, seed=3, flags=jr.JR_FLAG_MALA, chain_offset=first)
+        ch.set_execution("mega")
+        ch.advance(5)
+        assert ch.stats()["status_word"] == 0
+        x.append(ch.get_state())
+    assert np.array_equal(x[0][0][:, -100:], x[1][0])
+    assert np.array_equal(x[0][1][:, -100:], x[1][1])
