@@ -463,7 +463,10 @@ jr_status jr_flow_get_params(jr_flow* flow, float* params, void* stream);
  * status word instead.  Synchronises. */
 jr_status jr_flow_get_status(jr_flow* flow, uint32_t* status_out, void* stream);
 
-/* log q(x) for n rows of x_dev [D][n] (device, SoA) into lq_dev [n].  Async. */
+/* log q(x) for n rows of x_dev [D][n] (device, SoA) into lq_dev [n].  q is a
+ * density on [0,1)^D; a row outside of it is no error and changes no other row,
+ * and its own value means nothing (a coordinate below 0 counts as in a bin of the
+ * least mass, one of 1 or more as in the last bin).  Async. */
 jr_status jr_flow_log_density(jr_flow* flow, const float* x_dev, uint64_t n, float* lq_dev, void* stream);
 /* In place: rows z of xz_dev [D][n] in [0,1)^D become x = T^{-1}(z); lq_dev
  * [n] gets log q(x).  Async. */

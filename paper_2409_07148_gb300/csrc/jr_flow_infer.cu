@@ -244,7 +244,10 @@ __device__ __forceinline__ float cdf_row(const float* tile, int key, float& v) {
             }
         }
     }
-    const float qb_e = exp2_approx(tile[4 * (key ^ (b >> 2)) + (b & 3)] - m);
+    // A density coordinate below 0 has b < 0 and no bin: as with a select over the bins,
+    // only the floor's mass E/K is left of it, and the tile is not read.
+    float qb_e = 0.f;
+    if (kSample || b >= 0) qb_e = exp2_approx(tile[4 * (key ^ (b >> 2)) + (b & 3)] - m);
     const float lo = fmaf(sc, lo_e, (float)b * (kFE / kFK));
     const float qb = fmaf(sc, qb_e, kFE / kFK);
     if (!kSample) {
