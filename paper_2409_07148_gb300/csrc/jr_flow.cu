@@ -325,12 +325,13 @@ __global__ void __launch_bounds__(kTrainThreads) flow_train_kernel(FlowView f, c
                 float* xv = sm.x + row * kXs + pm[A + j + lj];
                 const float tt = *xv;
                 const int b = min((int)(tt * (float)kFK), kFK - 1);
+                const int at = max(b, 0);  // a coordinate below 0 (b < 0) continues bin 0
                 float lo = 0.f, qb = 0.f;
 #pragma unroll
                 for (int k = 0; k < kFK; ++k) {
                     const float q = Q[k] * sc + kFE / kFK;
                     if (k < b) lo += q;
-                    if (k == b) qb = q;
+                    if (k == at) qb = q;
                 }
                 *xv = lo + (tt * (float)kFK - (float)b) * qb;
                 dlq += __logf((float)kFK * qb);
@@ -390,21 +391,22 @@ __global__ void __launch_bounds__(kTrainThreads) flow_train_kernel(FlowView f, c
                 const int cb = pm[A + j + lj];
                 const float tt = sm.x[row * kXs + cb];
                 const int b = min((int)(tt * (float)kFK), kFK - 1);
+                const int at = max(b, 0);  // as in the forward pass
                 float pb = 0.f;
 #pragma unroll
-                for (int k = 0; k < kFK; ++k) pb = k == b ? P[k] : pb;
+                for (int k = 0; k < kFK; ++k) pb = k == at ? P[k] : pb;
                 const float qb = (1.0f - kFE) * pb + kFE / kFK;
                 const float up = sm.g[row * kXs + cb];  // dL/d(output coordinate)
                 const float at_b = up * (tt * (float)kFK - (float)b) + sm.s[row] / qb;
-                // dL/dQ_k = up ([k < b] + [k == b](tK - b)) + s [k == b] / Q_b
+                // dL/dQ_k = up ([k < b] + [k == at](tK - b)) + s [k == at] / Q_at
                 float dot = 0.f;
 #pragma unroll
-                for (int k = 0; k < kFK; ++k) dot += P[k] * (k < b ? up : k == b ? at_b : 0.f);
+                for (int k = 0; k < kFK; ++k) dot += P[k] * (k < b ? up : k == at ? at_b : 0.f);
                 uint32_t o[kFK / 2];
 #pragma unroll
                 for (int k = 0; k < kFK; k += 2) {
-                    const float d0 = k < b ? up : k == b ? at_b : 0.f;
-                    const float d1 = k + 1 < b ? up : k + 1 == b ? at_b : 0.f;
+                    const float d0 = k < b ? up : k == at ? at_b : 0.f;
+                    const float d1 = k + 1 < b ? up : k + 1 == at ? at_b : 0.f;
                     const __nv_bfloat162 v = __floats2bfloat162_rn((1.0f - kFE) * P[k] * (d0 - dot),
                                                                    (1.0f - kFE) * P[k + 1] * (d1 - dot));
                     o[k / 2] = *reinterpret_cast<const uint32_t*>(&v);

@@ -68,3 +68,35 @@ def test_density_rows_outside_the_cube(D):
     small = [r for r, v in rows.items() if np.isfinite(v) and abs(v) <= 2.0]
     want = _log_density(perm, w, bad[small].astype(np.float64))
     assert np.all(np.abs(got[small] - want) <= 0.05), np.abs(got[small] - want).max()
+
+
+# a batch below one tile and one of three; rows below 0 in one coordinate, or in all of them
+@pytest.mark.parametrize("D,rows", [(2, 40), (8, 150)])
+def test_training_rows_below_zero(D, rows):
+    """The training loss continues bin 0 to coordinates below it: finite, and the
+    continuation's value.  The gradient stays finite."""
+    import torch
+    from paper_2409_07148_gb300 import jr
+    perm, w = _flow(D, 60 + D)
+    rng = np.random.default_rng(D)
+    x = rng.random((rows, D)).astype(np.float32)
+    for k, v in enumerate([-2.0 ** -4, -0.5, -1.0, -17.25]):
+        x[3 + 8 * k, int(rng.integers(D))] = v
+        x[4 + 8 * k] = v
+    wt = (rng.random(rows) + 0.05).astype(np.float32)
+    loss, g = jr.Flow(D, perm, w).gradient(torch.from_numpy(np.ascontiguousarray(x.T)).cuda(),
+                                           torch.from_numpy(wt).cuda())
+    y, lq, A = x.astype(np.float64), np.zeros(rows), D // 2
+    for l in range(len(perm)):
+        ca, cb = perm[l][:A], perm[l][A:]
+        Q = FL.bins(w[l], y[:, ca], D)
+        t = y[:, cb]
+        b = np.minimum(np.trunc(t * K), K - 1).astype(np.int64)
+        at = np.maximum(b, 0)[..., None]
+        cum = np.concatenate([np.zeros((rows, A, 1)), np.cumsum(Q, axis=2)], axis=2)
+        qb = np.take_along_axis(Q, at, axis=2)[..., 0]
+        y[:, cb] = np.take_along_axis(cum, at, axis=2)[..., 0] + (t * K - b) * qb
+        lq += np.log(K * qb).sum(axis=1)
+    want = -(wt * lq).sum() / wt.sum()
+    assert abs(loss - want) <= 1e-3 * max(1.0, abs(want)), (loss, want)  # test_gpu_flow_train's bound
+    assert np.isfinite(g).all()
