@@ -312,7 +312,10 @@ jr_status jr_get_state(jr_chains* chains, float* x_out, float* fpu_out, void* st
  * fpu_in (the cached F, p, u of jr_get_state) may be NULL, in which case F, p
  * and u are re-evaluated on the device.  A checkpoint restored with
  * jr_set_state(x, fpu) + jr_set_counters continues bit-identically, because
- * the Philox counters depend only on (seed, chain id, step index).
+ * the Philox counters depend only on (seed, chain id, step index) and a step's
+ * state does not depend on the kernel that ran it, so neither on the execution
+ * mode nor on how the steps are split into calls.  (The image is a sum in FP32
+ * and FP64, in no fixed order.)
  * Synchronises `stream`. */
 jr_status jr_set_state(jr_chains* chains, const float* x_in, const float* fpu_in, void* stream);
 

@@ -37,7 +37,7 @@
 // evaluation.
 //
 // The draws, the arithmetic and the order of a chain's steps are the other modes',
-// so the chains are the same.
+// so the chains are the same, bit for bit.
 #include <cuda_runtime.h>
 #include <stdint.h>
 

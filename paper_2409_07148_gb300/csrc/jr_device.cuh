@@ -360,7 +360,60 @@ __device__ __forceinline__ float fresnel(float cos_i, float eta_i, float eta_t, 
     return 0.5f * (rs * rs + rp * rp);
 }
 
-// Sample the continuation direction; returns false when the path ends.
+// The modified Phong lobe about the mirror direction, weight rho (n+2)/(n+1) cos_i,
+// with every rounding written out: left to the compiler, which product of a sum of
+// two becomes the fused one differs between kernels, and a step's state would depend
+// on the kernel that ran it (21 of 2^20 chains after 16 steps of Cornell + spheres
+// differed in the last bit of F, and a restored checkpoint with them).  The order
+// is the one that the compiler most often takes; it costs nothing (9.41 ms for
+// those steps before and after; a call that is not inlined fixes it, too, at 9.51).
+__device__ __forceinline__ float dot_rn(float3 a, float3 b) {
+    return __fmaf_rn(a.z, b.z, __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)));
+}
+__device__ __forceinline__ float mix_rn(float t, float st, float b, float sb, float r, float sr) {
+    return __fmaf_rn(r, sr, __fmaf_rn(t, st, __fmul_rn(b, sb)));
+}
+struct PhongFrame {
+    float3 r, t, b;  // mirror direction and the basis around it
+    float cos_a, sin_a, sn, cs;
+};
+__device__ __forceinline__ PhongFrame phong_frame(const Material& m, float3 d, float3 ns, float u1, float u2) {
+    PhongFrame q;
+    const float k = -__fmul_rn(2.0f, dot_rn(d, ns));
+    q.r = f3(__fmaf_rn(ns.x, k, d.x), __fmaf_rn(ns.y, k, d.y), __fmaf_rn(ns.z, k, d.z));
+    q.cos_a = powf(__fsub_rn(1.0f, u1), m.phong_inv_n1);
+    q.sin_a = sqrtf(fmaxf(__fmaf_rn(-q.cos_a, q.cos_a, 1.0f), 0.0f));
+    sincospif(__fmul_rn(2.0f, u2), &q.sn, &q.cs);
+    const float sign = copysignf(1.0f, q.r.z);  // onb
+    const float a = __fdiv_rn(-1.0f, __fadd_rn(sign, q.r.z));
+    const float bb = __fmul_rn(__fmul_rn(q.r.x, q.r.y), a);
+    q.t = f3(__fmaf_rn(__fmul_rn(__fmul_rn(sign, q.r.x), q.r.x), a, 1.0f), __fmul_rn(sign, bb),
+             __fmul_rn(-sign, q.r.x));
+    q.b = f3(bb, __fmaf_rn(__fmul_rn(q.r.y, q.r.y), a, sign), -q.r.y);
+    return q;
+}
+__device__ __forceinline__ float3 phong_direction(const PhongFrame& q) {
+    const float st = __fmul_rn(q.sin_a, q.cs), sb = __fmul_rn(q.sin_a, q.sn);
+    return f3(mix_rn(q.t.x, st, q.b.x, sb, q.r.x, q.cos_a), mix_rn(q.t.y, st, q.b.y, sb, q.r.y, q.cos_a),
+              mix_rn(q.t.z, st, q.b.z, sb, q.r.z, q.cos_a));
+}
+__device__ __forceinline__ float3 phong_weight(const Material& m, float cos_i) {
+    const float k = __fmul_rn(m.phong_scale, cos_i);
+    return f3(__fmul_rn(m.albedo.x, k), __fmul_rn(m.albedo.y, k), __fmul_rn(m.albedo.z, k));
+}
+__device__ __forceinline__ bool phong_lobe(const Material& m, float3 d, float3 ns, float u1, float u2, float3& wi,
+                                           float3& w) {
+    wi = phong_direction(phong_frame(m, d, ns, u1, u2));
+    const float cos_i = dot_rn(wi, ns);
+    if (cos_i <= 0.0f) return false;
+    w = phong_weight(m, cos_i);
+    return true;
+}
+
+// Sample the continuation direction; returns false when the path ends.  kPinned =
+// false: path tracing's own evaluation (render_pt_each_kernel), whose FP64 sums keep
+// the roundings that they have always had.
+template <bool kPinned = true>
 __device__ __forceinline__ bool scatter(const Material& m, float3 d, float3 ng, float u1, float u2, float3& wi,
                                         float3& w) {
     if (m.type == JR_MAT_DIELECTRIC) {
@@ -397,7 +450,8 @@ __device__ __forceinline__ bool scatter(const Material& m, float3 d, float3 ng, 
         w = m.albedo;
         return m.albedo.x > 0.0f || m.albedo.y > 0.0f || m.albedo.z > 0.0f;
     }
-    // modified Phong lobe about the mirror direction; weight rho (n+2)/(n+1) cos_i
+    if constexpr (kPinned) return phong_lobe(m, d, ns, u1, u2, wi, w);
+    // phong_lobe's steps, rounded as the compiler contracts them
     const float3 r = d - ns * (2.0f * dot(d, ns));
     const float cos_a = powf(1.0f - u1, m.phong_inv_n1);
     const float sin_a = sqrtf(fmaxf(1.0f - cos_a * cos_a, 0.0f));
@@ -428,6 +482,7 @@ __device__ __forceinline__ void camera_ray(const SceneView& s, float y0, float y
 // one-sided emission T * L_e to F, and unless v == depth samples the
 // continuation with (u1, u2) = (y_{2+2v}, y_{3+2v}).  Returns true if the path
 // continues, with (o, d, T) updated to the next ray.
+template <bool kPinned = true>
 __device__ __forceinline__ bool shade_vertex(const SceneView& s, int k, float t, int v, int depth, float u1,
                                              float u2, float3& o, float3& d, float3& T, float3& F) {
     const TriRecord* tr = s.tris + k;
@@ -438,7 +493,7 @@ __device__ __forceinline__ bool shade_vertex(const SceneView& s, int k, float t,
     if (m.emits && -dot(d, ng) > 0.0f) F = F + mul(T, m.emission);
     if (v == depth) return false;
     float3 wi, w;
-    if (!scatter(m, d, ng, u1, u2, wi, w)) return false;
+    if (!scatter<kPinned>(m, d, ng, u1, u2, wi, w)) return false;
     T = mul(T, w);
     if (T.x == 0.0f && T.y == 0.0f && T.z == 0.0f) return false;
     const float3 off = dot(wi, ng) >= 0.0f ? ng : ng * -1.0f;
@@ -459,7 +514,7 @@ __device__ __forceinline__ float3 finite_or_zero(float3 F, unsigned& status) {
 // The integrand for the lanes in `mask` (all of which must call together;
 // lanes with want = false only keep the warp in step).  The bounce loop runs
 // until no lane in the warp has a live path.
-template <int kCheck, bool kCount>
+template <int kCheck, bool kCount, bool kPinned = true>
 __device__ __forceinline__ float3 eval_path_w(const SceneView& s, unsigned mask, bool want, int depth, const float* y,
                                               uint32_t ys, int32_t* ids, uint64_t id_stride, unsigned& status,
                                               Work& work) {
@@ -480,18 +535,18 @@ __device__ __forceinline__ float3 eval_path_w(const SceneView& s, unsigned mask,
                 if (ids) ids[v * id_stride] = __float_as_int(__ldg(&s.tris[k].v0_id.w));
                 const float u1 = v < depth ? y[(2 + 2 * v) * ys] : 0.0f;
                 const float u2 = v < depth ? y[(3 + 2 * v) * ys] : 0.0f;
-                alive = shade_vertex(s, k, t, v, depth, u1, u2, o, d, T, F);
+                alive = shade_vertex<kPinned>(s, k, t, v, depth, u1, u2, o, d, T, F);
             }
         }
     }
     return want ? finite_or_zero(F, status) : F;
 }
 
-template <int kCheck>
+template <int kCheck, bool kPinned = true>
 __device__ __forceinline__ float3 eval_path(const SceneView& s, unsigned mask, bool want, int depth, const float* y,
                                             uint32_t ys, int32_t* ids, uint64_t id_stride, unsigned& status) {
     Work w;
-    return eval_path_w<kCheck, false>(s, mask, want, depth, y, ys, ids, id_stride, status, w);
+    return eval_path_w<kCheck, false, kPinned>(s, mask, want, depth, y, ys, ids, id_stride, status, w);
 }
 
 // ------------------------------------------------------------------ persistent path tracing
@@ -874,14 +929,13 @@ __device__ inline bool scatter_grad(const Material& m, float3 d, float3 ng, floa
         return m.albedo.x > 0.0f || m.albedo.y > 0.0f || m.albedo.z > 0.0f;
     }
     // modified Phong: r = d - 2 (d.ns) ns, basis around r, lobe angle from u1, azimuth from u2
-    const float3 r = d - ns * (2.0f * dot(d, ns));
-    const float cos_a = powf(1.0f - u1, m.phong_inv_n1);
-    const float sin_a = sqrtf(fmaxf(1.0f - cos_a * cos_a, 0.0f));
-    float sn, cs;
-    sincospif(2.0f * u2, &sn, &cs);
-    onb(r, t, b);
-    wi = t * (sin_a * cs) + b * (sin_a * sn) + r * cos_a;
-    const float cos_i = dot(wi, ns);
+    const PhongFrame q = phong_frame(m, d, ns, u1, u2);
+    const float3 r = q.r;
+    const float cos_a = q.cos_a, sin_a = q.sin_a, sn = q.sn, cs = q.cs;
+    t = q.t;
+    b = q.b;
+    wi = phong_direction(q);
+    const float cos_i = dot_rn(wi, ns);
     if (cos_i <= 0.0f) return false;
     const float sign = copysignf(1.0f, r.z);
     const float a = -1.0f / (sign + r.z);  // the basis's a; its bb term is differentiated in the loop
@@ -917,7 +971,7 @@ __device__ inline bool scatter_grad(const Material& m, float3 d, float3 ng, floa
         Jw.c[1][k] = m.albedo.y * m.phong_scale * dci;
         Jw.c[2][k] = m.albedo.z * m.phong_scale * dci;
     }
-    w = m.albedo * (m.phong_scale * cos_i);
+    w = phong_weight(m, cos_i);
     return true;
 }
 

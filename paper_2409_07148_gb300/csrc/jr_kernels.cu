@@ -875,7 +875,7 @@ __global__ void render_pt_each_kernel(SceneView s, uint32_t W, uint32_t H, uint3
             if (4 * b + q < D) y[(4 * b + q) * B] = u01(rr[q]);
     }
     unsigned status = 0;
-    const float3 F = eval_path<kCheck>(s, mask, true, (int)depth, y, B, nullptr, 0, status);
+    const float3 F = eval_path<kCheck, false>(s, mask, true, (int)depth, y, B, nullptr, 0, status);
     uint32_t px = min((uint32_t)((double)y[0] * (double)W), W - 1);
     uint32_t py = min((uint32_t)((double)y[B] * (double)H), H - 1);
     const double WH = (double)W * (double)H;
@@ -1179,8 +1179,8 @@ cudaError_t launch_eval_states(const SceneView& s, uint32_t depth, float c_tilde
 // of the caustic 129 / 144; 100 000 of the 24-triangle box 35 / 41, 200 000 55 / 56, at depth 6
 // 53 / 53 and 85 / 76; 200 000 of the terrain 206 / 193, of the caustic 214 / 187).
 //
-// Scenes with a modified Phong material: the lobe's arithmetic rounds in the last bit
-// as the compiler contracts it, and it does so differently in the two kernels; the
+// Scenes with a modified Phong material: one thread per path rounds the lobe as the
+// compiler contracts it, which no one order of roundings written out gives, and the
 // FP64 sums would differ by 3e-9.  So there the persistent kernel only finds the lit
 // samples (1 % of them on Cornell + spheres), and one thread per path evaluates those.
 // The second pass moves the line (one thread per path / listed, Cornell + spheres:
