@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(32, 16) mala_tail_kernel(SceneView s, ChainVie
     }
 }
 
-// Sum of p over the chains (double), for the estimate of p_lambda.
+// Sum of p over the initial states (double), for the estimate of p_lambda.
 __global__ void __launch_bounds__(256) sum_p_kernel(ChainView c, double* out) {
     double s = 0.0;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < c.n; i += (uint64_t)gridDim.x * blockDim.x)
@@ -576,7 +576,8 @@ cudaError_t resident(K kernel, int threads, size_t shm, long long* blocks) {
 
 }  // namespace
 
-cudaError_t launch_sum_p(const ChainView& c, double* out, cudaStream_t st) {
+cudaError_t launch_sum_p(const ChainView& c, cudaStream_t st) {
+    double* out = reinterpret_cast<double*>(c.counters + kCounterMuP);
     const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(double), st);
     if (e != cudaSuccess) return e;
     sum_p_kernel<<<(unsigned)std::min<uint64_t>(608, (c.n + 255) / 256), 256, 0, st>>>(c, out);

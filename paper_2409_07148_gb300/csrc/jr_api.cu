@@ -264,6 +264,7 @@ jr_status jr_chains_create(const jr_scene* scene, const jr_params* params, void*
         ((v.flags & JR_FLAG_MALA) && (e = dev_alloc(&v.drift, (size_t)v.dim * v.n)) != cudaSuccess) ||
         (e = launch_init(scene->view, v, st)) != cudaSuccess ||
         ((v.flags & JR_FLAG_MALA) && (e = launch_mala_reeval(scene->view, v, st)) != cudaSuccess) ||
+        (!(v.flags & JR_FLAG_MH) && (e = launch_sum_p(v, st)) != cudaSuccess) ||
         (e = prepare_static_scratch()) != cudaSuccess) {  // jr_advance_static's array, see jr_wavefront.cu
         delete c;
         return cuda_fail(e, "jr_chains_create");
@@ -346,9 +347,12 @@ static bool warp_per_chain(const jr_chains* c) {
 //
 // It pays while few steps are local, because a local step's regeneration candidate
 // is traced for nothing.  The stationary share of local steps is p_lambda /
-// (p_lambda + c~) (Section 6.1); p_lambda = E_mu[p] is estimated once, from the chains'
-// own states (at first samples of mu).  Where the buffers cannot be had, or the
-// stream is being captured before they exist, the other modes run.
+// (p_lambda + c~) (Section 6.1); p_lambda = E_mu[p] is estimated from the initial states,
+// which are samples of mu (later ones follow the jump chain, which favours large p: 40
+// steps on, the 24-triangle box reads as 0.64 local instead of 0.14).  So the answer is
+// the same whatever the set has done before, and after a restore.  Where the buffers
+// cannot be had, or the stream is being captured before they exist, the other modes
+// run.
 constexpr double kAheadShare = 0.25;
 
 // Lets this thread allocate while some other stream of it captures in the global mode.
@@ -379,12 +383,11 @@ static bool use_ahead(jr_chains* c, uint32_t n_steps, cudaStream_t st) {
     RelaxedCapture relaxed;  // another stream of this thread may be capturing
     if (c->ahead_use == jr_chains::kUnknown) {
         double sum = 0.0;
-        double* at = reinterpret_cast<double*>(c->view.counters + kCounterDrain);
-        c->ahead_use = jr_chains::kNo;
-        if (launch_sum_p(c->view, at, st) != cudaSuccess ||
-            cudaMemcpyAsync(&sum, at, sizeof(sum), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        if (cudaMemcpyAsync(&sum, c->view.counters + kCounterMuP, sizeof(sum), cudaMemcpyDeviceToHost, st) !=
+                cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess)
             return false;
+        c->ahead_use = jr_chains::kNo;
         const double p = sum / (double)n;
         if (!(p / (p + (double)c->view.c_tilde) < kAheadShare)) return false;
         c->ahead_use = jr_chains::kYes;
@@ -690,7 +693,12 @@ jr_status jr_set_counters(jr_chains* c, const jr_stats* in, const double* acc_ho
     unsigned long long cnt[kCounters] = {in->regenerations, in->local_steps, in->accepted, 0, 0, 0, 0, 0};
     std::memcpy(&cnt[kCounterPSum], &in->p_sum_large, sizeof(double));
     unsigned int status = in->status_word;
-    JR_CUDA(cudaMemcpyAsync(c->view.counters, cnt, sizeof(cnt), cudaMemcpyHostToDevice, st), "jr_set_counters");
+    // all but kCounterMuP, which belongs to the set and not to the run
+    JR_CUDA(cudaMemcpyAsync(c->view.counters, cnt, sizeof(cnt[0]) * kCounterMuP, cudaMemcpyHostToDevice, st),
+            "jr_set_counters");
+    JR_CUDA(cudaMemcpyAsync(c->view.counters + kCounterMuP + 1, cnt + kCounterMuP + 1,
+                            sizeof(cnt[0]) * (kCounters - kCounterMuP - 1), cudaMemcpyHostToDevice, st),
+            "jr_set_counters");
     JR_CUDA(cudaMemcpyAsync(c->view.status, &status, sizeof(status), cudaMemcpyHostToDevice, st), "jr_set_counters");
     if (acc_host)
         JR_CUDA(cudaMemcpyAsync(c->view.acc64, acc_host, sizeof(double4_32a) * (size_t)c->view.width * c->view.height,
