@@ -72,6 +72,7 @@ struct Window {
 // kTail = false: a launch without a tail (1 to 2 % faster without its code).
 template <bool kTail>
 struct MixedPaths {
+    static constexpr bool kFusedMirror = true;
     const ChainView& c;
     Window next, tail;          // next.K = 0: no candidates; tail_count = 0: no tail
     uint32_t tail_count;

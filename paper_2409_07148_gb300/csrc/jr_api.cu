@@ -187,7 +187,6 @@ jr_status jr_scene_create(const jr_scene_desc* desc, void* stream, jr_scene** ou
     s->view.visit_budget = kNodeVisitBudget;
     s->view.stack_limit = kStackSize;
     s->view.stack_need = bvh.stack_need;
-    s->view.phong = std::any_of(mats.begin(), mats.end(), [](const Material& m) { return m.type == JR_MAT_PHONG; });
     std::memcpy(s->view.cam, desc->camera, sizeof(float) * 12);
     s->info.n_tris = desc->n_tris;
     s->info.n_nodes = (uint32_t)bvh.nodes.size();

@@ -367,6 +367,8 @@ __device__ __forceinline__ float fresnel(float cos_i, float eta_i, float eta_t, 
 // differed in the last bit of F, and a restored checkpoint with them).  The order
 // is the one that the compiler most often takes; it costs nothing (9.41 ms for
 // those steps before and after; a call that is not inlined fixes it, too, at 9.51).
+// kFusedMirror: the mirror direction's product is fused for the chains; path
+// tracing, whose FP64 sums keep the bits they have always had, rounds it by itself.
 __device__ __forceinline__ float dot_rn(float3 a, float3 b) {
     return __fmaf_rn(a.z, b.z, __fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)));
 }
@@ -377,10 +379,15 @@ struct PhongFrame {
     float3 r, t, b;  // mirror direction and the basis around it
     float cos_a, sin_a, sn, cs;
 };
+template <bool kFusedMirror = true>
 __device__ __forceinline__ PhongFrame phong_frame(const Material& m, float3 d, float3 ns, float u1, float u2) {
     PhongFrame q;
     const float k = -__fmul_rn(2.0f, dot_rn(d, ns));
-    q.r = f3(__fmaf_rn(ns.x, k, d.x), __fmaf_rn(ns.y, k, d.y), __fmaf_rn(ns.z, k, d.z));
+    if constexpr (kFusedMirror)
+        q.r = f3(__fmaf_rn(ns.x, k, d.x), __fmaf_rn(ns.y, k, d.y), __fmaf_rn(ns.z, k, d.z));
+    else
+        q.r = f3(__fadd_rn(d.x, __fmul_rn(ns.x, k)), __fadd_rn(d.y, __fmul_rn(ns.y, k)),
+                 __fadd_rn(d.z, __fmul_rn(ns.z, k)));
     q.cos_a = powf(__fsub_rn(1.0f, u1), m.phong_inv_n1);
     q.sin_a = sqrtf(fmaxf(__fmaf_rn(-q.cos_a, q.cos_a, 1.0f), 0.0f));
     sincospif(__fmul_rn(2.0f, u2), &q.sn, &q.cs);
@@ -401,19 +408,18 @@ __device__ __forceinline__ float3 phong_weight(const Material& m, float cos_i) {
     const float k = __fmul_rn(m.phong_scale, cos_i);
     return f3(__fmul_rn(m.albedo.x, k), __fmul_rn(m.albedo.y, k), __fmul_rn(m.albedo.z, k));
 }
+template <bool kFusedMirror>
 __device__ __forceinline__ bool phong_lobe(const Material& m, float3 d, float3 ns, float u1, float u2, float3& wi,
                                            float3& w) {
-    wi = phong_direction(phong_frame(m, d, ns, u1, u2));
+    wi = phong_direction(phong_frame<kFusedMirror>(m, d, ns, u1, u2));
     const float cos_i = dot_rn(wi, ns);
     if (cos_i <= 0.0f) return false;
     w = phong_weight(m, cos_i);
     return true;
 }
 
-// Sample the continuation direction; returns false when the path ends.  kPinned =
-// false: path tracing's own evaluation (render_pt_each_kernel), whose FP64 sums keep
-// the roundings that they have always had.
-template <bool kPinned = true>
+// Sample the continuation direction; returns false when the path ends.
+template <bool kFusedMirror = true>
 __device__ __forceinline__ bool scatter(const Material& m, float3 d, float3 ng, float u1, float u2, float3& wi,
                                         float3& w) {
     if (m.type == JR_MAT_DIELECTRIC) {
@@ -450,19 +456,7 @@ __device__ __forceinline__ bool scatter(const Material& m, float3 d, float3 ng, 
         w = m.albedo;
         return m.albedo.x > 0.0f || m.albedo.y > 0.0f || m.albedo.z > 0.0f;
     }
-    if constexpr (kPinned) return phong_lobe(m, d, ns, u1, u2, wi, w);
-    // phong_lobe's steps, rounded as the compiler contracts them
-    const float3 r = d - ns * (2.0f * dot(d, ns));
-    const float cos_a = powf(1.0f - u1, m.phong_inv_n1);
-    const float sin_a = sqrtf(fmaxf(1.0f - cos_a * cos_a, 0.0f));
-    float sn, cs;
-    sincospif(2.0f * u2, &sn, &cs);
-    onb(r, t, b);
-    wi = t * (sin_a * cs) + b * (sin_a * sn) + r * cos_a;
-    const float cos_i = dot(wi, ns);
-    if (cos_i <= 0.0f) return false;
-    w = m.albedo * (m.phong_scale * cos_i);
-    return true;
+    return phong_lobe<kFusedMirror>(m, d, ns, u1, u2, wi, w);
 }
 
 // ------------------------------------------------------------------ integrand
@@ -482,7 +476,7 @@ __device__ __forceinline__ void camera_ray(const SceneView& s, float y0, float y
 // one-sided emission T * L_e to F, and unless v == depth samples the
 // continuation with (u1, u2) = (y_{2+2v}, y_{3+2v}).  Returns true if the path
 // continues, with (o, d, T) updated to the next ray.
-template <bool kPinned = true>
+template <bool kFusedMirror = true>
 __device__ __forceinline__ bool shade_vertex(const SceneView& s, int k, float t, int v, int depth, float u1,
                                              float u2, float3& o, float3& d, float3& T, float3& F) {
     const TriRecord* tr = s.tris + k;
@@ -493,7 +487,7 @@ __device__ __forceinline__ bool shade_vertex(const SceneView& s, int k, float t,
     if (m.emits && -dot(d, ng) > 0.0f) F = F + mul(T, m.emission);
     if (v == depth) return false;
     float3 wi, w;
-    if (!scatter<kPinned>(m, d, ng, u1, u2, wi, w)) return false;
+    if (!scatter<kFusedMirror>(m, d, ng, u1, u2, wi, w)) return false;
     T = mul(T, w);
     if (T.x == 0.0f && T.y == 0.0f && T.z == 0.0f) return false;
     const float3 off = dot(wi, ng) >= 0.0f ? ng : ng * -1.0f;
@@ -514,7 +508,7 @@ __device__ __forceinline__ float3 finite_or_zero(float3 F, unsigned& status) {
 // The integrand for the lanes in `mask` (all of which must call together;
 // lanes with want = false only keep the warp in step).  The bounce loop runs
 // until no lane in the warp has a live path.
-template <int kCheck, bool kCount, bool kPinned = true>
+template <int kCheck, bool kCount, bool kFusedMirror = true>
 __device__ __forceinline__ float3 eval_path_w(const SceneView& s, unsigned mask, bool want, int depth, const float* y,
                                               uint32_t ys, int32_t* ids, uint64_t id_stride, unsigned& status,
                                               Work& work) {
@@ -535,18 +529,18 @@ __device__ __forceinline__ float3 eval_path_w(const SceneView& s, unsigned mask,
                 if (ids) ids[v * id_stride] = __float_as_int(__ldg(&s.tris[k].v0_id.w));
                 const float u1 = v < depth ? y[(2 + 2 * v) * ys] : 0.0f;
                 const float u2 = v < depth ? y[(3 + 2 * v) * ys] : 0.0f;
-                alive = shade_vertex<kPinned>(s, k, t, v, depth, u1, u2, o, d, T, F);
+                alive = shade_vertex<kFusedMirror>(s, k, t, v, depth, u1, u2, o, d, T, F);
             }
         }
     }
     return want ? finite_or_zero(F, status) : F;
 }
 
-template <int kCheck, bool kPinned = true>
+template <int kCheck, bool kFusedMirror = true>
 __device__ __forceinline__ float3 eval_path(const SceneView& s, unsigned mask, bool want, int depth, const float* y,
                                             uint32_t ys, int32_t* ids, uint64_t id_stride, unsigned& status) {
     Work w;
-    return eval_path_w<kCheck, false, kPinned>(s, mask, want, depth, y, ys, ids, id_stride, status, w);
+    return eval_path_w<kCheck, false, kFusedMirror>(s, mask, want, depth, y, ys, ids, id_stride, status, w);
 }
 
 // ------------------------------------------------------------------ persistent path tracing
@@ -575,6 +569,7 @@ __device__ __forceinline__ float3 eval_path(const SceneView& s, unsigned mask, b
 //   keep(F)          called while the path goes on: what emission() returns next
 //   finish(F, status)  the path has ended
 //   batch_done()     all lanes call after a shading batch
+//   kFusedMirror     see phong_frame
 // Sources keep F out of the traversal's registers where they have memory for it:
 // it is almost always 0.
 constexpr int kRefill = 4;  // refill a warp once this many lanes are idle
@@ -615,7 +610,7 @@ __device__ __forceinline__ void trace_paths(const SceneView& s, Source& src, uns
                     const int depth = src.depth();
                     const float2 uv = v < depth ? src.coords(v) : make_float2(0.f, 0.f);
                     float3 o = r.o, d = r.d;
-                    live = shade_vertex(s, r.best, r.tb, v, depth, uv.x, uv.y, o, d, T, F);
+                    live = shade_vertex<Source::kFusedMirror>(s, r.best, r.tb, v, depth, uv.x, uv.y, o, d, T, F);
                     if (live) {
                         ++v;
                         trav_begin_at(r, o, d, src.root(s));

@@ -72,7 +72,6 @@ struct SceneView {
     uint32_t visit_budget;  // node visits per ray before the watchdog stops it (kNodeVisitBudget)
     int stack_limit;        // traversal stack entries a ray may use (<= kStackSize)
     int stack_need;         // the most entries a traversal of this tree can hold (HostBvh::stack_need)
-    int phong;              // the scene has a modified Phong material
 };
 
 // The traversal watchdogs that can fire on a view (TravCheck in jr_device.cuh).

@@ -765,22 +765,20 @@ __global__ void eval_states_kernel(SceneView s, uint32_t depth, float c_tilde, c
 // Plain path tracing by persistent warps (trace_paths).  Warp w of the grid traces
 // samples [w n / warps, (w + 1) n / warps): no cursor in memory, so calls on
 // several streams share nothing.  The coordinates are drawn where they are used (one Philox
-// block per vertex), so a path reads and writes nothing but its pixel.  list (scenes
-// with a modified Phong material, see launch_render_pt): the lit samples are listed
-// instead of accumulated.  Bound by the divergent traversal's L1/L2 latency and issue,
-// as the chains' path kernel.  Against one thread per path, whose warp waits for the
-// longest ray of every vertex and for its longest path: 3.16 -> 1.40 ms for 2^21
-// samples of Cornell + spheres (with the list), 97.7 -> 37.8 ms for 2^26.
+// block per two vertices), so a path reads and writes nothing but its pixel.  Bound by
+// the divergent traversal's L1/L2 latency and issue, as the chains' path kernel.
+// Against one thread per path, whose warp waits for the longest ray of every vertex
+// and for its longest path: 2 649 -> 1 182 us for 2 10^6 samples of Cornell + spheres,
+// 10.26 -> 4.36 ms for 8 10^6.
 struct PtPaths {
+    static constexpr bool kFusedMirror = false;
     uint32_t W, H;
     int dep;
     uint64_t seed, next, end;  // next sample of the warp, end of its range
     double* accum;
-    uint32_t* list;              // offsets from sample `begin`
-    unsigned int* listed;
-    uint64_t begin;
-    bool drained = false, lit = false;
+    bool drained = false;
     uint64_t smp = 0;
+    uint2 spare{};  // the second half of the path's latest block
     float3 F = f3(0.f, 0.f, 0.f);
 
     __device__ __forceinline__ uint4 block(uint32_t b) const {
@@ -794,6 +792,7 @@ struct PtPaths {
         smp = j;
         F = f3(0.f, 0.f, 0.f);
         const uint4 r = block(0);
+        spare = make_uint2(r.z, r.w);
         y0 = u01(r.x);
         y1 = u01(r.y);
         return true;
@@ -801,18 +800,16 @@ struct PtPaths {
     __device__ __forceinline__ const SceneView& camera(const SceneView& s) const { return s; }
     __device__ __forceinline__ int root(const SceneView& s) const { return s.root; }
     __device__ __forceinline__ int depth() const { return dep; }
-    __device__ __forceinline__ float2 coords(int v) const {  // coordinates 2 + 2v, 3 + 2v
+    __device__ __forceinline__ float2 coords(int v) {  // coordinates 2 + 2v, 3 + 2v, in order of v
+        if (!(v & 1)) return make_float2(u01(spare.x), u01(spare.y));
         const uint4 r = block((uint32_t)(1 + v) >> 1);
-        return v & 1 ? make_float2(u01(r.x), u01(r.y)) : make_float2(u01(r.z), u01(r.w));
+        spare = make_uint2(r.z, r.w);
+        return make_float2(u01(r.x), u01(r.y));
     }
     __device__ __forceinline__ float3 emission() const { return F; }
     __device__ __forceinline__ void keep(float3 f) { F = f; }
     __device__ __forceinline__ void finish(float3 f, unsigned& status) {
         if (f.x == 0.f && f.y == 0.f && f.z == 0.f) return;
-        if (list) {
-            lit = true;
-            return;
-        }
         f = finite_or_zero(f, status);
         const uint4 r = block(0);
         const uint32_t px = min((uint32_t)((double)u01(r.x) * (double)W), W - 1);
@@ -824,49 +821,35 @@ struct PtPaths {
         if (f.z != 0.f) atomicAdd(a + 2, WH * f.z);
         // channel 3 is left to the caller: the sample count is n, known on the host
     }
-    __device__ __forceinline__ void batch_done() {
-        if (!list) return;
-        const unsigned m = __ballot_sync(0xffffffffu, lit);
-        if (m) {
-            const int lane = threadIdx.x & 31;
-            unsigned base = 0;
-            if (lane == 0) base = atomicAdd(listed, (unsigned)__popc(m));
-            base = __shfl_sync(0xffffffffu, base, 0);
-            if (lit) list[base + __popc(m & ((1u << lane) - 1u))] = (uint32_t)(smp - begin);
-        }
-        lit = false;
-    }
+    __device__ __forceinline__ void batch_done() const {}
 };
 
 template <int kCheck>
 __global__ void __launch_bounds__(128, 7) render_pt_kernel(SceneView s, uint32_t W, uint32_t H, uint32_t depth,
                                                            uint64_t seed, uint64_t sample_begin, uint64_t n,
-                                                           double* accum, uint32_t* list, unsigned int* listed) {
+                                                           double* accum) {
     const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
     const uint64_t w = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
     const uint64_t per = n / warps, more = n % warps;  // the first `more` warps take one sample more
     const uint64_t first = sample_begin + w * per + min(w, more);
-    PtPaths src{W, H, (int)depth, seed, first, first + per + (w < more ? 1 : 0), accum, list, listed, sample_begin};
+    PtPaths src{W, H, (int)depth, seed, first, first + per + (w < more ? 1 : 0), accum};
     unsigned status = 0;
     src.drained = src.next >= src.end;
     trace_paths<kCheck>(s, src, status);
 }
 
-// One thread per path: samples sample_begin + list[i] for i < *listed, or sample_begin
-// + i for i < n when list is null.
+// One thread per path.
 template <int kCheck>
 __global__ void render_pt_each_kernel(SceneView s, uint32_t W, uint32_t H, uint32_t depth, uint64_t seed,
-                                      uint64_t sample_begin, uint64_t n, double* accum, const uint32_t* list,
-                                      const unsigned int* listed) {
+                                      uint64_t sample_begin, uint64_t n, double* accum) {
     extern __shared__ float sh[];
     const uint32_t B = blockDim.x, tid = threadIdx.x;
     const uint64_t i = blockIdx.x * (uint64_t)B + tid;
-    const uint64_t count = list ? *listed : n;
-    const unsigned mask = __ballot_sync(0xffffffffu, i < count);
-    if (i >= count) return;
+    const unsigned mask = __ballot_sync(0xffffffffu, i < n);
+    if (i >= n) return;
     const int D = 2 + 2 * (int)depth;
     float* y = sh + tid;
-    const uint64_t smp = sample_begin + (list ? list[i] : i);
+    const uint64_t smp = sample_begin + i;
     for (int b = 0; 4 * b < D; ++b) {
         const uint4 r = draw(seed, kTagPt, (uint32_t)(b + 1), (uint32_t)smp, smp >> 32);
         const uint32_t rr[4] = {r.x, r.y, r.z, r.w};
@@ -1175,49 +1158,36 @@ cudaError_t launch_eval_states(const SceneView& s, uint32_t depth, float c_tilde
 }
 
 // Small calls keep one thread per path: the persistent warps' tail is then most of the
-// launch (one thread per path against persistent: 60 000 samples of the terrain 125 / 135 us,
-// of the caustic 129 / 144; 100 000 of the 24-triangle box 35 / 41, 200 000 55 / 56, at depth 6
-// 53 / 53 and 85 / 76; 200 000 of the terrain 206 / 193, of the caustic 214 / 187).
-//
-// Scenes with a modified Phong material: one thread per path rounds the lobe as the
-// compiler contracts it, which no one order of roundings written out gives, and the
-// FP64 sums would differ by 3e-9.  So there the persistent kernel only finds the lit
-// samples (1 % of them on Cornell + spheres), and one thread per path evaluates those.
-// The second pass moves the line (one thread per path / listed, Cornell + spheres:
-// 60 000 samples 157 / 253 us, 200 000 317 / 346, 400 000 535 / 435, 600 000 754 / 522).
-constexpr uint64_t kRenderPersistentMin = 1u << 17, kRenderListMin = 1u << 18, kRenderListMax = 1u << 24;
+// launch.  One thread per path / persistent, us, at 100 000, 160 000, 262 144 and 2 10^6 samples:
+//   Cornell + spheres, depth 8   219, 204   313, 220   429, 305   2 649, 1 182
+//   slit caustic, depth 10       186, 195   200, 200   272, 231   1 383,   602
+//   2M-triangle terrain          180, 194   209, 206   282, 241   1 564,   892
+//   5 000 boxes, depth 8         191, 226   272, 279   374, 358   2 386, 2 063
+// In scenes of a few triangles rays are short and alike, so that a warp waits for
+// nobody unless some of its paths leave the scene early and the others go on for long
+// (24-triangle box, depth 2: 54, 63 at 200 000, 318, 327 at 2 10^6; depth 4: 78, 83; 508, 433;
+// depth 8: 118, 109; 835, 541).  Where no path leaves (100 boxes in a room, depth 6: 1 318,
+// 1 398; the 12-triangle furnace: 435, 526) the persistent warps only cost.
+constexpr uint64_t kRenderPersistentMin = 5u << 15, kRenderPersistentMinSmall = 1u << 18;
+constexpr uint32_t kRenderSmallDepth = 4;
 
 cudaError_t launch_render_pt(const SceneView& s, uint32_t width, uint32_t height, uint32_t depth, uint64_t seed,
                              uint64_t sample_begin, uint64_t n, double* accum, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     cudaError_t e = cudaSuccess;
-    // A captured call keeps to one launch (a graph that allocates can't be a child graph).
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    bool each = n < (s.phong ? kRenderListMin : kRenderPersistentMin) ||
-                (s.phong && (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone));
-    const size_t shm = sizeof(float) * (2 + 2 * depth) * 128;
-    unsigned int* listed = nullptr;  // the count, then the list (256 bytes on)
-    uint32_t* list = nullptr;
-    if (s.phong && !each) {
-        const uint64_t most = std::min(n, kRenderListMax);
-        if (cudaMallocAsync((void**)&listed, 256 + sizeof(uint32_t) * most, st) == cudaSuccess) {
-            list = listed + 64;
-        } else {  // no memory for the list: every sample by its own thread
-            (void)cudaGetLastError();
-            listed = nullptr;
-            each = true;
-        }
-    }
+    const bool small = s.n_tris <= kWarpChainMaxTris;
+    const bool each = small ? n < kRenderPersistentMinSmall || depth < kRenderSmallDepth : n < kRenderPersistentMin;
     with_checks(trav_checks(s), [&](auto k) {
         if (each) {
+            const size_t shm = sizeof(float) * (2 + 2 * depth) * 128;
             render_pt_each_kernel<k()><<<grid_for(n, 128), 128, shm, st>>>(s, width, height, depth, seed, sample_begin,
-                                                                           n, accum, nullptr, nullptr);
+                                                                           n, accum);
             e = cudaGetLastError();
             return;
         }
         static DeviceOnce once;  // per device and variant: the persistent grid
         const auto kernel = render_pt_kernel<decltype(k)::value>;
-        long long packed = 0;    // SMs, and resident blocks per SM above them
+        long long blocks = 0;
         e = once.get(
             [&](int dev, long long* v) {
                 int sms = 0, per_sm = 0;
@@ -1225,29 +1195,16 @@ cudaError_t launch_render_pt(const SceneView& s, uint32_t width, uint32_t height
                 if ((r = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
                     (r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 128, 0)) != cudaSuccess)
                     return r;
-                *v = sms + ((long long)(per_sm > 0 ? per_sm : 1) << 32);
+                *v = (long long)sms * (per_sm > 0 ? per_sm : 1);
                 return cudaSuccess;
             },
-            &packed);
-        const long long sms = packed & 0xffffffffll;
-        const uint64_t blocks = (uint64_t)(sms * (packed >> 32));
-        for (uint64_t done = 0; done < n && e == cudaSuccess;) {
-            const uint64_t m = list ? std::min(n - done, kRenderListMax) : n;
-            const uint64_t want = (m + 255) / 256;  // two samples per lane: a warp that refills hides its longest path
-            if (list && (e = cudaMemsetAsync(listed, 0, sizeof(unsigned int), st)) != cudaSuccess) break;
-            kernel<<<(unsigned)std::min(blocks, want), 128, 0, st>>>(s, width, height, depth, seed, sample_begin + done,
-                                                                     m, accum, list, listed);
-            if (list)
-                render_pt_each_kernel<k()><<<grid_for(m, 128), 128, shm, st>>>(
-                    s, width, height, depth, seed, sample_begin + done, m, accum, list, listed);
-            e = cudaGetLastError();
-            done += m;
-        }
+            &blocks);
+        if (e != cudaSuccess) return;
+        const uint64_t want = (n + 255) / 256;  // two samples per lane: a warp that refills hides its longest path
+        kernel<<<(unsigned)std::min<uint64_t>((uint64_t)blocks, want), 128, 0, st>>>(s, width, height, depth, seed,
+                                                                                    sample_begin, n, accum);
+        e = cudaGetLastError();
     });
-    if (listed) {
-        const cudaError_t f = cudaFreeAsync(listed, st);
-        if (e == cudaSuccess) e = f;
-    }
     return e;
 }
 

@@ -348,6 +348,7 @@ __global__ void __launch_bounds__(128, 10) wf_step_kernel(ChainView c, uint64_t 
 // evict-first (ld/st .cs): each is touched once per launch, and L1 is better kept
 // for the BVH nodes, the triangles and the traversal stacks (measured: +0.3 %).
 struct ChainPaths {
+    static constexpr bool kFusedMirror = true;
     const ChainView& c;
     unsigned count;
     bool ident;
@@ -490,6 +491,7 @@ __global__ void __launch_bounds__(128) wf_batch_step_kernel(const BatchEntry* en
 // set, its depth, the candidate buffer and its stride, and starts each ray at the
 // set's root in the merged scene.
 struct BatchPaths {
+    static constexpr bool kFusedMirror = true;
     const BatchEntry* entries;
     const int* roots;
     const uint64_t* off;   // shared memory
