@@ -598,8 +598,7 @@ __device__ __forceinline__ void chain_steps_mala(const SceneView& s, const Chain
     }
 }
 
-// One-warp blocks of per_warp chains, as in step_kernel_spread (4 steps of 1 000
-// chains on Cornell + spheres 728 -> 285 us, 8 steps of 32 768 1 930 -> 1 687 us).
+// One-warp blocks of per_warp chains, as in step_kernel_spread (chains_per_warp).
 template <int kCheck, bool kTrace>
 __global__ void __launch_bounds__(32, 16) step_kernel_mala(SceneView s, ChainView c, uint64_t step_begin,
                                                            uint32_t n_steps, uint32_t per_warp, uint8_t* tr_flags,
@@ -910,16 +909,19 @@ inline unsigned grid_for(uint64_t n, unsigned b) { return (unsigned)((n + b - 1)
 // 1 600 at 16; 30 000 chains, 16 steps: 1 431, 1 357, 1 375 us; 6 000 chains in the
 // 24-triangle box, 64 steps: 785, 842, 892 us).
 //
-// kSpreadWarpsMalaSmall: MALA in scenes of at most kWarpChainMaxTris triangles.  There a
-// step is the gradient's Jacobians in local memory, whose lines a warp with few lanes
-// fills with as few of its chains; and the rays, which end after a visit or two, do not
-// hold one another up (24-triangle box, depth 6, 8 steps, warps per SM 4 / 8 / 12 / full
-// warps: 2 522 chains 272, 349, 391, 332 us; 8 000 chains 317, 498, 549, 333 us; 20 925
-// chains 458, 586, 668, 461 us; but 2 steps of 16 000 chains on Cornell + spheres 448,
-// 432, 419 and on the terrain 326, 309, 304 us).
-constexpr int kSpreadWarps = 12, kSpreadWarpsMalaSmall = 4;
+// MALA: a step's gradient keeps four 3 x D Jacobians per lane in local memory, whose
+// lines a warp with few lanes fills with as few of its chains (1536 D bytes a warp, beside
+// 512 D of shared memory).  So the warps per SM are as many as their lines fit L1 with, and the launch asks
+// for no more shared memory than they take (left alone, the split is made for 16 of
+// them, and L1 has 28 to 90 of its 256 KB): 4 warps, 3 beyond D = 24.  Times of one thread per
+// chain in blocks of 128 over this, and over 12 warps per SM without the request, 2 500 and 10 000
+// chains: Cornell + spheres depth 8 2.3, 1.7 (1.8, 1.2), depth 15 3.0, 2.0 (1.5, 1.2); 2M-triangle
+// terrain's kind 2.2, 1.7 (1.4, 1.2); glass furnace depth 12 2.4, 1.9 (1.2, 0.98); 24-triangle box
+// depth 15 3.2, 2.4 (1.1, 1.0); furnace depth 8 1.5, 1.4 (0.76, 0.75).  Up to kCarveWarps one-warp
+// blocks per SM the request still pays (30 000 chains 1.2, 1.05); beyond it costs.
+constexpr int kSpreadWarps = 12, kSpreadWarpsMala = 4, kSpreadWarpsMalaDeep = 3, kCarveWarps = 12;
 template <class K>
-cudaError_t chains_per_warp(K kernel, size_t shm, uint64_t n, int most, unsigned* per_warp) {
+cudaError_t chains_per_warp(K kernel, size_t shm, uint64_t n, int most, unsigned* per_warp, long long* sm_count = nullptr) {
     static DeviceOnce once;  // per device: its SM count
     long long sms = 0;
     cudaError_t e = once.get(
@@ -936,6 +938,7 @@ cudaError_t chains_per_warp(K kernel, size_t shm, uint64_t n, int most, unsigned
     const uint64_t warps = (uint64_t)sms * (uint64_t)std::min(per_sm, most);
     const bool fits = per_sm > 0 && n <= 32 * (uint64_t)sms * (uint64_t)per_sm;
     *per_warp = fits ? (unsigned)std::min<uint64_t>(32, (n + warps - 1) / warps) : 0u;
+    if (sm_count) *sm_count = sms;
     return cudaSuccess;
 }
 
@@ -1074,12 +1077,25 @@ cudaError_t launch_step_mala(const SceneView& s, const ChainView& c, uint64_t st
     const size_t shm = sizeof(float) * 4 * c.dim * 32;  // <= 16 KB
     const auto run = [&](auto kernel) {
         unsigned per_warp = 0;
-        const cudaError_t e = chains_per_warp(
-            kernel, shm, c.n, s.n_tris <= kWarpChainMaxTris ? kSpreadWarpsMalaSmall : kSpreadWarps, &per_warp);
+        long long sms = 0;
+        const cudaError_t e = chains_per_warp(kernel, shm, c.n, c.dim <= 24 ? kSpreadWarpsMala : kSpreadWarpsMalaDeep,
+                                              &per_warp, &sms);
         if (e != cudaSuccess) return e;
         if (per_warp == 0) per_warp = 32;
-        kernel<<<grid_for(c.n, per_warp), 32, shm, st>>>(s, c, step_begin, n_steps, per_warp, tr_flags, tr_dt, tr_pix);
-        return cudaGetLastError();
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(grid_for(c.n, per_warp));
+        cfg.blockDim = dim3(32);
+        cfg.dynamicSmemBytes = shm;
+        cfg.stream = st;
+        cudaLaunchAttribute carve;
+        const long long warps = (cfg.gridDim.x + sms - 1) / sms;
+        if (warps <= kCarveWarps) {  // percent of the SM's 228 KB; a block takes 1 KB beside its own
+            carve.id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+            carve.val.sharedMemCarveout = (unsigned)std::min<size_t>(100, 100 * warps * (shm + 1024) / (228 * 1024) + 1);
+            cfg.attrs = &carve;
+            cfg.numAttrs = 1;
+        }
+        return cudaLaunchKernelEx(&cfg, kernel, s, c, step_begin, n_steps, (uint32_t)per_warp, tr_flags, tr_dt, tr_pix);
     };
     if (tr_flags || tr_dt || tr_pix) return run(step_kernel_mala<kCheckAll, true>);
     cudaError_t e = cudaSuccess;
