@@ -182,11 +182,16 @@ __device__ __forceinline__ void plane4(const float4 p, float i, float o, float (
 //  * Three comparators instead of a full sorting network: the nearest child is
 //    exact, and so is the order of two hits; with three or more the order of
 //    the others is approximate, which costs fewer visits than the two
-//    comparators cost instructions (11.78 -> 11.70 ms; 2.76 -> 2.69 ms in the
-//    path-tracing kernel).  The closest hit does not depend on the order.
+//    comparators cost instructions (16 steps of 2^20 chains on Cornell + spheres 9.41
+//    ms against 9.53, 2^21 samples of path tracing 1.24 ms against 1.27).  That is not so
+//    where the rays cross many boxes that overlap: with kSorted, the full network, the
+//    batch megakernel takes 3 rooms of 10 % of their pixels in 519 us instead of 702,
+//    16 whole rooms in 20.6 ms instead of 22.0.  The closest hit does not depend on the order;
+//    which rays a limit stops does, so where one can fire the order is always the
+//    full one (the 2M-triangle terrain, 4 steps of 2^20 chains: 3.02 -> 3.00 ms).
 enum TravCheck { kCheckNone = 0, kCheckVisits = 1, kCheckAll = 2 };
 
-template <int kCheck, bool kCount>
+template <int kCheck, bool kCount, bool kSorted = false>
 __device__ __forceinline__ bool trav_node(const SceneView& s, Trav& r, int* stack, unsigned& status, Work& work) {
     if constexpr (kCheck != kCheckNone) ++r.visits;
     if constexpr (kCheck == kCheckAll) {
@@ -229,6 +234,10 @@ __device__ __forceinline__ bool trav_node(const SceneView& s, Trav& r, int* stac
     cswap(t[0], rf.x, t[1], rf.y);
     cswap(t[2], rf.z, t[3], rf.w);
     cswap(t[0], rf.x, t[2], rf.z);
+    if constexpr (kSorted || kCheck != kCheckNone) {
+        cswap(t[1], rf.y, t[3], rf.w);
+        cswap(t[1], rf.y, t[2], rf.z);
+    }
     if constexpr (kCheck == kCheckAll) {
         const int pushes = (t[1] < INFINITY) + (t[2] < INFINITY) + (t[3] < INFINITY);
         if (r.sp + pushes > s.stack_limit) {
@@ -317,7 +326,7 @@ __device__ __forceinline__ bool search_done(unsigned searching, unsigned tracing
 // a __any_sync over `mask`, so the lanes reconverge every iteration instead of
 // drifting apart under independent thread scheduling.  Returns the leaf-order
 // record index or -1; t_out gets the hit distance.
-template <int kCheck, bool kCount>
+template <int kCheck, bool kCount, bool kSorted = false>
 __device__ __forceinline__ int closest_hit(const SceneView& s, unsigned mask, bool want, float3 o, float3 d,
                                            float& t_out, unsigned& status, Work& work) {
     Trav r;
@@ -329,7 +338,7 @@ __device__ __forceinline__ int closest_hit(const SceneView& s, unsigned mask, bo
         const unsigned tracing = __ballot_sync(mask, active);
         if (__any_sync(mask, active && r.ref >= 0)) {
             do {  // one vote per node visit: it ends the loop when nobody searches, too
-                if (active && r.ref >= 0 && !trav_node<kCheck, kCount>(s, r, stack, status, work)) {
+                if (active && r.ref >= 0 && !trav_node<kCheck, kCount, kSorted>(s, r, stack, status, work)) {
                     active = false;
                     r.best = -1;
                 }
@@ -508,7 +517,7 @@ __device__ __forceinline__ float3 finite_or_zero(float3 F, unsigned& status) {
 // The integrand for the lanes in `mask` (all of which must call together;
 // lanes with want = false only keep the warp in step).  The bounce loop runs
 // until no lane in the warp has a live path.
-template <int kCheck, bool kCount, bool kFusedMirror = true>
+template <int kCheck, bool kCount, bool kFusedMirror = true, bool kSorted = false>
 __device__ __forceinline__ float3 eval_path_w(const SceneView& s, unsigned mask, bool want, int depth, const float* y,
                                               uint32_t ys, int32_t* ids, uint64_t id_stride, unsigned& status,
                                               Work& work) {
@@ -521,7 +530,7 @@ __device__ __forceinline__ float3 eval_path_w(const SceneView& s, unsigned mask,
     for (int v = 0; v <= depth; ++v) {
         if (!__any_sync(mask, alive)) break;
         float t;
-        const int k = closest_hit<kCheck, kCount>(s, mask, alive, o, d, t, status, work);
+        const int k = closest_hit<kCheck, kCount, kSorted>(s, mask, alive, o, d, t, status, work);
         if (alive) {
             if (k < 0) {
                 alive = false;

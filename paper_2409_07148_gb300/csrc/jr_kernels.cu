@@ -75,7 +75,7 @@ __global__ void reeval_kernel(SceneView s, ChainView c) {
 // n_steps of Alg. 2 for chain i of set c (thread tid of the block; `active`
 // false for threads without a chain).  Every thread of the block calls it;
 // sh holds [2][D][blockDim] floats.
-template <int kCheck, bool kTrace, bool kCount>
+template <int kCheck, bool kTrace, bool kCount, bool kSorted = false>
 __device__ __forceinline__ void chain_steps(const SceneView& s, const ChainView& c, uint64_t i, bool active, float* sh,
                                             uint64_t step_begin, uint32_t n_steps, uint8_t* tr_flags, float* tr_dt,
                                             int32_t* tr_pix, unsigned long long* work_out) {
@@ -125,7 +125,8 @@ __device__ __forceinline__ void chain_steps(const SceneView& s, const ChainView&
                 atomicAdd(c.fb + pix, make_float4(wgt * Fr, wgt * Fg, wgt * Fb, dt));
             }
             propose(c, chain, step, local, cur, cand, B);
-            const float3 Fy = eval_path_w<kCheck, kCount>(s, mask, true, (int)c.depth, cand, B, nullptr, 0, status, work);
+            const float3 Fy = eval_path_w<kCheck, kCount, true, kSorted>(s, mask, true, (int)c.depth, cand, B, nullptr, 0,
+                                                                         status, work);
             const float py_ = lum(Fy);
             bool accept;
             if (mh) {  // Alg. 1: U < min(1, p(y)/p(x)), 1 if p(x) = 0
@@ -670,7 +671,8 @@ __global__ void __launch_bounds__(256, 4) batch_step_kernel(const BatchEntry* en
         const BatchItem wi = items[it];
         const BatchEntry& e = entries[wi.set];  // descriptor fields are read where used
         const uint64_t i = wi.begin + threadIdx.x;
-        chain_steps<kCheck, false, false>(e.s, e.c, i, i < wi.end, sh, e.step, n_steps, nullptr, nullptr, nullptr, nullptr);
+        chain_steps<kCheck, false, false, true>(e.s, e.c, i, i < wi.end, sh, e.step, n_steps, nullptr, nullptr, nullptr,
+                                                nullptr);
         __syncthreads();  // the shared state buffers are reused by the next item
     }
 }
