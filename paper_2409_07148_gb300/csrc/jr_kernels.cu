@@ -200,13 +200,17 @@ __device__ __forceinline__ void chain_steps(const SceneView& s, const ChainView&
 // per SM): the 4-wide traversal would take 110, and the occupancy the cap buys
 // outweighs its small spill (measured: 5.0 -> 5.9e8 chain steps/s for the
 // megakernel, 5.9 -> 6.1e8 for the 64-scene batch).
+// The traced and the counted variant hold more and run with few chains, so they may
+// take 80 registers, and sort fully (5 000 chains, 8 steps, traced: Cornell + spheres 1 032 ->
+// 906 us, glass furnace 1 358 -> 930, 180 000-triangle terrain 726 -> 548).
 template <int kCheck, bool kTrace, bool kCount>
-__global__ void __launch_bounds__(256, 4) step_kernel(SceneView s, ChainView c, uint64_t step_begin, uint32_t n_steps,
+__global__ void __launch_bounds__(256, kTrace || kCount ? 3 : 4) step_kernel(SceneView s, ChainView c, uint64_t step_begin, uint32_t n_steps,
                                                    uint8_t* tr_flags, float* tr_dt, int32_t* tr_pix,
                                                    unsigned long long* work_out) {
     extern __shared__ float sh[];
     const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    chain_steps<kCheck, kTrace, kCount>(s, c, i, i < c.n, sh, step_begin, n_steps, tr_flags, tr_dt, tr_pix, work_out);
+    chain_steps<kCheck, kTrace, kCount, kTrace || kCount>(s, c, i, i < c.n, sh, step_begin, n_steps, tr_flags, tr_dt,
+                                                          tr_pix, work_out);
 }
 
 // The megakernel where all chains fit on the device at once: a warp holds only
@@ -1015,7 +1019,6 @@ cudaError_t launch_step(const SceneView& s, const ChainView& c, uint64_t step_be
     const unsigned B = (unsigned)block;
     const size_t shm = sizeof(float) * 2 * c.dim * B;  // <= 2 * 32 * 256 * 4 = 64 KB
     const unsigned G = grid_for(c.n, B);
-    // The traced and the counted variant always check both watchdogs.
     const auto run = [&](auto kernel, uint8_t* f, float* dt, int32_t* pix, unsigned long long* work) {
         static DeviceOnce once;  // per device and variant: opt in to > 48 KB of dynamic shared memory
         const cudaError_t e = once.get(
@@ -1028,10 +1031,15 @@ cudaError_t launch_step(const SceneView& s, const ChainView& c, uint64_t step_be
         kernel.value<<<G, B, shm, st>>>(s, c, step_begin, n_steps, f, dt, pix, work);
         return cudaGetLastError();
     };
-    if (work_out) return run(Kernel<step_kernel<kCheckAll, false, true>>{}, nullptr, nullptr, nullptr, work_out);
-    if (tr_flags || tr_dt || tr_pix)
-        return run(Kernel<step_kernel<kCheckAll, true, false>>{}, tr_flags, tr_dt, tr_pix, nullptr);
     cudaError_t e = cudaSuccess;
+    if (work_out || tr_flags || tr_dt || tr_pix) {  // both watchdogs checked, or neither
+        with_checks(trav_checks(s) == kCheckNone ? kCheckNone : kCheckAll, [&](auto k) {
+            if constexpr (k() != kCheckVisits)
+                e = work_out ? run(Kernel<step_kernel<k(), false, true>>{}, nullptr, nullptr, nullptr, work_out)
+                             : run(Kernel<step_kernel<k(), true, false>>{}, tr_flags, tr_dt, tr_pix, nullptr);
+        });
+        return e;
+    }
     with_checks(trav_checks(s), [&](auto k) {
         const auto spread = step_kernel_spread<decltype(k)::value>;
         const size_t wshm = sizeof(float) * 2 * c.dim * 32;  // <= 8 KB
