@@ -914,6 +914,11 @@ inline unsigned grid_for(uint64_t n, unsigned b) { return (unsigned)((n + b - 1)
 // (10 007 chains, 32 steps of Cornell + spheres: 1 702 us at 8, 1 578 at 12,
 // 1 600 at 16; 30 000 chains, 16 steps: 1 431, 1 357, 1 375 us; 6 000 chains in the
 // 24-triangle box, 64 steps: 785, 842, 892 us).
+// kSpreadWarpsSmall: scenes of at most kWarpChainMaxTris triangles, whose rays are short
+// and alike, so that the lanes of a warp hardly wait for one another: two warps per
+// scheduler (10 steps of 5 000 and 12 000 chains, 8 / 12 warps: 24-triangle box, depth 6,
+// 218, 219 and 250, 261 us; 100 boxes in a room 361, 361 and 444, 455; the furnace, depth
+// 8, where the lanes never part, 194, 220 and 203, 221, and in blocks of 128 198 and 199).
 //
 // MALA: a step's gradient keeps four 3 x D Jacobians per lane in local memory, whose
 // lines a warp with few lanes fills with as few of its chains (1536 D bytes a warp, beside
@@ -925,7 +930,7 @@ inline unsigned grid_for(uint64_t n, unsigned b) { return (unsigned)((n + b - 1)
 // terrain's kind 2.2, 1.7 (1.4, 1.2); glass furnace depth 12 2.4, 1.9 (1.2, 0.98); 24-triangle box
 // depth 15 3.2, 2.4 (1.1, 1.0); furnace depth 8 1.5, 1.4 (0.76, 0.75).  Up to kCarveWarps one-warp
 // blocks per SM the request still pays (30 000 chains 1.2, 1.05); beyond it costs.
-constexpr int kSpreadWarps = 12, kSpreadWarpsMala = 4, kSpreadWarpsMalaDeep = 3, kCarveWarps = 12;
+constexpr int kSpreadWarps = 12, kSpreadWarpsSmall = 8, kSpreadWarpsMala = 4, kSpreadWarpsMalaDeep = 3, kCarveWarps = 12;
 template <class K>
 cudaError_t chains_per_warp(K kernel, size_t shm, uint64_t n, int most, unsigned* per_warp, long long* sm_count = nullptr) {
     static DeviceOnce once;  // per device: its SM count
@@ -1044,7 +1049,8 @@ cudaError_t launch_step(const SceneView& s, const ChainView& c, uint64_t step_be
         const auto spread = step_kernel_spread<decltype(k)::value>;
         const size_t wshm = sizeof(float) * 2 * c.dim * 32;  // <= 8 KB
         unsigned per_warp = 0;
-        if ((e = chains_per_warp(spread, wshm, c.n, kSpreadWarps, &per_warp)) != cudaSuccess) return;
+        if ((e = chains_per_warp(spread, wshm, c.n,
+                                 s.n_tris <= kWarpChainMaxTris ? kSpreadWarpsSmall : kSpreadWarps, &per_warp)) != cudaSuccess) return;
         if (per_warp) {
             spread<<<grid_for(c.n, per_warp), 32, wshm, st>>>(s, c, step_begin, n_steps, per_warp);
             e = cudaGetLastError();

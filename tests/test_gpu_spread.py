@@ -29,3 +29,14 @@ def _alone_and_together(sc, n, **kw):
 def test_mala_chains_do_not_depend_on_their_warps(depth, n, flags):
     sc = scenes.cornell_spheres(width=32, height=32, depth=depth, n_lon=24, n_lat=25)
     _alone_and_together(sc, n, flags=flags, sigma=0.02, burn_in=0)
+
+
+# 8 warps per SM up to 128 triangles, 12 above (152 SMs): the sizes at which a warp takes one chain more, and the
+# largest that is spread at all
+@pytest.mark.parametrize("name,n", [("box", 1216), ("box", 1217), ("box", 38913), ("box", 77824), ("box", 77825),
+                                    ("spheres", 1824), ("spheres", 1825), ("spheres", 58369)])
+@pytest.mark.parametrize("flags", [0, jr.JR_FLAG_MH])
+def test_chains_do_not_depend_on_their_warps(name, n, flags):
+    sc = scenes.cornell(width=32, height=32, depth=4) if name == "box" else \
+        scenes.cornell_spheres(width=32, height=32, depth=4, n_lon=24, n_lat=25)
+    _alone_and_together(sc, n, flags=flags, burn_in=0)
