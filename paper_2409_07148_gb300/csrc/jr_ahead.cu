@@ -551,15 +551,6 @@ __global__ void __launch_bounds__(32, 16) mala_tail_kernel(SceneView s, ChainVie
     }
 }
 
-// Sum of p over the initial states (double), for the estimate of p_lambda.
-__global__ void __launch_bounds__(256) sum_p_kernel(ChainView c, double* out) {
-    double s = 0.0;
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < c.n; i += (uint64_t)gridDim.x * blockDim.x)
-        s += (double)c.fpu[3 * c.n + i];
-    s = warp_sum(s);
-    if ((threadIdx.x & 31) == 0 && s != 0.0) atomicAdd(out, s);
-}
-
 inline unsigned grid_for(uint64_t n, unsigned b) { return (unsigned)((n + b - 1) / b); }
 
 // Resident one-warp or 128-thread blocks of a kernel on the current device.
@@ -576,14 +567,6 @@ cudaError_t resident(K kernel, int threads, size_t shm, long long* blocks) {
 }
 
 }  // namespace
-
-cudaError_t launch_sum_p(const ChainView& c, cudaStream_t st) {
-    double* out = reinterpret_cast<double*>(c.counters + kCounterMuP);
-    const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(double), st);
-    if (e != cudaSuccess) return e;
-    sum_p_kernel<<<(unsigned)std::min<uint64_t>(608, (c.n + 255) / 256), 256, 0, st>>>(c, out);
-    return cudaGetLastError();
-}
 
 cudaError_t launch_ahead(const SceneView& s, const ChainView& c, const AheadView& a, uint64_t step_begin,
                          uint32_t n_steps, bool warp_tail, cudaStream_t st, KernelTimer* tm) {

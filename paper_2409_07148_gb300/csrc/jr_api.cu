@@ -263,7 +263,6 @@ jr_status jr_chains_create(const jr_scene* scene, const jr_params* params, void*
         ((v.flags & JR_FLAG_MALA) && (e = dev_alloc(&v.drift, (size_t)v.dim * v.n)) != cudaSuccess) ||
         (e = launch_init(scene->view, v, st)) != cudaSuccess ||
         ((v.flags & JR_FLAG_MALA) && (e = launch_mala_reeval(scene->view, v, st)) != cudaSuccess) ||
-        (!(v.flags & JR_FLAG_MH) && (e = launch_sum_p(v, st)) != cudaSuccess) ||
         (e = prepare_static_scratch()) != cudaSuccess) {  // jr_advance_static's array, see jr_wavefront.cu
         delete c;
         return cuda_fail(e, "jr_chains_create");

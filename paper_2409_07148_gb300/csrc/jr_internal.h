@@ -21,7 +21,7 @@ constexpr uint32_t kNodeVisitBudget = 1u << 16;  // per ray; exceeding it is a w
 
 constexpr uint32_t kTagStep = 0, kTagInit = 1, kTagPt = 2, kTagRestart = 3;
 constexpr int kCounters = 8;   // ChainView::counters entries
-constexpr int kCounterMuP = 4;    // sum of p over the initial states (a double's bits; not MH)
+constexpr int kCounterMuP = 4;    // sum of p over the initial states (a double's bits)
 constexpr int kCounterDrain = 6;  // [6], [7]: launch_drain's ctl
 constexpr int kCounterPSum = 5;  // MH: sum of p over the large-step proposals (double)
 constexpr uint64_t kWavefrontMinChains = 1u << 18;  // JR_EXEC_AUTO picks the wavefront from here up
@@ -345,12 +345,10 @@ cudaError_t launch_runs_tail(const SceneView& s, const ChainView& c, uint64_t st
 cudaError_t launch_runs_drain(const SceneView& s, const ChainView& c, uint64_t step_begin, uint32_t n_steps,
                               unsigned long long* ctl, cudaStream_t st);
 
-// jr_ahead.cu: n steps of Alg. 2 in look-ahead windows (uniform mu, no flow, not
-// MH or MALA).  warp_tail: one warp per chain settles the window (small scenes).
+// jr_ahead.cu: n steps of Alg. 2 in look-ahead windows (uniform mu, no flow, not MH;
+// MALA Restore included).  warp_tail: one warp per chain settles the window (small scenes).
 cudaError_t launch_ahead(const SceneView& s, const ChainView& c, const AheadView& a, uint64_t step_begin,
                          uint32_t n_steps, bool warp_tail, cudaStream_t st, KernelTimer* tm = nullptr);
-// Sum of p over the chains' states into counters[kCounterMuP].
-cudaError_t launch_sum_p(const ChainView& c, cudaStream_t st);
 // Paths per look-ahead window (128 MB of F; an advance of several windows keeps two).
 // Shorter windows pay the path launch's end more often, longer ones a longer last
 // tail: 16 steps of 2^20 chains on Cornell + spheres 10.19 (2^21), 9.68 (2^22), 9.64

@@ -25,34 +25,47 @@ namespace jr {
 namespace {
 
 // ------------------------------------------------------------------ kernels
-// x0 ~ mu (tag 1); y built in shared memory, then written to the SoA state.
+// x0 ~ mu (tag 1); y built in shared memory, then written to the SoA state.  The sum
+// of p goes to counters[kCounterMuP], one atomic per block (a launch of its own
+// took 6 to 30 us of a set's creation).
 template <int kCheck>
 __global__ void init_kernel(SceneView s, ChainView c) {
     extern __shared__ float sh[];
+    __shared__ double sum_p;
     const uint32_t B = blockDim.x, tid = threadIdx.x;
     const uint64_t i = blockIdx.x * (uint64_t)B + tid;
-    const unsigned mask = __ballot_sync(0xffffffffu, i < c.n);  // lanes that trace together
-    if (i >= c.n) return;
+    const bool valid = i < c.n;
+    if (tid == 0) sum_p = 0.0;
+    __syncthreads();
     const int D = (int)c.dim;
     float* y = sh + tid;
-    const uint32_t chain = c.chain_offset + (uint32_t)i;
-    for (int b = 0; 4 * b < D; ++b) {
-        const uint4 r = draw(c.seed, kTagInit, (uint32_t)(b + 1), chain, 0);
-        const uint32_t rr[4] = {r.x, r.y, r.z, r.w};
+    if (valid) {
+        const uint32_t chain = c.chain_offset + (uint32_t)i;
+        for (int b = 0; 4 * b < D; ++b) {
+            const uint4 r = draw(c.seed, kTagInit, (uint32_t)(b + 1), chain, 0);
+            const uint32_t rr[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (4 * b + q < D) y[(4 * b + q) * B] = u01(rr[q]);
+            for (int q = 0; q < 4; ++q)
+                if (4 * b + q < D) y[(4 * b + q) * B] = u01(rr[q]);
+        }
     }
     unsigned status = 0;
-    const float3 F = eval_path<kCheck>(s, mask, true, (int)c.depth, y, B, nullptr, 0, status);
-    float2* x2 = reinterpret_cast<float2*>(c.x);
-    for (int k = 0; 2 * k < D; ++k) x2[(uint64_t)k * c.n + i] = make_float2(y[2 * k * B], y[(2 * k + 1) * B]);
-    c.fpu[0 * c.n + i] = F.x;
-    c.fpu[1 * c.n + i] = F.y;
-    c.fpu[2 * c.n + i] = F.z;
-    c.fpu[3 * c.n + i] = lum(F);
-    c.fpu[4 * c.n + i] = 1.0f;  // u of uniform mu
-    flush_status(status, c.status);
+    const float3 F = eval_path<kCheck>(s, 0xffffffffu, valid, (int)c.depth, y, B, nullptr, 0, status);
+    const float p = valid ? lum(F) : 0.0f;
+    if (valid) {
+        float2* x2 = reinterpret_cast<float2*>(c.x);
+        for (int k = 0; 2 * k < D; ++k) x2[(uint64_t)k * c.n + i] = make_float2(y[2 * k * B], y[(2 * k + 1) * B]);
+        c.fpu[0 * c.n + i] = F.x;
+        c.fpu[1 * c.n + i] = F.y;
+        c.fpu[2 * c.n + i] = F.z;
+        c.fpu[3 * c.n + i] = p;
+        c.fpu[4 * c.n + i] = 1.0f;  // u of uniform mu
+        flush_status(status, c.status);
+    }
+    const double v = warp_sum((double)p);
+    if ((tid & 31) == 0 && v != 0.0) atomicAdd(&sum_p, v);
+    __syncthreads();
+    if (tid == 0 && sum_p != 0.0) atomicAdd(reinterpret_cast<double*>(c.counters + kCounterMuP), sum_p);
 }
 
 // Re-evaluate F, p, u of the stored states (after jr_set_state).
