@@ -235,7 +235,9 @@ jr_status jr_set_block_size(jr_chains* chains, uint32_t block);
  *                       Jump Restore chains without a flow, uniform or MALA, few
  *                       local steps expected, enough steps in the call; it holds
  *                       16 bytes per chain and step of the window, 256 MB at
- *                       most, until the chains are destroyed, and the first such
+ *                       most (128 MB with MALA or one warp per chain), and 16
+ *                       bytes per chain until the chains are destroyed, from 2^18
+ *                       chains up beside the wavefront's buffers; the first such
  *                       advance reads one number back).  Otherwise, also where
  *                       that memory is not to be had and while a capture has
  *                       nothing to use, wavefront from 2^18 chains up; below

@@ -408,19 +408,34 @@ static bool use_ahead(jr_chains* c, uint32_t n_steps, cudaStream_t st) {
     uint64_t window = least;  // a power of two, so that advances of growing lengths rarely grow it
     while (window < n_steps) window *= 2;
     window = std::min<uint64_t>(window, kAheadItems / n);
-    const uint32_t buffers = n_steps > window ? 2 : 1;
-    if ((a.window < window || a.buffers < buffers) && !c->ahead_fixed) {
-        AheadView b;
-        b.window = (uint32_t)std::max<uint64_t>(window, a.window);
-        b.buffers = std::max(buffers, a.buffers);
-        if (dev_alloc(&b.F, (size_t)b.buffers * b.window * n) == cudaSuccess && dev_alloc(&b.queue, n) == cudaSuccess &&
-            dev_alloc(&b.ctl, 4) == cudaSuccess)
-            std::swap(a, b);
-        else
+    // Two only where a window's tail waits for the next window's paths (launch_ahead).
+    const uint32_t buffers = n_steps > window && !mala && !warp_per_chain(c) ? 2 : 1;
+    if (c->ahead_fixed) return a.window != 0;
+    if (!a.queue && (dev_alloc(&a.queue, n) != cudaSuccess || dev_alloc(&a.ctl, kCtlCount) != cudaSuccess)) {
+        (void)cudaGetLastError();
+        cudaFree(a.queue);
+        a.queue = nullptr;
+        return false;
+    }
+    if (a.window < window || a.buffers < buffers) {
+        // The old buffer goes first (this waits for the launches that use it), so that no
+        // more than one is held; where the new one cannot be had, one of the old size may.
+        const AheadView old = a;
+        cudaFree(a.F);
+        a.F = nullptr;
+        a.window = (uint32_t)std::max<uint64_t>(window, old.window);
+        a.buffers = std::max(buffers, old.buffers);
+        if (dev_alloc(&a.F, (size_t)a.buffers * a.window * n) != cudaSuccess) {
             (void)cudaGetLastError();
-        cudaFree(b.F);  // the old buffers (this waits for the launches that use them), or a part of the new ones
-        cudaFree(b.queue);
-        cudaFree(b.ctl);
+            a.F = nullptr;
+            a.window = old.window;
+            a.buffers = old.buffers;
+            if (a.window == 0 || dev_alloc(&a.F, (size_t)a.buffers * a.window * n) != cudaSuccess) {
+                (void)cudaGetLastError();
+                a.F = nullptr;
+                a.window = a.buffers = 0;
+            }
+        }
     }
     return a.window != 0;
 }
