@@ -1576,7 +1576,7 @@ jr_status drain_impl(jr_chains* c, uint32_t max_steps, uint64_t* remaining, cuda
         const uint32_t g = std::min(runs ? kDrainTailSteps : len, max_steps - k);
         unsigned long long* ctl = c->view.counters + kCounterDrain;
         if (runs) JR_CUDA(launch_runs_drain(c->scene_view(), c->view, s0 + k, g, ctl, st), who);
-        else JR_CUDA(launch_drain(c->scene_view(), c->view, c->view.wf.done, s0 + k, g, ctl, st), who);
+        else JR_CUDA(launch_drain(c->scene_view(), c->view, s0 + k, g, ctl, st), who);
         k += g;
         unsigned long long open = 0;
         JR_CUDA(cudaMemcpyAsync(&open, ctl + 1, sizeof(open), cudaMemcpyDeviceToHost, st), who);

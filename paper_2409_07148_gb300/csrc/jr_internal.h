@@ -290,11 +290,11 @@ cudaError_t launch_step_warp(const SceneView& s, const ChainView& c, uint64_t st
 cudaError_t launch_step(const SceneView& s, const ChainView& c, uint64_t step_begin, uint32_t n_steps,
                         uint8_t* tr_flags, float* tr_dt, int32_t* tr_pix, unsigned long long* work_out, int block,
                         cudaStream_t st);
-// The open tours of a drain to their ends (no flow): every chain with skip[i] = 0
-// (all of them when skip is null) takes up to n_steps drain steps from step_begin.
+// The open tours of a drain to their ends (no flow): every chain with c.wf.done[i] = 0
+// takes up to n_steps drain steps from step_begin.
 // ctl [2]: fetch cursor, chains still open afterwards.  Sets c.wf.done.
-cudaError_t launch_drain(const SceneView& s, const ChainView& c, const uint8_t* skip, uint64_t step_begin,
-                         uint32_t n_steps, unsigned long long* ctl, cudaStream_t st);
+cudaError_t launch_drain(const SceneView& s, const ChainView& c, uint64_t step_begin, uint32_t n_steps,
+                         unsigned long long* ctl, cudaStream_t st);
 cudaError_t launch_fold(const ChainView& c, cudaStream_t st);
 // JR_FLAG_MALA chain sets: n steps with Langevin local moves (megakernel, one
 // chain per thread, one-warp blocks); F, p and drift of stored states;
@@ -341,7 +341,7 @@ cudaError_t launch_runs_settle(const SceneView& s, const ChainView& c, uint64_t 
 // tail_kernel takes them otherwise.
 cudaError_t launch_runs_tail(const SceneView& s, const ChainView& c, uint64_t step0, uint32_t K, const float4* F,
                              const uint4* queue, unsigned int* ctl, uint32_t* most, cudaStream_t st);
-// As launch_drain with skip = c.wf.done, for few open tours.
+// As launch_drain, for few open tours.
 cudaError_t launch_runs_drain(const SceneView& s, const ChainView& c, uint64_t step_begin, uint32_t n_steps,
                               unsigned long long* ctl, cudaStream_t st);
 

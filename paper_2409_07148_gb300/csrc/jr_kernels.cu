@@ -257,9 +257,8 @@ __global__ void __launch_bounds__(32, 16) step_kernel_spread(SceneView s, ChainV
 // paths and for three launches over all chains; here a chain waits for no other
 // but the few in its warp, so the drain lasts as long as its longest tour.
 template <int kCheck>
-__global__ void __launch_bounds__(32, 16) drain_kernel(SceneView s, ChainView c, const uint8_t* skip,
-                                                       uint64_t step_begin, uint32_t n_steps,
-                                                       unsigned long long* ctl) {
+__global__ void __launch_bounds__(32, 16) drain_kernel(SceneView s, ChainView c, uint64_t step_begin,
+                                                       uint32_t n_steps, unsigned long long* ctl) {
     extern __shared__ float sh[];
     constexpr uint32_t B = 32;
     const int lane = threadIdx.x;
@@ -300,7 +299,7 @@ __global__ void __launch_bounds__(32, 16) drain_kernel(SceneView s, ChainView c,
             if (!live && !drained) {
                 i = base + __popc(want & ((1u << lane) - 1u));
                 drained = i >= c.n;
-                if (!drained && !(skip && skip[i])) {
+                if (!drained && !c.wf.done[i]) {
                     p = c.fpu[3 * c.n + i];
                     step = step_begin;
                     if (!(p > 0.0f)) {  // k = inf: killed at once, nothing to splat
@@ -1074,8 +1073,8 @@ cudaError_t launch_step(const SceneView& s, const ChainView& c, uint64_t step_be
     return e;
 }
 
-cudaError_t launch_drain(const SceneView& s, const ChainView& c, const uint8_t* skip, uint64_t step_begin,
-                         uint32_t n_steps, unsigned long long* ctl, cudaStream_t st) {
+cudaError_t launch_drain(const SceneView& s, const ChainView& c, uint64_t step_begin, uint32_t n_steps,
+                         unsigned long long* ctl, cudaStream_t st) {
     const size_t shm = sizeof(float) * 2 * c.dim * 32;  // <= 8 KB
     cudaError_t e = cudaMemsetAsync(ctl, 0, 2 * sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
@@ -1095,7 +1094,7 @@ cudaError_t launch_drain(const SceneView& s, const ChainView& c, const uint8_t* 
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32, shm);
         if (e != cudaSuccess) return;
         const uint64_t blocks = std::min<uint64_t>((uint64_t)sms * (per_sm > 0 ? per_sm : 1), (c.n + 31) / 32);
-        kernel<<<(unsigned)blocks, 32, shm, st>>>(s, c, skip, step_begin, n_steps, ctl);
+        kernel<<<(unsigned)blocks, 32, shm, st>>>(s, c, step_begin, n_steps, ctl);
         e = cudaGetLastError();
     });
     return e;
