@@ -118,6 +118,37 @@ static uint64_t mh_samples(const jr_chains* c) {
     return c->steps > c->view.burn_in ? (c->steps - c->view.burn_in) * c->view.n : 0;
 }
 
+// Whether a scene of at most kWarpChainMaxTris triangles is a closed surface, which no path
+// leaves: every edge (by the positions of its ends) is walked as often one way as the
+// other.  Each way adds or takes one hash of the edge, so that the sum is 0 then, and
+// otherwise with a chance of 2^-64, which costs speed only.
+static bool closed_surface(const jr_scene_desc* d) {
+    if (d->n_tris == 0 || d->n_tris > kWarpChainMaxTris) return false;
+    const auto point = [&](uint32_t v) {
+        uint64_t h = 0;
+        for (int a = 0; a < 3; ++a) {
+            const float x = d->verts[3 * (size_t)v + a] + 0.0f;  // -0 as 0
+            uint32_t bits;
+            std::memcpy(&bits, &x, sizeof(bits));
+            h = (h ^ bits) * 0x9E3779B97F4A7C15ull;  // splitmix64's constants
+            h ^= h >> 29;
+        }
+        return h;
+    };
+    uint64_t sum = 0;
+    for (uint32_t t = 0; t < d->n_tris; ++t) {
+        const uint32_t* tri = d->tris + 3 * (size_t)t;
+        const uint64_t h[3] = {point(tri[0]), point(tri[1]), point(tri[2])};
+        for (int k = 0; k < 3; ++k) {
+            const uint64_t a = std::min(h[k], h[(k + 1) % 3]), b = std::max(h[k], h[(k + 1) % 3]);
+            uint64_t e = (a ^ (b * 0xBF58476D1CE4E5B9ull)) * 0x94D049BB133111EBull;
+            e ^= e >> 31;
+            if (a != b) sum += h[k] == a ? e : 0 - e;
+        }
+    }
+    return sum == 0;
+}
+
 extern "C" {
 
 const char* jr_last_error(void) { return g_err.c_str(); }
@@ -152,9 +183,11 @@ jr_status jr_scene_create(const jr_scene_desc* desc, void* stream, jr_scene** ou
     }
     HostBvh bvh;
     std::string err;
+    bool closed = false;
     try {
         if (!build_bvh(desc->verts, desc->n_verts, desc->tris, desc->n_tris, desc->tri_material, &bvh, &err))
             return fail(JR_ERR_INVALID_ARG, "jr_scene_create: " + err);
+        closed = closed_surface(desc);
     } catch (const std::bad_alloc&) {
         return fail(JR_ERR_OOM, "jr_scene_create: host allocation failed in the BVH build");
     } catch (const std::exception& ex) {
@@ -187,6 +220,7 @@ jr_status jr_scene_create(const jr_scene_desc* desc, void* stream, jr_scene** ou
     s->view.visit_budget = kNodeVisitBudget;
     s->view.stack_limit = kStackSize;
     s->view.stack_need = bvh.stack_need;
+    s->view.closed = closed;
     std::memcpy(s->view.cam, desc->camera, sizeof(float) * 12);
     s->info.n_tris = desc->n_tris;
     s->info.n_nodes = (uint32_t)bvh.nodes.size();

@@ -72,6 +72,7 @@ struct SceneView {
     uint32_t visit_budget;  // node visits per ray before the watchdog stops it (kNodeVisitBudget)
     int stack_limit;        // traversal stack entries a ray may use (<= kStackSize)
     int stack_need;         // the most entries a traversal of this tree can hold (HostBvh::stack_need)
+    int closed;             // at most kWarpChainMaxTris triangles, and no path can leave them
 };
 
 // The traversal watchdogs that can fire on a view (TravCheck in jr_device.cuh).

@@ -1210,8 +1210,9 @@ cudaError_t launch_eval_states(const SceneView& s, uint32_t depth, float c_tilde
 // In scenes of a few triangles rays are short and alike, so that a warp waits for
 // nobody unless some of its paths leave the scene early and the others go on for long
 // (24-triangle box, depth 2: 54, 63 at 200 000, 318, 327 at 2 10^6; depth 4: 78, 83; 508, 433;
-// depth 8: 118, 109; 835, 541).  Where no path leaves (100 boxes in a room, depth 6: 1 318,
-// 1 398; the 12-triangle furnace: 435, 526) the persistent warps only cost.
+// depth 8: 118, 109; 835, 541).  Where no path can leave (100 boxes in a room, depth 6: 211,
+// 243 at 262 144, 1 318, 1 398 at 2 10^6; the 12-triangle furnace, depth 8: 79, 94; 435, 526) the
+// persistent warps only cost.
 constexpr uint64_t kRenderPersistentMin = 5u << 15, kRenderPersistentMinSmall = 1u << 18;
 constexpr uint32_t kRenderSmallDepth = 4;
 
@@ -1220,7 +1221,8 @@ cudaError_t launch_render_pt(const SceneView& s, uint32_t width, uint32_t height
     if (n == 0) return cudaSuccess;
     cudaError_t e = cudaSuccess;
     const bool small = s.n_tris <= kWarpChainMaxTris;
-    const bool each = small ? n < kRenderPersistentMinSmall || depth < kRenderSmallDepth : n < kRenderPersistentMin;
+    const bool each = small ? s.closed || n < kRenderPersistentMinSmall || depth < kRenderSmallDepth
+                            : n < kRenderPersistentMin;
     with_checks(trav_checks(s), [&](auto k) {
         if (each) {
             const size_t shm = sizeof(float) * (2 + 2 * depth) * 128;
