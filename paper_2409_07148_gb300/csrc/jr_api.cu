@@ -118,6 +118,18 @@ static uint64_t mh_samples(const jr_chains* c) {
     return c->steps > c->view.burn_in ? (c->steps - c->view.burn_in) * c->view.n : 0;
 }
 
+// swizzle_nodes_kernel's moves on the host: chunk c of node i to c ^ (i & 7).  For few
+// nodes, whose launch would be a seventh of the scene's creation.
+constexpr size_t kHostSwizzleNodes = 256;
+static void swizzle_nodes_host(Bvh4Node* nodes, size_t n) {
+    for (size_t i = 0; i < n; ++i) {
+        unsigned char from[sizeof(Bvh4Node)], to[sizeof(Bvh4Node)];
+        std::memcpy(from, nodes + i, sizeof(from));
+        for (size_t c = 0; c < sizeof(Bvh4Node) / 16; ++c) std::memcpy(to + 16 * (c ^ (i & 7)), from + 16 * c, 16);
+        std::memcpy(nodes + i, to, sizeof(to));
+    }
+}
+
 // Whether a scene of at most kWarpChainMaxTris triangles is a closed surface, which no path
 // leaves: every edge (by the positions of its ends) is walked as often one way as the
 // other.  Each way adds or takes one hash of the edge, so that the sum is 0 then, and
@@ -196,13 +208,15 @@ jr_status jr_scene_create(const jr_scene_desc* desc, void* stream, jr_scene** ou
     jr_scene* s = new (std::nothrow) jr_scene();
     if (!s) return fail(JR_ERR_OOM, "jr_scene_create: host allocation failed");
     cudaStream_t st = (cudaStream_t)stream;
+    const bool on_host = bvh.nodes.size() <= kHostSwizzleNodes;
+    if (on_host) swizzle_nodes_host(bvh.nodes.data(), bvh.nodes.size());
     cudaError_t e;
     if ((e = dev_alloc(&s->nodes, bvh.nodes.size())) != cudaSuccess ||
         (e = dev_alloc(&s->tris, bvh.tris.size())) != cudaSuccess ||
         (e = dev_alloc(&s->mats, mats.size())) != cudaSuccess ||
         (e = cudaMemcpyAsync(s->nodes, bvh.nodes.data(), sizeof(Bvh4Node) * bvh.nodes.size(), cudaMemcpyHostToDevice,
                              st)) != cudaSuccess ||
-        (e = launch_swizzle_nodes(s->nodes, (uint32_t)bvh.nodes.size(), st)) != cudaSuccess ||
+        (!on_host && (e = launch_swizzle_nodes(s->nodes, (uint32_t)bvh.nodes.size(), st)) != cudaSuccess) ||
         (e = cudaMemcpyAsync(s->tris, bvh.tris.data(), sizeof(TriRecord) * bvh.tris.size(), cudaMemcpyHostToDevice,
                              st)) != cudaSuccess ||
         (e = cudaMemcpyAsync(s->mats, mats.data(), sizeof(Material) * mats.size(), cudaMemcpyHostToDevice, st)) !=
