@@ -79,8 +79,8 @@ struct jr_chains {
     uint64_t flow_gen = 0;      // bumped whenever the attached flow (or its weight) changes
     uint32_t visit_budget = 0;  // traversal watchdog limits of this set's launches (0: the scene's)
     int stack_limit = 0;
-    AheadView ahead{};          // look-ahead buffers (JR_EXEC_AUTO), and whether they are worth having
-    enum Ahead { kUnknown, kYes, kNo } ahead_use = kUnknown;
+    AheadView ahead{};          // look-ahead buffers (JR_EXEC_AUTO)
+    double ahead_share = -1.0;  // the expected share of local steps (< 0: not read back yet)
     bool ahead_fixed = false;   // a captured graph holds the buffers' addresses: they stay as they are
     // The scene as this set's launches see it (with the set's traversal limits).
     SceneView scene_view() const {
@@ -349,6 +349,21 @@ static jr_status ensure_wavefront(jr_chains* c, cudaStream_t st) {
     return JR_OK;
 }
 
+// The current device's SM count (0 where it cannot be had).
+static uint64_t sm_count() {
+    static DeviceOnce once;
+    long long sms = 0;
+    const cudaError_t e = once.get(
+        [](int dev, long long* v) {
+            int n = 0;
+            const cudaError_t r = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+            *v = n;
+            return r;
+        },
+        &sms);
+    return e == cudaSuccess ? (uint64_t)sms : 0;
+}
+
 // One warp per chain: asked for, or (auto) a small scene with fewer chains
 // than 32 per SM -- while one thread per chain would leave the SMs without
 // even one warp each (measured on the Cornell box and a depth-6 furnace: one
@@ -359,18 +374,7 @@ static bool warp_per_chain(const jr_chains* c) {
     if (c->view.flow.D != 0) return false;
     if (c->exec == JR_EXEC_WARP) return true;
     if (c->exec != JR_EXEC_AUTO || c->scene->view.n_tris > kWarpChainMaxTris) return false;
-    static DeviceOnce once;  // per device: its SM count
-    long long sms = 0;
-    if (once.get(
-            [](int dev, long long* v) {
-                int n = 0;
-                cudaError_t e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-                *v = n;
-                return e;
-            },
-            &sms) != cudaSuccess)
-        return false;
-    return c->view.n < (uint64_t)(32 * sms);
+    return c->view.n < 32 * sm_count();
 }
 
 // Whether JR_EXEC_AUTO runs this advance in look-ahead windows (jr_ahead.cu); sets
@@ -410,7 +414,14 @@ static bool warp_per_chain(const jr_chains* c) {
 // 1.73 1.37 1.18, terrain 1.68 1.39 1.12 1.02, slit caustic 1.09 0.93 0.89 0.94 (1 000 chains
 // 1.04 0.95 0.77 0.80), from 7 000 chains up above 1 everywhere.  A quarter is where the
 // scene that gains least breaks even.
-constexpr double kAheadShare = 0.25;
+//
+// One warp per chain beyond 4 chains per SM (up to there a block per chain takes a
+// window's local steps two or three at a time): a window settled by a warp per chain
+// gains only what its path launch saves, so with less than kAheadShareSteps steps the limit
+// is lower in proportion (24-triangle box, one warp per chain over look-ahead at shares
+// of 0.05, 0.1, 0.15, 0.2: 1 000 chains x 32 steps 1.11 1.02 0.96 0.88, x 48 1.50 1.16 0.99
+// 0.93, x 64 1.77 1.18 1.10 1.04; depth 8, 2 000 x 32 1.28 1.04 0.95 0.81, x 64 above 1).
+constexpr double kAheadShare = 0.25, kAheadShareSteps = 96.0;
 
 // Lets this thread allocate while some other stream of it captures in the global mode.
 struct RelaxedCapture {
@@ -422,15 +433,17 @@ struct RelaxedCapture {
 };
 
 static bool use_ahead(jr_chains* c, uint32_t n_steps, cudaStream_t st) {
-    if (c->exec != JR_EXEC_AUTO || c->view.flow.D != 0 || (c->view.flags & JR_FLAG_MH) ||
-        c->ahead_use == jr_chains::kNo)
-        return false;
+    if (c->exec != JR_EXEC_AUTO || c->view.flow.D != 0 || (c->view.flags & JR_FLAG_MH)) return false;
     const uint64_t n = c->view.n;
     const bool mala = (c->view.flags & JR_FLAG_MALA) != 0;
     const uint32_t least = mala ? (n >= (1u << 17) ? 2 : n >= (1u << 15) ? 4 : n >= (1u << 13) ? 8 : 32)
                                 : n >= (1u << 18) ? 2 : n >= (1u << 16) ? 8 : n >= (1u << 14) ? 16 : 32;
     if (n_steps < least || n > kAheadItems / least) return false;
-    if (c->scene->view.n_tris <= kWarpChainMaxTris && (mala || !warp_per_chain(c))) return false;
+    const bool warp = !mala && warp_per_chain(c);
+    if (c->scene->view.n_tris <= kWarpChainMaxTris && !warp) return false;
+    const double limit =
+        warp && n > 4 * sm_count() ? kAheadShare * std::min(1.0, n_steps / kAheadShareSteps) : kAheadShare;
+    if (c->ahead_share >= limit) return false;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const bool captured = cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
     if (captured) {  // with the buffers an advance outside a capture left, or not at all
@@ -438,26 +451,27 @@ static bool use_ahead(jr_chains* c, uint32_t n_steps, cudaStream_t st) {
         return c->ahead.window != 0;
     }
     RelaxedCapture relaxed;  // another stream of this thread may be capturing
-    if (c->ahead_use == jr_chains::kUnknown) {
+    if (c->ahead_share < 0.0) {
         double sum = 0.0;
         if (cudaMemcpyAsync(&sum, c->view.counters + kCounterMuP, sizeof(sum), cudaMemcpyDeviceToHost, st) !=
                 cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess)
             return false;
-        c->ahead_use = jr_chains::kNo;
         const double p = sum / (double)n;
-        if (!(p / (p + (double)c->view.c_tilde) < kAheadShare)) return false;
-        c->ahead_use = jr_chains::kYes;
+        const double share = p / (p + (double)c->view.c_tilde);
+        c->ahead_share = share >= 0.0 ? share : 1.0;
         // A later advance of fewer steps is the wavefront's, and may be captured: its
         // buffers have to exist by then.
-        if (!mala && n >= kWavefrontMinChains && ensure_wavefront(c, st) != JR_OK) (void)cudaGetLastError();
+        if (c->ahead_share < kAheadShare && !mala && n >= kWavefrontMinChains && ensure_wavefront(c, st) != JR_OK)
+            (void)cudaGetLastError();
+        if (!(c->ahead_share < limit)) return false;
     }
     AheadView& a = c->ahead;
     uint64_t window = least;  // a power of two, so that advances of growing lengths rarely grow it
     while (window < n_steps) window *= 2;
     window = std::min<uint64_t>(window, kAheadItems / n);
     // Two only where a window's tail waits for the next window's paths (launch_ahead).
-    const uint32_t buffers = n_steps > window && !mala && !warp_per_chain(c) ? 2 : 1;
+    const uint32_t buffers = n_steps > window && !mala && !warp ? 2 : 1;
     if (c->ahead_fixed) return a.window != 0;
     if (!a.queue && (dev_alloc(&a.queue, n) != cudaSuccess || dev_alloc(&a.ctl, kCtlCount) != cudaSuccess)) {
         (void)cudaGetLastError();

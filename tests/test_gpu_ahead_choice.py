@@ -44,3 +44,14 @@ def test_many_local_steps_do_not_look_ahead(n):
     ch = jr.Chains(jr.Scene(sc), sc.width, sc.height, sc.depth, n, seed=4, c_tilde=0.02)
     assert not _looks_ahead(ch, 100)
     assert not _looks_ahead(ch, 100)
+
+
+# a share of local steps of about 0.2 (c~ = 0.65): 256 and 608 chains are settled by blocks, 609 and 2000 by a
+# warp each (152 SMs), where it takes more steps for a window to pay
+@pytest.mark.parametrize("n,steps,expected", [(256, 32, True), (608, 32, True), (609, 32, False), (2000, 64, False),
+                                              (609, 96, True), (2000, 96, True)])
+def test_few_steps_of_a_warp_per_chain(n, steps, expected):
+    sc = SCENES["box"]()
+    ch = jr.Chains(jr.Scene(sc), sc.width, sc.height, sc.depth, n, seed=4, c_tilde=0.65)
+    assert _looks_ahead(ch, steps) == expected
+    assert _looks_ahead(ch, 200)  # asked again by every call

@@ -23,7 +23,7 @@ def _advance(scene, sc, n, mode, advances, **kw):
 # of 27 steps).
 @pytest.mark.parametrize("name,n,advances,other,c_tilde", [
     ("box", 256, [3, 33, 64], "warp", 1.0), ("box", 256, [40], "warp", 0.7), ("box", 500, [3, 40], "warp", 1.0),
-    ("box", 2000, [40, 32], "warp", 0.7), ("spheres", 3000, [2, 40], "mega", 0.05),
+    ("box", 2000, [100, 96], "warp", 0.7), ("spheres", 3000, [2, 40], "mega", 0.05),
     ("spheres", 100000, [9, 16], "mega", 0.05), ("spheres", 300000, [60], "wave", 0.05),
 ])
 @pytest.mark.parametrize("flags", [0, RAO])
