@@ -87,7 +87,8 @@ typedef enum {
  * the forward-mode derivative of the path contribution (it flows through the
  * directions and the modified Phong weights; Lambertian and dielectric weights
  * are constant).  MALA is pi-invariant, so MALA Restore keeps k = c~ u / p.
- * Runs in the megakernel only (jr_advance picks it; 128 threads per block); not
+ * Runs in a megakernel of one-warp blocks, and MALA Restore also in look-ahead
+ * windows (jr_advance picks); not
  * with JR_FLAG_RAO_BLACKWELL, flows, drains, batches or jr_advance_static. */
 #define JR_FLAG_MALA 4u
 
@@ -369,9 +370,8 @@ jr_status jr_philox(uint64_t seed, uint32_t tag, uint32_t block, uint64_t chain_
  * (depth + 1) x log2(triangles), longest first.  Or, with JR_BATCH_WAVEFRONT,
  * by shared wavefront launches over all the sets.  Every set advances as
  * jr_advance would advance it on its own (same Philox streams, same
- * per-chain arithmetic; Alg. 2 of Section 7.2 per chain): the same states,
- * with F and p equal up to the rounding of separately compiled kernels (one
- * may contract a multiply-add into an FMA where the other does not).  The sets stay owned
+ * per-chain arithmetic; Alg. 2 of Section 7.2 per chain): the same states, F
+ * and p, bit for bit (where no traversal limit stops a ray).  The sets stay owned
  * by the caller and must outlive the batch; a set may still be advanced,
  * resolved or inspected on its own between batch advances.
  * Sets with a learned regeneration flow attached (jr_chains_set_flow, before or
@@ -526,7 +526,7 @@ jr_status jr_flow_train_rows(jr_flow* flow, const float* x_dev, const float* w_d
  * the chains whose tour is still open after them (0: every tour completed, and
  * the accumulated image is the completed-tour estimator).  Then each chain
  * starts a new tour from mu (Philox tag 3, keyed by a restart count; not a
- * regeneration).  Wavefront mode; synchronises `stream` once per drain step. */
+ * regeneration).  Synchronises `stream`, several times while tours are open. */
 jr_status jr_complete_tours(jr_chains* chains, uint32_t max_steps, uint64_t* remaining, void* stream);
 
 /* Attach a flow (or detach with flow = NULL) with mixture weight beta in

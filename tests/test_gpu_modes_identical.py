@@ -87,3 +87,22 @@ def test_mala_splits_are_bit_identical(name, n, steps):
     rest.set_counters(first.stats(), first.accumulator())
     rest.advance(steps - steps // 3)
     _same(rest, mega)
+
+
+# the batched wavefront and the batch megakernel, every material, over sets of uneven size
+@pytest.mark.parametrize("block", [0, 64])
+@pytest.mark.parametrize("flags", [0, jr.JR_FLAG_MH])
+def test_batches_are_bit_identical(block, flags):
+    scs = [SCENES[name]() for name in ("box", "spheres", "caustic", "glass")]
+    alone, together = [], []
+    for sc, n in zip(scs, (100, 3001, 20000, 700)):
+        scene = jr.Scene(sc)
+        for sets in (alone, together):
+            sets.append(_set(scene, sc, n, c_tilde=0.1, flags=flags, burn_in=0))
+    batch = jr.Batch(together)
+    batch.set_block(block)
+    batch.advance(12)
+    for a, b in zip(alone, together):
+        a.set_execution("mega")
+        a.advance(12)
+        _same(b, a)
