@@ -934,14 +934,15 @@ inline unsigned grid_for(uint64_t n, unsigned b) { return (unsigned)((n + b - 1)
 //
 // MALA: a step's gradient keeps four 3 x D Jacobians per lane in local memory, whose
 // lines a warp with few lanes fills with as few of its chains (1536 D bytes a warp, beside
-// 512 D of shared memory).  So the warps per SM are as many as their lines fit L1 with, and the launch asks
-// for no more shared memory than they take (left alone, the split is made for 16 of
-// them, and L1 has 28 to 90 of its 256 KB): 4 warps, 3 beyond D = 24.  Times of one thread per
-// chain in blocks of 128 over this, and over 12 warps per SM without the request, 2 500 and 10 000
-// chains: Cornell + spheres depth 8 2.3, 1.7 (1.8, 1.2), depth 15 3.0, 2.0 (1.5, 1.2); 2M-triangle
-// terrain's kind 2.2, 1.7 (1.4, 1.2); glass furnace depth 12 2.4, 1.9 (1.2, 0.98); 24-triangle box
-// depth 15 3.2, 2.4 (1.1, 1.0); furnace depth 8 1.5, 1.4 (0.76, 0.75).  Up to kCarveWarps one-warp
-// blocks per SM the request still pays (30 000 chains 1.2, 1.05); beyond it costs.
+// 512 D of shared memory).  So the warps per SM are as many as their lines fit L1 with:
+// 4, or 3 beyond D = 24; and the launch asks for no more shared memory than they take
+// (left alone, the split is made for 16 of them, and L1 has 28 to 90 of its 256 KB).  Gain
+// over one thread per chain in blocks of 128 (in brackets 12 warps per SM, in scenes of at
+// most 128 triangles 4, without the request), 2 500 and 10 000 chains: Cornell + spheres,
+// depth 8, 2.3, 1.7 (1.8, 1.2), depth 15 3.0, 2.0 (1.5, 1.2); 180 000-triangle terrain 2.2, 1.7
+// (1.4, 1.2); glass furnace, depth 12, 2.4, 1.9 (1.2, 0.98); 24-triangle box, depth 15, 3.2, 2.4
+// (1.1, 1.0); furnace, depth 8, 1.5, 1.4 (0.76, 0.75).  Up to kCarveWarps one-warp blocks
+// per SM the request still pays (30 000 chains 1.2, 1.05); beyond it costs.
 constexpr int kSpreadWarps = 12, kSpreadWarpsSmall = 8, kSpreadWarpsMala = 4, kSpreadWarpsMalaDeep = 3, kCarveWarps = 12;
 template <class K>
 cudaError_t chains_per_warp(K kernel, size_t shm, uint64_t n, int most, unsigned* per_warp, long long* sm_count = nullptr) {
